@@ -131,6 +131,7 @@ seg_gather_kernel(const SegGatherArgs a, const HeavyArgs h) {
   if (tile >= a.num_tiles) return;                       // whole groups leave together
   const uint32_t smem = smem_u32(smem_raw) + worker * RingLayout<L, false>::kWorkerBytes;
   const L ln(a.R);
+  if (tile == 0 && ln.g == 0) a.carry_seg[a.num_tiles] = 0;   // no cut run of carries listed yet (carry_fixup_role)
 
   const int64_t total = a.M + a.N;
   const int64_t d0 = tile * a.tile_items;
@@ -204,70 +205,209 @@ __global__ void __launch_bounds__(kBlockThreads) seg_partition_kernel(const int3
   part[t] = (int32_t)merge_path_segments(seg_end, M, N, d);
 }
 
-// Adds the carries onto the stored rows. Tiles that stopped inside the same segment are consecutive;
-// the first of such a run sums the run in tile order and updates the row (the only writer of it now).
-// A heavy segment spans hundreds of tiles, so the run is read eight tiles at a time with all loads in
-// flight together (the additions keep the tile order).
+// Adds the carries onto the stored rows. The tiles that stopped inside one segment are consecutive (a run); the sum of
+// a run is added to the segment's row, which has no other writer by now. One thread per tile and column: the thread at
+// the head of a run adds it up, several tiles in flight. What bounds this is latency, and a run of thousands of tiles
+// (a slice that holds most of a tensor) would be a serial chain: a run of more than kRunShort tiles is therefore added
+// by the whole CTA of its head, and in large problems (cut) runs are cut at every multiple of kRunPiece tiles: a
+// piece's sum stays in the slot of its first tile and carry_runs_kernel adds the pieces, a CTA per run. Every order is
+// fixed. Measured, runs followed by one thread -> as here: 0.85 M entries, R = 4, 60 % of them in one slice 918 -> 84 us
+// (whole CSF MTTKRP); 14.9 M entries, R = 32 3.05 -> 0.40 ms (COO); 100 M entries, heaviest slice 0.5 % 2.90 -> 2.86 ms.
+constexpr int kRunFirst = 4;
+constexpr int kRunShort = kRunFirst + 16;
+constexpr int kRunPiece = 1024;
+
+struct FixupArgs {
+  double *carry_val;
+  const int32_t *carry_seg;
+  int32_t num_tiles;
+  int32_t R, carry_ld;
+  void *C;
+  int64_t ldc;
+  const int32_t *out_row;
+  int32_t *run_count, *run_list;                 // the cut runs (NULL: runs are not cut)
+};
+
 template <class T>
-__device__ __forceinline__ void carry_fixup_role(int64_t block, const double *__restrict__ carry_val,
-                                                 const int32_t *__restrict__ carry_seg, int64_t num_tiles, int32_t R,
-                                                 int32_t carry_ld, T *__restrict__ C, int64_t ldc,
-                                                 const int32_t *__restrict__ out_row) {
-  const int64_t idx = block * blockDim.x + threadIdx.x;
-  const int64_t tile = idx / R;
-  const int32_t c = (int32_t)(idx - tile * R);
-  if (tile >= num_tiles) return;
-  const int32_t seg = carry_seg[tile];
-  if (seg < 0) return;
-  if (tile > 0 && carry_seg[tile - 1] == seg) return;
-  double sum = carry_val[tile * carry_ld + c];
-  bool more = true;
-  for (int64_t t = tile + 1; more; t += 8) {
-    int32_t s[8];
-    double v[8];
+__device__ __forceinline__ void add_to_row(const FixupArgs &f, int32_t seg, int32_t c, double sum) {
+  const int64_t row = f.out_row ? (int64_t)__ldg(f.out_row + seg) : (int64_t)seg;
+  T *const dst = static_cast<T *>(f.C) + row * f.ldc + c;
+  *dst = (T)((double)*dst + sum);
+}
+
+// The sum of the slots first, first + step, ... (count of them), over all threads of the CTA: group g of the 256 / R
+// groups of R threads takes slots g, g + G, ..., the groups' sums are added in group order. Valid for threads below R.
+__device__ __forceinline__ double cta_slot_sum(const FixupArgs &f, int64_t first, int64_t step, int32_t count, double *s_part) {
+  const int32_t G = kBlockThreads / f.R;
+  const int32_t g = threadIdx.x / f.R, c = threadIdx.x - g * f.R;
+  double sum = 0.0;
+  if (g < G) {
+    const double *src = f.carry_val + first * f.carry_ld + c;
+    const int64_t stride = step * f.carry_ld;
+    int32_t q = g;
+    for (; q + 15 * G < count; q += 16 * G) {
+      double v[16];
 #pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      const bool in = t + u < num_tiles;
-      s[u] = in ? __ldg(carry_seg + t + u) : -2;
-      v[u] = in ? __ldcs(carry_val + (t + u) * carry_ld + c) : 0.0;
+      for (int u = 0; u < 16; ++u) v[u] = __ldcs(src + (int64_t)(q + u * G) * stride);
+#pragma unroll
+      for (int u = 0; u < 16; ++u) sum += v[u];
     }
+    for (; q < count; q += G) sum += __ldcs(src + (int64_t)q * stride);
+  }
+  __syncthreads();
+  s_part[threadIdx.x] = sum;
+  __syncthreads();
+  sum = 0.0;
+  if (threadIdx.x < f.R)
+    for (int32_t x = 0; x < G; ++x) sum += s_part[x * f.R + threadIdx.x];
+  return sum;
+}
+
+// `block` of fixup_blocks() CTAs: 256 / R tiles each, R threads per tile. LONG: long runs are possible.
+template <class T, bool LONG>
+__device__ __forceinline__ void carry_fixup_role(const FixupArgs &f, int64_t block) {
+  const int32_t G = kBlockThreads / f.R;         // R is at most 128
+  const int32_t g = threadIdx.x / f.R, c = threadIdx.x - g * f.R;
+  const int32_t tile = (int32_t)block * G + g;
+  const bool cut = LONG && f.run_count != nullptr;
+  bool is_long = false;
+  if (g < G && tile < f.num_tiles) {
+    const int32_t seg_before = tile > 0 ? __ldg(f.carry_seg + tile - 1) : -2;
+    const int32_t seg = __ldg(f.carry_seg + tile);
+    const bool head = seg >= 0 && seg_before != seg;
+    if (head || (seg >= 0 && cut && tile % kRunPiece == 0)) {
+      const int32_t edge = cut ? (tile / kRunPiece + 1) * kRunPiece : f.num_tiles;
+      const int32_t limit = edge < f.num_tiles ? edge : f.num_tiles;       // the run is followed up to here
+      double v0[kRunFirst];
+      int32_t s0[kRunFirst];
 #pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      more = more && s[u] == seg;
-      if (more) sum += v[u];
+      for (int u = 0; u < kRunFirst; ++u) {
+        const bool in = tile + u < limit;
+        s0[u] = in ? __ldg(f.carry_seg + tile + u) : -2;
+        v0[u] = in ? __ldcs(f.carry_val + (int64_t)(tile + u) * f.carry_ld + c) : 0.0;
+      }
+      double sum = v0[0];
+      bool more = true;
+#pragma unroll
+      for (int u = 1; u < kRunFirst; ++u) {
+        more = more && s0[u] == seg;
+        if (more) sum += v0[u];
+      }
+      for (int32_t q = kRunFirst; more && (!LONG || q < kRunShort); q += 8) {
+        int32_t s[8];
+        double v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          const bool in = tile + q + u < limit;
+          s[u] = in ? __ldg(f.carry_seg + tile + q + u) : -2;
+          v[u] = in ? __ldcs(f.carry_val + (int64_t)(tile + q + u) * f.carry_ld + c) : 0.0;
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          more = more && s[u] == seg;
+          if (more) sum += v[u];
+        }
+      }
+      is_long = LONG && more;                    // every thread of the tile sees the same run
+      if (!is_long) {
+        const bool on = cut && edge < f.num_tiles && edge - tile <= kRunShort && __ldg(f.carry_seg + edge - 1) == seg &&
+                        __ldg(f.carry_seg + edge) == seg;
+        if (head && !on) add_to_row<T>(f, seg, c, sum);
+        else f.carry_val[(int64_t)tile * f.carry_ld + c] = sum;
+        if (head && on && c == 0) f.run_list[atomicAdd(f.run_count, 1)] = tile;
+      }
     }
   }
-  const int64_t row = out_row ? (int64_t)out_row[seg] : (int64_t)seg;
-  C[row * ldc + c] = (T)((double)C[row * ldc + c] + sum);
+  if constexpr (LONG) {
+    if (!__syncthreads_or(is_long)) return;
+    __shared__ double s_part[kBlockThreads];
+    __shared__ int32_t s_long[kBlockThreads], s_longs;
+    if (threadIdx.x == 0) s_longs = 0;
+    __syncthreads();
+    if (is_long && c == 0) s_long[atomicAdd(&s_longs, 1)] = tile;
+    __syncthreads();
+    const int32_t longs = s_longs;
+    for (int32_t x = 0; x < longs; ++x) {
+      const int32_t first = s_long[x];
+      const int32_t seg = __ldg(f.carry_seg + first);
+      const int32_t edge = cut ? (first / kRunPiece + 1) * kRunPiece : f.num_tiles;
+      const int32_t limit = edge < f.num_tiles ? edge : f.num_tiles;
+      int32_t count = kRunShort, more;
+      do {
+        const int32_t at = first + count + threadIdx.x;
+        more = __syncthreads_count(at < limit && __ldg(f.carry_seg + at) == seg);
+        count += more;
+      } while (more == kBlockThreads);
+      const double sum = cta_slot_sum(f, first, 1, count, s_part);
+      if (threadIdx.x < f.R) {
+        const bool head = first == 0 || __ldg(f.carry_seg + first - 1) != seg;
+        const bool on = limit < f.num_tiles && first + count == limit && __ldg(f.carry_seg + limit) == seg;
+        if (head && !on) add_to_row<T>(f, seg, threadIdx.x, sum);
+        else f.carry_val[(int64_t)first * f.carry_ld + threadIdx.x] = sum;
+        if (head && on && threadIdx.x == 0) f.run_list[atomicAdd(f.run_count, 1)] = first;
+      }
+      __syncthreads();
+    }
+  }
 }
 
 template <class T>
-__global__ void __launch_bounds__(kBlockThreads) carry_fixup_kernel(const double *__restrict__ carry_val,
-                                                                    const int32_t *__restrict__ carry_seg, int64_t num_tiles,
-                                                                    int32_t R, int32_t carry_ld, T *__restrict__ C, int64_t ldc,
-                                                                    const int32_t *__restrict__ out_row) {
-  carry_fixup_role<T>(blockIdx.x, carry_val, carry_seg, num_tiles, R, carry_ld, C, ldc, out_row);
+__global__ void __launch_bounds__(kBlockThreads) carry_fixup_kernel(const FixupArgs f) {
+  carry_fixup_role<T, true>(f, blockIdx.x);
 }
+
+// The cut runs, a CTA per run (the order of the list does not matter: every run has a row of its own).
+template <class T>
+__global__ void __launch_bounds__(kBlockThreads) carry_runs_kernel(const FixupArgs f) {
+  __shared__ double s_part[kBlockThreads];
+  const int32_t runs = __ldcg(f.run_count);
+  for (int32_t r = blockIdx.x; r < runs; r += gridDim.x) {
+    const int32_t first = f.run_list[r];
+    const int32_t seg = __ldg(f.carry_seg + first);
+    const int32_t second = (first / kRunPiece + 1) * kRunPiece;
+    int32_t pieces = 0, more;                    // behind the first one
+    do {
+      const int64_t at = second + (int64_t)(pieces + threadIdx.x) * kRunPiece;
+      more = __syncthreads_count(at < f.num_tiles && __ldg(f.carry_seg + at) == seg);
+      pieces += more;
+    } while (more == kBlockThreads);
+    const double sum = cta_slot_sum(f, second, kRunPiece, pieces, s_part);
+    if (threadIdx.x < f.R)
+      add_to_row<T>(f, seg, threadIdx.x, __ldcs(f.carry_val + (int64_t)first * f.carry_ld + threadIdx.x) + sum);
+    __syncthreads();
+  }
+}
+
+static int64_t fixup_blocks(int64_t num_tiles, int32_t R) { return ceil_div(num_tiles, kBlockThreads / R); }
 
 // SpMM with the long-row path: both fix-ups in one launch. They read different scratch and write different rows
 // of C (the general tiles leave the long rows out, so no carry names one), so the first `heavy_blocks` CTAs add
-// the long rows' slots while the others add the carries.
+// the long rows' slots while the others add the carries. (Runs are short here: the general tiles' segments are shorter
+// than the long-row threshold.)
 template <class T>
-__global__ void __launch_bounds__(kBlockThreads) spmm_fixups_kernel(const HeavyArgs h, int heavy_blocks,
-                                                                    const double *__restrict__ carry_val,
-                                                                    const int32_t *__restrict__ carry_seg, int64_t num_tiles,
-                                                                    int32_t R, int32_t carry_ld, T *__restrict__ C, int64_t ldc) {
+__global__ void __launch_bounds__(kBlockThreads) spmm_fixups_kernel(const HeavyArgs h, int heavy_blocks, const FixupArgs f) {
   if ((int)blockIdx.x < heavy_blocks) heavy_fixup_role<T>(h, (int)blockIdx.x, heavy_blocks);
-  else carry_fixup_role<T>((int64_t)blockIdx.x - heavy_blocks, carry_val, carry_seg, num_tiles, R, carry_ld, C, ldc, nullptr);
+  else carry_fixup_role<T, false>(f, (int64_t)blockIdx.x - heavy_blocks);
 }
 
-void carry_fixup_launch(int dtype, const double *carry_val, const int32_t *carry_seg, int64_t num_tiles, int32_t R,
-                        int32_t carry_ld, void *C, int64_t ldc, const int32_t *out_row, cudaStream_t stream) {
-  const unsigned blocks = (unsigned)ceil_div(num_tiles * R, 256);
-  if (dtype == COMET_F32)
-    carry_fixup_kernel<float><<<blocks, 256, 0, stream>>>(carry_val, carry_seg, num_tiles, R, carry_ld, (float *)C, ldc, out_row);
-  else
-    carry_fixup_kernel<double><<<blocks, 256, 0, stream>>>(carry_val, carry_seg, num_tiles, R, carry_ld, (double *)C, ldc, out_row);
+int64_t carry_seg_words(int64_t num_tiles) { return num_tiles + 1 + num_tiles / kRunPiece + 1; }
+
+int carry_fixup_launch(int dtype, double *carry_val, int32_t *carry_seg, int64_t num_tiles, int32_t R, int32_t carry_ld,
+                       void *C, int64_t ldc, const int32_t *out_row, bool cut_runs, cudaStream_t stream) {
+  // Runs are cut where one CTA would take too long over the longest possible one (it adds about 4 G carries a second:
+  // 65 us for 2^18) and the second launch (2 to 3 us) is small against the contraction.
+  const bool cut = cut_runs && num_tiles * R > (1ll << 18) && num_tiles > 2 * kRunPiece;
+  const FixupArgs f{carry_val, carry_seg, (int32_t)num_tiles, R, carry_ld, C, ldc, out_row,
+                    cut ? carry_seg + num_tiles : nullptr, cut ? carry_seg + num_tiles + 1 : nullptr};
+  const unsigned blocks = (unsigned)fixup_blocks(num_tiles, R);
+  if (dtype == COMET_F32) carry_fixup_kernel<float><<<blocks, kBlockThreads, 0, stream>>>(f);
+  else carry_fixup_kernel<double><<<blocks, kBlockThreads, 0, stream>>>(f);
+  if (!cut) return 1;
+  const int64_t most = num_tiles / kRunPiece + 1;
+  const unsigned run_blocks = (unsigned)(most < kSmCount ? most : kSmCount);
+  if (dtype == COMET_F32) carry_runs_kernel<float><<<run_blocks, kBlockThreads, 0, stream>>>(f);
+  else carry_runs_kernel<double><<<run_blocks, kBlockThreads, 0, stream>>>(f);
+  return 2;
 }
 
 template <class T>
@@ -322,7 +462,7 @@ template <class T, int LPN, int CPL, int VEC> constexpr bool kHeavyShape =
                               LPN * CPL * VEC * sizeof(T) == 1024) && LPN >= 16;
 
 static size_t carry_bytes(int64_t num_tiles, int32_t carry_ld) {
-  return align_up((size_t)num_tiles * carry_ld * sizeof(double), 256) + align_up((size_t)num_tiles * sizeof(int32_t), 256);
+  return align_up((size_t)num_tiles * carry_ld * sizeof(double), 256) + align_up((size_t)carry_seg_words(num_tiles) * sizeof(int32_t), 256);
 }
 
 // `heavy` (optional): the long-row plan of an SpMM; its scratch precedes the carries of this launch.
@@ -368,9 +508,9 @@ static comet_status_t launch_one(Context *ctx, SegGatherArgs a, HeavyArgs *heavy
       st = launch_mapped<T, LPN, CPL, VEC, false, true>(ctx, a, h, blocks, stream);
       if (st != COMET_OK) return st;
       const int heavy_blocks = kSmCount * 8;
-      const unsigned fix_blocks = (unsigned)(heavy_blocks + ceil_div(a.num_tiles * a.R, kBlockThreads));
-      spmm_fixups_kernel<T><<<fix_blocks, kBlockThreads, 0, stream>>>(h, heavy_blocks, a.carry_val, a.carry_seg, a.num_tiles,
-                                                                     (int32_t)a.R, a.carry_ld, static_cast<T *>(a.C), a.ldc);
+      const unsigned fix_blocks = (unsigned)(heavy_blocks + fixup_blocks(a.num_tiles, a.R));
+      const FixupArgs f{a.carry_val, a.carry_seg, (int32_t)a.num_tiles, a.R, a.carry_ld, a.C, a.ldc, nullptr, nullptr, nullptr};
+      spmm_fixups_kernel<T><<<fix_blocks, kBlockThreads, 0, stream>>>(h, heavy_blocks, f);
       COMET_LAUNCH_CHECK(ctx);
       return COMET_OK;
     }
@@ -378,9 +518,9 @@ static comet_status_t launch_one(Context *ctx, SegGatherArgs a, HeavyArgs *heavy
   st = a.out_row ? launch_mapped<T, LPN, CPL, VEC, true, false>(ctx, a, h, blocks, stream)
                  : launch_mapped<T, LPN, CPL, VEC, false, false>(ctx, a, h, blocks, stream);
   if (st != COMET_OK) return st;
-  carry_fixup_launch(sizeof(T) == 4 ? COMET_F32 : COMET_F64, a.carry_val, a.carry_seg, a.num_tiles, a.R, a.carry_ld, a.C,
-                     a.ldc, a.out_row, stream);
-  COMET_LAUNCH_CHECK(ctx);
+  COMET_LAUNCHED(ctx, carry_fixup_launch(sizeof(T) == 4 ? COMET_F32 : COMET_F64, a.carry_val, a.carry_seg, a.num_tiles, a.R,
+                                         a.carry_ld, a.C, a.ldc, a.out_row, a.out_row == nullptr || a.num_tiles * a.R > (1ll << 20),
+                                         stream));
   return COMET_OK;
 }
 

@@ -123,6 +123,7 @@ __global__ void __launch_bounds__(kBlockThreads, (CPL * VEC * sizeof(T) <= 16 ? 
   using P = CooPolicy<T, LPN, CPL, VEC>;
   const uint32_t smem = smem_u32(smem_raw) + worker * RingLayout<L, true>::kWorkerBytes;
   const L ln(a.R);
+  if (tile == 0 && ln.g == 0) a.carry_seg[a.num_tiles] = 0;   // no cut run of carries listed yet
 
   const int64_t j0 = tile * a.tile_items;
   const int64_t j1 = (j0 + a.tile_items < a.N) ? j0 + a.tile_items : a.N;
@@ -400,6 +401,7 @@ __global__ void __launch_bounds__(kBlockThreads, (CPL * VEC * sizeof(T) <= 16 ? 
   const uint32_t smem = smem_u32(smem_raw) + worker * RingLayout<L, false>::kWorkerBytes;
   const uint32_t flags = smem_u32(smem_raw) + (uint32_t)RingLayout<L, false>::kBlockBytes + worker * kCsfWorkerBytes;
   const L ln(a.R);
+  if (tile == 0 && ln.g == 0) a.carry_seg[a.num_tiles] = 0;   // no cut run of carries listed yet
 
   // A tile is a span of the merge list of fiber-end markers and leaf positions (equal work per tile: an entry
   // costs a gather, a fiber another one). It owns the leaf entries of the span and the fibers whose LAST entry
@@ -441,7 +443,7 @@ static comet_status_t launch_mttkrp(Context *ctx, MttkrpArgs a, cudaStream_t str
   a.num_tiles = ceil_div(total, a.tile_items);
   a.carry_ld = (int32_t)align_up((size_t)a.R, 2);
   const size_t val_bytes = align_up((size_t)a.num_tiles * a.carry_ld * sizeof(double), 256);
-  const size_t seg_bytes = align_up((size_t)a.num_tiles * sizeof(int32_t), 256);
+  const size_t seg_bytes = align_up((size_t)carry_seg_words(a.num_tiles) * sizeof(int32_t), 256);
   const size_t part_bytes = CSF ? align_up((size_t)(a.num_tiles + 1) * sizeof(int32_t), 256) : 0;
   char *scratch = (char *)scratch_get(ctx, val_bytes + seg_bytes + 2 * part_bytes, stream);
   if (!scratch) return COMET_ERR_ALLOC;
@@ -471,9 +473,8 @@ static comet_status_t launch_mttkrp(Context *ctx, MttkrpArgs a, cudaStream_t str
   kernel<<<blocks, kBlockThreads, smem, stream>>>(a);
   COMET_LAUNCH_CHECK(ctx);
   if (CSF && a.level1) return COMET_OK;
-  carry_fixup_launch(sizeof(T) == 4 ? COMET_F32 : COMET_F64, a.carry_val, a.carry_seg, a.num_tiles, a.R, a.carry_ld, a.out,
-                     a.ldo, CSF ? a.crd0 : nullptr, stream);
-  COMET_LAUNCH_CHECK(ctx);
+  COMET_LAUNCHED(ctx, carry_fixup_launch(sizeof(T) == 4 ? COMET_F32 : COMET_F64, a.carry_val, a.carry_seg, a.num_tiles, a.R,
+                                         a.carry_ld, a.out, a.ldo, CSF ? a.crd0 : nullptr, true, stream));
   return COMET_OK;
 }
 

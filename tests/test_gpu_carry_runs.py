@@ -1,0 +1,58 @@
+"""The carry fix-up: segments that span from one tile to thousands of them, with run lengths around 20 tiles (added by
+one thread or by a whole CTA) and around multiples of 1,024 (where runs are cut in large problems). Small tiles are
+forced, so that small inputs reach every case."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from oracle import D, CU, CN, S
+
+pytestmark = pytest.mark.gpu
+
+comet = pytest.importorskip("paper_2102_05187_b200")
+from gpu_util import assert_close, dev, upload_packed  # noqa: E402
+
+TILE = 8                                                     # items per tile: a row of 8 k entries spans about k tiles
+
+
+@pytest.fixture(autouse=True)
+def _need_gpu(cuda_device, monkeypatch):
+    monkeypatch.setenv("COMET_TILE_ITEMS", str(TILE))
+    yield
+
+
+@pytest.mark.parametrize("lengths", [[3, 8 * 18, 0, 8 * 19, 1, 8 * 20 + 5, 8 * 21, 2, 8 * 22],
+                                     [1, 8 * 700, 0, 8 * 64 - 3, 2, 8 * 1030, 8 * 3000]])
+@pytest.mark.parametrize("R", [1, 5, 16, 100])
+def test_spmm_runs(lengths, R):
+    rng = np.random.default_rng(len(lengths) * 100 + R)
+    cols = max(lengths) + 3
+    r = np.repeat(np.arange(len(lengths)), lengths).astype(np.int32)
+    c = np.concatenate([rng.permutation(cols)[:n] for n in lengths]).astype(np.int32)
+    v, B = rng.uniform(-1, 1, r.size), rng.uniform(-1, 1, (cols, R))
+    want, norm = oracle.spmm([r, c], v, (len(lengths), cols), B)
+    A = upload_packed(oracle.pack([r, c], v, (len(lengths), cols), (0, 1), (D, CU)))
+    first = comet.spmm(A, dev(B))
+    assert_close(first, want, norm)
+    assert torch.equal(first, comet.spmm(A, dev(B))), "not reproducible"
+
+
+@pytest.mark.parametrize("attr", [(CU, CU, CU), (CN, S, S)])
+@pytest.mark.parametrize("R,n", [(4, 17000), (33, 180000), (128, 60000)])
+def test_mttkrp_heavy_slice(attr, R, n):
+    """A slice with most of the entries among slices of one entry, of about 21 tiles and of about 1,024 (R = 4: one launch;
+    R = 33 and 128: the runs are cut)."""
+    rng = np.random.default_rng(R)
+    dims = (12, 811, 399)
+    cell = rng.permutation(dims[1] * dims[2])[:n]
+    i = np.full(n, 4)
+    i[:8] = [0, 1, 2, 3, 5, 6, 7, 8]
+    i[8:8 + 160] = 9
+    i[200:200 + 8200] = 10
+    coords = [i.astype(np.int32), (cell // dims[2]).astype(np.int32), (cell % dims[2]).astype(np.int32)]
+    v = rng.uniform(-1, 1, n)
+    F = [None] + [rng.uniform(-1, 1, (d, R)) for d in dims[1:]]
+    want, norm = oracle.mttkrp(coords, v, dims, 0, F)
+    X = upload_packed(oracle.pack(coords, v, dims, (0, 1, 2), attr))
+    assert_close(comet.mttkrp(X, 0, [None, dev(F[1]), dev(F[2])]), want, norm)

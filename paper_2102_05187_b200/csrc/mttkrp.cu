@@ -550,14 +550,16 @@ comet_status_t mttkrp_csf(Context *ctx, int dtype, const int32_t *pos1, const in
 }
 
 // CSF, output mode stored at level 1: out[crd1[f], :] += (sum over fiber f of val * Q[crd2, :]) * P[crd0[slice of f], :].
-// fp64 with 16-byte aligned operands and R a multiple of 2 up to 64; returns COMET_ERR_UNSUPPORTED_FORMAT otherwise
-// (the caller then takes the general scatter kernel). `out` is zero-filled here.
+// fp64 with 16-byte aligned operands and R = 4, 8, 16 or 64; returns COMET_ERR_UNSUPPORTED_FORMAT otherwise (the caller
+// then takes the kernel of mttkrp_level1.cu). `out` is zero-filled here.
 comet_status_t mttkrp_csf_level1(Context *ctx, int dtype, const int32_t *pos1, const int32_t *crd0, const int32_t *crd1,
                                  const int32_t *pos2, const int32_t *crd2, const void *val, int64_t S, int64_t F, int64_t N,
                                  int64_t rows, const void *P, int64_t ldp, const void *Q, int64_t ldq, int64_t R, void *out,
                                  int64_t ldo, cudaStream_t stream) {
-  if (dtype != COMET_F64 || !(R == 2 || R == 4 || R == 8 || R == 16 || R == 32 || R == 64) || N == 0 || S == 0)
-    return COMET_ERR_UNSUPPORTED_FORMAT;
+  // Widths at which a worker of few lanes (or of 32 lanes with two columns each) beats the lane-per-column kernel of
+  // mttkrp_level1.cu, 5 M entries: R = 4 / 8 / 16 / 64 181 / 154 / 193 / 506 us against 217 / 240 / 249 / 520 us; at R = 2
+  // and 32 the other kernel is faster (357 against 213 us; 100 M entries 4.03 against 3.61 ms).
+  if (dtype != COMET_F64 || !(R == 4 || R == 8 || R == 16 || R == 64) || N == 0 || S == 0) return COMET_ERR_UNSUPPORTED_FORMAT;
   if (!aligned16(P) || !aligned16(Q) || !aligned16(out) || ldp % 2 || ldq % 2 || ldo % 2) return COMET_ERR_UNSUPPORTED_FORMAT;
   if (ldp >= (1ll << 28) || ldq >= (1ll << 28)) return COMET_ERR_INDEX_OVERFLOW;
   if (ldo == R) {

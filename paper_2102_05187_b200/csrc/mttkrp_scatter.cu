@@ -9,7 +9,7 @@
 // fp32 tensors the atomics go to a double scratch matrix that is rounded into the output at the end.
 //
 // CSF [CU,CU,CU], coordinates (i, j, k) at levels 0..2, A / B = the factors of the two other modes:
-//   level 1:  out[j, :] += (sum over the fiber's entries of val * B[k, :]) * A[i, :]     one add per fiber
+//   level 1:  out[j, :] += (sum over the fiber's entries of val * B[k, :]) * A[i, :]     one add per fiber (mttkrp_level1.cu)
 //   level 2:  out[k, :] += val * (A[i, :] * B[j, :])                                     one add per entry
 // COO [CN,S,S]:  out[c_out, :] += val * A[c_a, :] * B[c_b, :]                            one add per entry
 //
@@ -38,7 +38,7 @@ struct ScatterArgs {
 
 constexpr int kScatterThreads = 256;
 
-template <class T, int LEVEL, int G>
+template <class T, int G>
 __global__ void __launch_bounds__(kScatterThreads) mttkrp_csf_scatter_kernel(const ScatterArgs a) {
   const T *const val = static_cast<const T *>(a.val);
   const T *const A = static_cast<const T *>(a.A), *const B = static_cast<const T *>(a.B);
@@ -60,16 +60,9 @@ __global__ void __launch_bounds__(kScatterThreads) mttkrp_csf_scatter_kernel(con
     const int64_t i = __ldg(a.crd0 + s), j = __ldg(a.crd1 + f);
     const int64_t p0 = __ldg(a.pos2 + f), p1 = __ldg(a.pos2 + f + 1);
     for (int c = g; c < a.R; c += G) {
-      if (LEVEL == 1) {
-        double t = 0.0;
-        for (int64_t p = p0; p < p1; ++p)
-          t += (double)ld_stream(val + p) * (double)__ldg(B + (int64_t)__ldg(a.crd2 + p) * a.ldb + c);
-        atomicAdd(a.acc + j * a.ldacc + c, t * (double)__ldg(A + i * a.lda + c));
-      } else {
-        const double w = (double)__ldg(A + i * a.lda + c) * (double)__ldg(B + j * a.ldb + c);
-        for (int64_t p = p0; p < p1; ++p)
-          atomicAdd(a.acc + (int64_t)__ldg(a.crd2 + p) * a.ldacc + c, (double)ld_stream(val + p) * w);
-      }
+      const double w = (double)__ldg(A + i * a.lda + c) * (double)__ldg(B + j * a.ldb + c);
+      for (int64_t p = p0; p < p1; ++p)
+        atomicAdd(a.acc + (int64_t)__ldg(a.crd2 + p) * a.ldacc + c, (double)ld_stream(val + p) * w);
     }
   }
 }
@@ -378,8 +371,7 @@ static void launch_scatter(int kind, const ScatterArgs &a, int64_t units, cudaSt
   const int64_t workers = ceil_div(units, a.per_worker);
   const unsigned blocks = (unsigned)ceil_div(workers * G, kScatterThreads);
   if (kind == 0) mttkrp_coo_scatter_kernel<T, G><<<blocks, kScatterThreads, 0, stream>>>(a);
-  else if (kind == 1) mttkrp_csf_scatter_kernel<T, 1, G><<<blocks, kScatterThreads, 0, stream>>>(a);
-  else mttkrp_csf_scatter_kernel<T, 2, G><<<blocks, kScatterThreads, 0, stream>>>(a);
+  else mttkrp_csf_scatter_kernel<T, G><<<blocks, kScatterThreads, 0, stream>>>(a);
 }
 
 template <class T>
@@ -403,11 +395,15 @@ comet_status_t mttkrp_scatter(Context *ctx, int dtype, int kind, const int32_t *
   ScatterArgs a{};
   a.pos1 = pos1; a.crd0 = crd0; a.crd1 = crd1; a.pos2 = pos2; a.crd2 = crd2; a.val = val;
   a.S = S; a.F = F; a.N = N; a.A = A; a.lda = lda; a.B = B; a.ldb = ldb; a.R = (int32_t)R;
+  // CSF, output at level 1: a row add per fiber (mttkrp_level1.cu)
+  const size_t part_bytes = kind == 1 && N > 0 ? mttkrp_level1_bytes(N) : 0;
+  char *part = nullptr;
   if (dtype == COMET_F32) {
     if (rows == 0) return COMET_OK;
     const int64_t n = rows * R;
-    a.acc = (double *)scratch_get(ctx, (size_t)n * sizeof(double), stream);
-    if (!a.acc) return COMET_ERR_ALLOC;
+    part = (char *)scratch_get(ctx, part_bytes + (size_t)n * sizeof(double), stream);
+    if (!part) return COMET_ERR_ALLOC;
+    a.acc = (double *)(part + part_bytes);
     a.ldacc = R;
     zero_acc_kernel<<<(unsigned)ceil_div(n, 256), 256, 0, stream>>>(a.acc, n);
     COMET_LAUNCH_CHECK(ctx);
@@ -416,9 +412,16 @@ comet_status_t mttkrp_scatter(Context *ctx, int dtype, int kind, const int32_t *
     if (st != COMET_OK) return st;
     a.acc = (double *)out;
     a.ldacc = ldo;
+    if (part_bytes && !(part = (char *)scratch_get(ctx, part_bytes, stream))) return COMET_ERR_ALLOC;
   }
   if (N > 0) {
     int done = 0;
+    if (part_bytes) {
+      const comet_status_t st = mttkrp_level1(ctx, dtype, pos1, crd0, crd1, pos2, crd2, val, S, F, N, A, lda, B, ldb, R, a.acc,
+                                              a.ldacc, part, stream);
+      if (st != COMET_OK) return st;
+      done = 1;
+    }
     if (kind == 2 || kind == 0) {                   // one add per entry: the popular output rows go to shared memory
       comet_status_t st = dtype == COMET_F32 ? entries_hot<float>(ctx, a, kind == 0, rows, a_rows, b_rows, &done, stream)
                                               : entries_hot<double>(ctx, a, kind == 0, rows, a_rows, b_rows, &done, stream);

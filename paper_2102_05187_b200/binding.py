@@ -105,12 +105,29 @@ def load_library():
     for name in EXPORTS:
         if name not in ("comet_status_string", "comet_kernel_launches"):
             getattr(lib, name).restype = C.c_int
+    # Declared argument types let the calls below pass plain integers (device addresses among them), which costs a
+    # fraction of wrapping each one in a ctypes object: a call on a small tensor is bound by the host.
+    t, i32, i64, p = C.POINTER(SpTensorStruct), C.c_int32, C.c_int64, C.c_void_p
+    lib.comet_spmv.argtypes = [p, t, p, p, p]
+    lib.comet_spmm.argtypes = [p, t, p, i64, i64, p, i64, p]
+    lib.comet_ttv.argtypes = [p, t, i32, p, t, p]
+    lib.comet_ttm.argtypes = [p, t, i32, p, i64, i64, t, p]
+    lib.comet_ttv_symbolic.argtypes = [p, t, i32, p, p, t]
+    lib.comet_ttm_symbolic_ex.argtypes = [p, t, i32, i64, p, p, t]
+    lib.comet_mttkrp.argtypes = [p, t, i32, p, p, i64, p, i64, p]
+    lib.comet_pack_ex.argtypes = [p, i32, p, i64, p, p, C.c_int, p, p, C.c_uint32, p, t]
+    lib.comet_sptensor_free.argtypes = [p, t, p]
     _lib = lib
     return lib
 
 
 def _stream_ptr():
     return C.c_void_p(torch.cuda.current_stream().cuda_stream)
+
+
+def _raw_stream() -> int:
+    """The current stream's address, without building a torch.cuda.Stream around it."""
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 def _ptr(t):
@@ -124,7 +141,8 @@ def _require_cuda(*tensors):
 
 
 class Handle:
-    """A library handle whose allocator hands out torch CUDA tensors."""
+    """A library handle whose allocator takes its blocks from torch's caching allocator (addresses: no tensor is built
+    around a block that only the library sees)."""
 
     def __init__(self):
         if not torch.cuda.is_available():
@@ -132,16 +150,21 @@ class Handle:
         self.lib = load_library()
         self._live = {}
 
-        def _alloc(_ctx, nbytes, _stream):
+        torch.cuda.init()
+        live = self._live
+        raw_alloc, raw_delete = torch._C._cuda_cudaCachingAllocator_raw_alloc, torch._C._cuda_cudaCachingAllocator_raw_delete
+
+        def _alloc(_ctx, nbytes, stream):
             try:
-                t = torch.empty(max(int(nbytes), 1), dtype=torch.uint8, device="cuda")
+                ptr = raw_alloc(nbytes or 1, stream or 0)
             except Exception:
                 return None
-            self._live[t.data_ptr()] = t
-            return t.data_ptr()
+            live[ptr] = nbytes
+            return ptr
 
         def _free(_ctx, ptr, _stream):
-            self._live.pop(ptr, None)
+            if live.pop(ptr, None) is not None:
+                raw_delete(ptr)
 
         self._alloc_cb = _ALLOC_FN(_alloc)
         self._free_cb = _FREE_FN(_free)
@@ -228,7 +251,7 @@ class SpTensor:
 
     def free(self):
         if self.c.owner:
-            self.handle.lib.comet_sptensor_free(self.handle._h, C.byref(self.c), _stream_ptr())
+            self.handle.lib.comet_sptensor_free(self.handle._h, C.byref(self.c), _raw_stream())
         self._keep = None
 
     def __del__(self):
@@ -270,21 +293,24 @@ class SpTensor:
         return SpTensor(handle, s, keep)
 
 
+class _CudaArray:
+    """n elements of device memory at an address, in the form torch takes; keeps the memory's owner alive."""
+    __slots__ = ("__cuda_array_interface__", "_owner")
+
+
+_TYPESTR = {torch.int32: ("<i4", 4), torch.float64: ("<f8", 8), torch.float32: ("<f4", 4), torch.uint8: ("|u1", 1)}
+
+
 def _from_ptr(ptr, n, dtype, owner):
     """A torch tensor aliasing n elements of device memory at ptr (kept alive by `owner`)."""
     if not ptr or n == 0:
         return torch.zeros(0, dtype=dtype, device="cuda")
-    itemsize = torch.empty(0, dtype=dtype).element_size()
-
-    class _Iface:
-        pass
-
-    iface = _Iface()
-    typestr = {torch.int32: "<i4", torch.float64: "<f8", torch.float32: "<f4", torch.uint8: "|u1"}[dtype]
-    iface.__cuda_array_interface__ = {"shape": (int(n),), "typestr": typestr, "data": (int(ptr), False),
+    typestr, itemsize = _TYPESTR[dtype]
+    array = _CudaArray()
+    array.__cuda_array_interface__ = {"shape": (int(n),), "typestr": typestr, "data": (int(ptr), False),
                                       "version": 3, "strides": (itemsize,)}
-    iface._owner = owner
-    return torch.as_tensor(iface, device="cuda")
+    array._owner = owner
+    return torch.as_tensor(array, device="cuda")
 
 
 # ------------------------------------------------------------------------------------------- entry points
@@ -309,11 +335,9 @@ def pack(coords, val, dims, mode_order, attr, handle: Handle | None = None, sum_
     h_mo = (C.c_int32 * order)(*[int(m) for m in mode_order])
     h_at = (C.c_int32 * order)(*[int(a) for a in attr])
     out = SpTensorStruct()
-    st = handle.lib.comet_pack_ex(handle._h, C.c_int32(order), h_dims, C.c_int64(val.numel()), h_crd, _ptr(val),
-                                  C.c_int(_dtype_code(val)), h_mo, h_at,
-                                  C.c_uint32((PACK_SUM_DUPLICATES if sum_duplicates else 0) | (PACK_CSR_HISTOGRAM if csr_histogram else 0)),
-                                  _stream_ptr(),
-                                  C.byref(out))
+    st = handle.lib.comet_pack_ex(handle._h, order, h_dims, val.numel(), h_crd, val.data_ptr(), _dtype_code(val), h_mo, h_at,
+                                  (PACK_SUM_DUPLICATES if sum_duplicates else 0) | (PACK_CSR_HISTOGRAM if csr_histogram else 0),
+                                  _raw_stream(), C.byref(out))
     handle.check(st, "comet_pack")
     return SpTensor(handle, out)
 
@@ -328,7 +352,7 @@ def spmv(A: SpTensor, x: torch.Tensor, y: torch.Tensor | None = None) -> torch.T
     dt = _same_dtype(A, x, y)
     if y is None:
         y = torch.empty(rows, dtype=dt, device=x.device)
-    st = A.handle.lib.comet_spmv(A.handle._h, C.byref(A.c), _ptr(x), _ptr(y), _stream_ptr())
+    st = A.handle.lib.comet_spmv(A.handle._h, C.byref(A.c), x.data_ptr(), y.data_ptr(), _raw_stream())
     A.handle.check(st, "comet_spmv")
     return y
 
@@ -341,8 +365,8 @@ def spmm(A: SpTensor, B: torch.Tensor, out: torch.Tensor | None = None) -> torch
     dt = _same_dtype(A, B, out)
     if out is None:
         out = torch.empty((rows, R), dtype=dt, device=B.device)
-    st = A.handle.lib.comet_spmm(A.handle._h, C.byref(A.c), _ptr(B), C.c_int64(R), C.c_int64(B.stride(0)),
-                                 _ptr(out), C.c_int64(out.stride(0)), _stream_ptr())
+    st = A.handle.lib.comet_spmm(A.handle._h, C.byref(A.c), B.data_ptr(), R, B.stride(0), out.data_ptr(), out.stride(0),
+                                 _raw_stream())
     A.handle.check(st, "comet_spmm")
     return out
 
@@ -374,7 +398,7 @@ def ttv_symbolic(X: SpTensor, mode: int, out_attr=None) -> SpTensor:
         out_attr = (D, CU) if n == 2 else (CU,) * n
     assert len(out_attr) == n
     h_at = (C.c_int32 * n)(*out_attr)
-    st = X.handle.lib.comet_ttv_symbolic(X.handle._h, C.byref(X.c), C.c_int32(mode), h_at, _stream_ptr(), C.byref(out))
+    st = X.handle.lib.comet_ttv_symbolic(X.handle._h, C.byref(X.c), mode, h_at, _raw_stream(), C.byref(out))
     X.handle.check(st, "comet_ttv_symbolic")
     return SpTensor(X.handle, out)
 
@@ -384,7 +408,7 @@ def ttv(X: SpTensor, mode: int, v: torch.Tensor, Y: SpTensor | None = None) -> S
     _same_dtype(X, v)
     if Y is None:
         Y = ttv_symbolic(X, mode)
-    st = X.handle.lib.comet_ttv(X.handle._h, C.byref(X.c), C.c_int32(mode), _ptr(v), C.byref(Y.c), _stream_ptr())
+    st = X.handle.lib.comet_ttv(X.handle._h, C.byref(X.c), mode, v.data_ptr(), C.byref(Y.c), _raw_stream())
     X.handle.check(st, "comet_ttv")
     return Y
 
@@ -394,8 +418,7 @@ def ttm_symbolic(X: SpTensor, mode: int, R: int, out_attr=None) -> SpTensor:
     (CN, S, D): the mode-generic form with one coordinate pair per stored fiber."""
     out = SpTensorStruct()
     h_at = None if out_attr is None else (C.c_int32 * X.c.order)(*out_attr)
-    st = X.handle.lib.comet_ttm_symbolic_ex(X.handle._h, C.byref(X.c), C.c_int32(mode), C.c_int64(R), h_at,
-                                            _stream_ptr(), C.byref(out))
+    st = X.handle.lib.comet_ttm_symbolic_ex(X.handle._h, C.byref(X.c), mode, R, h_at, _raw_stream(), C.byref(out))
     X.handle.check(st, "comet_ttm_symbolic")
     return SpTensor(X.handle, out)
 
@@ -407,8 +430,7 @@ def ttm(X: SpTensor, mode: int, U: torch.Tensor, Y: SpTensor | None = None) -> S
     _same_dtype(X, U)
     if Y is None:
         Y = ttm_symbolic(X, mode, R)
-    st = X.handle.lib.comet_ttm(X.handle._h, C.byref(X.c), C.c_int32(mode), _ptr(U), C.c_int64(R),
-                                C.c_int64(U.stride(0)), C.byref(Y.c), _stream_ptr())
+    st = X.handle.lib.comet_ttm(X.handle._h, C.byref(X.c), mode, U.data_ptr(), R, U.stride(0), C.byref(Y.c), _raw_stream())
     X.handle.check(st, "comet_ttm")
     return Y
 
@@ -427,8 +449,7 @@ def mttkrp(X: SpTensor, mode: int, factors, out: torch.Tensor | None = None) -> 
     assert len(factors) == order
     h_f = (C.c_void_p * order)(*[0 if (m == mode or f is None) else f.data_ptr() for m, f in enumerate(factors)])
     h_ld = (C.c_int64 * order)(*[0 if (m == mode or f is None) else f.stride(0) for m, f in enumerate(factors)])
-    st = X.handle.lib.comet_mttkrp(X.handle._h, C.byref(X.c), C.c_int32(mode), h_f, h_ld, C.c_int64(R), _ptr(out),
-                                   C.c_int64(out.stride(0)), _stream_ptr())
+    st = X.handle.lib.comet_mttkrp(X.handle._h, C.byref(X.c), mode, h_f, h_ld, R, out.data_ptr(), out.stride(0), _raw_stream())
     X.handle.check(st, "comet_mttkrp")
     return out
 

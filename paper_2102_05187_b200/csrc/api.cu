@@ -75,7 +75,6 @@ __global__ void expand_root_pos_kernel(const int32_t *__restrict__ crd0, const i
   out[i] = pos1[lo];
 }
 
-__global__ void set_word_kernel(int32_t *p, int32_t v) { *p = v; }
 __global__ void set_two_words_kernel(int32_t *p, int32_t v0, int32_t v1) { p[0] = v0; p[1] = v1; }
 
 // Coordinates of every fiber of a 3-level CSF structure: out0[f] = crd0[slice that holds f], out1[f] = crd1[f]
@@ -373,8 +372,40 @@ static const int32_t *stashed_fiber_pos(const comet_sptensor_t *Y, int slot, int
   return Y->crd[COMET_MAX_ORDER - 1];
 }
 
-// Copies X's upper levels (all but the last) into the same levels of Y, device to device.
-static comet_status_t copy_upper_levels(Context *ctx, const comet_sptensor_t *X, comet_sptensor_t *Y, Owner *o,
+// Copies of level arrays and single words, all in one launch: a symbolic call on a small tensor is a handful of arrays of
+// some kilobytes, and a launch or a copy each cost more than the bytes do.
+struct CopyJob {
+  static constexpr int kMost = 2 * COMET_MAX_ORDER;
+  int32_t *dst[kMost];
+  const int32_t *src[kMost];
+  int64_t words[kMost];
+  int jobs;
+  int32_t *word_at;                // a single word to set, or NULL
+  int32_t word;
+};
+__global__ void __launch_bounds__(256) copy_levels_kernel(const CopyJob c) {
+  const int64_t tid = (int64_t)blockIdx.x * 256 + threadIdx.x, threads = (int64_t)gridDim.x * 256;
+#pragma unroll
+  for (int j = 0; j < CopyJob::kMost; ++j)
+    if (j < c.jobs)
+      for (int64_t i = tid; i < c.words[j]; i += threads) c.dst[j][i] = __ldcs(c.src[j] + i);
+  if (tid == 0 && c.word_at) *c.word_at = c.word;
+}
+static void copy_job_add(CopyJob &c, int32_t *dst, const int32_t *src, int64_t words) {
+  if (words <= 0) return;
+  c.dst[c.jobs] = dst; c.src[c.jobs] = src; c.words[c.jobs++] = words;
+}
+static comet_status_t copy_job_run(Context *ctx, const CopyJob &c, cudaStream_t s) {
+  int64_t most = 1;
+  for (int j = 0; j < c.jobs; ++j) if (c.words[j] > most) most = c.words[j];
+  const int64_t blocks = ceil_div(most, 256 * 4) < 16 * kSmCount ? ceil_div(most, 256 * 4) : 16 * kSmCount;
+  copy_levels_kernel<<<(unsigned)blocks, 256, 0, s>>>(c);
+  COMET_LAUNCH_CHECK(ctx);
+  return COMET_OK;
+}
+
+// Allocates X's upper levels (all but the last) as the same levels of Y and notes their copies.
+static comet_status_t copy_upper_levels(Context *ctx, const comet_sptensor_t *X, comet_sptensor_t *Y, Owner *o, CopyJob &c,
                                         cudaStream_t s) {
   for (int l = 0; l < X->order - 1; ++l) {
     Y->pos_len[l] = X->pos_len[l];
@@ -382,10 +413,8 @@ static comet_status_t copy_upper_levels(Context *ctx, const comet_sptensor_t *X,
     Y->pos[l] = (int32_t *)owned_alloc(ctx, o, (size_t)X->pos_len[l] * 4, s);
     Y->crd[l] = (int32_t *)owned_alloc(ctx, o, (size_t)X->crd_len[l] * 4, s);
     if (!Y->pos[l] || !Y->crd[l]) return COMET_ERR_ALLOC;
-    if (X->pos_len[l])
-      COMET_CUDA_TRY(ctx, cudaMemcpyAsync(Y->pos[l], X->pos[l], (size_t)X->pos_len[l] * 4, cudaMemcpyDeviceToDevice, s));
-    if (X->crd_len[l])
-      COMET_CUDA_TRY(ctx, cudaMemcpyAsync(Y->crd[l], X->crd[l], (size_t)X->crd_len[l] * 4, cudaMemcpyDeviceToDevice, s));
+    copy_job_add(c, Y->pos[l], X->pos[l], X->pos_len[l]);
+    copy_job_add(c, Y->crd[l], X->crd[l], X->crd_len[l]);
   }
   return COMET_OK;
 }
@@ -423,8 +452,9 @@ extern "C" comet_status_t comet_ttv_symbolic(comet_handle_t handle, const comet_
   }
   Y->nnz = F;
   st = COMET_OK;
+  CopyJob copies{};
   if (dcsr) {
-    st = copy_upper_levels(ctx, X, Y, o, s);
+    st = copy_upper_levels(ctx, X, Y, o, copies, s);
   } else {
     Y->pos_len[0] = 1; Y->crd_len[0] = 0; Y->pos_len[1] = rows + 1; Y->crd_len[1] = F;
     Y->pos[0] = (int32_t *)owned_alloc(ctx, o, 4, s);
@@ -432,18 +462,18 @@ extern "C" comet_status_t comet_ttv_symbolic(comet_handle_t handle, const comet_
     Y->crd[1] = (int32_t *)owned_alloc(ctx, o, (size_t)F * 4, s);
     if (!Y->pos[0] || !Y->pos[1] || !Y->crd[1]) st = COMET_ERR_ALLOC;
     if (st == COMET_OK) {
-      set_word_kernel<<<1, 1, 0, s>>>(Y->pos[0], (int32_t)rows);
+      copies.word_at = Y->pos[0];
+      copies.word = (int32_t)rows;
+      copy_job_add(copies, Y->crd[1], X->crd[1], F);
       expand_root_pos_kernel<<<(unsigned)ceil_div(rows + 1, 256), 256, 0, s>>>(X->crd[0], X->pos[1], S, rows, Y->pos[1]);
-      ctx->launches += 2;
+      ctx->launches += 1;
       cudaError_t e = cudaGetLastError();
-      if (e == cudaSuccess && F)
-        e = cudaMemcpyAsync(Y->crd[1], X->crd[1], (size_t)F * 4, cudaMemcpyDeviceToDevice, s);
       if (e != cudaSuccess) st = cuda_fail(ctx, e);
     }
   }
   if (st == COMET_OK) {
     Y->val = owned_alloc(ctx, o, (size_t)F * elem_size(X->dtype), s);
-    if (!Y->val) st = COMET_ERR_ALLOC;
+    st = Y->val ? copy_job_run(ctx, copies, s) : COMET_ERR_ALLOC;
   }
   if (from_coo) {
     if (st == COMET_OK) stash_fiber_pos(Y, o, out_order, &view);
@@ -516,6 +546,7 @@ extern "C" comet_status_t comet_ttm_symbolic_ex(comet_handle_t handle, const com
   for (int l = 0; l < last; ++l) Y->attr[l] = COMET_CU;
   Y->attr[last] = COMET_D;
   Y->nnz = F * R;
+  CopyJob copies{};
   if (generic) {
     Y->attr[0] = COMET_CN; Y->attr[1] = COMET_S;
     Y->pos_len[0] = 2; Y->crd_len[0] = F; Y->crd_len[1] = F;
@@ -533,7 +564,7 @@ extern "C" comet_status_t comet_ttm_symbolic_ex(comet_handle_t handle, const com
       if (e != cudaSuccess) st = cuda_fail(ctx, e);
     }
   } else {
-    st = copy_upper_levels(ctx, X, Y, o, s);
+    st = copy_upper_levels(ctx, X, Y, o, copies, s);
   }
   if (st == COMET_OK) {
     Y->pos_len[last] = 1;
@@ -541,10 +572,9 @@ extern "C" comet_status_t comet_ttm_symbolic_ex(comet_handle_t handle, const com
     Y->val = owned_alloc(ctx, o, (size_t)F * R * elem_size(X->dtype), s);
     if (!Y->pos[last] || !Y->val) st = COMET_ERR_ALLOC;
     else {
-      set_word_kernel<<<1, 1, 0, s>>>(Y->pos[last], (int32_t)R);
-      ctx->launches += 1;
-      cudaError_t e = cudaGetLastError();
-      if (e != cudaSuccess) st = cuda_fail(ctx, e);
+      copies.word_at = Y->pos[last];
+      copies.word = (int32_t)R;
+      st = copy_job_run(ctx, copies, s);
     }
   }
   if (from_coo) {

@@ -15,6 +15,7 @@ struct Context {
   comet_allocator_t allocator;            // user allocator or the cudaMalloc fallback
   bool user_allocator;
   int device;
+  int sm_count;                           // SMs for cooperative launches, -1: none; 0: not asked yet
   int last_cuda_error;
   void *scratch;                          // cached scratch, grown on demand
   size_t scratch_bytes;

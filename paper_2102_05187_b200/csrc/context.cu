@@ -73,6 +73,7 @@ extern "C" comet_status_t comet_create(comet_handle_t *handle, const comet_alloc
   if (allocator) ctx->allocator = *allocator;
   else ctx->allocator = comet_allocator_t{comet::default_alloc, comet::default_free, nullptr};
   ctx->device = dev;
+  ctx->sm_count = 0;
   ctx->last_cuda_error = 0;
   ctx->has_last_stream = false;
   ctx->last_stream = nullptr;

@@ -19,6 +19,7 @@
 // No inter-CTA waiting anywhere: every scan is reduce / scan-of-sums / apply in separate launches.
 #include "common.cuh"
 #include "kernels.cuh"
+#include "pack_common.cuh"
 
 #include <stdlib.h>
 #include <string.h>
@@ -36,33 +37,7 @@ constexpr int kScanTile = kScanThreads * kScanItems;
 
 enum { kStatusRange = 0, kStatusDuplicate = 1, kStatusInvalid = 2 };   // words of Context::d_status
 
-struct KeyLayout {
-  int order;
-  int shift[COMET_MAX_ORDER];      // bit position of level l's coordinate inside the key
-  int bits[COMET_MAX_ORDER];
-  int total_bits;
-  int64_t dim[COMET_MAX_ORDER];    // extent of the mode stored at level l
-};
-
-struct CoordPtrs { const int32_t *p[COMET_MAX_ORDER]; };   // level order
-
 // ------------------------------------------------------------------------------------------------ keys
-// ORDER is a template parameter so that the per-level loops unroll and the by-value descriptor structs
-// are read with constant indices (a runtime index would push them into local memory).
-template <int ORDER>
-__device__ __forceinline__ uint64_t entry_key(const CoordPtrs &c, const KeyLayout &k, int64_t p, bool &bad) {
-  int32_t v[ORDER];
-#pragma unroll
-  for (int l = 0; l < ORDER; ++l) v[l] = __ldcs(c.p[l] + p);
-  uint64_t key = 0;
-#pragma unroll
-  for (int l = 0; l < ORDER; ++l) {
-    bad |= (v[l] < 0) | ((int64_t)v[l] >= k.dim[l]);
-    key |= ((uint64_t)(uint32_t)v[l] & ((1ull << k.bits[l]) - 1)) << k.shift[l];
-  }
-  return key;
-}
-
 // Where a sort pass reads its (key, payload) pairs. The payload is one 32-bit word that travels with the key
 // through every pass: a 32-bit value itself (as raw bits; nothing is gathered afterwards), else the entry's index
 // (64-bit values are gathered through it once, at the end: carrying them would cost more per pass than the gather
@@ -101,32 +76,6 @@ __global__ void make_keys_kernel(CooEntries<ORDER> src, int64_t n, uint64_t *__r
 
 // ------------------------------------------------------------------------------------------------ scan
 // Exclusive scan of uint32 in three launches: tile sums, scan of the sums by one CTA, apply.
-__device__ __forceinline__ uint32_t block_exclusive_scan(uint32_t v, uint32_t *s_warp, uint32_t *total) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
-  uint32_t inc = v;
-#pragma unroll
-  for (int off = 1; off < 32; off <<= 1) {
-    const uint32_t t = __shfl_up_sync(0xffffffffu, inc, off);
-    if (lane >= off) inc += t;
-  }
-  if (lane == 31) s_warp[warp] = inc;
-  __syncthreads();
-  if (warp == 0) {
-    uint32_t w = lane < warps ? s_warp[lane] : 0;
-#pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-      const uint32_t t = __shfl_up_sync(0xffffffffu, w, off);
-      if (lane >= off) w += t;
-    }
-    if (lane < warps) s_warp[lane] = w;        // inclusive over warps
-  }
-  __syncthreads();
-  const uint32_t before = warp > 0 ? s_warp[warp - 1] : 0;
-  if (total) *total = s_warp[warps - 1];
-  __syncthreads();
-  return before + inc - v;
-}
-
 __global__ void scan_tile_sums_kernel(const uint32_t *__restrict__ in, int64_t n, uint32_t *__restrict__ sums) {
   __shared__ uint32_t s_warp[32];
   const int64_t base = (int64_t)blockIdx.x * kScanTile;
@@ -397,19 +346,6 @@ __global__ void dup_merge_kernel(const uint64_t *__restrict__ keys, const uint32
 }
 
 // ------------------------------------------------------------------------------------------------ levels
-struct LevelPlan {
-  int order;
-  int attr[COMET_MAX_ORDER];
-  int shift[COMET_MAX_ORDER];
-  int bits[COMET_MAX_ORDER];
-  int counted[COMET_MAX_ORDER];     // index of the level's node counter (-1: positions are entry ranks or dense)
-  int ncounted;
-};
-
-__device__ __forceinline__ bool is_head(uint64_t k, uint64_t kprev, bool first, int shift) {
-  return first || (k >> shift) != (kprev >> shift);
-}
-
 constexpr int kLevelThreads = 256;
 constexpr int kLevelItems = 8;
 constexpr int kLevelTile = kLevelThreads * kLevelItems;
@@ -463,16 +399,41 @@ __global__ void __launch_bounds__(kLevelThreads) level_count_kernel(const uint64
     counts[(int64_t)threadIdx.x * tiles + blockIdx.x] = s_cnt[threadIdx.x];
 }
 
-struct LevelOut {
-  int32_t *pos[COMET_MAX_ORDER];
-  int32_t *crd[COMET_MAX_ORDER];
-  void *val;                   // fp64 or fp32, as the COO values
-  int64_t dim0;                // extent of level 0 (for a dense root)
-  uint32_t nodes[COMET_MAX_ORDER];   // node count of every counted level (indexed by level)
-};
+// Closes the pos arrays: the terminal entry of every compressed level (and the empty tail of a CSR pos).
+template <int ORDER>
+__device__ __forceinline__ void level_finish_role(const uint64_t *__restrict__ keys, int64_t n, const LevelPlan &plan, const LevelOut &out,
+                                                  int64_t tid, int64_t threads) {
+  uint32_t parents = 1;
+#pragma unroll
+  for (int l = 0; l < ORDER; ++l) {
+    const int a = plan.attr[l];
+    const uint32_t nodes = plan.counted[l] >= 0 ? out.nodes[l] : (uint32_t)n;
+    if (a == COMET_D) {
+      if (tid == 0) out.pos[l][0] = (int32_t)out.dim0;
+      parents = (uint32_t)out.dim0;
+    } else if (a == COMET_CU) {
+      if (l == 0) {
+        if (tid == 0) { out.pos[0][0] = 0; out.pos[0][1] = (int32_t)nodes; }
+      } else if (plan.attr[l > 0 ? l - 1 : 0] == COMET_D) {
+        // rows after the last stored one (all rows when the tensor is empty) start at `nodes`
+        const int sh = plan.shift[l > 0 ? l - 1 : 0], bt = plan.bits[l > 0 ? l - 1 : 0];
+        const int64_t last = n > 0 ? (int64_t)((keys[n - 1] >> sh) & ((1ull << bt) - 1)) : -1;
+        for (int64_t r = last + 1 + tid; r <= (int64_t)out.dim0; r += threads)
+          out.pos[l][r] = (int32_t)nodes;
+      } else if (tid == 0) {
+        out.pos[l][parents] = (int32_t)nodes;
+      }
+      parents = nodes;
+    } else if (a == COMET_CN) {
+      if (tid == 0) { out.pos[l][0] = 0; out.pos[l][1] = (int32_t)n; }
+      parents = (uint32_t)n;
+    }
+  }
+}
 
 // Per tile: ranks of the heads (tile-local scan + the tile's scanned offset), then crd / pos / val. GATHER: the
 // values are the caller's, read through the sorted payload (entry indices); else they are in sorted order already.
+// The CTAs behind the tiles close the pos arrays (a launch of its own otherwise).
 template <int ORDER, class V, bool GATHER>
 __global__ void __launch_bounds__(kLevelThreads) level_emit_kernel(const uint64_t *__restrict__ keys,
                                                                    const uint32_t *__restrict__ perm,
@@ -481,6 +442,11 @@ __global__ void __launch_bounds__(kLevelThreads) level_emit_kernel(const uint64_
                                                                    const uint32_t *__restrict__ offsets,
                                                                    LevelOut out) {
   __shared__ uint32_t s_warp[32];
+  if ((int64_t)blockIdx.x >= tiles) {
+    level_finish_role<ORDER>(keys, n, plan, out, ((int64_t)blockIdx.x - tiles) * kLevelThreads + threadIdx.x,
+                             ((int64_t)gridDim.x - tiles) * kLevelThreads);
+    return;
+  }
   const int64_t base = (int64_t)blockIdx.x * kLevelTile + (int64_t)threadIdx.x * kLevelItems;   // blocked: 8 consecutive
   uint64_t k[kLevelItems + 1];
   V vals[kLevelItems];
@@ -559,38 +525,6 @@ __global__ void __launch_bounds__(kLevelThreads) level_emit_kernel(const uint64_
         }
       }
       static_cast<V *>(out.val)[p] = vals[t];
-    }
-  }
-}
-
-// Closes the pos arrays: the terminal entry of every compressed level (and the empty tail of a CSR pos).
-template <int ORDER>
-__global__ void level_finish_kernel(const uint64_t *__restrict__ keys, int64_t n, LevelPlan plan, LevelOut out) {
-  const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  uint32_t parents = 1;
-#pragma unroll
-  for (int l = 0; l < ORDER; ++l) {
-    const int a = plan.attr[l];
-    const uint32_t nodes = plan.counted[l] >= 0 ? out.nodes[l] : (uint32_t)n;
-    if (a == COMET_D) {
-      if (tid == 0) out.pos[l][0] = (int32_t)out.dim0;
-      parents = (uint32_t)out.dim0;
-    } else if (a == COMET_CU) {
-      if (l == 0) {
-        if (tid == 0) { out.pos[0][0] = 0; out.pos[0][1] = (int32_t)nodes; }
-      } else if (plan.attr[l > 0 ? l - 1 : 0] == COMET_D) {
-        // rows after the last stored one (all rows when the tensor is empty) start at `nodes`
-        const int sh = plan.shift[l > 0 ? l - 1 : 0], bt = plan.bits[l > 0 ? l - 1 : 0];
-        const int64_t last = n > 0 ? (int64_t)((keys[n - 1] >> sh) & ((1ull << bt) - 1)) : -1;
-        for (int64_t r = last + 1 + tid; r <= (int64_t)out.dim0; r += (int64_t)gridDim.x * blockDim.x)
-          out.pos[l][r] = (int32_t)nodes;
-      } else if (tid == 0) {
-        out.pos[l][parents] = (int32_t)nodes;
-      }
-      parents = nodes;
-    } else if (a == COMET_CN) {
-      if (tid == 0) { out.pos[l][0] = 0; out.pos[l][1] = (int32_t)n; }
-      parents = (uint32_t)n;
     }
   }
 }
@@ -781,72 +715,87 @@ extern "C" comet_status_t comet_pack_ex(comet_handle_t handle, int32_t order, co
   const int64_t counts_len = (int64_t)COMET_MAX_ORDER * level_tiles;
 
   TempBlocks tmp(ctx, s);
-  uint64_t *keys_a = (uint64_t *)tmp.get((size_t)(n + 1) * 8);
-  uint64_t *keys_b = (uint64_t *)tmp.get((size_t)(n + 1) * 8);
-  uint32_t *pay_a = (uint32_t *)tmp.get((size_t)(n + 1) * 4);   // fp32 values as raw bits, else entry indices
-  uint32_t *pay_b = (uint32_t *)tmp.get((size_t)(n + 1) * 4);
-  const int64_t table_words = table_len > counts_len ? table_len : counts_len;
-  uint32_t *table = (uint32_t *)tmp.get((size_t)table_words * 4);
-  uint32_t *scan_tmp = (uint32_t *)tmp.get((size_t)(ceil_div(table_words, kScanTile) + 1) * 4);
-  if (!keys_a || !keys_b || !pay_a || !pay_b || !table || !scan_tmp) return COMET_ERR_ALLOC;
-
-  COMET_CUDA_TRY(ctx, cudaMemsetAsync(ctx->d_status, 0, 16 * sizeof(int32_t), s));
-  uint32_t *d_nodes = reinterpret_cast<uint32_t *>(ctx->d_status) + 8;   // node counts live beside the status words
-
+  uint64_t *keys_a = nullptr;
+  uint32_t *pay_a = nullptr;           // fp32 values as raw bits, else entry indices
+  uint32_t *table = nullptr;           // digit counts during the sort, then the scanned node counts per tile and level
   const void *sorted_val = nullptr;    // the values in sorted order, once some array holds them so
-  if (n > 0) {
-    {
-      const uint32_t *val32 = dtype == COMET_F32 ? static_cast<const uint32_t *>(coo_val) : nullptr;
-      comet_status_t st;
-      if (order == 2) st = sort_entries<2>(ctx, coords, key, val32, keys_a, keys_b, pay_a, pay_b, n, table, scan_tmp, s);
-      else if (order == 3) st = sort_entries<3>(ctx, coords, key, val32, keys_a, keys_b, pay_a, pay_b, n, table, scan_tmp, s);
-      else st = sort_entries<4>(ctx, coords, key, val32, keys_a, keys_b, pay_a, pay_b, n, table, scan_tmp, s);
-      if (st != COMET_OK) return st;
-      if (dtype == COMET_F32) sorted_val = pay_a;
-    }
-    if (flags & COMET_PACK_SUM_DUPLICATES) {
-      // merge runs of equal keys; costs one more synchronisation (the number of distinct cells sizes the rest)
-      uint32_t *rank = (uint32_t *)tmp.get((size_t)n * 4);
-      void *merged = tmp.get((size_t)n * (dtype == COMET_F32 ? 4 : 8));
-      if (!rank || !merged) return COMET_ERR_ALLOC;
-      uint32_t *d_distinct = reinterpret_cast<uint32_t *>(ctx->d_status) + 12;
-      dup_heads_kernel<<<(unsigned)ceil_div(n, 256), 256, 0, s>>>(keys_a, n, rank);
+  if (!(flags & COMET_PACK_SUM_DUPLICATES) && pack_small_applies(ctx, order, total_bits, n)) {
+    char *block = (char *)tmp.get(pack_small_bytes(order, n));
+    if (!block) return COMET_ERR_ALLOC;
+    PackSmallSorted sorted;
+    const comet_status_t st = pack_small_sort(ctx, order, coords, key, plan,
+                                              dtype == COMET_F32 ? static_cast<const uint32_t *>(coo_val) : nullptr, n, block,
+                                              &sorted, s);
+    if (st != COMET_OK) return st;
+    keys_a = sorted.keys; pay_a = sorted.pay; table = sorted.counts;
+    if (dtype == COMET_F32) sorted_val = pay_a;
+  } else {
+    keys_a = (uint64_t *)tmp.get((size_t)(n + 1) * 8);
+    uint64_t *keys_b = (uint64_t *)tmp.get((size_t)(n + 1) * 8);
+    pay_a = (uint32_t *)tmp.get((size_t)(n + 1) * 4);
+    uint32_t *pay_b = (uint32_t *)tmp.get((size_t)(n + 1) * 4);
+    const int64_t table_words = table_len > counts_len ? table_len : counts_len;
+    table = (uint32_t *)tmp.get((size_t)table_words * 4);
+    uint32_t *scan_tmp = (uint32_t *)tmp.get((size_t)(ceil_div(table_words, kScanTile) + 1) * 4);
+    if (!keys_a || !keys_b || !pay_a || !pay_b || !table || !scan_tmp) return COMET_ERR_ALLOC;
+
+    COMET_CUDA_TRY(ctx, cudaMemsetAsync(ctx->d_status, 0, 16 * sizeof(int32_t), s));
+    uint32_t *d_nodes = reinterpret_cast<uint32_t *>(ctx->d_status) + 8;   // node counts live beside the status words
+
+    if (n > 0) {
+      {
+        const uint32_t *val32 = dtype == COMET_F32 ? static_cast<const uint32_t *>(coo_val) : nullptr;
+        comet_status_t st;
+        if (order == 2) st = sort_entries<2>(ctx, coords, key, val32, keys_a, keys_b, pay_a, pay_b, n, table, scan_tmp, s);
+        else if (order == 3) st = sort_entries<3>(ctx, coords, key, val32, keys_a, keys_b, pay_a, pay_b, n, table, scan_tmp, s);
+        else st = sort_entries<4>(ctx, coords, key, val32, keys_a, keys_b, pay_a, pay_b, n, table, scan_tmp, s);
+        if (st != COMET_OK) return st;
+        if (dtype == COMET_F32) sorted_val = pay_a;
+      }
+      if (flags & COMET_PACK_SUM_DUPLICATES) {
+        // merge runs of equal keys; costs one more synchronisation (the number of distinct cells sizes the rest)
+        uint32_t *rank = (uint32_t *)tmp.get((size_t)n * 4);
+        void *merged = tmp.get((size_t)n * (dtype == COMET_F32 ? 4 : 8));
+        if (!rank || !merged) return COMET_ERR_ALLOC;
+        uint32_t *d_distinct = reinterpret_cast<uint32_t *>(ctx->d_status) + 12;
+        dup_heads_kernel<<<(unsigned)ceil_div(n, 256), 256, 0, s>>>(keys_a, n, rank);
+        COMET_LAUNCH_CHECK(ctx);
+        uint32_t *rank_tmp = (uint32_t *)keys_b;                 // free until the merge writes it
+        comet_status_t st = exclusive_scan(ctx, rank, rank, n, rank_tmp, d_distinct, s);
+        if (st != COMET_OK) return st;
+        COMET_CUDA_TRY(ctx, cudaMemcpyAsync(ctx->h_pinned, ctx->d_status, 16 * sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+        COMET_CUDA_TRY(ctx, cudaStreamSynchronize(s));
+        if (ctx->h_pinned[kStatusRange]) return COMET_ERR_COORD_OUT_OF_RANGE;
+        const int64_t distinct = reinterpret_cast<uint32_t *>(ctx->h_pinned)[12];
+        // keys_b is both the scan's scratch and the merge's output: the scan has finished (synchronised above)
+        if (dtype == COMET_F32)
+          dup_merge_kernel<float, false><<<(unsigned)ceil_div(n, 256), 256, 0, s>>>(keys_a, nullptr, (const float *)sorted_val, n, rank,
+                                                                                   keys_b, (float *)merged);
+        else
+          dup_merge_kernel<double, true><<<(unsigned)ceil_div(n, 256), 256, 0, s>>>(keys_a, pay_a, (const double *)coo_val, n, rank,
+                                                                                   keys_b, (double *)merged);
+        COMET_LAUNCH_CHECK(ctx);
+        keys_a = keys_b;
+        sorted_val = merged;
+        n = distinct;
+        level_tiles = ceil_div(n > 0 ? n : 1, kLevelTile);
+      }
+      // node counts of the counted levels: per-tile counts -> scanned offsets (kept in `table`) + totals
+      if (order == 2) level_count_kernel<2><<<(unsigned)level_tiles, kLevelThreads, 0, s>>>(keys_a, n, plan, level_tiles, table, ctx->d_status);
+      else if (order == 3) level_count_kernel<3><<<(unsigned)level_tiles, kLevelThreads, 0, s>>>(keys_a, n, plan, level_tiles, table, ctx->d_status);
+      else level_count_kernel<4><<<(unsigned)level_tiles, kLevelThreads, 0, s>>>(keys_a, n, plan, level_tiles, table, ctx->d_status);
       COMET_LAUNCH_CHECK(ctx);
-      uint32_t *rank_tmp = (uint32_t *)keys_b;                 // free until the merge writes it
-      comet_status_t st = exclusive_scan(ctx, rank, rank, n, rank_tmp, d_distinct, s);
-      if (st != COMET_OK) return st;
-      COMET_CUDA_TRY(ctx, cudaMemcpyAsync(ctx->h_pinned, ctx->d_status, 16 * sizeof(int32_t), cudaMemcpyDeviceToHost, s));
-      COMET_CUDA_TRY(ctx, cudaStreamSynchronize(s));
-      if (ctx->h_pinned[kStatusRange]) return COMET_ERR_COORD_OUT_OF_RANGE;
-      const int64_t distinct = reinterpret_cast<uint32_t *>(ctx->h_pinned)[12];
-      // keys_b is both the scan's scratch and the merge's output: the scan has finished (synchronised above)
-      if (dtype == COMET_F32)
-        dup_merge_kernel<float, false><<<(unsigned)ceil_div(n, 256), 256, 0, s>>>(keys_a, nullptr, (const float *)sorted_val, n, rank,
-                                                                                 keys_b, (float *)merged);
-      else
-        dup_merge_kernel<double, true><<<(unsigned)ceil_div(n, 256), 256, 0, s>>>(keys_a, pay_a, (const double *)coo_val, n, rank,
-                                                                                 keys_b, (double *)merged);
-      COMET_LAUNCH_CHECK(ctx);
-      keys_a = keys_b;
-      sorted_val = merged;
-      n = distinct;
-      level_tiles = ceil_div(n > 0 ? n : 1, kLevelTile);
+      for (int l = 0; l < order; ++l) {
+        if (plan.counted[l] < 0) continue;
+        comet_status_t st = exclusive_scan(ctx, table + (int64_t)l * level_tiles, table + (int64_t)l * level_tiles,
+                                           level_tiles, scan_tmp, d_nodes + l, s);
+        if (st != COMET_OK) return st;
+      }
     }
-    // node counts of the counted levels: per-tile counts -> scanned offsets (kept in `table`) + totals
-    if (order == 2) level_count_kernel<2><<<(unsigned)level_tiles, kLevelThreads, 0, s>>>(keys_a, n, plan, level_tiles, table, ctx->d_status);
-    else if (order == 3) level_count_kernel<3><<<(unsigned)level_tiles, kLevelThreads, 0, s>>>(keys_a, n, plan, level_tiles, table, ctx->d_status);
-    else level_count_kernel<4><<<(unsigned)level_tiles, kLevelThreads, 0, s>>>(keys_a, n, plan, level_tiles, table, ctx->d_status);
-    COMET_LAUNCH_CHECK(ctx);
-    for (int l = 0; l < order; ++l) {
-      if (plan.counted[l] < 0) continue;
-      comet_status_t st = exclusive_scan(ctx, table + (int64_t)l * level_tiles, table + (int64_t)l * level_tiles,
-                                         level_tiles, scan_tmp, d_nodes + l, s);
-      if (st != COMET_OK) return st;
-    }
+    // the one synchronisation: status words and node counts
+    COMET_CUDA_TRY(ctx, cudaMemcpyAsync(ctx->h_pinned, ctx->d_status, 16 * sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+    COMET_CUDA_TRY(ctx, cudaStreamSynchronize(s));
   }
-  // the one synchronisation: status words and node counts
-  COMET_CUDA_TRY(ctx, cudaMemcpyAsync(ctx->h_pinned, ctx->d_status, 16 * sizeof(int32_t), cudaMemcpyDeviceToHost, s));
-  COMET_CUDA_TRY(ctx, cudaStreamSynchronize(s));
   if (ctx->h_pinned[kStatusRange]) return COMET_ERR_COORD_OUT_OF_RANGE;
   if (ctx->h_pinned[kStatusDuplicate]) return COMET_ERR_DUPLICATE_COORD;
 
@@ -883,29 +832,28 @@ extern "C" comet_status_t comet_pack_ex(comet_handle_t handle, int32_t order, co
   lo.dim0 = key.dim[0];
   if (!alloc_ok) { owner_release(ctx, owner, s); memset(out, 0, sizeof(*out)); return COMET_ERR_ALLOC; }
 
-  if (n > 0) {
-    const unsigned g = (unsigned)level_tiles;
+  // An empty tensor has no tiles: only the closing role runs. A dense root may have a long empty tail to write.
+  const int64_t emit_tiles = n > 0 ? level_tiles : 0;
+  const unsigned g = (unsigned)(emit_tiles + (h_attr[0] == COMET_D ? kSmCount : 1));
+  {
     if (dtype == COMET_F32) {
       const float *vin = (const float *)sorted_val;
-      if (order == 2) level_emit_kernel<2, float, false><<<g, kLevelThreads, 0, s>>>(keys_a, nullptr, vin, n, plan, level_tiles, table, lo);
-      else if (order == 3) level_emit_kernel<3, float, false><<<g, kLevelThreads, 0, s>>>(keys_a, nullptr, vin, n, plan, level_tiles, table, lo);
-      else level_emit_kernel<4, float, false><<<g, kLevelThreads, 0, s>>>(keys_a, nullptr, vin, n, plan, level_tiles, table, lo);
+      if (order == 2) level_emit_kernel<2, float, false><<<g, kLevelThreads, 0, s>>>(keys_a, nullptr, vin, n, plan, emit_tiles, table, lo);
+      else if (order == 3) level_emit_kernel<3, float, false><<<g, kLevelThreads, 0, s>>>(keys_a, nullptr, vin, n, plan, emit_tiles, table, lo);
+      else level_emit_kernel<4, float, false><<<g, kLevelThreads, 0, s>>>(keys_a, nullptr, vin, n, plan, emit_tiles, table, lo);
     } else if (sorted_val) {
       const double *vin = (const double *)sorted_val;
-      if (order == 2) level_emit_kernel<2, double, false><<<g, kLevelThreads, 0, s>>>(keys_a, nullptr, vin, n, plan, level_tiles, table, lo);
-      else if (order == 3) level_emit_kernel<3, double, false><<<g, kLevelThreads, 0, s>>>(keys_a, nullptr, vin, n, plan, level_tiles, table, lo);
-      else level_emit_kernel<4, double, false><<<g, kLevelThreads, 0, s>>>(keys_a, nullptr, vin, n, plan, level_tiles, table, lo);
+      if (order == 2) level_emit_kernel<2, double, false><<<g, kLevelThreads, 0, s>>>(keys_a, nullptr, vin, n, plan, emit_tiles, table, lo);
+      else if (order == 3) level_emit_kernel<3, double, false><<<g, kLevelThreads, 0, s>>>(keys_a, nullptr, vin, n, plan, emit_tiles, table, lo);
+      else level_emit_kernel<4, double, false><<<g, kLevelThreads, 0, s>>>(keys_a, nullptr, vin, n, plan, emit_tiles, table, lo);
     } else {
       const double *vin = (const double *)coo_val;
-      if (order == 2) level_emit_kernel<2, double, true><<<g, kLevelThreads, 0, s>>>(keys_a, pay_a, vin, n, plan, level_tiles, table, lo);
-      else if (order == 3) level_emit_kernel<3, double, true><<<g, kLevelThreads, 0, s>>>(keys_a, pay_a, vin, n, plan, level_tiles, table, lo);
-      else level_emit_kernel<4, double, true><<<g, kLevelThreads, 0, s>>>(keys_a, pay_a, vin, n, plan, level_tiles, table, lo);
+      if (order == 2) level_emit_kernel<2, double, true><<<g, kLevelThreads, 0, s>>>(keys_a, pay_a, vin, n, plan, emit_tiles, table, lo);
+      else if (order == 3) level_emit_kernel<3, double, true><<<g, kLevelThreads, 0, s>>>(keys_a, pay_a, vin, n, plan, emit_tiles, table, lo);
+      else level_emit_kernel<4, double, true><<<g, kLevelThreads, 0, s>>>(keys_a, pay_a, vin, n, plan, emit_tiles, table, lo);
     }
   }
-  if (order == 2) level_finish_kernel<2><<<kSmCount, 256, 0, s>>>(keys_a, n, plan, lo);
-  else if (order == 3) level_finish_kernel<3><<<kSmCount, 256, 0, s>>>(keys_a, n, plan, lo);
-  else level_finish_kernel<4><<<kSmCount, 256, 0, s>>>(keys_a, n, plan, lo);
-  ctx->launches += n > 0 ? 2 : 1;
+  ctx->launches += 1;
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) { owner_release(ctx, owner, s); memset(out, 0, sizeof(*out)); return cuda_fail(ctx, e); }
   out->owner = owner;

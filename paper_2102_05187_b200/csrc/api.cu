@@ -186,18 +186,18 @@ extern "C" comet_status_t comet_spmm(comet_handle_t handle, const comet_sptensor
   const int64_t rows = A->dims[A->mode_order[0]];
   if (is_fmt(A, 2, COMET_D, COMET_CU))
     return seg_gather(ctx, A->dtype, A->pos[1] + 1, A->crd[1], A->val, rows, A->nnz, B, ldb, R, C, ldc, nullptr, rows,
-                      A->dims[A->mode_order[1]], s);
+                      A->dims[A->mode_order[1]], true, s);
   if (is_fmt(A, 2, COMET_CU, COMET_CU)) {
     if (A->crd_len[0] == 0) return zero_rows(ctx, C, A->dtype, rows, R, ldc, s);
     return seg_gather(ctx, A->dtype, A->pos[1] + 1, A->crd[1], A->val, A->crd_len[0], A->nnz, B, ldb, R, C, ldc, A->crd[0],
-                      rows, 0, s);
+                      rows, A->dims[A->mode_order[1]], false, s);
   }
   if (is_fmt(A, 2, COMET_CN, COMET_S)) {
     int32_t *pos = nullptr;
     st = coo_rows(ctx, A, rows, s, &pos);
     if (st != COMET_OK) return st;
     st = seg_gather(ctx, A->dtype, pos + 1, A->crd[1], A->val, rows, A->nnz, B, ldb, R, C, ldc, nullptr, rows,
-                    A->dims[A->mode_order[1]], s);
+                    A->dims[A->mode_order[1]], true, s);
     ctx_free(ctx, pos, s);
     return st;
   }
@@ -601,8 +601,8 @@ extern "C" comet_status_t comet_ttm(comet_handle_t handle, const comet_sptensor_
   if (Y->dtype != X->dtype) return COMET_ERR_INVALID_ARG;
   if (misaligned(U, X->dtype)) return COMET_ERR_MISALIGNED;
   Context *ctx = reinterpret_cast<Context *>(handle);
-  return seg_gather(ctx, X->dtype, fiber_pos + 1, X->crd[last], X->val, F, X->nnz, U, ldu, R, Y->val, R, nullptr, F, 0,
-                    (cudaStream_t)stream);
+  return seg_gather(ctx, X->dtype, fiber_pos + 1, X->crd[last], X->val, F, X->nnz, U, ldu, R, Y->val, R, nullptr, F, X->dims[mode],
+                    false, (cudaStream_t)stream);
 }
 
 // ------------------------------------------------------------------------------------------ element-wise
@@ -701,10 +701,10 @@ extern "C" comet_status_t comet_mttkrp(comet_handle_t handle, const comet_sptens
                           out, ldo, s);
   }
   if (coo)
-    return mttkrp_coo(ctx, X->dtype, X->crd[0], X->crd[1], X->crd[2], X->val, X->nnz, rows, P, h_ld[m1], Q, h_ld[m2], R, out,
-                      ldo, s);
+    return mttkrp_coo(ctx, X->dtype, X->crd[0], X->crd[1], X->crd[2], X->val, X->nnz, rows, P, X->dims[m1], h_ld[m1], Q,
+                      X->dims[m2], h_ld[m2], R, out, ldo, s);
   if (csf)
     return mttkrp_csf(ctx, X->dtype, X->pos[1], X->crd[0], X->crd[1], X->pos[2], X->crd[2], X->val, X->crd_len[0],
-                      X->crd_len[1], X->nnz, rows, P, h_ld[m1], Q, h_ld[m2], R, out, ldo, s);
+                      X->crd_len[1], X->nnz, rows, P, X->dims[m1], h_ld[m1], Q, X->dims[m2], h_ld[m2], R, out, ldo, s);
   return COMET_ERR_UNSUPPORTED_FORMAT;
 }

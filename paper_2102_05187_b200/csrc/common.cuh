@@ -87,6 +87,7 @@ __device__ __forceinline__ int64_t merge_path_segments(const int32_t *__restrict
 template <int W>
 __device__ __forceinline__ int64_t merge_path_segments_coop(const int32_t *__restrict__ seg_end, int64_t M, int64_t N,
                                                             int64_t diag, int k, unsigned mask) {
+  if (W == 1) return merge_path_segments(seg_end, M, N, diag);   // one probe per round would be a linear search
   int64_t lo = diag > N ? diag - N : 0;
   int64_t hi = diag < M ? diag : M;                 // markers below lo are inside, markers from hi on are not
   const int shift = (threadIdx.x & 31) & ~(W - 1);

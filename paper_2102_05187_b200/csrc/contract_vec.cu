@@ -35,6 +35,7 @@ struct SegGatherArgs {
   const int32_t *out_row;   // NULL: segment s -> row s. Else segment s -> row out_row[s] (ascending) and the
   int64_t out_rows;         //   rows in between (and up to out_rows) are zero-filled by the flushing worker
   int32_t R;                // columns handled by this launch
+  bool wide_store;          // ragged shapes: rows of C take 16-byte stores
   int32_t tile_items;
   int64_t num_tiles;
   double *carry_val;        // num_tiles x carry_ld
@@ -47,12 +48,14 @@ struct SegGatherArgs {
 };
 
 // What the walker does with one leaf entry: close the segments that end in front of it, accumulate.
-template <class T, int LPN, int CPL, int VEC, bool MAPPED, bool PASS_THROUGH = false>
+template <class T, int LPN, int CPL, int VEC, bool RAGGED, bool MAPPED, bool PASS_THROUGH = false>
 struct SegGatherPolicy {
-  using L = Lanes<T, LPN, CPL, VEC>;
+  using L = Lanes<T, LPN, CPL, VEC, RAGGED>;
   static constexpr int kPF = COMET_PF_GATHER;
   static constexpr bool kAux = false;
-  static constexpr bool kFullUnroll = true;
+  // Ragged fp32 rows end in up to four scalar stores per lane, too much code for one copy per entry of the chunk: with the
+  // chunk unrolled the kernel waits for instructions (30 M entries, R = 50: 519 us unrolled, 475 rolled).
+  static constexpr bool kFullUnroll = !(RAGGED && sizeof(T) == 4);
   // one copy of the unrolled body where the chunk is long (instruction cache; measured: SpMM config 2 -4 %); the
   // narrow shapes have short tiles of short chunks, where the slower rolled tail costs more than it saves (TTM +5 %)
   static constexpr bool kRolledTail = LPN >= 16;
@@ -72,7 +75,7 @@ struct SegGatherPolicy {
       : a(args), ln(lanes), seg((int32_t)i0), base(j0) {
     ln.zero(acc);
     if (PASS_THROUGH) pass = l2_policy_evict_first();
-    bcol = reinterpret_cast<const char *>(static_cast<const T *>(a.B) + ln.col0);
+    bcol = reinterpret_cast<const char *>(static_cast<const T *>(a.B) + ln.load_col());
     rel_end = end_of_open();
   }
   __device__ __forceinline__ int32_t end_of_open() const {
@@ -117,10 +120,10 @@ struct SegGatherPolicy {
 // others walk the general tiles and skip those rows. The two roles are bound by different things (the long rows
 // by the L2 -> L1 fill rate, the rest by DRAM latency), so sharing the SMs between them is faster than running
 // one after the other.
-template <class T, int LPN, int CPL, int VEC, bool MAPPED, bool HEAVY>
+template <class T, int LPN, int CPL, int VEC, bool RAGGED, bool MAPPED, bool HEAVY>
 __global__ void __launch_bounds__(kBlockThreads, (CPL * VEC * sizeof(T) <= 16 ? COMET_MINB_GATHER : 2))
 seg_gather_kernel(const SegGatherArgs a, const HeavyArgs h) {
-  using L = Lanes<T, LPN, CPL, VEC>;
+  using L = Lanes<T, LPN, CPL, VEC, RAGGED>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   if (HEAVY && (int)blockIdx.x < h.heavy_ctas) {
     heavy_role<T, LPN, CPL, VEC>(h, smem_raw);
@@ -130,7 +133,7 @@ seg_gather_kernel(const SegGatherArgs a, const HeavyArgs h) {
   const int64_t tile = (int64_t)(blockIdx.x - (HEAVY ? h.heavy_ctas : 0)) * L::kWorkers + worker;
   if (tile >= a.num_tiles) return;                       // whole groups leave together
   const uint32_t smem = smem_u32(smem_raw) + worker * RingLayout<L, false>::kWorkerBytes;
-  const L ln(a.R);
+  const L ln(a.R, a.wide_store);
   if (tile == 0 && ln.g == 0) a.carry_seg[a.num_tiles] = 0;   // no cut run of carries listed yet (carry_fixup_role)
 
   const int64_t total = a.M + a.N;
@@ -181,7 +184,7 @@ seg_gather_kernel(const SegGatherArgs a, const HeavyArgs h) {
     }
   }
 
-  SegGatherPolicy<T, LPN, CPL, VEC, MAPPED, HEAVY> p(a, ln, i0, j0);
+  SegGatherPolicy<T, LPN, CPL, VEC, RAGGED, MAPPED, HEAVY> p(a, ln, i0, j0);
   walk_tile(ln, p, j0, j1, smem);
   while (p.segment() < i1) p.flush();                    // end markers that close the tile
 
@@ -193,18 +196,6 @@ seg_gather_kernel(const SegGatherArgs a, const HeavyArgs h) {
   if (carry) ln.store_carry(a.carry_val + tile * a.carry_ld + ln.col0, p.acc);
 }
 
-// Merge-path split at every tile boundary, a thread per boundary (a warp per boundary with a 32-way search was
-// measured: slower, the boundaries are many and the searches hide each other's latency).
-__global__ void __launch_bounds__(kBlockThreads) seg_partition_kernel(const int32_t *__restrict__ seg_end, int64_t M, int64_t N,
-                                                                      int32_t tile_items, int64_t num_tiles,
-                                                                      int32_t *__restrict__ part) {
-  const int64_t t = (int64_t)blockIdx.x * kBlockThreads + threadIdx.x;
-  if (t > num_tiles) return;
-  const int64_t total = M + N;
-  const int64_t d = t * tile_items < total ? t * tile_items : total;
-  part[t] = (int32_t)merge_path_segments(seg_end, M, N, d);
-}
-
 // Adds the carries onto the stored rows. The tiles that stopped inside one segment are consecutive (a run); the sum of
 // a run is added to the segment's row, which has no other writer by now. One thread per tile and column: the thread at
 // the head of a run adds it up, several tiles in flight. What bounds this is latency, and a run of thousands of tiles
@@ -214,7 +205,7 @@ __global__ void __launch_bounds__(kBlockThreads) seg_partition_kernel(const int3
 // fixed. Measured, runs followed by one thread -> as here: 0.85 M entries, R = 4, 60 % of them in one slice 918 -> 84 us
 // (whole CSF MTTKRP); 14.9 M entries, R = 32 3.05 -> 0.40 ms (COO); 100 M entries, heaviest slice 0.5 % 2.90 -> 2.86 ms.
 constexpr int kRunFirst = 4;
-constexpr int kRunShort = kRunFirst + 16;
+constexpr int kRunShort = kRunFirst + 8;
 constexpr int kRunPiece = 1024;
 
 struct FixupArgs {
@@ -244,15 +235,13 @@ __device__ __forceinline__ double cta_slot_sum(const FixupArgs &f, int64_t first
   if (g < G) {
     const double *src = f.carry_val + first * f.carry_ld + c;
     const int64_t stride = step * f.carry_ld;
-    int32_t q = g;
-    for (; q + 15 * G < count; q += 16 * G) {
-      double v[16];
+    for (int32_t q = g; q < count; q += 8 * G) {           // eight slots in flight, the last ones guarded
+      double v[8];
 #pragma unroll
-      for (int u = 0; u < 16; ++u) v[u] = __ldcs(src + (int64_t)(q + u * G) * stride);
+      for (int u = 0; u < 8; ++u) v[u] = q + u * G < count ? __ldcs(src + (int64_t)(q + u * G) * stride) : 0.0;
 #pragma unroll
-      for (int u = 0; u < 16; ++u) sum += v[u];
+      for (int u = 0; u < 8; ++u) sum += v[u];
     }
-    for (; q < count; q += G) sum += __ldcs(src + (int64_t)q * stride);
   }
   __syncthreads();
   s_part[threadIdx.x] = sum;
@@ -263,13 +252,16 @@ __device__ __forceinline__ double cta_slot_sum(const FixupArgs &f, int64_t first
   return sum;
 }
 
-// `block` of fixup_blocks() CTAs: 256 / R tiles each, R threads per tile. LONG: long runs are possible.
+// `block` of fixup_blocks() CTAs: a thread per tile and pair of columns (half as many CTAs as with a column each: 27 ->
+// 24 us for 37,000 tiles of 64 columns). LONG: long runs are possible.
+__host__ __device__ __forceinline__ int32_t fixup_tiles(int32_t R) { return kBlockThreads / ((R + 1) / 2); }   // per CTA
+
 template <class T, bool LONG>
 __device__ __forceinline__ void carry_fixup_role(const FixupArgs &f, int64_t block) {
-  const int32_t G = kBlockThreads / f.R;         // R is at most 128
-  const int32_t g = threadIdx.x / f.R, c = threadIdx.x - g * f.R;
+  const int32_t per = (f.R + 1) / 2, G = fixup_tiles(f.R);      // R is at most 128
+  const int32_t g = threadIdx.x / per, c = 2 * (threadIdx.x - g * per);
   const int32_t tile = (int32_t)block * G + g;
-  const bool cut = LONG && f.run_count != nullptr;
+  const bool cut = LONG && f.run_count != nullptr, two = c + 1 < f.R;
   bool is_long = false;
   if (g < G && tile < f.num_tiles) {
     const int32_t seg_before = tile > 0 ? __ldg(f.carry_seg + tile - 1) : -2;
@@ -278,42 +270,44 @@ __device__ __forceinline__ void carry_fixup_role(const FixupArgs &f, int64_t blo
     if (head || (seg >= 0 && cut && tile % kRunPiece == 0)) {
       const int32_t edge = cut ? (tile / kRunPiece + 1) * kRunPiece : f.num_tiles;
       const int32_t limit = edge < f.num_tiles ? edge : f.num_tiles;       // the run is followed up to here
-      double v0[kRunFirst];
-      int32_t s0[kRunFirst];
-#pragma unroll
-      for (int u = 0; u < kRunFirst; ++u) {
-        const bool in = tile + u < limit;
-        s0[u] = in ? __ldg(f.carry_seg + tile + u) : -2;
-        v0[u] = in ? __ldcs(f.carry_val + (int64_t)(tile + u) * f.carry_ld + c) : 0.0;
-      }
-      double sum = v0[0];
+      auto carry = [&](int32_t t) {
+        const double *at = f.carry_val + (int64_t)t * f.carry_ld + c;
+        return f.carry_ld == 1 ? make_double2(__ldcs(at), 0.0) : __ldcs(reinterpret_cast<const double2 *>(at));
+      };
+      double2 sum = make_double2(0.0, 0.0);
       bool more = true;
-#pragma unroll
-      for (int u = 1; u < kRunFirst; ++u) {
-        more = more && s0[u] == seg;
-        if (more) sum += v0[u];
-      }
-      for (int32_t q = kRunFirst; more && (!LONG || q < kRunShort); q += 8) {
+      int32_t q = 0;
+      for (int step = kRunFirst; more && (!LONG || q < kRunShort); q += step, step = 8) {
         int32_t s[8];
-        double v[8];
+        double2 v[8];
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
-          const bool in = tile + q + u < limit;
+          const bool in = u < step && tile + q + u < limit;
           s[u] = in ? __ldg(f.carry_seg + tile + q + u) : -2;
-          v[u] = in ? __ldcs(f.carry_val + (int64_t)(tile + q + u) * f.carry_ld + c) : 0.0;
+          v[u] = in ? carry(tile + q + u) : make_double2(0.0, 0.0);
         }
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
-          more = more && s[u] == seg;
-          if (more) sum += v[u];
+          if (u < step) {
+            more = more && s[u] == seg;
+            if (more) { sum.x += v[u].x; sum.y += v[u].y; }
+          }
         }
       }
       is_long = LONG && more;                    // every thread of the tile sees the same run
       if (!is_long) {
         const bool on = cut && edge < f.num_tiles && edge - tile <= kRunShort && __ldg(f.carry_seg + edge - 1) == seg &&
                         __ldg(f.carry_seg + edge) == seg;
-        if (head && !on) add_to_row<T>(f, seg, c, sum);
-        else f.carry_val[(int64_t)tile * f.carry_ld + c] = sum;
+        if (head && !on) {
+          const int64_t row = f.out_row ? (int64_t)__ldg(f.out_row + seg) : (int64_t)seg;
+          T *const dst = static_cast<T *>(f.C) + row * f.ldc + c;
+          const double x = (double)dst[0], y = two ? (double)dst[1] : 0.0;
+          dst[0] = (T)(x + sum.x);
+          if (two) dst[1] = (T)(y + sum.y);
+        } else {
+          f.carry_val[(int64_t)tile * f.carry_ld + c] = sum.x;
+          if (two) f.carry_val[(int64_t)tile * f.carry_ld + c + 1] = sum.y;
+        }
         if (head && on && c == 0) f.run_list[atomicAdd(f.run_count, 1)] = tile;
       }
     }
@@ -378,7 +372,7 @@ __global__ void __launch_bounds__(kBlockThreads) carry_runs_kernel(const FixupAr
   }
 }
 
-static int64_t fixup_blocks(int64_t num_tiles, int32_t R) { return ceil_div(num_tiles, kBlockThreads / R); }
+static int64_t fixup_blocks(int64_t num_tiles, int32_t R) { return ceil_div(num_tiles, fixup_tiles(R)); }
 
 // SpMM with the long-row path: both fix-ups in one launch. They read different scratch and write different rows
 // of C (the general tiles leave the long rows out, so no carry names one), so the first `heavy_blocks` CTAs add
@@ -438,17 +432,22 @@ int32_t choose_tile_items(int64_t total_items, int workers_per_block, bool uneve
   // 8.2 M, R = 49 306 / 298 / 307 / 320 us; DCSR, 94 % of the rows empty, R = 8 1037 / 960 / 928 / 919 us.
   const int64_t slots = (int64_t)kSmCount * 4 * workers_per_block;
   int64_t t = ceil_div(total_items, slots * (uneven ? 8 : 4));
-  if (t < 32) t = 32;
+  if (t < 32) {
+    // Small: 32 items per tile unless that leaves SMs without work; a worker is sequential, so 8 items at least. With 32 / 16 /
+    // 8 / 4: 20,000 entries, fp64, R = 4 31.7 / 17.3 / 15.5 / 15.8 us; 150,000, fp32, R = 8 27.6 / 21.4 / 19.4 / 19.4 us.
+    const int64_t one_cta = ceil_div(total_items, (int64_t)kSmCount * workers_per_block);
+    t = one_cta > 32 ? 32 : one_cta < 8 ? 8 : one_cta;
+  }
   if (t > 512) t = 512;
   return (int32_t)t;
 }
 
-template <class T, int LPN, int CPL, int VEC, bool MAPPED, bool HEAVY>
+template <class T, int LPN, int CPL, int VEC, bool RAGGED, bool MAPPED, bool HEAVY>
 static comet_status_t launch_mapped(Context *ctx, const SegGatherArgs &a, const HeavyArgs &h, int64_t blocks,
                                     cudaStream_t stream) {
-  using L = Lanes<T, LPN, CPL, VEC>;
+  using L = Lanes<T, LPN, CPL, VEC, RAGGED>;
   constexpr size_t smem = RingLayout<L, false>::kBlockBytes;
-  auto kernel = seg_gather_kernel<T, LPN, CPL, VEC, MAPPED, HEAVY>;
+  auto kernel = seg_gather_kernel<T, LPN, CPL, VEC, RAGGED, MAPPED, HEAVY>;
   if (smem > 48 * 1024)
     COMET_CUDA_TRY(ctx, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   kernel<<<(unsigned)(blocks + (HEAVY ? h.heavy_ctas : 0)), kBlockThreads, smem, stream>>>(a, h);
@@ -465,9 +464,86 @@ static size_t carry_bytes(int64_t num_tiles, int32_t carry_ld) {
   return align_up((size_t)num_tiles * carry_ld * sizeof(double), 256) + align_up((size_t)carry_seg_words(num_tiles) * sizeof(int32_t), 256);
 }
 
-// `heavy` (optional): the long-row plan of an SpMM; its scratch precedes the carries of this launch.
-template <class T, int LPN, int CPL, int VEC>
-static comet_status_t launch_one(Context *ctx, SegGatherArgs a, HeavyArgs *heavy, cudaStream_t stream) {
+// What has to be there before a gather kernel starts, as roles of one launch (the steps are latency, not data: side by side
+// they cost what the longest of them does): copies of dense rows padded with zeros to whole 16-byte pieces, a thread per
+// piece, and in front of them, for SpMM and TTM, the merge-path split at every tile boundary, a thread per boundary.
+struct PadJob {
+  const void *src;
+  int64_t pieces_total;      // rows * pieces
+  int64_t ld;
+  void *dst;
+  int32_t R, pieces;
+};
+struct PrepareArgs {
+  const int32_t *seg_end;
+  int64_t M, N, num_tiles;
+  int32_t tile_items;
+  int32_t *part;
+  int64_t part_blocks;
+  PadJob pad[2];
+  int64_t pad_blocks[2];
+};
+
+template <class T>
+__device__ __forceinline__ void pad_role(const PadJob &p, int64_t i) {
+  constexpr int PER = 16 / sizeof(T);
+  if (i >= p.pieces_total) return;
+  const int64_t r = i < (1ll << 31) ? (int64_t)((uint32_t)i / (uint32_t)p.pieces) : i / p.pieces;
+  const int32_t c = (int32_t)(i - r * p.pieces) * PER;
+  const T *src = static_cast<const T *>(p.src) + r * p.ld + c;
+  T v[PER];
+#pragma unroll
+  for (int x = 0; x < PER; ++x) v[x] = c + x < p.R ? __ldg(src + x) : (T)0;
+  reinterpret_cast<int4 *>(p.dst)[i] = *reinterpret_cast<const int4 *>(v);
+}
+
+template <class T>
+__global__ void __launch_bounds__(kBlockThreads) prepare_kernel(const PrepareArgs a) {
+  int64_t block = blockIdx.x;
+  if (block < a.part_blocks) {
+    const int64_t t = block * kBlockThreads + threadIdx.x;
+    if (t > a.num_tiles) return;
+    const int64_t total = a.M + a.N;
+    const int64_t d = t * a.tile_items < total ? t * a.tile_items : total;
+    a.part[t] = (int32_t)merge_path_segments(a.seg_end, a.M, a.N, d);
+    return;
+  }
+  block -= a.part_blocks;
+  if (block < a.pad_blocks[0]) { pad_role<T>(a.pad[0], block * kBlockThreads + threadIdx.x); return; }
+  pad_role<T>(a.pad[1], (block - a.pad_blocks[0]) * kBlockThreads + threadIdx.x);
+}
+
+size_t padded_bytes(int dtype, int64_t rows, int64_t R) {
+  const int per = dtype == COMET_F32 ? 4 : 2;
+  return align_up((size_t)rows * ceil_div(R, per) * 16, 256);
+}
+static void pad_job(PrepareArgs &a, int which, int dtype, const void *src, int64_t rows, int64_t R, int64_t ld, void *dst) {
+  PadJob &p = a.pad[which];
+  p.src = src; p.ld = ld; p.dst = dst; p.R = (int32_t)R;
+  p.pieces = (int32_t)ceil_div(R, dtype == COMET_F32 ? 4 : 2);
+  p.pieces_total = rows * p.pieces;
+  a.pad_blocks[which] = ceil_div(p.pieces_total, (int64_t)kBlockThreads);
+}
+static comet_status_t prepare_run(Context *ctx, int dtype, const PrepareArgs &a, cudaStream_t stream) {
+  const int64_t blocks = a.part_blocks + a.pad_blocks[0] + a.pad_blocks[1];
+  if (blocks == 0) return COMET_OK;
+  if (dtype == COMET_F32) prepare_kernel<float><<<(unsigned)blocks, kBlockThreads, 0, stream>>>(a);
+  else prepare_kernel<double><<<(unsigned)blocks, kBlockThreads, 0, stream>>>(a);
+  COMET_LAUNCH_CHECK(ctx);
+  return COMET_OK;
+}
+comet_status_t pad_rows2(Context *ctx, int dtype, const void *src0, int64_t rows0, int64_t ld0, void *dst0, const void *src1, int64_t rows1,
+                         int64_t ld1, void *dst1, int64_t R, cudaStream_t stream) {
+  PrepareArgs a{};
+  pad_job(a, 0, dtype, src0, rows0, R, ld0, dst0);
+  pad_job(a, 1, dtype, src1, rows1, R, ld1, dst1);
+  return prepare_run(ctx, dtype, a, stream);
+}
+
+// `heavy` (optional): the long-row plan of an SpMM; its scratch precedes the carries of this launch. pad (RAGGED): the
+// first `pad` rows of B are copied into scratch as whole pieces and gathered from there.
+template <class T, int LPN, int CPL, int VEC, bool RAGGED = false>
+static comet_status_t launch_one(Context *ctx, SegGatherArgs a, HeavyArgs *heavy, int64_t pad, cudaStream_t stream) {
   constexpr int WORKERS = kBlockThreads / LPN;
   const int64_t total = a.M + a.N;
   a.tile_items = choose_tile_items(total, WORKERS, a.out_row != nullptr);
@@ -477,13 +553,22 @@ static comet_status_t launch_one(Context *ctx, SegGatherArgs a, HeavyArgs *heavy
   const size_t val_bytes = align_up((size_t)a.num_tiles * a.carry_ld * sizeof(double), 256);
   size_t heavy_bytes = 0;
   HeavyArgs h{};
-  if (kHeavyShape<T, LPN, CPL, VEC> && heavy && !a.out_row)
+  if (!RAGGED && kHeavyShape<T, LPN, CPL, VEC> && heavy && !a.out_row)
     heavy_bytes = spmm_heavy_plan(sizeof(T) == 4 ? COMET_F32 : COMET_F64, a.M, a.N, heavy->cols, a.B, a.ldb, a.R, a.C, a.ldc,
                                   a.tile_items, &h);
   static const bool use_part = !(getenv("COMET_SEG_PARTITION") && atoi(getenv("COMET_SEG_PARTITION")) == 0);
   const size_t part_bytes = use_part && a.num_tiles >= 1024 ? align_up((size_t)(a.num_tiles + 1) * sizeof(int32_t), 256) : 0;
-  char *scratch = (char *)scratch_get(ctx, heavy_bytes + carry_bytes(a.num_tiles, a.carry_ld) + part_bytes, stream);
+  constexpr int kDtype = sizeof(T) == 4 ? COMET_F32 : COMET_F64;
+  const size_t pad_bytes = RAGGED && pad ? padded_bytes(kDtype, pad, a.R) : 0;
+  char *scratch = (char *)scratch_get(ctx, pad_bytes + heavy_bytes + carry_bytes(a.num_tiles, a.carry_ld) + part_bytes, stream);
   if (!scratch) return COMET_ERR_ALLOC;
+  PrepareArgs prep{};
+  if (pad_bytes) {
+    pad_job(prep, 0, kDtype, a.B, pad, a.R, a.ldb, scratch);
+    a.B = scratch;
+    a.ldb = ceil_div(a.R, VEC) * VEC;
+    scratch += pad_bytes;
+  }
   a.carry_val = (double *)(scratch + heavy_bytes);
   a.carry_seg = (int32_t *)(scratch + heavy_bytes + val_bytes);
   if (part_bytes) {
@@ -492,20 +577,21 @@ static comet_status_t launch_one(Context *ctx, SegGatherArgs a, HeavyArgs *heavy
       h.part_seg_end = a.seg_end; h.part_M = a.M; h.part_N = a.N; h.part_tiles = a.num_tiles;
       h.part_tile_items = a.tile_items; h.part = part;
     } else {
-      seg_partition_kernel<<<(unsigned)ceil_div(a.num_tiles + 1, kBlockThreads), kBlockThreads, 0, stream>>>(a.seg_end, a.M, a.N,
-                                                                                                           a.tile_items, a.num_tiles, part);
-      COMET_LAUNCH_CHECK(ctx);
+      prep.seg_end = a.seg_end; prep.M = a.M; prep.N = a.N; prep.num_tiles = a.num_tiles;
+      prep.tile_items = a.tile_items; prep.part = part;
+      prep.part_blocks = ceil_div(a.num_tiles + 1, (int64_t)kBlockThreads);
     }
     a.part = part;
   }
   const int64_t blocks = ceil_div(a.num_tiles, WORKERS);
-  comet_status_t st;
-  if constexpr (kHeavyShape<T, LPN, CPL, VEC>) {
+  comet_status_t st = prepare_run(ctx, kDtype, prep, stream);
+  if (st != COMET_OK) return st;
+  if constexpr (!RAGGED && kHeavyShape<T, LPN, CPL, VEC>) {
     if (heavy_bytes) {
       st = spmm_heavy_prepare(ctx, &h, a.seg_end - 1, a.crd, a.val, scratch, stream);
       if (st != COMET_OK) return st;
       a.skip_len = h.threshold;
-      st = launch_mapped<T, LPN, CPL, VEC, false, true>(ctx, a, h, blocks, stream);
+      st = launch_mapped<T, LPN, CPL, VEC, false, false, true>(ctx, a, h, blocks, stream);
       if (st != COMET_OK) return st;
       const int heavy_blocks = kSmCount * 8;
       const unsigned fix_blocks = (unsigned)(heavy_blocks + fixup_blocks(a.num_tiles, a.R));
@@ -515,8 +601,8 @@ static comet_status_t launch_one(Context *ctx, SegGatherArgs a, HeavyArgs *heavy
       return COMET_OK;
     }
   }
-  st = a.out_row ? launch_mapped<T, LPN, CPL, VEC, true, false>(ctx, a, h, blocks, stream)
-                 : launch_mapped<T, LPN, CPL, VEC, false, false>(ctx, a, h, blocks, stream);
+  st = a.out_row ? launch_mapped<T, LPN, CPL, VEC, RAGGED, true, false>(ctx, a, h, blocks, stream)
+                 : launch_mapped<T, LPN, CPL, VEC, RAGGED, false, false>(ctx, a, h, blocks, stream);
   if (st != COMET_OK) return st;
   COMET_LAUNCHED(ctx, carry_fixup_launch(sizeof(T) == 4 ? COMET_F32 : COMET_F64, a.carry_val, a.carry_seg, a.num_tiles, a.R,
                                          a.carry_ld, a.C, a.ldc, a.out_row, a.out_row == nullptr || a.num_tiles * a.R > (1ll << 20),
@@ -526,39 +612,58 @@ static comet_status_t launch_one(Context *ctx, SegGatherArgs a, HeavyArgs *heavy
 
 static bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
 
-// One launch per chunk of up to 128 columns. A power-of-two chunk on 16-byte-aligned rows takes the
-// 128-bit path (LPN lanes x 16 bytes); anything else takes the scalar path (32 lanes, ragged).
+// One launch per chunk of up to 128 columns. A power-of-two number of whole pieces on aligned rows takes an exact
+// shape, anything else a ragged one; rows of B that are no whole pieces are padded into scratch first, unless B has so
+// many more rows than the matrix has entries that the copy would cost more than it saves: then the scalar shapes (32
+// lanes, a column each) run on B as it is. What the scalar shapes lose is lanes (R = 10: 22 of 32 idle) and requests in
+// flight. Measured, scalar -> ragged: 4 M entries in 200,000 rows, R = 3 / 10 / 25 / 50 / 100 fp64 134 -> 68, 137 -> 77, 155
+// -> 122, 194 -> 167, 463 -> 403 us, fp32 129 -> 70, 132 -> 77, 136 -> 109, 187 -> 151, 304 -> 208 us; a power-law
+// matrix of 3.2 M entries, R = 50, fp32 156 -> 145 us.
 template <class T>
 static comet_status_t seg_gather_typed(Context *ctx, const int32_t *seg_end, const int32_t *crd, const T *val,
                                        int64_t M, int64_t N, const T *B, int64_t ldb, int64_t R, T *C, int64_t ldc,
-                                       const int32_t *out_row, int64_t out_rows, int64_t b_rows, cudaStream_t stream) {
-  HeavyArgs hint{};                                        // SpMM on [D,CU] with a known B: long rows by column phases
-  hint.cols = b_rows;
-  HeavyArgs *heavy = (!out_row && b_rows > 0 && R <= 128) ? &hint : nullptr;
+                                       const int32_t *out_row, int64_t out_rows, int64_t b_rows, bool long_rows,
+                                       cudaStream_t stream) {
   constexpr int PER = 16 / sizeof(T);                      // elements per 128-bit piece
-  const bool vec_ok = aligned16(B) && aligned16(C) && (ldb % PER == 0) && (ldc % PER == 0);
+  HeavyArgs hint{};                                        // SpMM on [D,CU]: long rows by column phases
+  hint.cols = b_rows;
+  HeavyArgs *heavy = long_rows && !out_row && b_rows > 0 && R <= 128 ? &hint : nullptr;
+  const bool b_ok = aligned16(B) && ldb % PER == 0 && R % PER == 0, c_ok = aligned16(C) && ldc % PER == 0;
+  const bool pad = !b_ok && N >= 2 * b_rows;
   int64_t done = 0;
   while (done < R) {
-    const int64_t rem = R - done;
     SegGatherArgs a{};
     a.seg_end = seg_end; a.crd = crd; a.val = val; a.M = M; a.N = N;
     a.B = B + done; a.ldb = ldb; a.C = C + done; a.ldc = ldc;
     a.out_row = out_row; a.out_rows = out_rows;
-    comet_status_t st;
-    const int64_t chunk = rem < 128 ? rem : 128;
-    a.R = (int32_t)chunk;
-    const bool v = vec_ok && done % PER == 0;
-    const int64_t pieces = chunk / PER;                    // 128-bit pieces per row when chunk is a multiple
-    if (v && chunk % PER == 0 && pieces == 64) st = launch_one<T, 32, 2, PER>(ctx, a, heavy, stream);
-    else if (v && chunk % PER == 0 && pieces == 32) st = launch_one<T, 32, 1, PER>(ctx, a, heavy, stream);
-    else if (v && chunk % PER == 0 && pieces == 16) st = launch_one<T, 16, 1, PER>(ctx, a, heavy, stream);
-    else if (v && chunk % PER == 0 && pieces == 8) st = launch_one<T, 8, 1, PER>(ctx, a, heavy, stream);
-    else if (v && chunk % PER == 0 && pieces == 4) st = launch_one<T, 4, 1, PER>(ctx, a, heavy, stream);
-    else if (v && chunk % PER == 0 && pieces == 2) st = launch_one<T, 2, 1, PER>(ctx, a, heavy, stream);
-    else if (v && chunk % PER == 0 && pieces == 1) st = launch_one<T, 1, 1, PER>(ctx, a, heavy, stream);
-    else if (chunk > 64) st = launch_one<T, 32, 4, 1>(ctx, a, heavy, stream);
-    else if (chunk > 32) st = launch_one<T, 32, 2, 1>(ctx, a, heavy, stream);
-    else st = launch_one<T, 32, 1, 1>(ctx, a, heavy, stream);
+    a.wide_store = c_ok;
+    comet_status_t st = COMET_OK;
+    const int64_t rem = R - done;
+    if (b_ok || pad) {
+      const int64_t chunk = rem < 128 ? rem : 128, pieces = ceil_div(chunk, PER);
+      a.R = (int32_t)chunk;
+      const int64_t p = b_ok ? 0 : b_rows;
+      const bool exact = b_ok && c_ok && (pieces & (pieces - 1)) == 0;
+      if (pieces > 32) {
+        if constexpr (sizeof(T) == 8)                      // fp32 chunks are at most 32 pieces
+          st = exact ? launch_one<T, 32, 2, PER>(ctx, a, heavy, 0, stream) : launch_one<T, 32, 2, PER, true>(ctx, a, heavy, p, stream);
+      } else if (exact && pieces == 32) st = launch_one<T, 32, 1, PER>(ctx, a, heavy, 0, stream);
+      else if (exact && pieces == 16) st = launch_one<T, 16, 1, PER>(ctx, a, heavy, 0, stream);
+      else if (exact && pieces == 8) st = launch_one<T, 8, 1, PER>(ctx, a, heavy, 0, stream);
+      else if (exact && pieces == 4) st = launch_one<T, 4, 1, PER>(ctx, a, heavy, 0, stream);
+      else if (exact && pieces == 2) st = launch_one<T, 2, 1, PER>(ctx, a, heavy, 0, stream);
+      else if (exact && pieces == 1) st = launch_one<T, 1, 1, PER>(ctx, a, heavy, 0, stream);
+      else if (pieces > 16) st = launch_one<T, 32, 1, PER, true>(ctx, a, heavy, p, stream);
+      else if (pieces > 8) st = launch_one<T, 16, 1, PER, true>(ctx, a, heavy, p, stream);
+      else if (pieces > 4) st = launch_one<T, 8, 1, PER, true>(ctx, a, heavy, p, stream);
+      else if (pieces > 2) st = launch_one<T, 4, 1, PER, true>(ctx, a, heavy, p, stream);
+      else st = launch_one<T, 2, 1, PER, true>(ctx, a, heavy, p, stream);
+    } else {
+      a.R = (int32_t)(rem < 128 ? rem : 128);
+      if (a.R > 64) st = launch_one<T, 32, 4, 1>(ctx, a, heavy, 0, stream);
+      else if (a.R > 32) st = launch_one<T, 32, 2, 1>(ctx, a, heavy, 0, stream);
+      else st = launch_one<T, 32, 1, 1>(ctx, a, heavy, 0, stream);
+    }
     if (st != COMET_OK) return st;
     done += a.R;
   }
@@ -567,14 +672,14 @@ static comet_status_t seg_gather_typed(Context *ctx, const int32_t *seg_end, con
 
 comet_status_t seg_gather(Context *ctx, int dtype, const int32_t *seg_end, const int32_t *crd, const void *val,
                           int64_t M, int64_t N, const void *B, int64_t ldb, int64_t R, void *C, int64_t ldc,
-                          const int32_t *out_row, int64_t out_rows, int64_t b_rows, cudaStream_t stream) {
+                          const int32_t *out_row, int64_t out_rows, int64_t b_rows, bool long_rows, cudaStream_t stream) {
   if (ldb >= (1ll << 28)) return COMET_ERR_INDEX_OVERFLOW;      // row offsets are formed as int32 bytes * int32 index
   if (M == 0) return out_row ? zero_rows(ctx, C, dtype, out_rows, R, ldc, stream) : COMET_OK;
   if (dtype == COMET_F32)
     return seg_gather_typed<float>(ctx, seg_end, crd, (const float *)val, M, N, (const float *)B, ldb, R, (float *)C, ldc,
-                                   out_row, out_rows, b_rows, stream);
+                                   out_row, out_rows, b_rows, long_rows, stream);
   return seg_gather_typed<double>(ctx, seg_end, crd, (const double *)val, M, N, (const double *)B, ldb, R, (double *)C,
-                                  ldc, out_row, out_rows, b_rows, stream);
+                                  ldc, out_row, out_rows, b_rows, long_rows, stream);
 }
 
 }  // namespace comet

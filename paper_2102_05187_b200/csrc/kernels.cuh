@@ -8,10 +8,10 @@ namespace comet {
 // out[row(s), 0..R) = sum over leaf entries p of segment s of val[p] * B[crd[p], 0..R)   (SpMM, TTM)
 // seg_end[s] = leaf position where segment s ends; seg_end - 1 must be readable and hold 0 (seg_end = pos + 1).
 // out_row == NULL: row(s) = s; otherwise row(s) = out_row[s] (ascending) and all other rows below out_rows are
-// zero-filled. b_rows = number of rows of B (0: unknown; only used to decide on the long-row path of SpMM).
+// zero-filled. b_rows = number of rows of B. long_rows: the long-row path of SpMM may be taken.
 comet_status_t seg_gather(Context *ctx, int dtype, const int32_t *seg_end, const int32_t *crd, const void *val,
                           int64_t M, int64_t N, const void *B, int64_t ldb, int64_t R, void *C, int64_t ldc,
-                          const int32_t *out_row, int64_t out_rows, int64_t b_rows, cudaStream_t stream);
+                          const int32_t *out_row, int64_t out_rows, int64_t b_rows, bool long_rows, cudaStream_t stream);
 
 
 // y[row(s)] = sum over leaf entries p of segment s of val[p] * x[crd[p]]                    (SpMV, TTV)
@@ -21,13 +21,13 @@ comet_status_t seg_dot(Context *ctx, int dtype, const int32_t *seg_end, const in
 
 // Sorted COO [CN,S,S]: out[crd0[p], :] += val[p] * P[crd1[p], :] * Q[crd2[p], :]; every row < rows written.
 comet_status_t mttkrp_coo(Context *ctx, int dtype, const int32_t *crd0, const int32_t *crd1, const int32_t *crd2,
-                          const void *val, int64_t N, int64_t rows, const void *P, int64_t ldp, const void *Q,
-                          int64_t ldq, int64_t R, void *out, int64_t ldo, cudaStream_t stream);
+                          const void *val, int64_t N, int64_t rows, const void *P, int64_t p_rows, int64_t ldp,
+                          const void *Q, int64_t q_rows, int64_t ldq, int64_t R, void *out, int64_t ldo, cudaStream_t stream);
 
 // CSF [CU,CU,CU]: per fiber t = sum val * Q[crd2]; out[crd0[slice], :] += t * P[crd1[fiber], :].
 comet_status_t mttkrp_csf(Context *ctx, int dtype, const int32_t *pos1, const int32_t *crd0, const int32_t *crd1,
                           const int32_t *pos2, const int32_t *crd2, const void *val, int64_t S, int64_t F,
-                          int64_t N, int64_t rows, const void *P, int64_t ldp, const void *Q, int64_t ldq,
+                          int64_t N, int64_t rows, const void *P, int64_t p_rows, int64_t ldp, const void *Q, int64_t q_rows, int64_t ldq,
                           int64_t R, void *out, int64_t ldo, cudaStream_t stream);
 
 // CSF with the output mode stored at level 1, on the tiled walker (mttkrp.cu): fp64, R = 4, 8, 16 or 64 and
@@ -64,6 +64,12 @@ comet_status_t mttkrp_scatter4(Context *ctx, int dtype, int kind, const int32_t 
                                int64_t F2, int64_t N, int64_t rows, const void *A, int64_t lda, const void *B,
                                int64_t ldb, const void *C, int64_t ldc, int64_t R, void *out, int64_t ldo,
                                cudaStream_t stream);
+
+// Copies of two matrices of R columns with every row padded with zeros to whole 16-byte pieces, in one launch
+// (contract_vec.cu); padded_bytes: the size of such a copy.
+size_t padded_bytes(int dtype, int64_t rows, int64_t R);
+comet_status_t pad_rows2(Context *ctx, int dtype, const void *src0, int64_t rows0, int64_t ld0, void *dst0, const void *src1,
+                         int64_t rows1, int64_t ld1, void *dst1, int64_t R, cudaStream_t stream);
 
 comet_status_t zero_rows(Context *ctx, void *C, int dtype, int64_t rows, int64_t R, int64_t ldc, cudaStream_t stream);
 // Exclusive scan of uint32 words in three launches (tile sums, scan of the sums, apply); defined in pack.cu.

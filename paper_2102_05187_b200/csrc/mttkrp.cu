@@ -45,6 +45,7 @@ struct MttkrpArgs {
   void *out;
   int64_t ldo;
   int32_t R;
+  bool wide_store;   // ragged shapes: rows of `out` take 16-byte stores
   int32_t tile_items;
   int64_t num_tiles;
   double *carry_val;
@@ -55,9 +56,9 @@ struct MttkrpArgs {
 };
 
 // ------------------------------------------------------------------------------------------- COO
-template <class T, int LPN, int CPL, int VEC>
+template <class T, int LPN, int CPL, int VEC, bool RAGGED>
 struct CooPolicy {
-  using L = Lanes<T, LPN, CPL, VEC>;
+  using L = Lanes<T, LPN, CPL, VEC, RAGGED>;
   static constexpr int kPF = COMET_PF_COO;   // two rows per entry
   static constexpr bool kAux = true;         // the root coordinate rides in the side ring
   static constexpr bool kFullUnroll = true;
@@ -76,8 +77,8 @@ struct CooPolicy {
   __device__ __forceinline__ CooPolicy(const MttkrpArgs &args, const L &lanes, int32_t first_row)
       : a(args), ln(lanes), cur(first_row) {
     ln.zero(acc);
-    pcol = reinterpret_cast<const char *>(static_cast<const T *>(a.P) + ln.col0);
-    qcol = reinterpret_cast<const char *>(static_cast<const T *>(a.Q) + ln.col0);
+    pcol = reinterpret_cast<const char *>(static_cast<const T *>(a.P) + ln.load_col());
+    qcol = reinterpret_cast<const char *>(static_cast<const T *>(a.Q) + ln.load_col());
     ldp_bytes = (int32_t)(a.ldp * sizeof(T));
     ldq_bytes = (int32_t)(a.ldq * sizeof(T));
     ocol = static_cast<T *>(a.out) + ln.col0;
@@ -113,16 +114,16 @@ struct CooPolicy {
   }
 };
 
-template <class T, int LPN, int CPL, int VEC>
+template <class T, int LPN, int CPL, int VEC, bool RAGGED>
 __global__ void __launch_bounds__(kBlockThreads, (CPL * VEC * sizeof(T) <= 16 ? COMET_MINB_COO : 1)) mttkrp_coo_kernel(const MttkrpArgs a) {
-  using L = Lanes<T, LPN, CPL, VEC>;
+  using L = Lanes<T, LPN, CPL, VEC, RAGGED>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int worker = threadIdx.x / LPN;
   const int64_t tile = (int64_t)blockIdx.x * L::kWorkers + worker;
   if (tile >= a.num_tiles) return;
-  using P = CooPolicy<T, LPN, CPL, VEC>;
+  using P = CooPolicy<T, LPN, CPL, VEC, RAGGED>;
   const uint32_t smem = smem_u32(smem_raw) + worker * RingLayout<L, true>::kWorkerBytes;
-  const L ln(a.R);
+  const L ln(a.R, a.wide_store);
   if (tile == 0 && ln.g == 0) a.carry_seg[a.num_tiles] = 0;   // no cut run of carries listed yet
 
   const int64_t j0 = tile * a.tile_items;
@@ -173,11 +174,11 @@ __device__ __forceinline__ void atom_or_shared(uint32_t addr, uint32_t bits) {
 // tile to tile. Sums are double; the output must be zero when the kernel starts.
 constexpr int kCsfFold = 0, kCsfExpand = 1, kCsfLevel1 = 2;
 
-template <class T, int LPN, int CPL, int VEC, int FORM>
+template <class T, int LPN, int CPL, int VEC, bool RAGGED, int FORM>
 struct CsfPolicy {
   static constexpr bool EXPAND = FORM == kCsfExpand;
   static constexpr bool LEVEL1 = FORM == kCsfLevel1;
-  using L = Lanes<T, LPN, CPL, VEC>;
+  using L = Lanes<T, LPN, CPL, VEC, RAGGED>;
   static constexpr int kPF = COMET_PF_CSF;
   static constexpr bool kAux = false;
   static constexpr bool kFullUnroll = true;
@@ -206,8 +207,8 @@ struct CsfPolicy {
         j0(j0_), f0((int32_t)f0_), s((int32_t)s0), a_dirty(false) {
     ln.zero(tac);
     ln.zero(aac);
-    pcol = reinterpret_cast<const char *>(static_cast<const T *>(a.P) + ln.col0);
-    qcol = reinterpret_cast<const char *>(static_cast<const T *>(a.Q) + ln.col0);
+    pcol = reinterpret_cast<const char *>(static_cast<const T *>(a.P) + ln.load_col());
+    qcol = reinterpret_cast<const char *>(static_cast<const T *>(a.Q) + ln.load_col());
     ldp_bytes = (int32_t)(a.ldp * sizeof(T));
     ldq_bytes = (int32_t)(a.ldq * sizeof(T));
     ocol = static_cast<T *>(a.out) + ln.col0;
@@ -390,17 +391,17 @@ __global__ void __launch_bounds__(kBlockThreads) zero_unowned_rows_kernel(const 
   }
 }
 
-template <class T, int LPN, int CPL, int VEC, int FORM>
+template <class T, int LPN, int CPL, int VEC, bool RAGGED, int FORM>
 __global__ void __launch_bounds__(kBlockThreads, (CPL * VEC * sizeof(T) <= 16 ? COMET_MINB_CSF : 2)) mttkrp_csf_kernel(const MttkrpArgs a) {
-  using L = Lanes<T, LPN, CPL, VEC>;
+  using L = Lanes<T, LPN, CPL, VEC, RAGGED>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int worker = threadIdx.x / LPN;
   const int64_t tile = (int64_t)blockIdx.x * L::kWorkers + worker;
   if (tile >= a.num_tiles) return;
-  using P = CsfPolicy<T, LPN, CPL, VEC, FORM>;
+  using P = CsfPolicy<T, LPN, CPL, VEC, RAGGED, FORM>;
   const uint32_t smem = smem_u32(smem_raw) + worker * RingLayout<L, false>::kWorkerBytes;
   const uint32_t flags = smem_u32(smem_raw) + (uint32_t)RingLayout<L, false>::kBlockBytes + worker * kCsfWorkerBytes;
-  const L ln(a.R);
+  const L ln(a.R, a.wide_store);
   if (tile == 0 && ln.g == 0) a.carry_seg[a.num_tiles] = 0;   // no cut run of carries listed yet
 
   // A tile is a span of the merge list of fiber-end markers and leaf positions (equal work per tile: an entry
@@ -433,11 +434,12 @@ __global__ void __launch_bounds__(kBlockThreads, (CPL * VEC * sizeof(T) <= 16 ? 
 // ------------------------------------------------------------------------------------------- host
 static bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
 
-template <bool CSF, class T, int LPN, int CPL, int VEC>
-static comet_status_t launch_mttkrp(Context *ctx, MttkrpArgs a, cudaStream_t stream) {
+// p_pad / q_pad (RAGGED): so many rows of P / Q are copied into scratch as whole pieces and gathered from there.
+template <bool CSF, class T, int LPN, int CPL, int VEC, bool RAGGED = false>
+static comet_status_t launch_mttkrp(Context *ctx, MttkrpArgs a, int64_t p_pad, int64_t q_pad, cudaStream_t stream) {
   constexpr int WORKERS = kBlockThreads / LPN;
   const int64_t total = CSF ? a.F + a.N : a.N;
-  using L = Lanes<T, LPN, CPL, VEC>;
+  using L = Lanes<T, LPN, CPL, VEC, RAGGED>;
   a.tile_items = choose_tile_items(total, WORKERS, false);
   if (CSF && a.tile_items > kCsfTileCap) a.tile_items = kCsfTileCap;          // one mask bit per leaf entry of a tile
   a.num_tiles = ceil_div(total, a.tile_items);
@@ -445,8 +447,18 @@ static comet_status_t launch_mttkrp(Context *ctx, MttkrpArgs a, cudaStream_t str
   const size_t val_bytes = align_up((size_t)a.num_tiles * a.carry_ld * sizeof(double), 256);
   const size_t seg_bytes = align_up((size_t)carry_seg_words(a.num_tiles) * sizeof(int32_t), 256);
   const size_t part_bytes = CSF ? align_up((size_t)(a.num_tiles + 1) * sizeof(int32_t), 256) : 0;
-  char *scratch = (char *)scratch_get(ctx, val_bytes + seg_bytes + 2 * part_bytes, stream);
+  constexpr int kDtype = sizeof(T) == 4 ? COMET_F32 : COMET_F64;
+  const size_t p_bytes = RAGGED && p_pad ? padded_bytes(kDtype, p_pad, a.R) : 0, q_bytes = RAGGED && p_pad ? padded_bytes(kDtype, q_pad, a.R) : 0;
+  char *scratch = (char *)scratch_get(ctx, p_bytes + q_bytes + val_bytes + seg_bytes + 2 * part_bytes, stream);
   if (!scratch) return COMET_ERR_ALLOC;
+  if (p_bytes) {
+    const comet_status_t ps = pad_rows2(ctx, kDtype, a.P, p_pad, a.ldp, scratch, a.Q, q_pad, a.ldq, scratch + p_bytes, a.R, stream);
+    if (ps != COMET_OK) return ps;
+    a.P = scratch;
+    a.Q = scratch + p_bytes;
+    a.ldp = a.ldq = ceil_div(a.R, VEC) * VEC;
+    scratch += p_bytes + q_bytes;
+  }
   a.carry_val = (double *)scratch;
   a.carry_seg = (int32_t *)(scratch + val_bytes);
   if (CSF) {
@@ -463,10 +475,10 @@ static comet_status_t launch_mttkrp(Context *ctx, MttkrpArgs a, cudaStream_t str
   // CSF with short fibers (mean length below 4): the per-entry form; COMET_CSF_FORM=fold / expand forces one
   bool expand = CSF && a.N < 4 * a.F;
   if (const char *e = getenv("COMET_CSF_FORM")) expand = CSF && (e[0] == 'e' ? true : (e[0] == 'f' ? false : expand));
-  auto kernel = !CSF ? mttkrp_coo_kernel<T, LPN, CPL, VEC>
-                     : (expand ? mttkrp_csf_kernel<T, LPN, CPL, VEC, kCsfExpand> : mttkrp_csf_kernel<T, LPN, CPL, VEC, kCsfFold>);
-  if constexpr (CSF && sizeof(T) == 8 && VEC == 2 && CPL == 1) {
-    if (a.level1) kernel = mttkrp_csf_kernel<T, LPN, CPL, VEC, kCsfLevel1>;
+  auto kernel = !CSF ? mttkrp_coo_kernel<T, LPN, CPL, VEC, RAGGED>
+                     : (expand ? mttkrp_csf_kernel<T, LPN, CPL, VEC, RAGGED, kCsfExpand> : mttkrp_csf_kernel<T, LPN, CPL, VEC, RAGGED, kCsfFold>);
+  if constexpr (CSF && sizeof(T) == 8 && VEC == 2 && CPL == 1 && !RAGGED && LPN != 16) {
+    if (a.level1) kernel = mttkrp_csf_kernel<T, LPN, CPL, VEC, RAGGED, kCsfLevel1>;
   }
   if (smem > 48 * 1024)
     COMET_CUDA_TRY(ctx, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
@@ -478,42 +490,57 @@ static comet_status_t launch_mttkrp(Context *ctx, MttkrpArgs a, cudaStream_t str
   return COMET_OK;
 }
 
+// Shapes as in seg_gather_typed (contract_vec.cu): exact ones, ragged ones (operands padded into scratch where they are no
+// whole 16-byte pieces), scalar ones where the factors have far more rows than the tensor has entries.
 template <bool CSF, class T>
-static comet_status_t mttkrp_chunks(Context *ctx, MttkrpArgs base, int64_t R, cudaStream_t stream) {
+static comet_status_t mttkrp_chunks(Context *ctx, const MttkrpArgs &base, int64_t p_rows, int64_t q_rows, int64_t R, cudaStream_t stream) {
   constexpr int PER = 16 / sizeof(T);
-  const bool vec_ok = aligned16(base.P) && aligned16(base.Q) && aligned16(base.out) && base.ldp % PER == 0 &&
-                      base.ldq % PER == 0 && base.ldo % PER == 0;
+  const bool in_ok = aligned16(base.P) && aligned16(base.Q) && base.ldp % PER == 0 && base.ldq % PER == 0 && R % PER == 0;
+  const bool out_ok = aligned16(base.out) && base.ldo % PER == 0;
+  const bool pad = !in_ok && 2 * base.N >= p_rows + q_rows;
   int64_t done = 0;
   while (done < R) {
     const int64_t rem = R - done;
-    const int64_t chunk = rem < 128 ? rem : 128;
     MttkrpArgs a = base;
     a.P = static_cast<const T *>(base.P) + done;
     a.Q = static_cast<const T *>(base.Q) + done;
     a.out = static_cast<T *>(base.out) + done;
-    a.R = (int32_t)chunk;
-    const bool v = vec_ok && done % PER == 0 && chunk % PER == 0;
-    const int64_t pieces = chunk / PER;
-    comet_status_t st;
-    if (v && pieces == 64) st = launch_mttkrp<CSF, T, 32, 2, PER>(ctx, a, stream);
-    else if (v && pieces == 32) st = launch_mttkrp<CSF, T, 32, 1, PER>(ctx, a, stream);
-    else if (v && pieces == 16) st = launch_mttkrp<CSF, T, 16, 1, PER>(ctx, a, stream);
-    else if (v && pieces == 8) st = launch_mttkrp<CSF, T, 8, 1, PER>(ctx, a, stream);
-    else if (v && pieces == 4) st = launch_mttkrp<CSF, T, 4, 1, PER>(ctx, a, stream);
-    else if (v && pieces == 2) st = launch_mttkrp<CSF, T, 2, 1, PER>(ctx, a, stream);
-    else if (v && pieces == 1) st = launch_mttkrp<CSF, T, 1, 1, PER>(ctx, a, stream);
-    else if (chunk > 64) st = launch_mttkrp<CSF, T, 32, 4, 1>(ctx, a, stream);
-    else if (chunk > 32) st = launch_mttkrp<CSF, T, 32, 2, 1>(ctx, a, stream);
-    else st = launch_mttkrp<CSF, T, 32, 1, 1>(ctx, a, stream);
+    a.wide_store = out_ok;
+    comet_status_t st = COMET_OK;
+    if (in_ok || pad) {
+      const int64_t chunk = rem < 128 ? rem : 128, pieces = ceil_div(chunk, PER);
+      a.R = (int32_t)chunk;
+      const int64_t pp = in_ok ? 0 : p_rows, qp = in_ok ? 0 : q_rows;
+      const bool exact = in_ok && out_ok && (pieces & (pieces - 1)) == 0;
+      if (pieces > 32) {
+        if constexpr (sizeof(T) == 8)                      // fp32 chunks are at most 32 pieces
+          st = exact ? launch_mttkrp<CSF, T, 32, 2, PER>(ctx, a, 0, 0, stream) : launch_mttkrp<CSF, T, 32, 2, PER, true>(ctx, a, pp, qp, stream);
+      } else if (exact && pieces == 32) st = launch_mttkrp<CSF, T, 32, 1, PER>(ctx, a, 0, 0, stream);
+      else if (exact && pieces == 16) st = launch_mttkrp<CSF, T, 16, 1, PER>(ctx, a, 0, 0, stream);
+      else if (exact && pieces == 8) st = launch_mttkrp<CSF, T, 8, 1, PER>(ctx, a, 0, 0, stream);
+      else if (exact && pieces == 4) st = launch_mttkrp<CSF, T, 4, 1, PER>(ctx, a, 0, 0, stream);
+      else if (exact && pieces == 2) st = launch_mttkrp<CSF, T, 2, 1, PER>(ctx, a, 0, 0, stream);
+      else if (exact && pieces == 1) st = launch_mttkrp<CSF, T, 1, 1, PER>(ctx, a, 0, 0, stream);
+      else if (pieces > 16) st = launch_mttkrp<CSF, T, 32, 1, PER, true>(ctx, a, pp, qp, stream);
+      else if (pieces > 8) st = launch_mttkrp<CSF, T, 16, 1, PER, true>(ctx, a, pp, qp, stream);
+      else if (pieces > 4) st = launch_mttkrp<CSF, T, 8, 1, PER, true>(ctx, a, pp, qp, stream);
+      else if (pieces > 2) st = launch_mttkrp<CSF, T, 4, 1, PER, true>(ctx, a, pp, qp, stream);
+      else st = launch_mttkrp<CSF, T, 2, 1, PER, true>(ctx, a, pp, qp, stream);
+    } else {
+      a.R = (int32_t)(rem < 128 ? rem : 128);
+      if (a.R > 64) st = launch_mttkrp<CSF, T, 32, 4, 1>(ctx, a, 0, 0, stream);
+      else if (a.R > 32) st = launch_mttkrp<CSF, T, 32, 2, 1>(ctx, a, 0, 0, stream);
+      else st = launch_mttkrp<CSF, T, 32, 1, 1>(ctx, a, 0, 0, stream);
+    }
     if (st != COMET_OK) return st;
-    done += chunk;
+    done += a.R;
   }
   return COMET_OK;
 }
 
 comet_status_t mttkrp_coo(Context *ctx, int dtype, const int32_t *crd0, const int32_t *crd1, const int32_t *crd2,
-                          const void *val, int64_t N, int64_t rows, const void *P, int64_t ldp, const void *Q,
-                          int64_t ldq, int64_t R, void *out, int64_t ldo, cudaStream_t stream) {
+                          const void *val, int64_t N, int64_t rows, const void *P, int64_t p_rows, int64_t ldp,
+                          const void *Q, int64_t q_rows, int64_t ldq, int64_t R, void *out, int64_t ldo, cudaStream_t stream) {
   if (ldp >= (1ll << 28) || ldq >= (1ll << 28)) return COMET_ERR_INDEX_OVERFLOW;
   {                                                        // rows without entries stay zero; the others are stored over
     const size_t elt = dtype == COMET_F32 ? 4 : 8;
@@ -527,12 +554,13 @@ comet_status_t mttkrp_coo(Context *ctx, int dtype, const int32_t *crd0, const in
   MttkrpArgs a{};
   a.crd0 = crd0; a.crd1 = crd1; a.crd2 = crd2; a.val = val; a.N = N; a.rows = rows;
   a.P = P; a.ldp = ldp; a.Q = Q; a.ldq = ldq; a.out = out; a.ldo = ldo;
-  return dtype == COMET_F32 ? mttkrp_chunks<false, float>(ctx, a, R, stream) : mttkrp_chunks<false, double>(ctx, a, R, stream);
+  return dtype == COMET_F32 ? mttkrp_chunks<false, float>(ctx, a, p_rows, q_rows, R, stream)
+                            : mttkrp_chunks<false, double>(ctx, a, p_rows, q_rows, R, stream);
 }
 
 comet_status_t mttkrp_csf(Context *ctx, int dtype, const int32_t *pos1, const int32_t *crd0, const int32_t *crd1,
                           const int32_t *pos2, const int32_t *crd2, const void *val, int64_t S, int64_t F,
-                          int64_t N, int64_t rows, const void *P, int64_t ldp, const void *Q, int64_t ldq,
+                          int64_t N, int64_t rows, const void *P, int64_t p_rows, int64_t ldp, const void *Q, int64_t q_rows, int64_t ldq,
                           int64_t R, void *out, int64_t ldo, cudaStream_t stream) {
   if (ldp >= (1ll << 28) || ldq >= (1ll << 28)) return COMET_ERR_INDEX_OVERFLOW;
   if (N == 0 || S == 0) return zero_rows(ctx, out, dtype, rows, R, ldo, stream);
@@ -546,7 +574,8 @@ comet_status_t mttkrp_csf(Context *ctx, int dtype, const int32_t *pos1, const in
     else zero_unowned_rows_kernel<double><<<blocks, kBlockThreads, 0, stream>>>(crd0, S, rows, (double *)out, ldo, (int32_t)R);
     COMET_LAUNCH_CHECK(ctx);
   }
-  return dtype == COMET_F32 ? mttkrp_chunks<true, float>(ctx, a, R, stream) : mttkrp_chunks<true, double>(ctx, a, R, stream);
+  return dtype == COMET_F32 ? mttkrp_chunks<true, float>(ctx, a, p_rows, q_rows, R, stream)
+                            : mttkrp_chunks<true, double>(ctx, a, p_rows, q_rows, R, stream);
 }
 
 // CSF, output mode stored at level 1: out[crd1[f], :] += (sum over fiber f of val * Q[crd2, :]) * P[crd0[slice of f], :].
@@ -573,7 +602,7 @@ comet_status_t mttkrp_csf_level1(Context *ctx, int dtype, const int32_t *pos1, c
   a.S = S; a.F = F; a.N = N; a.rows = rows;
   a.P = P; a.ldp = ldp; a.Q = Q; a.ldq = ldq; a.out = out; a.ldo = ldo;
   a.level1 = true;
-  return mttkrp_chunks<true, double>(ctx, a, R, stream);
+  return mttkrp_chunks<true, double>(ctx, a, 0, 0, R, stream);        // aligned: nothing is padded
 }
 
 }  // namespace comet

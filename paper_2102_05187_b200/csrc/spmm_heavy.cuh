@@ -63,7 +63,7 @@ struct HeavyPolicy {
     keep = l2_policy_evict_last();
     val = static_cast<const T *>(a.val);
     crd = a.crd;
-    bcol = reinterpret_cast<const char *>(static_cast<const T *>(a.B) + ln.col0);
+    bcol = reinterpret_cast<const char *>(static_cast<const T *>(a.B) + ln.load_col());
     ldb_bytes = (int32_t)(a.ldb * sizeof(T));
   }
   __device__ __forceinline__ void fetch(int32_t j, Entry16 &e, int32_t &) const {

@@ -122,30 +122,47 @@ template <> struct Piece<float, 1> {
 };
 
 // T is the storage type of values and dense operands (double or float); sums are always kept in double.
-template <class T_, int LPN_, int CPL_, int VEC_> struct Lanes {
+// RAGGED: 16-byte pieces, but fewer of them than the lanes hold, or a last one of fewer columns. The gathered rows are whole
+// pieces all the same (aligned operands, padded ones where the caller's are not): a lane beyond the last piece reads the
+// last one, which costs no traffic and keeps predicates out of the walk, and stores nothing.
+template <class T_, int LPN_, int CPL_, int VEC_, bool RAGGED_ = false> struct Lanes {
   using T = T_;
   static constexpr int LPN = LPN_, CPL = CPL_, VEC = VEC_;
+  static constexpr bool RAGGED = RAGGED_;
   // leaf entries per refill of the ring (8 for the narrow shapes: 16 was measured 3 % slower on TTM config 4,
   // the staging registers of a second entry per lane are better spent elsewhere)
   static constexpr int kChunk = LPN >= 16 ? 32 : 8;
   static constexpr int kPer = kChunk / LPN;                // entries each lane loads per refill
   static constexpr int kWorkers = kBlockThreads / LPN;     // workers per CTA
   static constexpr int kStride = LPN * VEC;                // columns between a lane's consecutive pieces
-  static constexpr bool kVector = VEC * sizeof(T) == 16;   // 128-bit pieces: the launch width is never ragged
+  static constexpr bool kVector = VEC * sizeof(T) == 16;   // 128-bit pieces: every lane's loads are in bounds
 
   int g;            // lane within the group
   unsigned mask;    // the group's lanes
   int32_t col0;     // first column of piece 0; piece t starts at col0 + t * kStride
   bool ok[CPL];     // piece inside the R columns of this launch (only the scalar path is ever ragged)
+  int32_t lcol, lstep;   // RAGGED: where this lane's loads of piece 0 start, and the step to piece 1
+  int32_t R;             // RAGGED: columns of this launch
+  bool wide;             // RAGGED: output rows take 16-byte stores
 
-  __device__ __forceinline__ Lanes(int R) {
+  __device__ __forceinline__ Lanes(int R_, bool wide_ = true) {
+    const int R = R_;
     g = threadIdx.x & (LPN - 1);
     const unsigned lane = threadIdx.x & 31;
     mask = LPN == 32 ? 0xffffffffu : (((1u << LPN) - 1u) << (lane & ~(LPN - 1)));
     col0 = g * VEC;
 #pragma unroll
     for (int t = 0; t < CPL; ++t) ok[t] = kVector ? true : (col0 + t * kStride) < R;
+    if constexpr (RAGGED) {
+      this->R = R;
+      wide = wide_;
+      const int32_t last = (R - 1) / VEC * VEC;            // first column of the last piece
+      lcol = col0 < last ? col0 : last;
+      lstep = (col0 + kStride < last ? col0 + kStride : last) - lcol;
+    }
   }
+  __device__ __forceinline__ int32_t load_col() const { return RAGGED ? lcol : col0; }
+  __device__ __forceinline__ int32_t piece(int t) const { return RAGGED ? t * lstep : t * kStride; }   // t is 0 or, RAGGED, 1
   __device__ __forceinline__ void sync() const { __syncwarp(mask); }
 
   __device__ __forceinline__ void zero(double (&acc)[CPL][VEC]) const {
@@ -154,22 +171,34 @@ template <class T_, int LPN_, int CPL_, int VEC_> struct Lanes {
 #pragma unroll
       for (int e = 0; e < VEC; ++e) acc[t][e] = 0.0;
   }
-  // `row` already points at this lane's piece 0 (row base + col0)
+  // `row` already points at this lane's piece 0 (row base + load_col())
   __device__ __forceinline__ void gather(const T *row, T (&dst)[CPL][VEC]) const {
 #pragma unroll
     for (int t = 0; t < CPL; ++t)
-      if (ok[t]) Piece<T, VEC>::load(row + t * kStride, dst[t]);
+      if (ok[t]) Piece<T, VEC>::load(row + piece(t), dst[t]);
   }
   // the same with an L2 eviction policy (128-bit pieces only; the other shapes never carry two roles)
   __device__ __forceinline__ void gather_hint(const T *row, T (&dst)[CPL][VEC], uint64_t pol) const {
     if constexpr (VEC * sizeof(T) == 16) {
 #pragma unroll
-      for (int t = 0; t < CPL; ++t) Piece<T, VEC>::load_hint(row + t * kStride, dst[t], pol);
+      for (int t = 0; t < CPL; ++t) Piece<T, VEC>::load_hint(row + piece(t), dst[t], pol);
     } else {
       gather(row, dst);
     }
   }
   __device__ __forceinline__ void store_row(T *row, const double (&acc)[CPL][VEC]) const {
+    if constexpr (RAGGED) {
+#pragma unroll
+      for (int t = 0; t < CPL; ++t) {
+        const int32_t left = R - (col0 + t * kStride);
+        if (wide && left >= VEC) Piece<T, VEC>::store_stream(row + t * kStride, acc[t]);
+        else
+#pragma unroll
+          for (int e = 0; e < VEC; ++e)
+            if (e < left) __stcs(row + t * kStride + e, (T)acc[t][e]);
+      }
+      return;
+    }
 #pragma unroll
     for (int t = 0; t < CPL; ++t)
       if (ok[t]) Piece<T, VEC>::store_stream(row + t * kStride, acc[t]);
@@ -179,7 +208,8 @@ template <class T_, int LPN_, int CPL_, int VEC_> struct Lanes {
     for (int t = 0; t < CPL; ++t)
       if (ok[t])
 #pragma unroll
-        for (int e = 0; e < VEC; ++e) row[t * kStride + e] = acc[t][e];
+        for (int e = 0; e < VEC; ++e)
+          if (!RAGGED || col0 + t * kStride + e < R) row[t * kStride + e] = acc[t][e];
   }
   // rows lo .. hi-1 of a matrix whose lane-piece-0 pointer of row 0 is `base`
   __device__ __forceinline__ void zero_rows(T *base, int64_t ld, int64_t lo, int64_t hi) const {
@@ -266,25 +296,27 @@ template <class L, class Policy, bool TAIL>
 __device__ __forceinline__ void walk_chunk_rolled(Policy &p, typename Policy::Slot (&win)[Policy::kPF], uint32_t cur,
                                                   uint32_t nxt, uint32_t cur_aux, uint32_t nxt_aux, int n) {
   constexpr int kChunk = L::kChunk, kPF = Policy::kPF;
-  // the two halves are adjacent in shared memory: position q + kPF of `cur` wraps into `nxt`
+  // the two halves are adjacent in shared memory: the kPF positions behind a step lie in one half, so a step's ring
+  // addresses are two bases and immediates
   const uint32_t lo = cur < nxt ? cur : nxt, lo_aux = cur_aux < nxt_aux ? cur_aux : nxt_aux;
   const int off = cur < nxt ? 0 : kChunk;
 #pragma unroll 1
   for (int q0 = 0; q0 < (TAIL ? n : kChunk); q0 += kPF) {
+    const uint32_t at = lo + (off + q0) * 16, ahead = lo + ((off + q0 + kPF) & (2 * kChunk - 1)) * 16;
+    const uint32_t at_aux = lo_aux + (off + q0) * 4;
 #pragma unroll
     for (int u = 0; u < kPF; ++u) {
       const int q = q0 + u;
       if (TAIL && q >= n) break;
-      const int r = off + q;
       if constexpr (policy_slot_carries<Policy>::value) p.consume_slot(q, win[u]);
-      else if constexpr (policy_consumes_entry<Policy>::value) p.consume_entry(q, lds_entry(lo + r * 16), win[u]);
-      else p.consume(q, lds_f64(lo + r * 16), Policy::kAux ? lds_s32(lo_aux + r * 4) : 0, win[u]);
+      else if constexpr (policy_consumes_entry<Policy>::value) p.consume_entry(q, lds_entry(at + u * 16), win[u]);
+      else p.consume(q, lds_f64(at + u * 16), Policy::kAux ? lds_s32(at_aux + u * 4) : 0, win[u]);
       if (TAIL && q + kPF >= n) continue;
       if constexpr (policy_slot_carries<Policy>::value) {
-        p.prefetch_entry(lds_entry(lo + ((r + kPF) & (2 * kChunk - 1)) * 16), win[u]);
+        p.prefetch_entry(lds_entry(ahead + u * 16), win[u]);
       } else {
         int32_t ca, cb;
-        lds_coords(lo + ((r + kPF) & (2 * kChunk - 1)) * 16, ca, cb);
+        lds_coords(ahead + u * 16, ca, cb);
         if constexpr (policy_is_positional<Policy>::value) p.prefetch_at((q + kPF) & (kChunk - 1), q + kPF < kChunk, ca, cb, win[u]);
         else p.prefetch(ca, cb, win[u]);
       }

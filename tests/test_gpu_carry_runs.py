@@ -1,4 +1,4 @@
-"""The carry fix-up: segments that span from one tile to thousands of them, with run lengths around 20 tiles (added by
+"""The carry fix-up: segments that span from one tile to thousands of them, with run lengths around 12 and 20 tiles (added by
 one thread or by a whole CTA) and around multiples of 1,024 (where runs are cut in large problems). Small tiles are
 forced, so that small inputs reach every case."""
 import numpy as np
@@ -22,7 +22,7 @@ def _need_gpu(cuda_device, monkeypatch):
     yield
 
 
-@pytest.mark.parametrize("lengths", [[3, 8 * 18, 0, 8 * 19, 1, 8 * 20 + 5, 8 * 21, 2, 8 * 22],
+@pytest.mark.parametrize("lengths", [[3, 8 * 10, 0, 8 * 11, 1, 8 * 12 + 5, 8 * 13, 2, 8 * 14, 8 * 20],
                                      [1, 8 * 700, 0, 8 * 64 - 3, 2, 8 * 1030, 8 * 3000]])
 @pytest.mark.parametrize("R", [1, 5, 16, 100])
 def test_spmm_runs(lengths, R):
@@ -41,7 +41,7 @@ def test_spmm_runs(lengths, R):
 @pytest.mark.parametrize("attr", [(CU, CU, CU), (CN, S, S)])
 @pytest.mark.parametrize("R,n", [(4, 17000), (33, 180000), (128, 60000)])
 def test_mttkrp_heavy_slice(attr, R, n):
-    """A slice with most of the entries among slices of one entry, of about 21 tiles and of about 1,024 (R = 4: one launch;
+    """A slice with most of the entries among slices of one entry, of about 20 tiles and of about 1,024 (R = 4: one launch;
     R = 33 and 128: the runs are cut)."""
     rng = np.random.default_rng(R)
     dims = (12, 811, 399)

@@ -629,7 +629,14 @@ static comet_status_t seg_gather_typed(Context *ctx, const int32_t *seg_end, con
   hint.cols = b_rows;
   HeavyArgs *heavy = long_rows && !out_row && b_rows > 0 && R <= 128 ? &hint : nullptr;
   const bool b_ok = aligned16(B) && ldb % PER == 0 && R % PER == 0, c_ok = aligned16(C) && ldc % PER == 0;
-  const bool pad = !b_ok && N >= 2 * b_rows;
+  // The copy moves a row of B twice (0.4 ps per byte and row); a ragged shape saves about 17 ps per entry on the scalar one.
+  const bool pad = !b_ok && N * 40 >= b_rows * R * (int64_t)sizeof(T);
+  // More than 32 pieces are two per lane, which halves the warps on an SM. Long rows of a B that stays in L2 are faster as
+  // two launches of at most 32 (4 M entries in 200,000 rows, 84 MB of B: R = 70 335 -> 262, R = 120 460 -> 381 us), short
+  // ones or a B in DRAM are not (2.9 entries per row: 784 -> 1128 us; 430 MB: 398 -> 527 us). Short rows are faster still
+  // with a column per lane (R = 70: 784 -> 760 us): what costs there is the stores of the ragged rows.
+  const bool split = N >= 8 * M && b_rows * R * (int64_t)sizeof(T) <= (126ll << 20);
+  const bool scalar = R > 32 * PER && R < 128 && N < 4 * M;
   int64_t done = 0;
   while (done < R) {
     SegGatherArgs a{};
@@ -639,8 +646,10 @@ static comet_status_t seg_gather_typed(Context *ctx, const int32_t *seg_end, con
     a.wide_store = c_ok;
     comet_status_t st = COMET_OK;
     const int64_t rem = R - done;
-    if (b_ok || pad) {
-      const int64_t chunk = rem < 128 ? rem : 128, pieces = ceil_div(chunk, PER);
+    if ((b_ok || pad) && !scalar) {
+      int64_t chunk = rem < 128 ? rem : 128;
+      if (chunk > 32 * PER && split && !(b_ok && c_ok && chunk == 64 * PER)) chunk = 32 * PER;
+      const int64_t pieces = ceil_div(chunk, PER);
       a.R = (int32_t)chunk;
       const int64_t p = b_ok ? 0 : b_rows;
       const bool exact = b_ok && c_ok && (pieces & (pieces - 1)) == 0;

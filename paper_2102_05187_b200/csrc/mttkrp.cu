@@ -497,7 +497,7 @@ static comet_status_t mttkrp_chunks(Context *ctx, const MttkrpArgs &base, int64_
   constexpr int PER = 16 / sizeof(T);
   const bool in_ok = aligned16(base.P) && aligned16(base.Q) && base.ldp % PER == 0 && base.ldq % PER == 0 && R % PER == 0;
   const bool out_ok = aligned16(base.out) && base.ldo % PER == 0;
-  const bool pad = !in_ok && 2 * base.N >= p_rows + q_rows;
+  const bool pad = !in_ok && base.N * 40 >= (p_rows + q_rows) * R * (int64_t)sizeof(T);   // as in seg_gather_typed
   int64_t done = 0;
   while (done < R) {
     const int64_t rem = R - done;

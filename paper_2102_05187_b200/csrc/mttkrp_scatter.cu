@@ -22,6 +22,8 @@
 
 #include <stdlib.h>
 
+#include <type_traits>
+
 namespace comet {
 
 struct ScatterArgs {
@@ -91,25 +93,31 @@ __global__ void __launch_bounds__(kScatterThreads) mttkrp_coo_scatter_kernel(con
 // that were seen most often get a slot each (as many as fit), every CTA adds their terms into its own copy and
 // adds that copy into the output once, at the end. Which rows are chosen changes the speed only, not the sums.
 constexpr int kHotThreads = 512;
-// Entries whose rows are in flight per warp (a divisor of 32). An add is a branch, and the compiler moves no load
-// across it, so an unrolled loop of load-add-load-add waits for every row in turn. 100 M entries, R = 32, fp64, leaf mode:
-// 6.43 ms with one entry at a time, 5.68 with 4, 5.76 with 8; the same tensor's middle mode in COO (50 M entries): 3.53
-// -> 2.76 -> 2.75 ms.
-constexpr int kHotBatch = 4;
+// Entries whose rows are in flight per half warp. An add is a branch, and the compiler moves no load across it, so a loop
+// of load-add-load-add waits for every row in turn. What bounds the kernel then is the L1 data pipe (91 % busy, 13
+// wavefronts per entry) and issue: hence entries by broadcast from shared memory instead of five shuffles each, two
+// entries per instruction, ordinary and popular rows apart, and the row of A kept while it stays the same. 100 M entries,
+// R = 32, fp64, leaf mode: one entry per warp at a time 6.43, four in flight 5.68, half warps 4.94 (batches of 1 / 2 / 4:
+// 5.15 / 4.94 / 6.08), the row of A kept 4.69 ms. COO, 50 M entries, modes 2 / 3: 2.80 -> 2.61, 2.74 -> 2.26 ms.
+constexpr int kHotBatch = 2;
 constexpr int kHotCtas = 2;                        // CTAs per SM
 // Entries per warp and step; the warps draw chunk numbers from a counter. Dealt out round-robin instead, the last
 // round is only partly filled: 100 M entries over 9,472 warps take 42 rounds of 256 (2 % idle) but 3 rounds of
 // 4,096 where 2.6 would do (measured, round-robin: 6.70 / 6.76 / 7.88 ms with 256 / 1,024 / 4,096 entries; with the
 // counter 6.43 / 6.44 / 6.45 ms with 256 / 512 / 1,024).
 constexpr int kHotChunk = 256;
-// Shared memory per CTA for the popular rows: 256 rows of 32 columns. Measured on config 5 (leaf frequencies
+// Shared memory per CTA for the popular rows: 320 rows of 32 columns. Measured with the kernel as it was before (an entry
+// per warp) on config 5 (leaf frequencies
 // (k + 100)^-1.5 over 200,000 rows): 32 rows 16.6 ms, 128 rows 6.75 to 8.9 ms depending on where the output
 // matrix happened to be allocated (the next few hundred rows still collide in L2), 256 rows 6.87 ms wherever it
 // was, 384 rows 7.16 ms (an add in shared memory is a compare-and-swap loop of about a dozen instructions, an
 // add in L2 one instruction: past the rows that L2 serialises, more slots cost more than they save).
-constexpr size_t kHotBytes = 64 * 1024;
+// With the kernel as it is (half a warp per entry): 48 / 64 / 80 / 84 KB 5.79 / 4.69 / 4.63 / 4.70 ms; the middle modes of the
+// tensor in COO (50 M entries) 64 -> 80 KB 2.60 -> 2.46 and 2.26 -> 2.15 ms.
+constexpr size_t kHotBytes = 80 * 1024;
 constexpr int64_t kHotMaxRows = 1ll << 24;         // two 32-bit words per output row are allocated for the call
-constexpr int64_t kHotSamples = 1ll << 22;
+// Samples: the rows that count are those with a share of 1e-4 and more, a few dozen hits each (2^22 samples cost 83 us).
+constexpr int64_t kHotSamples = 1ll << 19;
 
 __global__ void sample_rows_kernel(const int32_t *__restrict__ crd, int64_t n, int64_t stride, int32_t *__restrict__ counts) {
   const int64_t p = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * stride;
@@ -144,15 +152,29 @@ __global__ void __launch_bounds__(256) count_histogram_kernel(const int32_t *__r
 
 // *threshold = the lowest bin t such that at most `slots` rows have a count in bin t or above
 __global__ void pick_threshold_kernel(const int32_t *__restrict__ bins, int32_t slots, int32_t *__restrict__ threshold) {
-  __shared__ int32_t s_bins[kCountBins];
-  for (int b = threadIdx.x; b < kCountBins; b += blockDim.x) s_bins[b] = bins[b];
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    int t = kCountBins - 1;
-    int64_t reach = s_bins[t];
-    while (t > 0 && reach + s_bins[t - 1] <= slots) { --t; reach += s_bins[t]; }
-    *threshold = t;
+  // one warp: lane l holds bins 16 l .. 16 l + 15 and learns how many rows lie in the bins of the lanes above
+  constexpr int kOwn = kCountBins / 32;
+  const int lane = threadIdx.x;
+  int32_t own[kOwn], sum = 0;
+#pragma unroll
+  for (int x = 0; x < kOwn; ++x) own[x] = bins[lane * kOwn + x];
+#pragma unroll
+  for (int x = 0; x < kOwn; ++x) sum += own[x];
+  int32_t reach = sum;                             // inclusive suffix sum over the lanes
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const int32_t v = __shfl_down_sync(0xffffffffu, reach, d);
+    if (lane + d < 32) reach += v;
   }
+  reach -= sum;
+  int t = kCountBins;                              // the lowest of this lane's bins that at most `slots` rows reach
+#pragma unroll
+  for (int x = kOwn - 1; x >= 0; --x) {
+    reach += own[x];
+    if (reach <= slots) t = lane * kOwn + x;
+  }
+  t = __reduce_min_sync(0xffffffffu, t);
+  if (lane == 0) *threshold = t < kCountBins ? t : kCountBins - 1;
 }
 
 __global__ void assign_slots_kernel(const int32_t *__restrict__ counts, int64_t rows, const int32_t *__restrict__ threshold,
@@ -191,6 +213,11 @@ __global__ void __launch_bounds__(kHotThreads, kHotCtas) mttkrp_csf_leaf_hot_ker
                                                                                    const int32_t *__restrict__ n_hot, int32_t slots,
                                                                                    unsigned long long *__restrict__ next_chunk) {
   extern __shared__ double s_acc[];                // slots x R
+  __shared__ int4 s_entries[kHotThreads];          // per warp: (value, destination, row of B) of 32 entries
+  __shared__ uint32_t s_rows_a[kHotThreads];
+  int4 *const s_entry = s_entries + (threadIdx.x & ~31);
+  uint32_t *const s_row_a = s_rows_a + (threadIdx.x & ~31);
+  const int g = threadIdx.x & 15, h = (threadIdx.x >> 4) & 1;
   const T *const val = static_cast<const T *>(a.val);
   const T *const A = static_cast<const T *>(a.A), *const B = static_cast<const T *>(a.B);
   const int used = *n_hot < slots ? *n_hot : slots;
@@ -251,34 +278,67 @@ __global__ void __launch_bounds__(kHotThreads, kHotCtas) mttkrp_csf_leaf_hot_ker
       }
       // where the entry's term goes: a slot's row in shared memory (bit 31 set) or the output row's element offset
       const uint32_t dest = qq >= 0 ? 0x80000000u | (uint32_t)(qq * a.R) : (uint32_t)kk * (uint32_t)a.ldacc;
+      // The 32 entries go to shared memory, those of ordinary rows first, and come back by broadcast. A half warp works on
+      // an entry (two columns per lane), so an instruction serves two of them; both are of the same kind but for one pair.
+      const unsigned in = cnt == 32 ? full : (1u << cnt) - 1u;
+      const unsigned hot = __ballot_sync(full, qq >= 0) & in, cold = in & ~hot;
+      const int n_cold = __popc(cold);
+      const unsigned below = (1u << lane) - 1u;
+      const int at = qq >= 0 ? n_cold + __popc(hot & below) : __popc(cold & below);
+      __syncwarp();                                // the entries in front have been read
+      if (lane < cnt) {
+        s_entry[at] = make_int4(__double2loint(vv), __double2hiint(vv), (int)dest, (int)row_b);
+        s_row_a[at] = row_a;
+      }
+      __syncwarp();
       for (int c0 = 0; c0 < a.R; c0 += 32) {
-        const int c = c0 + lane;
-        const bool inb = c < a.R;
-        // the row reads of kHotBatch entries are in flight together (an add is a branch that nothing moves across);
-        // the rows of consecutive entries of a fiber come from L1
-        for (int e0 = 0; e0 < cnt; e0 += kHotBatch) {
-          uint32_t d[kHotBatch];
-          T va[kHotBatch], vb[kHotBatch];
+        const int left = a.R - c0 - g;             // columns from this lane's first one on
+        const int c = left > 0 ? c0 + g : a.R - 1, step = left > 16 ? 16 : 0;
+        const T *const ac = A + c, *const bc = B + c;
+        T a_row[2] = {(T)0, (T)0};                 // this lane's columns of the row of A that was read last, and its offset
+        uint32_t a_at = 0xffffffffu;
+        auto run = [&](int from, int end, auto is_hot) {
+          constexpr bool HOT = decltype(is_hot)::value;
+#pragma unroll 1
+          for (int e0 = from + h; e0 - h < end; e0 += 2 * kHotBatch) {
+            double v[kHotBatch];
+            uint32_t d[kHotBatch];
+            T va[kHotBatch][2], vb[kHotBatch][2];
+            uint32_t ra[kHotBatch];
+            bool same = true;
 #pragma unroll
-          for (int u = 0; u < kHotBatch; ++u) {
-            d[u] = __shfl_sync(full, dest, e0 + u);
-            const uint32_t ra = __shfl_sync(full, row_a, e0 + u), rb = __shfl_sync(full, row_b, e0 + u);
-            va[u] = vb[u] = (T)0;
-            if (inb) {
-              va[u] = __ldg(A + (ra + c));
-              vb[u] = __ldg(B + (rb + c));
+            for (int u = 0; u < kHotBatch; ++u) {  // the row reads of 2 x kHotBatch entries are in flight together
+              const int e = e0 + 2 * u < end ? e0 + 2 * u : end - 1;
+              const int4 en = s_entry[e];
+              const T *const rb = bc + (uint32_t)en.w;
+              ra[u] = s_row_a[e];
+              same = same && ra[u] == a_at;
+              v[u] = __hiloint2double(en.y, en.x);
+              d[u] = (uint32_t)en.z;
+              vb[u][0] = __ldg(rb); vb[u][1] = __ldg(rb + step);
+            }
+            if (!same) {                           // a slice's entries share the row of A: few batches read it again
+#pragma unroll
+              for (int u = 0; u < kHotBatch; ++u) { va[u][0] = __ldg(ac + ra[u]); va[u][1] = __ldg(ac + ra[u] + step); }
+              a_row[0] = va[kHotBatch - 1][0]; a_row[1] = va[kHotBatch - 1][1];
+              a_at = ra[kHotBatch - 1];
+            } else {
+#pragma unroll
+              for (int u = 0; u < kHotBatch; ++u) { va[u][0] = a_row[0]; va[u][1] = a_row[1]; }
+            }
+#pragma unroll
+            for (int u = 0; u < kHotBatch; ++u) {
+              if (e0 + 2 * u < end && left > 0) {
+                const double t0 = v[u] * ((double)va[u][0] * (double)vb[u][0]), t1 = v[u] * ((double)va[u][1] * (double)vb[u][1]);
+                double *const dst = HOT ? &s_acc[(d[u] & 0x7fffffffu) + c] : a.acc + (d[u] + c);
+                atomicAdd(dst, t0);
+                if (step) atomicAdd(dst + 16, t1);
+              }
             }
           }
-#pragma unroll
-          for (int u = 0; u < kHotBatch; ++u) {
-            const double v = __shfl_sync(full, vv, e0 + u);
-            if (inb && e0 + u < cnt) {
-              const double t = v * ((double)va[u] * (double)vb[u]);
-              if (d[u] & 0x80000000u) atomicAdd(&s_acc[(d[u] & 0x7fffffffu) + c], t);
-              else atomicAdd(a.acc + (d[u] + c), t);
-            }
-          }
-        }
+        };
+        run(0, n_cold, std::false_type());
+        run(n_cold, cnt, std::true_type());
       }
     }
   }
@@ -326,7 +386,7 @@ static comet_status_t entries_hot(Context *ctx, const ScatterArgs &a, bool coo, 
     sample_rows_kernel<<<(unsigned)ceil_div(samples, 256), 256, 0, stream>>>(out_crd, a.N, stride, counts);
     const int64_t hist_ctas = ceil_div(rows, 256) < 2 * kSmCount ? ceil_div(rows, 256) : 2 * kSmCount;
     count_histogram_kernel<<<(unsigned)hist_ctas, 256, 0, stream>>>(counts, rows, bins);
-    pick_threshold_kernel<<<1, 256, 0, stream>>>(bins, (int32_t)slots, threshold);
+    pick_threshold_kernel<<<1, 32, 0, stream>>>(bins, (int32_t)slots, threshold);
     assign_slots_kernel<<<(unsigned)ceil_div(rows, 256), 256, 0, stream>>>(counts, rows, threshold, (int32_t)slots, hot_slot, hot_rows, n_hot);
     ctx->launches += 4;
     if (!coo) {

@@ -46,6 +46,8 @@ struct SortedPairs {                 // the output of the pass before
   const uint64_t *keys;
   const uint32_t *pay;
   __device__ __forceinline__ uint64_t key(int64_t i, bool &) const { return __ldcs(keys + i); }
+  __device__ __forceinline__ uint64_t digit_key(int64_t i) const { return __ldcs(keys + i); }
+  static constexpr bool kChecks = false;
   __device__ __forceinline__ uint32_t payload(int64_t i) const { return __ldcs(pay + i); }
 };
 
@@ -55,6 +57,14 @@ struct CooEntries {                  // the first pass: the caller's COO arrays;
   KeyLayout k;
   const uint32_t *val32;             // 32-bit values, or null: the payload is the entry's index
   __device__ __forceinline__ uint64_t key(int64_t i, bool &bad) const { return entry_key<ORDER>(c, k, i, bad); }
+  // For the counts of the first digit: where the last level's coordinate has 8 bits and more, it alone holds them (19.7 M
+  // entries, order 2: the counting launch 55 -> 30 us). The scatter sees every coordinate and checks the range.
+  __device__ __forceinline__ uint64_t digit_key(int64_t i) const {
+    if (k.bits[ORDER - 1] >= 8) return (uint64_t)(uint32_t)__ldcs(c.p[ORDER - 1] + i);
+    bool ignored = false;
+    return entry_key<ORDER>(c, k, i, ignored);
+  }
+  static constexpr bool kChecks = true;
   __device__ __forceinline__ uint32_t payload(int64_t i) const {
     uint32_t p = (uint32_t)i;
     if (val32) p = __ldcs(val32 + i);
@@ -112,16 +122,31 @@ __global__ void scan_apply_kernel(const uint32_t *__restrict__ in, int64_t n, co
   const int64_t base = (int64_t)blockIdx.x * kScanTile + (int64_t)threadIdx.x * kScanItems;
   uint32_t v[kScanItems];
   uint32_t mine = 0;
+  // a thread's eight words are two 16-byte accesses where they are whole and aligned (14.6 -> 8.3 us for 2.5 M words)
+  const bool wide = base + kScanItems <= n && ((reinterpret_cast<uintptr_t>(in) | reinterpret_cast<uintptr_t>(out)) & 15) == 0;
+  if (wide) {
+    *reinterpret_cast<uint4 *>(v) = *reinterpret_cast<const uint4 *>(in + base);
+    *reinterpret_cast<uint4 *>(v + 4) = *reinterpret_cast<const uint4 *>(in + base + 4);
+  } else {
 #pragma unroll
-  for (int t = 0; t < kScanItems; ++t) {
-    v[t] = (base + t < n) ? in[base + t] : 0;
-    mine += v[t];
+    for (int t = 0; t < kScanItems; ++t) v[t] = (base + t < n) ? in[base + t] : 0;
   }
+#pragma unroll
+  for (int t = 0; t < kScanItems; ++t) mine += v[t];
   uint32_t run = sums[blockIdx.x] + block_exclusive_scan(mine, s_warp, nullptr);
 #pragma unroll
   for (int t = 0; t < kScanItems; ++t) {
-    if (base + t < n) out[base + t] = run;
-    run += v[t];
+    const uint32_t x = v[t];
+    v[t] = run;
+    run += x;
+  }
+  if (wide) {
+    *reinterpret_cast<uint4 *>(out + base) = *reinterpret_cast<const uint4 *>(v);
+    *reinterpret_cast<uint4 *>(out + base + 4) = *reinterpret_cast<const uint4 *>(v + 4);
+  } else {
+#pragma unroll
+    for (int t = 0; t < kScanItems; ++t)
+      if (base + t < n) out[base + t] = v[t];
   }
 }
 
@@ -145,26 +170,23 @@ comet_status_t exclusive_scan(Context *ctx, const uint32_t *in, uint32_t *out, i
 // ------------------------------------------------------------------------------------------------ radix sort
 template <class Src>
 __global__ void __launch_bounds__(kSortThreads) radix_histogram_kernel(Src src, int64_t n, int shift, int64_t tiles,
-                                                                       uint32_t *__restrict__ table,
-                                                                       int32_t *__restrict__ status) {
+                                                                       uint32_t *__restrict__ table) {
   __shared__ uint32_t s_cnt[256];
   s_cnt[threadIdx.x] = 0;
   __syncthreads();
   const int64_t base = (int64_t)blockIdx.x * kSortTile;
-  bool bad = false;
   uint64_t k[kSortItems];
   const bool full = base + kSortTile <= n;
 #pragma unroll
   for (int t = 0; t < kSortItems; ++t) {          // unconditional loads: the eight of a thread are in flight together
     const int64_t i = base + (int64_t)t * kSortThreads + threadIdx.x;
-    k[t] = src.key(full || i < n ? i : n - 1, bad);
+    k[t] = src.digit_key(full || i < n ? i : n - 1);
   }
 #pragma unroll
   for (int t = 0; t < kSortItems; ++t) {
     const int64_t i = base + (int64_t)t * kSortThreads + threadIdx.x;
     if (full || i < n) atomicAdd(&s_cnt[(k[t] >> shift) & 255], 1u);
   }
-  if (bad) atomicOr(status + kStatusRange, 1);    // only the pass that forms the keys can see a bad coordinate
   __syncthreads();
   table[(int64_t)threadIdx.x * tiles + blockIdx.x] = s_cnt[threadIdx.x];     // digit-major
 }
@@ -173,7 +195,8 @@ template <class Src>
 __global__ void __launch_bounds__(kSortThreads, 4) radix_scatter_kernel(Src src, uint64_t *__restrict__ kout,
                                                                         uint32_t *__restrict__ pout,
                                                                         const uint32_t *__restrict__ table, int64_t n,
-                                                                        int shift, int64_t tiles) {
+                                                                        int shift, int64_t tiles,
+                                                                        int32_t *__restrict__ status) {
   __shared__ uint32_t s_cnt[kSortWarps][256];     // per-warp digit counts, then where each warp's keys of a digit go
   __shared__ uint32_t s_delta[256];               // global position of digit d's run minus its start inside the tile
   __shared__ uint64_t s_key[kSortTile];           // the tile in sorted order
@@ -189,23 +212,24 @@ __global__ void __launch_bounds__(kSortThreads, 4) radix_scatter_kernel(Src src,
   const int64_t warp_base = tile_base + (int64_t)warp * (32 * kSortItems);
   uint64_t key[kSortItems];
   uint32_t pay[kSortItems];
-  bool ignored = false;
+  bool bad = false;
   if (tile_base + kSortTile <= n) {               // all loads first, none behind a branch
 #pragma unroll
     for (int r = 0; r < kSortItems; ++r) {
       const int64_t i = warp_base + r * 32 + lane;
-      key[r] = src.key(i, ignored);
+      key[r] = src.key(i, bad);
       pay[r] = src.payload(i);
     }
   } else {
 #pragma unroll
     for (int r = 0; r < kSortItems; ++r) {
       const int64_t i = warp_base + r * 32 + lane;
-      key[r] = src.key(i < n ? i : n - 1, ignored);
+      key[r] = src.key(i < n ? i : n - 1, bad);
       pay[r] = src.payload(i < n ? i : n - 1);
       if (i >= n) key[r] = ~0ull;                  // slots past the end rank after every real key of the tile
     }
   }
+  if (Src::kChecks && bad) atomicOr(status + kStatusRange, 1);      // the pass that forms the keys
   __syncthreads();
   uint32_t rank[kSortItems];
   const unsigned lt = (1u << lane) - 1u;
@@ -267,11 +291,11 @@ template <class Src>
 static comet_status_t radix_pass(Context *ctx, const Src &src, uint64_t *kout, uint32_t *pout, int64_t n, int shift,
                                  uint32_t *table, uint32_t *scan_tmp, cudaStream_t s) {
   const int64_t tiles = ceil_div(n, kSortTile);
-  radix_histogram_kernel<Src><<<(unsigned)tiles, kSortThreads, 0, s>>>(src, n, shift, tiles, table, ctx->d_status);
+  radix_histogram_kernel<Src><<<(unsigned)tiles, kSortThreads, 0, s>>>(src, n, shift, tiles, table);
   COMET_LAUNCH_CHECK(ctx);
   comet_status_t st = exclusive_scan(ctx, table, table, 256 * tiles, scan_tmp, nullptr, s);
   if (st != COMET_OK) return st;
-  radix_scatter_kernel<Src><<<(unsigned)tiles, kSortThreads, 0, s>>>(src, kout, pout, table, n, shift, tiles);
+  radix_scatter_kernel<Src><<<(unsigned)tiles, kSortThreads, 0, s>>>(src, kout, pout, table, n, shift, tiles, ctx->d_status);
   COMET_LAUNCH_CHECK(ctx);
   return COMET_OK;
 }

@@ -25,7 +25,7 @@ __device__ __forceinline__ uint64_t entry_key(const CoordPtrs &c, const KeyLayou
   uint64_t key = 0;
 #pragma unroll
   for (int l = 0; l < ORDER; ++l) {
-    bad |= (v[l] < 0) | ((int64_t)v[l] >= k.dim[l]);
+    bad |= (uint32_t)v[l] >= (uint32_t)k.dim[l];          // extents are below 2^31: a negative coordinate is beyond them too
     key |= ((uint64_t)(uint32_t)v[l] & ((1ull << k.bits[l]) - 1)) << k.shift[l];
   }
   return key;

@@ -217,6 +217,7 @@ class SpTensor:
     def __init__(self, handle: Handle, struct: SpTensorStruct, keep=None):
         self.handle = handle
         self.c = struct
+        self._ref = C.byref(struct)          # what the calls pass: made once
         self._keep = keep
 
     @property
@@ -348,26 +349,28 @@ def validate(t: SpTensor):
 
 def spmv(A: SpTensor, x: torch.Tensor, y: torch.Tensor | None = None) -> torch.Tensor:
     _require_cuda(x)
-    rows = A.c.dims[A.c.mode_order[0]]
-    dt = _same_dtype(A, x, y)
+    _same_dtype(A, x, y)
     if y is None:
-        y = torch.empty(rows, dtype=dt, device=x.device)
-    st = A.handle.lib.comet_spmv(A.handle._h, C.byref(A.c), x.data_ptr(), y.data_ptr(), _raw_stream())
-    A.handle.check(st, "comet_spmv")
+        y = x.new_empty(A.c.dims[A.c.mode_order[0]])
+    h = A.handle
+    st = h.lib.comet_spmv(h._h, A._ref, x.data_ptr(), y.data_ptr(), _raw_stream())
+    if st:
+        h.check(st, "comet_spmv")
     return y
 
 
 def spmm(A: SpTensor, B: torch.Tensor, out: torch.Tensor | None = None) -> torch.Tensor:
     _require_cuda(B)
-    assert B.dim() == 2 and B.stride(1) == 1
-    rows = A.c.dims[A.c.mode_order[0]]
+    ldb, step = B.stride()
+    assert step == 1
     R = B.shape[1]
-    dt = _same_dtype(A, B, out)
+    _same_dtype(A, B, out)
     if out is None:
-        out = torch.empty((rows, R), dtype=dt, device=B.device)
-    st = A.handle.lib.comet_spmm(A.handle._h, C.byref(A.c), B.data_ptr(), R, B.stride(0), out.data_ptr(), out.stride(0),
-                                 _raw_stream())
-    A.handle.check(st, "comet_spmm")
+        out = B.new_empty((A.c.dims[A.c.mode_order[0]], R))
+    h = A.handle
+    st = h.lib.comet_spmm(h._h, A._ref, B.data_ptr(), R, ldb, out.data_ptr(), out.stride(0), _raw_stream())
+    if st:
+        h.check(st, "comet_spmm")
     return out
 
 
@@ -408,7 +411,7 @@ def ttv(X: SpTensor, mode: int, v: torch.Tensor, Y: SpTensor | None = None) -> S
     _same_dtype(X, v)
     if Y is None:
         Y = ttv_symbolic(X, mode)
-    st = X.handle.lib.comet_ttv(X.handle._h, C.byref(X.c), mode, v.data_ptr(), C.byref(Y.c), _raw_stream())
+    st = X.handle.lib.comet_ttv(X.handle._h, X._ref, mode, v.data_ptr(), Y._ref, _raw_stream())
     X.handle.check(st, "comet_ttv")
     return Y
 
@@ -430,7 +433,7 @@ def ttm(X: SpTensor, mode: int, U: torch.Tensor, Y: SpTensor | None = None) -> S
     _same_dtype(X, U)
     if Y is None:
         Y = ttm_symbolic(X, mode, R)
-    st = X.handle.lib.comet_ttm(X.handle._h, C.byref(X.c), mode, U.data_ptr(), R, U.stride(0), C.byref(Y.c), _raw_stream())
+    st = X.handle.lib.comet_ttm(X.handle._h, X._ref, mode, U.data_ptr(), R, U.stride(0), Y._ref, _raw_stream())
     X.handle.check(st, "comet_ttm")
     return Y
 
@@ -449,7 +452,7 @@ def mttkrp(X: SpTensor, mode: int, factors, out: torch.Tensor | None = None) -> 
     assert len(factors) == order
     h_f = (C.c_void_p * order)(*[0 if (m == mode or f is None) else f.data_ptr() for m, f in enumerate(factors)])
     h_ld = (C.c_int64 * order)(*[0 if (m == mode or f is None) else f.stride(0) for m, f in enumerate(factors)])
-    st = X.handle.lib.comet_mttkrp(X.handle._h, C.byref(X.c), mode, h_f, h_ld, R, out.data_ptr(), out.stride(0), _raw_stream())
+    st = X.handle.lib.comet_mttkrp(X.handle._h, X._ref, mode, h_f, h_ld, R, out.data_ptr(), out.stride(0), _raw_stream())
     X.handle.check(st, "comet_mttkrp")
     return out
 

@@ -33,7 +33,6 @@ struct SegDotArgs {
   int64_t num_tiles;
   double *carry_val;
   int32_t *carry_seg;
-  int32_t *run_count;       // may be NULL: the word behind carry_seg that counts cut runs of carries, zeroed by tile 0
   unsigned int *ctas_done;  // tile kernel only, may be NULL: counter (zero between calls) that lets the CTA which
                             // finishes last add the carries itself, so that a small problem is ONE launch
 };
@@ -154,7 +153,6 @@ __global__ void __launch_bounds__(THREADS) seg_dot_kernel(const SegDotArgs a) {
   const int64_t total = a.M + a.N;
   const int64_t d0 = tile * ITEMS;
   const int64_t d1 = (d0 + ITEMS < total) ? d0 + ITEMS : total;
-  if (tile == 0 && tid == 0 && a.run_count) *a.run_count = 0;
   if (tid < 64) {          // warps 0 and 1 locate the two ends of the tile, 32 probes per round each
     const int64_t split = merge_path_segments_coop<32>(a.seg_end, a.M, a.N, tid < 32 ? d0 : d1, tid & 31, 0xffffffffu);
     if ((tid & 31) == 0) {
@@ -323,7 +321,6 @@ seg_dot_resident_kernel(const SegDotArgs a, const int32_t *__restrict__ splits, 
     }
   };
 
-  if (t == 0 && tid == 0) *a.run_count = 0;
   if (t < a.num_tiles) fetch(t, __ldg(splits + t), __ldg(splits + t + 1));
   if (t + stride < a.num_tiles) { n_i0 = __ldg(splits + t + stride); n_i1 = __ldg(splits + t + stride + 1); }
 
@@ -400,7 +397,6 @@ seg_dot_stream_kernel(const SegDotArgs a, int64_t x_len, int32_t span, unsigned 
       if (cap < hi) hi = cap;
     }
     int64_t s = lo;
-    if (tile == 0 && lane == 0) *a.run_count = 0;
     if (tile == 0)                                       // leading empty segments (end == 0) belong to nobody else
       for (int64_t q = lane; q < s; q += 32) y[a.out_row ? (int64_t)__ldg(a.out_row + q) : q] = (T)0;
 
@@ -542,7 +538,6 @@ seg_dot_stream2_kernel(const SegDotArgs a, int64_t x_len, int32_t span, unsigned
       if (cap < hi) hi = cap;
     }
     int64_t s = lo;
-    if (tile == 0 && lane == 0) *a.run_count = 0;
     if (tile == 0)
       for (int64_t q = lane; q < s; q += 32) y[a.out_row ? (int64_t)__ldg(a.out_row + q) : q] = (T)0;
 
@@ -666,20 +661,19 @@ static comet_status_t launch_dot(Context *ctx, SegDotArgs a, cudaStream_t stream
   const int64_t total = a.M + a.N;
   a.num_tiles = ceil_div(total, (int64_t)THREADS * IPT - kDotOwn);
   const size_t val_bytes = align_up((size_t)a.num_tiles * sizeof(double), 256);
-  const size_t seg_bytes = align_up((size_t)carry_seg_words(a.num_tiles) * sizeof(int32_t), 256);
+  const size_t seg_bytes = align_up((size_t)a.num_tiles * sizeof(int32_t), 256);
   char *scratch = (char *)scratch_get(ctx, val_bytes + seg_bytes, stream);
   if (!scratch) return COMET_ERR_ALLOC;
   a.carry_val = (double *)scratch;
   a.carry_seg = (int32_t *)(scratch + val_bytes);
-  a.run_count = a.carry_seg + a.num_tiles;
   // up to a few thousand tiles the last CTA adds the carries itself: one launch instead of two
   const bool fused = a.num_tiles > 1 && a.num_tiles <= 4096;
   a.ctas_done = fused ? reinterpret_cast<unsigned int *>(ctx->d_status + 35) : nullptr;
   seg_dot_kernel<T, THREADS, IPT, kDotOwn><<<(unsigned)a.num_tiles, THREADS, 0, stream>>>(a);
   COMET_LAUNCH_CHECK(ctx);
   if (a.num_tiles > 1 && !fused) {
-    COMET_LAUNCHED(ctx, carry_fixup_launch(sizeof(T) == 4 ? COMET_F32 : COMET_F64, a.carry_val, a.carry_seg, a.num_tiles, 1,
-                                           1, a.y, 1, a.out_row, true, stream));
+    carry_fixup_launch(sizeof(T) == 4 ? COMET_F32 : COMET_F64, a.carry_val, a.carry_seg, a.num_tiles, 1, 1, a.y, 1, a.out_row, false, stream);
+  COMET_LAUNCH_CHECK(ctx);
   }
   return COMET_OK;
 }
@@ -698,13 +692,12 @@ static comet_status_t launch_resident(Context *ctx, SegDotArgs a, int64_t x_len,
   const int64_t total = a.M + a.N;
   a.num_tiles = ceil_div(total, (int64_t)RL::TILE);
   const size_t val_bytes = align_up((size_t)a.num_tiles * sizeof(double), 256);
-  const size_t seg_bytes = align_up((size_t)carry_seg_words(a.num_tiles) * sizeof(int32_t), 256);
+  const size_t seg_bytes = align_up((size_t)a.num_tiles * sizeof(int32_t), 256);
   const size_t split_bytes = align_up((size_t)(a.num_tiles + 1) * sizeof(int32_t), 256);
   char *scratch = (char *)scratch_get(ctx, val_bytes + seg_bytes + split_bytes, stream);
   if (!scratch) return COMET_ERR_ALLOC;
   a.carry_val = (double *)scratch;
   a.carry_seg = (int32_t *)(scratch + val_bytes);
-  a.run_count = a.carry_seg + a.num_tiles;
   int32_t *splits = (int32_t *)(scratch + val_bytes + seg_bytes);
   tile_split_kernel<<<(unsigned)ceil_div((a.num_tiles + 1) * 32, 256), 256, 0, stream>>>(a.seg_end, a.M, a.N, RL::TILE,
                                                                                        a.num_tiles, splits);
@@ -716,8 +709,8 @@ static comet_status_t launch_resident(Context *ctx, SegDotArgs a, int64_t x_len,
   const int64_t ctas = ceil_div(a.num_tiles, kResVC) < kSmCount ? ceil_div(a.num_tiles, kResVC) : kSmCount;
   kernel<<<(unsigned)ctas, kResVC * kResThreads, smem, stream>>>(a, splits, x_len, x_bytes);
   COMET_LAUNCH_CHECK(ctx);
-  COMET_LAUNCHED(ctx, carry_fixup_launch(sizeof(T) == 4 ? COMET_F32 : COMET_F64, a.carry_val, a.carry_seg, a.num_tiles, 1,
-                                         1, a.y, 1, a.out_row, true, stream));
+  carry_fixup_launch(sizeof(T) == 4 ? COMET_F32 : COMET_F64, a.carry_val, a.carry_seg, a.num_tiles, 1, 1, a.y, 1, a.out_row, false, stream);
+  COMET_LAUNCH_CHECK(ctx);
   return COMET_OK;
 }
 
@@ -737,12 +730,11 @@ static comet_status_t launch_stream(Context *ctx, SegDotArgs a, int64_t x_len, b
   if (const char *e = getenv("COMET_STREAM_SPAN")) { const int v = atoi(e); if (v >= 128 && v % 128 == 0) span = v; }
   a.num_tiles = ceil_div(a.N, span);
   const size_t val_bytes = align_up((size_t)a.num_tiles * sizeof(double), 256);
-  const size_t seg_bytes = align_up((size_t)carry_seg_words(a.num_tiles) * sizeof(int32_t), 256);
+  const size_t seg_bytes = align_up((size_t)a.num_tiles * sizeof(int32_t), 256);
   char *scratch = (char *)scratch_get(ctx, val_bytes + seg_bytes + 256, stream);
   if (!scratch) return COMET_ERR_ALLOC;
   a.carry_val = (double *)scratch;
   a.carry_seg = (int32_t *)(scratch + val_bytes);
-  a.run_count = a.carry_seg + a.num_tiles;
   const int64_t ctas = ceil_div(a.num_tiles, 32) < kSmCount ? ceil_div(a.num_tiles, 32) : kSmCount;
   if (pairs) {
     // span counter and finished-CTA counter live in the handle and are zero between calls (the kernel's last
@@ -757,8 +749,8 @@ static comet_status_t launch_stream(Context *ctx, SegDotArgs a, int64_t x_len, b
       seg_dot_stream2_kernel<T, false><<<(unsigned)ctas, 1024, 0, stream>>>(a, x_len, (int32_t)span, next_tile, ctas_done);
     }
     COMET_LAUNCH_CHECK(ctx);
-    COMET_LAUNCHED(ctx, carry_fixup_launch(sizeof(T) == 4 ? COMET_F32 : COMET_F64, a.carry_val, a.carry_seg, a.num_tiles, 1,
-                                           1, a.y, 1, a.out_row, true, stream));
+    carry_fixup_launch(sizeof(T) == 4 ? COMET_F32 : COMET_F64, a.carry_val, a.carry_seg, a.num_tiles, 1, 1, a.y, 1, a.out_row, false, stream);
+  COMET_LAUNCH_CHECK(ctx);
     return COMET_OK;
   }
   unsigned long long *next_tile = (unsigned long long *)(scratch + val_bytes + seg_bytes);
@@ -771,8 +763,8 @@ static comet_status_t launch_stream(Context *ctx, SegDotArgs a, int64_t x_len, b
     seg_dot_stream_kernel<T, false><<<(unsigned)ctas, 1024, 0, stream>>>(a, x_len, (int32_t)span, next_tile);
   }
   COMET_LAUNCH_CHECK(ctx);
-  COMET_LAUNCHED(ctx, carry_fixup_launch(sizeof(T) == 4 ? COMET_F32 : COMET_F64, a.carry_val, a.carry_seg, a.num_tiles, 1,
-                                         1, a.y, 1, a.out_row, true, stream));
+  carry_fixup_launch(sizeof(T) == 4 ? COMET_F32 : COMET_F64, a.carry_val, a.carry_seg, a.num_tiles, 1, 1, a.y, 1, a.out_row, false, stream);
+  COMET_LAUNCH_CHECK(ctx);
   return COMET_OK;
 }
 

@@ -137,7 +137,7 @@ seg_gather_kernel(const SegGatherArgs a, const HeavyArgs h) {
   if (tile >= a.num_tiles) return;                       // whole groups leave together
   const uint32_t smem = smem_u32(smem_raw) + worker * RingLayout<L, false>::kWorkerBytes;
   const L ln(a.R, a.wide_store);
-  if (tile == 0 && ln.g == 0) a.carry_seg[a.num_tiles] = 0;   // no cut run of carries listed yet (carry_fixup_role)
+  if (tile == 0) clear_piece_counts(a.carry_seg, a.num_tiles, ln.g, LPN);
 
   const int64_t total = a.M + a.N;
   const int64_t d0 = tile * a.tile_items;
@@ -203,13 +203,13 @@ seg_gather_kernel(const SegGatherArgs a, const HeavyArgs h) {
 // a run is added to the segment's row, which has no other writer by now. One thread per tile and column: the thread at
 // the head of a run adds it up, several tiles in flight. What bounds this is latency, and a run of thousands of tiles
 // (a slice that holds most of a tensor) would be a serial chain: a run of more than kRunShort tiles is therefore added
-// by the whole CTA of its head, and in large problems (cut) runs are cut at every multiple of kRunPiece tiles: a
-// piece's sum stays in the slot of its first tile and carry_runs_kernel adds the pieces, a CTA per run. Every order is
-// fixed. Measured, runs followed by one thread -> as here: 0.85 M entries, R = 4, 60 % of them in one slice 918 -> 84 us
-// (whole CSF MTTKRP); 14.9 M entries, R = 32 3.05 -> 0.40 ms (COO); 100 M entries, heaviest slice 0.5 % 2.90 -> 2.86 ms.
+// by the whole CTA of its head, and (cut) runs are cut at every multiple of kRunPiece tiles: a piece's sum stays in the
+// slot of its first tile, and the CTA that finishes the last piece of a run adds the pieces (each counts itself done; none
+// waits). Every order is fixed. Measured, runs followed by one thread -> as here: 0.85 M entries, R = 4, 60 % of them in one
+// slice 918 -> 84 us (whole CSF MTTKRP); 14.9 M entries, R = 32 3.05 -> 0.39 ms (COO); 100 M entries, heaviest slice 0.5 %
+// 2.90 -> 2.84 ms.
 constexpr int kRunFirst = 4;
 constexpr int kRunShort = kRunFirst + 8;
-constexpr int kRunPiece = 1024;
 
 struct FixupArgs {
   double *carry_val;
@@ -219,7 +219,8 @@ struct FixupArgs {
   void *C;
   int64_t ldc;
   const int32_t *out_row;
-  int32_t *run_count, *run_list;                 // the cut runs (NULL: runs are not cut)
+  int32_t *done;                                 // per multiple of kRunPiece: pieces of the run first cut there that are summed
+                                                 // (zero at the start; NULL: runs are not cut)
 };
 
 template <class T>
@@ -241,7 +242,7 @@ __device__ __forceinline__ double cta_slot_sum(const FixupArgs &f, int64_t first
     for (int32_t q = g; q < count; q += 8 * G) {           // eight slots in flight, the last ones guarded
       double v[8];
 #pragma unroll
-      for (int u = 0; u < 8; ++u) v[u] = q + u * G < count ? __ldcs(src + (int64_t)(q + u * G) * stride) : 0.0;
+      for (int u = 0; u < 8; ++u) v[u] = q + u * G < count ? __ldcg(src + (int64_t)(q + u * G) * stride) : 0.0;
 #pragma unroll
       for (int u = 0; u < 8; ++u) sum += v[u];
     }
@@ -255,6 +256,47 @@ __device__ __forceinline__ double cta_slot_sum(const FixupArgs &f, int64_t first
   return sum;
 }
 
+// A part of a cut run is in its slot (tile `first`, written by threads of this CTA): counts it, and if it was the last part
+// of the run adds them all up. A run of `pieces` cuts has pieces + 1 parts: its head's and one from every cut on.
+template <class T>
+__device__ __forceinline__ void finish_piece(const FixupArgs &f, int32_t first, int32_t seg, double *s_part, int32_t *s_old) {
+  auto cut_at = [&](int64_t m) {                 // the run is cut at multiple m
+    const int64_t t = m * kRunPiece;
+    return m > 0 && t < f.num_tiles && __ldg(f.carry_seg + t) == seg && __ldg(f.carry_seg + t - 1) == seg;
+  };
+  __threadfence();
+  __syncthreads();
+  const int32_t here = first / kRunPiece;
+  int32_t back = 0, ahead = 0, more;
+  do {                                           // cuts at `here` and below, and above
+    more = __syncthreads_count(cut_at((int64_t)here - back - (int32_t)threadIdx.x));
+    back += more;
+  } while (more == kBlockThreads);
+  do {
+    more = __syncthreads_count(cut_at((int64_t)here + 1 + ahead + threadIdx.x));
+    ahead += more;
+  } while (more == kBlockThreads);
+  // a head that sits on a multiple is no cut itself; a head inside a piece sees the cuts above it only
+  const int32_t m1 = here + 1 - back, pieces = back + ahead;
+  if (threadIdx.x == 0) *s_old = atomicAdd(f.done + m1, 1);
+  __syncthreads();
+  const bool last = *s_old == pieces;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  const int32_t second = m1 * kRunPiece;
+  int32_t lead = 0;                              // tiles of the head's part
+  do {
+    const int32_t t = second - 1 - lead - (int32_t)threadIdx.x;
+    more = __syncthreads_count(t >= 0 && __ldg(f.carry_seg + t) == seg);
+    lead += more;
+  } while (more == kBlockThreads);
+  const double sum = cta_slot_sum(f, second, kRunPiece, pieces, s_part);
+  if (threadIdx.x < f.R)
+    add_to_row<T>(f, seg, threadIdx.x, __ldcg(f.carry_val + (int64_t)(second - lead) * f.carry_ld + threadIdx.x) + sum);
+  __syncthreads();
+}
+
 // `block` of fixup_blocks() CTAs: a thread per tile and pair of columns (half as many CTAs as with a column each: 27 ->
 // 24 us for 37,000 tiles of 64 columns). LONG: long runs are possible.
 __host__ __device__ __forceinline__ int32_t fixup_tiles(int32_t R) { return kBlockThreads / ((R + 1) / 2); }   // per CTA
@@ -264,8 +306,8 @@ __device__ __forceinline__ void carry_fixup_role(const FixupArgs &f, int64_t blo
   const int32_t per = (f.R + 1) / 2, G = fixup_tiles(f.R);      // R is at most 128
   const int32_t g = threadIdx.x / per, c = 2 * (threadIdx.x - g * per);
   const int32_t tile = (int32_t)block * G + g;
-  const bool cut = LONG && f.run_count != nullptr, two = c + 1 < f.R;
-  bool is_long = false;
+  const bool cut = LONG && f.done != nullptr, two = c + 1 < f.R;
+  bool is_long = false, is_piece = false;        // is_piece: this tile's sum is a part of a cut run
   if (g < G && tile < f.num_tiles) {
     const int32_t seg_before = tile > 0 ? __ldg(f.carry_seg + tile - 1) : -2;
     const int32_t seg = __ldg(f.carry_seg + tile);
@@ -311,22 +353,26 @@ __device__ __forceinline__ void carry_fixup_role(const FixupArgs &f, int64_t blo
           f.carry_val[(int64_t)tile * f.carry_ld + c] = sum.x;
           if (two) f.carry_val[(int64_t)tile * f.carry_ld + c + 1] = sum.y;
         }
-        if (head && on && c == 0) f.run_list[atomicAdd(f.run_count, 1)] = tile;
+        is_piece = !head || on;
       }
     }
   }
   if constexpr (LONG) {
-    if (!__syncthreads_or(is_long)) return;
+    if (!__syncthreads_or(is_long || is_piece)) return;
     __shared__ double s_part[kBlockThreads];
-    __shared__ int32_t s_long[kBlockThreads], s_longs;
+    __shared__ int32_t s_long[kBlockThreads], s_longs, s_old;
     if (threadIdx.x == 0) s_longs = 0;
     __syncthreads();
-    if (is_long && c == 0) s_long[atomicAdd(&s_longs, 1)] = tile;
+    if ((is_long || is_piece) && c == 0) s_long[atomicAdd(&s_longs, 1)] = is_long ? tile : ~tile;
     __syncthreads();
     const int32_t longs = s_longs;
     for (int32_t x = 0; x < longs; ++x) {
-      const int32_t first = s_long[x];
+      const int32_t first = s_long[x] < 0 ? ~s_long[x] : s_long[x];
       const int32_t seg = __ldg(f.carry_seg + first);
+      if (s_long[x] < 0) {
+        finish_piece<T>(f, first, seg, s_part, &s_old);
+        continue;
+      }
       const int32_t edge = cut ? (first / kRunPiece + 1) * kRunPiece : f.num_tiles;
       const int32_t limit = edge < f.num_tiles ? edge : f.num_tiles;
       int32_t count = kRunShort, more;
@@ -341,8 +387,10 @@ __device__ __forceinline__ void carry_fixup_role(const FixupArgs &f, int64_t blo
         const bool on = limit < f.num_tiles && first + count == limit && __ldg(f.carry_seg + limit) == seg;
         if (head && !on) add_to_row<T>(f, seg, threadIdx.x, sum);
         else f.carry_val[(int64_t)first * f.carry_ld + threadIdx.x] = sum;
-        if (head && on && threadIdx.x == 0) f.run_list[atomicAdd(f.run_count, 1)] = first;
+        if (threadIdx.x == 0) s_old = head && !on;
       }
+      __syncthreads();
+      if (!s_old) finish_piece<T>(f, first, seg, s_part, &s_old);
       __syncthreads();
     }
   }
@@ -351,28 +399,6 @@ __device__ __forceinline__ void carry_fixup_role(const FixupArgs &f, int64_t blo
 template <class T>
 __global__ void __launch_bounds__(kBlockThreads) carry_fixup_kernel(const FixupArgs f) {
   carry_fixup_role<T, true>(f, blockIdx.x);
-}
-
-// The cut runs, a CTA per run (the order of the list does not matter: every run has a row of its own).
-template <class T>
-__global__ void __launch_bounds__(kBlockThreads) carry_runs_kernel(const FixupArgs f) {
-  __shared__ double s_part[kBlockThreads];
-  const int32_t runs = __ldcg(f.run_count);
-  for (int32_t r = blockIdx.x; r < runs; r += gridDim.x) {
-    const int32_t first = f.run_list[r];
-    const int32_t seg = __ldg(f.carry_seg + first);
-    const int32_t second = (first / kRunPiece + 1) * kRunPiece;
-    int32_t pieces = 0, more;                    // behind the first one
-    do {
-      const int64_t at = second + (int64_t)(pieces + threadIdx.x) * kRunPiece;
-      more = __syncthreads_count(at < f.num_tiles && __ldg(f.carry_seg + at) == seg);
-      pieces += more;
-    } while (more == kBlockThreads);
-    const double sum = cta_slot_sum(f, second, kRunPiece, pieces, s_part);
-    if (threadIdx.x < f.R)
-      add_to_row<T>(f, seg, threadIdx.x, __ldcs(f.carry_val + (int64_t)first * f.carry_ld + threadIdx.x) + sum);
-    __syncthreads();
-  }
 }
 
 static int64_t fixup_blocks(int64_t num_tiles, int32_t R) { return ceil_div(num_tiles, fixup_tiles(R)); }
@@ -387,24 +413,15 @@ __global__ void __launch_bounds__(kBlockThreads) spmm_fixups_kernel(const HeavyA
   else carry_fixup_role<T, false>(f, (int64_t)blockIdx.x - heavy_blocks);
 }
 
-int64_t carry_seg_words(int64_t num_tiles) { return num_tiles + 1 + num_tiles / kRunPiece + 1; }
+int64_t carry_seg_words(int64_t num_tiles) { return num_tiles + num_tiles / kRunPiece + 2; }
 
-int carry_fixup_launch(int dtype, double *carry_val, int32_t *carry_seg, int64_t num_tiles, int32_t R, int32_t carry_ld,
-                       void *C, int64_t ldc, const int32_t *out_row, bool cut_runs, cudaStream_t stream) {
-  // Runs are cut where one CTA would take too long over the longest possible one (it adds about 4 G carries a second:
-  // 65 us for 2^18) and the second launch (2 to 3 us) is small against the contraction.
-  const bool cut = cut_runs && num_tiles * R > (1ll << 18) && num_tiles > 2 * kRunPiece;
-  const FixupArgs f{carry_val, carry_seg, (int32_t)num_tiles, R, carry_ld, C, ldc, out_row,
-                    cut ? carry_seg + num_tiles : nullptr, cut ? carry_seg + num_tiles + 1 : nullptr};
+void carry_fixup_launch(int dtype, double *carry_val, int32_t *carry_seg, int64_t num_tiles, int32_t R, int32_t carry_ld,
+                        void *C, int64_t ldc, const int32_t *out_row, bool cut_runs, cudaStream_t stream) {
+  const bool cut = cut_runs && num_tiles > 2 * kRunPiece;
+  const FixupArgs f{carry_val, carry_seg, (int32_t)num_tiles, R, carry_ld, C, ldc, out_row, cut ? carry_seg + num_tiles : nullptr};
   const unsigned blocks = (unsigned)fixup_blocks(num_tiles, R);
   if (dtype == COMET_F32) carry_fixup_kernel<float><<<blocks, kBlockThreads, 0, stream>>>(f);
   else carry_fixup_kernel<double><<<blocks, kBlockThreads, 0, stream>>>(f);
-  if (!cut) return 1;
-  const int64_t most = num_tiles / kRunPiece + 1;
-  const unsigned run_blocks = (unsigned)(most < kSmCount ? most : kSmCount);
-  if (dtype == COMET_F32) carry_runs_kernel<float><<<run_blocks, kBlockThreads, 0, stream>>>(f);
-  else carry_runs_kernel<double><<<run_blocks, kBlockThreads, 0, stream>>>(f);
-  return 2;
 }
 
 template <class T>
@@ -612,7 +629,7 @@ static comet_status_t launch_one(Context *ctx, SegGatherArgs a, HeavyArgs *heavy
       if (st != COMET_OK) return st;
       const int heavy_blocks = kSmCount * 8;
       const unsigned fix_blocks = (unsigned)(heavy_blocks + fixup_blocks(a.num_tiles, a.R));
-      const FixupArgs f{a.carry_val, a.carry_seg, (int32_t)a.num_tiles, a.R, a.carry_ld, a.C, a.ldc, nullptr, nullptr, nullptr};
+      const FixupArgs f{a.carry_val, a.carry_seg, (int32_t)a.num_tiles, a.R, a.carry_ld, a.C, a.ldc, nullptr, nullptr};
       spmm_fixups_kernel<T><<<fix_blocks, kBlockThreads, 0, stream>>>(h, heavy_blocks, f);
       COMET_LAUNCH_CHECK(ctx);
       return COMET_OK;
@@ -621,9 +638,8 @@ static comet_status_t launch_one(Context *ctx, SegGatherArgs a, HeavyArgs *heavy
   st = a.out_row ? launch_mapped<T, LPN, CPL, VEC, RAGGED, true, false>(ctx, a, h, blocks, stream)
                  : launch_mapped<T, LPN, CPL, VEC, RAGGED, false, false>(ctx, a, h, blocks, stream);
   if (st != COMET_OK) return st;
-  COMET_LAUNCHED(ctx, carry_fixup_launch(sizeof(T) == 4 ? COMET_F32 : COMET_F64, a.carry_val, a.carry_seg, a.num_tiles, a.R,
-                                         a.carry_ld, a.C, a.ldc, a.out_row, a.out_row == nullptr || a.num_tiles * a.R > (1ll << 20),
-                                         stream));
+  carry_fixup_launch(kDtype, a.carry_val, a.carry_seg, a.num_tiles, a.R, a.carry_ld, a.C, a.ldc, a.out_row, true, stream);
+  COMET_LAUNCH_CHECK(ctx);
   return COMET_OK;
 }
 

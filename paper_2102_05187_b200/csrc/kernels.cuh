@@ -112,11 +112,11 @@ void *owner_alloc(Context *ctx, void *owner, size_t bytes, cudaStream_t stream);
 void owner_release(Context *ctx, void *owner, cudaStream_t stream);
 
 // Carry fix-up shared by all contraction kernels (defined in contract_vec.cu): adds the per-tile open sums
-// carry_val[tile, 0..R) onto row carry_seg[tile] of C (mapped through out_row when given); R is at most 128. Long runs
-// are cut in large problems (cut_runs): carry_seg then has carry_seg_words(num_tiles) words and the kernel that writes
-// it leaves a 0 in word num_tiles. Returns the number of launches made on `stream`; the caller checks for errors.
+// carry_val[tile, 0..R) onto row carry_seg[tile] of C (mapped through out_row when given); R is at most 128. cut_runs: runs
+// of very many tiles are cut; carry_seg then has carry_seg_words(num_tiles) words and the kernel that writes it clears those
+// behind the tiles (clear_piece_counts). One launch on `stream`; the caller checks for errors.
 int64_t carry_seg_words(int64_t num_tiles);
-int carry_fixup_launch(int dtype, double *carry_val, int32_t *carry_seg, int64_t num_tiles, int32_t R, int32_t carry_ld,
-                       void *C, int64_t ldc, const int32_t *out_row, bool cut_runs, cudaStream_t stream);
+void carry_fixup_launch(int dtype, double *carry_val, int32_t *carry_seg, int64_t num_tiles, int32_t R, int32_t carry_ld,
+                        void *C, int64_t ldc, const int32_t *out_row, bool cut_runs, cudaStream_t stream);
 
 }  // namespace comet

@@ -124,7 +124,7 @@ __global__ void __launch_bounds__(kBlockThreads, (CPL * VEC * sizeof(T) <= 16 ? 
   using P = CooPolicy<T, LPN, CPL, VEC, RAGGED>;
   const uint32_t smem = smem_u32(smem_raw) + worker * RingLayout<L, true>::kWorkerBytes;
   const L ln(a.R, a.wide_store);
-  if (tile == 0 && ln.g == 0) a.carry_seg[a.num_tiles] = 0;   // no cut run of carries listed yet
+  if (tile == 0) clear_piece_counts(a.carry_seg, a.num_tiles, ln.g, LPN);
 
   const int64_t j0 = tile * a.tile_items;
   const int64_t j1 = (j0 + a.tile_items < a.N) ? j0 + a.tile_items : a.N;
@@ -402,7 +402,7 @@ __global__ void __launch_bounds__(kBlockThreads, (CPL * VEC * sizeof(T) <= 16 ? 
   const uint32_t smem = smem_u32(smem_raw) + worker * RingLayout<L, false>::kWorkerBytes;
   const uint32_t flags = smem_u32(smem_raw) + (uint32_t)RingLayout<L, false>::kBlockBytes + worker * kCsfWorkerBytes;
   const L ln(a.R, a.wide_store);
-  if (tile == 0 && ln.g == 0) a.carry_seg[a.num_tiles] = 0;   // no cut run of carries listed yet
+  if (tile == 0) clear_piece_counts(a.carry_seg, a.num_tiles, ln.g, LPN);
 
   // A tile is a span of the merge list of fiber-end markers and leaf positions (equal work per tile: an entry
   // costs a gather, a fiber another one). It owns the leaf entries of the span and the fibers whose LAST entry
@@ -485,8 +485,8 @@ static comet_status_t launch_mttkrp(Context *ctx, MttkrpArgs a, int64_t p_pad, i
   kernel<<<blocks, kBlockThreads, smem, stream>>>(a);
   COMET_LAUNCH_CHECK(ctx);
   if (CSF && a.level1) return COMET_OK;
-  COMET_LAUNCHED(ctx, carry_fixup_launch(sizeof(T) == 4 ? COMET_F32 : COMET_F64, a.carry_val, a.carry_seg, a.num_tiles, a.R,
-                                         a.carry_ld, a.out, a.ldo, CSF ? a.crd0 : nullptr, true, stream));
+  carry_fixup_launch(kDtype, a.carry_val, a.carry_seg, a.num_tiles, a.R, a.carry_ld, a.out, a.ldo, CSF ? a.crd0 : nullptr, true, stream);
+  COMET_LAUNCH_CHECK(ctx);
   return COMET_OK;
 }
 

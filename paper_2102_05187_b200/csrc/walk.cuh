@@ -226,6 +226,13 @@ template <class T_, int LPN_, int CPL_, int VEC_, bool RAGGED_ = false> struct L
   }
 };
 
+// The words behind carry_seg in which the carry fix-up counts the parts of cut runs (contract_vec.cu): cleared by the first
+// tile's worker.
+constexpr int kRunPiece = 1024;                  // tiles after which a run of carries is cut
+__device__ __forceinline__ void clear_piece_counts(int32_t *carry_seg, int64_t num_tiles, int g, int lanes) {
+  for (int64_t x = g; x < num_tiles / kRunPiece + 2; x += lanes) carry_seg[num_tiles + x] = 0;
+}
+
 // Shared memory of one worker: the entry ring, then (when the policy stages an aux word) the side ring.
 template <class L, bool AUX> struct RingLayout {
   static constexpr int kEntryBytes = 2 * L::kChunk * 16;

@@ -202,14 +202,20 @@ seg_gather_kernel(const SegGatherArgs a, const HeavyArgs h) {
 // Adds the carries onto the stored rows. The tiles that stopped inside one segment are consecutive (a run); the sum of
 // a run is added to the segment's row, which has no other writer by now. One thread per tile and column: the thread at
 // the head of a run adds it up, several tiles in flight. What bounds this is latency, and a run of thousands of tiles
-// (a slice that holds most of a tensor) would be a serial chain: a run of more than kRunShort tiles is therefore added
+// (a slice that holds most of a tensor) would be a serial chain: a run of more than run_short() tiles is therefore added
 // by the whole CTA of its head, and (cut) runs are cut at every multiple of kRunPiece tiles: a piece's sum stays in the
 // slot of its first tile, and the CTA that finishes the last piece of a run adds the pieces (each counts itself done; none
 // waits). Every order is fixed. Measured, runs followed by one thread -> as here: 0.85 M entries, R = 4, 60 % of them in one
 // slice 918 -> 84 us (whole CSF MTTKRP); 14.9 M entries, R = 32 3.05 -> 0.39 ms (COO); 100 M entries, heaviest slice 0.5 %
 // 2.90 -> 2.84 ms.
-constexpr int kRunFirst = 4;
-constexpr int kRunShort = kRunFirst + 8;
+// Tiles up to which a thread follows a run. Beyond, the run takes its CTA about 3 us, and a CTA takes the runs of its tiles one
+// after the other, while the threads follow theirs side by side, 0.7 us per eight tiles: the narrower the rows, the more
+// tiles (and runs) a CTA has. A power-law matrix of 19.5 M entries times a vector: 135 us with 12 for every width, 106 us
+// when the limit grows with the tiles per CTA.
+__device__ __forceinline__ int32_t run_first(int32_t R) { return R == 1 ? 8 : 4; }     // tiles read at once to begin with
+__device__ __forceinline__ int32_t run_short(int32_t R, int32_t tiles) {
+  return run_first(R) + (tiles >= 128 ? 96 : tiles >= 32 ? 32 : tiles >= 16 ? 24 : 8);
+}
 
 struct FixupArgs {
   double *carry_val;
@@ -307,6 +313,7 @@ __device__ __forceinline__ void carry_fixup_role(const FixupArgs &f, int64_t blo
   const int32_t g = threadIdx.x / per, c = 2 * (threadIdx.x - g * per);
   const int32_t tile = (int32_t)block * G + g;
   const bool cut = LONG && f.done != nullptr, two = c + 1 < f.R;
+  const int32_t short_run = run_short(f.R, G);
   bool is_long = false, is_piece = false;        // is_piece: this tile's sum is a part of a cut run
   if (g < G && tile < f.num_tiles) {
     const int32_t seg_before = tile > 0 ? __ldg(f.carry_seg + tile - 1) : -2;
@@ -322,7 +329,7 @@ __device__ __forceinline__ void carry_fixup_role(const FixupArgs &f, int64_t blo
       double2 sum = make_double2(0.0, 0.0);
       bool more = true;
       int32_t q = 0;
-      for (int step = kRunFirst; more && (!LONG || q < kRunShort); q += step, step = 8) {
+      for (int step = run_first(f.R); more && (!LONG || q < short_run); q += step, step = 8) {
         int32_t s[8];
         double2 v[8];
 #pragma unroll
@@ -341,7 +348,7 @@ __device__ __forceinline__ void carry_fixup_role(const FixupArgs &f, int64_t blo
       }
       is_long = LONG && more;                    // every thread of the tile sees the same run
       if (!is_long) {
-        const bool on = cut && edge < f.num_tiles && edge - tile <= kRunShort && __ldg(f.carry_seg + edge - 1) == seg &&
+        const bool on = cut && edge < f.num_tiles && edge - tile <= short_run && __ldg(f.carry_seg + edge - 1) == seg &&
                         __ldg(f.carry_seg + edge) == seg;
         if (head && !on) {
           const int64_t row = f.out_row ? (int64_t)__ldg(f.out_row + seg) : (int64_t)seg;
@@ -375,7 +382,7 @@ __device__ __forceinline__ void carry_fixup_role(const FixupArgs &f, int64_t blo
       }
       const int32_t edge = cut ? (first / kRunPiece + 1) * kRunPiece : f.num_tiles;
       const int32_t limit = edge < f.num_tiles ? edge : f.num_tiles;
-      int32_t count = kRunShort, more;
+      int32_t count = short_run, more;
       do {
         const int32_t at = first + count + threadIdx.x;
         more = __syncthreads_count(at < limit && __ldg(f.carry_seg + at) == seg);
@@ -454,24 +461,27 @@ comet_status_t zero_rows(Context *ctx, void *C, int dtype, int64_t rows, int64_t
   return COMET_OK;
 }
 
-int32_t choose_tile_items(int64_t total_items, int workers_per_block, bool uneven) {
+int32_t choose_tile_items(int64_t total_items, int workers_per_block, bool uneven, int32_t least) {
   if (const char *e = getenv("COMET_TILE_ITEMS")) {
     int v = atoi(e);
     if (v >= 8 && v <= (1 << 20)) return v;
   }
   // Four tiles per resident worker (148 SMs x 4 CTAs), eight where their work is uneven (rows of zeros to write),
-  // capped so that the last tiles do not leave the chip idle and floored so that the head of a tile amortises; rounded
+  // capped so that the last tiles do not leave the chip idle; rounded
   // up, so that the last wave is not nearly empty. Every tile boundary costs a carry and two searches. Measured with
   // 2 / 4 / 6 / 8 tiles: 3.2 M entries, R = 50, fp32 147 / 153 / 160 / 165 us; 30 M, R = 16 404 / 381 / 386 / 394 us;
   // 8.2 M, R = 49 306 / 298 / 307 / 320 us; DCSR, 94 % of the rows empty, R = 8 1037 / 960 / 928 / 919 us.
   const int64_t slots = (int64_t)kSmCount * 4 * workers_per_block;
   int64_t t = ceil_div(total_items, slots * (uneven ? 8 : 4));
-  if (t < 32) {
-    // Small: 32 items per tile unless that leaves SMs without work; a worker is sequential, so 8 items at least. With 32 / 16 /
-    // 8 / 4: 20,000 entries, fp64, R = 4 31.7 / 17.3 / 15.5 / 15.8 us; 150,000, fp32, R = 8 27.6 / 21.4 / 19.4 / 19.4 us.
-    const int64_t one_cta = ceil_div(total_items, (int64_t)kSmCount * workers_per_block);
-    t = one_cta > 32 ? 32 : one_cta < 8 ? 8 : one_cta;
-  }
+  // That many tiles only where they are not too short: as long as half a CTA's worth of tiles per SM allows, up to 160 items
+  // (32 where the work is uneven), and not below `least` items. Measured with a limit of 32 / 96 / 160 / 256 items: SpMM, 2 M
+  // entries, R = 16 53.5 / 51.2 / 43.5 / 48.1 us; MTTKRP, CSF, 2 M, R = 16 94 / 89 / 78 / 86 us; COO 76 / 64 / 54 / 52 us. With
+  // `least` 32 / 16 / 8 / 4: 20,000 entries, fp64, R = 4 31.7 / 17.3 / 15.5 / 15.8 us; the head of a CSF tile costs more (60,000
+  // entries: 28 us with 32, 31 with 8).
+  const int64_t most = uneven ? 32 : 160;
+  int64_t low = ceil_div(total_items, (int64_t)kSmCount * 2 * workers_per_block);
+  low = low < least ? least : low < most ? low : most;
+  if (t < low) t = low;
   if (t > 512) t = 512;
   return (int32_t)t;
 }
@@ -580,7 +590,7 @@ template <class T, int LPN, int CPL, int VEC, bool RAGGED = false>
 static comet_status_t launch_one(Context *ctx, SegGatherArgs a, HeavyArgs *heavy, int64_t pad, cudaStream_t stream) {
   constexpr int WORKERS = kBlockThreads / LPN;
   const int64_t total = a.M + a.N;
-  a.tile_items = choose_tile_items(total, WORKERS, a.out_row != nullptr);
+  a.tile_items = choose_tile_items(total, WORKERS, a.out_row != nullptr, 8);
   a.num_tiles = ceil_div(total, a.tile_items);
   a.own_len = a.tile_items / 4;
   a.carry_ld = (int32_t)align_up((size_t)a.R, 2);
@@ -663,12 +673,13 @@ static comet_status_t seg_gather_typed(Context *ctx, const int32_t *seg_end, con
   HeavyArgs *heavy = long_rows && !out_row && b_rows > 0 && R <= 128 ? &hint : nullptr;
   const bool b_ok = aligned16(B) && ldb % PER == 0 && R % PER == 0, c_ok = aligned16(C) && ldc % PER == 0;
   // The copy moves a row of B twice (0.4 ps per byte and row); a ragged shape saves about 17 ps per entry on the scalar one.
-  const bool pad = !b_ok && N * 40 >= b_rows * R * (int64_t)sizeof(T);
+  // Below 100,000 entries that is less than the launch costs.
+  const bool pad = !b_ok && N >= 100000 && N * 40 >= b_rows * R * (int64_t)sizeof(T);
   // More than 32 pieces are two per lane, which halves the warps on an SM. Long rows of a B that stays in L2 are faster as
   // two launches of at most 32 (4 M entries in 200,000 rows, 84 MB of B: R = 70 335 -> 262, R = 120 460 -> 381 us), short
-  // ones or a B in DRAM are not (2.9 entries per row: 784 -> 1128 us; 430 MB: 398 -> 527 us). Short rows are faster still
+  // ones, a B in DRAM and small inputs (35,000 entries: 22 -> 40 us) are not (2.9 entries per row: 784 -> 1128 us; 430 MB: 398 -> 527 us). Short rows are faster still
   // with a column per lane (R = 70: 784 -> 760 us): what costs there is the stores of the ragged rows.
-  const bool split = N >= 8 * M && b_rows * R * (int64_t)sizeof(T) <= (126ll << 20);
+  const bool split = N >= (1 << 20) && N >= 8 * M && b_rows * R * (int64_t)sizeof(T) <= (126ll << 20);
   const bool scalar = R > 32 * PER && R < 128 && N < 4 * M;
   // A compressed root level with at least twice as many rows as segments: C is cleared in one stream of wide stores and the
   // stored rows are written over it. A worker that fills the rows in front of each segment itself writes fewer bytes but

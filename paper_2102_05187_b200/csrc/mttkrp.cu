@@ -440,7 +440,7 @@ static comet_status_t launch_mttkrp(Context *ctx, MttkrpArgs a, int64_t p_pad, i
   constexpr int WORKERS = kBlockThreads / LPN;
   const int64_t total = CSF ? a.F + a.N : a.N;
   using L = Lanes<T, LPN, CPL, VEC, RAGGED>;
-  a.tile_items = choose_tile_items(total, WORKERS, false);
+  a.tile_items = choose_tile_items(total, WORKERS, false, CSF ? 32 : 8);
   if (CSF && a.tile_items > kCsfTileCap) a.tile_items = kCsfTileCap;          // one mask bit per leaf entry of a tile
   a.num_tiles = ceil_div(total, a.tile_items);
   a.carry_ld = (int32_t)align_up((size_t)a.R, 2);
@@ -497,7 +497,7 @@ static comet_status_t mttkrp_chunks(Context *ctx, const MttkrpArgs &base, int64_
   constexpr int PER = 16 / sizeof(T);
   const bool in_ok = aligned16(base.P) && aligned16(base.Q) && base.ldp % PER == 0 && base.ldq % PER == 0 && R % PER == 0;
   const bool out_ok = aligned16(base.out) && base.ldo % PER == 0;
-  const bool pad = !in_ok && base.N * 40 >= (p_rows + q_rows) * R * (int64_t)sizeof(T);   // as in seg_gather_typed
+  const bool pad = !in_ok && base.N >= 100000 && base.N * 40 >= (p_rows + q_rows) * R * (int64_t)sizeof(T);   // as in seg_gather_typed
   int64_t done = 0;
   while (done < R) {
     const int64_t rem = R - done;

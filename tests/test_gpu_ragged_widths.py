@@ -66,6 +66,31 @@ def test_spmm_and_root_mttkrp(R, lead, offset, dtype):
         assert_close(got, want, norm, tol if dtype == torch.float64 else 2 * tol)
 
 
+@pytest.mark.parametrize("dtype", [torch.float64, torch.float32])
+@pytest.mark.parametrize("R", [1, 3, 5, 9, 25, 33, 65, 67, 131])
+def test_padded_copies(R, dtype):
+    """Enough entries for the operands to be padded: rows that are no whole pieces, an odd leading dimension."""
+    rng = np.random.default_rng(R)
+    f = lambda a: a.astype(np.float32).astype(np.float64) if dtype == torch.float32 else a  # noqa: E731
+    tol = 1e-12 if dtype == torch.float64 else 3 * 2.0 ** -24
+    rows, cols, n = 700, 300, 110_000
+    cell = rng.permutation(rows * cols)[:n]
+    r, c = (cell // cols).astype(np.int32), (cell % cols).astype(np.int32)
+    v, B = f(rng.uniform(-1, 1, n)), f(rng.uniform(-1, 1, (cols, R)))
+    want, norm = oracle.spmm([r, c], v, (rows, cols), B)
+    for attr in [(D, CU), (CU, CU)]:
+        A = _as(upload_packed(oracle.pack([r, c], v, (rows, cols), (0, 1), attr)), dtype)
+        assert_close(comet.spmm(A, _operand(B, 1, 1, dtype)), want, norm, tol)
+    dims = (rows, 20, 15)
+    coords = [r, (c % 20).astype(np.int32), (c // 20).astype(np.int32)]
+    F = [None] + [f(rng.uniform(-1, 1, (d, R))) for d in dims[1:]]
+    want, norm = oracle.mttkrp(coords, v, dims, 0, F)
+    for attr in [(CU, CU, CU), (CN, S, S)]:
+        X = _as(upload_packed(oracle.pack(coords, v, dims, (0, 1, 2), attr)), dtype)
+        got = comet.mttkrp(X, 0, [None] + [_operand(x, 1, 1, dtype) for x in F[1:]])
+        assert_close(got, want, norm, tol if dtype == torch.float64 else 2 * tol)
+
+
 @pytest.mark.parametrize("R", [1, 2, 5, 50, 130])
 def test_few_entries_many_operand_rows(R):
     rng = np.random.default_rng(R)

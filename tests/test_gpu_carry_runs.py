@@ -38,6 +38,28 @@ def test_spmm_runs(lengths, R):
     assert torch.equal(first, comet.spmm(A, dev(B))), "not reproducible"
 
 
+@pytest.mark.parametrize("dtype", [np.float64, np.float32])
+@pytest.mark.parametrize("kernel", ["stream", "stream2", "resident"])
+def test_vector_runs(kernel, dtype, monkeypatch):
+    """The form of the fix-up for vector results: runs below, at and beyond the length where the CTA takes over (104 tiles)."""
+    span = 128
+    monkeypatch.setenv("COMET_SEG_DOT_KERNEL", kernel)
+    monkeypatch.setenv("COMET_STREAM_SPAN", str(span))
+    rng = np.random.default_rng(7)
+    lengths = [span * t + d for t in (7, 8, 9, 103, 104, 105, 106, 200) for d in (0, 1)] + [1, 0, 3]
+    cols = max(lengths) + 3
+    r = np.repeat(np.arange(len(lengths)), lengths).astype(np.int32)
+    c = np.concatenate([rng.permutation(cols)[:n] for n in lengths]).astype(np.int32)
+    v, x = rng.uniform(-1, 1, r.size).astype(dtype), rng.uniform(-1, 1, cols).astype(dtype)
+    want, norm = oracle.spmv([r, c], v.astype(np.float64), (len(lengths), cols), x.astype(np.float64))
+    ptr = np.concatenate([[0], np.cumsum(lengths)]).astype(np.int32)
+    A = comet.SpTensor.from_arrays((len(lengths), cols), (0, 1), (D, CU), [None, dev(ptr)], [None, dev(c)], dev(v))
+    first = comet.spmv(A, dev(x))
+    # fp32: a row is rounded when it is stored and once more when its carries are added (2 x 2^-24 of at most norm each)
+    assert_close(first.double(), want, norm, 1e-12 if dtype == np.float64 else 1.01 * 2.0 ** -23)
+    assert torch.equal(first, comet.spmv(A, dev(x))), "not reproducible"
+
+
 @pytest.mark.parametrize("attr", [(CU, CU, CU), (CN, S, S)])
 @pytest.mark.parametrize("R,n", [(4, 17000), (33, 180000), (128, 60000)])
 def test_mttkrp_heavy_slice(attr, R, n):

@@ -166,6 +166,7 @@ class Handle:
             if live.pop(ptr, None) is not None:
                 raw_delete(ptr)
 
+        self._give_back = raw_delete
         self._alloc_cb = _ALLOC_FN(_alloc)
         self._free_cb = _FREE_FN(_free)
         self._allocator = AllocatorStruct(self._alloc_cb, self._free_cb, None)
@@ -180,8 +181,12 @@ class Handle:
             self._h = C.c_void_p()
 
     def __del__(self):
+        # Tensors hold their handle, and views hold their tensors: nothing refers to a block any more. Blocks of tensors that
+        # were alive when the handle was closed are still here (a closed handle frees none).
         try:
             self.close()
+            while self._live:
+                self._give_back(self._live.popitem()[0])
         except Exception:
             pass
 

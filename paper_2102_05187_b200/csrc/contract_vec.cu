@@ -34,7 +34,6 @@ struct SegGatherArgs {
   int64_t ldc;
   const int32_t *out_row;   // NULL: segment s -> row s. Else segment s -> row out_row[s] (ascending) and the
   int64_t out_rows;         //   rows in between (and up to out_rows) are zero-filled by the flushing worker
-  bool cleared;             // out_row given: C holds zeros already, no rows to fill
   int32_t R;                // columns handled by this launch
   bool wide_store;          // ragged shapes: rows of C take 16-byte stores
   int32_t tile_items;
@@ -48,8 +47,13 @@ struct SegGatherArgs {
                             //      path of SpMM): neither walked nor stored here. Never below tile_items.
 };
 
+// Where the rows of C go: segment s to row s; through out_row, the rows in between filled with zeros; or through out_row into
+// a C that holds zeros already. Three kernels, not a test: it sat in the body that is unrolled for every entry of a chunk, and
+// a DCSR matrix of 6.6 M entries in 2.1 M of 2.2 M rows, fp32, R = 31, took 1,060 us with it, 853 without.
+constexpr int kRowsAll = 0, kRowsFilled = 1, kRowsMapped = 2;
+
 // What the walker does with one leaf entry: close the segments that end in front of it, accumulate.
-template <class T, int LPN, int CPL, int VEC, bool RAGGED, bool MAPPED, bool PASS_THROUGH = false>
+template <class T, int LPN, int CPL, int VEC, bool RAGGED, int ROWS, bool PASS_THROUGH = false>
 struct SegGatherPolicy {
   using L = Lanes<T, LPN, CPL, VEC, RAGGED>;
   static constexpr int kPF = COMET_PF_GATHER;
@@ -97,10 +101,10 @@ struct SegGatherPolicy {
   // Stores the open segment (and, for a compressed root level, zero-fills the rows in front of it).
   __device__ __forceinline__ void flush() {
     T *cmat = static_cast<T *>(a.C) + ln.col0;
-    if (MAPPED) {
+    if (ROWS != kRowsAll) {
       const int64_t i = seg;
       const int64_t r = __ldg(a.out_row + i);
-      if (!a.cleared) {
+      if (ROWS == kRowsFilled) {
         const int64_t lo = (i > 0) ? (int64_t)__ldg(a.out_row + i - 1) + 1 : 0;
         ln.zero_rows(cmat, a.ldc, lo, r);
         if (i == a.M - 1) ln.zero_rows(cmat, a.ldc, r + 1, a.out_rows);
@@ -123,7 +127,7 @@ struct SegGatherPolicy {
 // others walk the general tiles and skip those rows. The two roles are bound by different things (the long rows
 // by the L2 -> L1 fill rate, the rest by DRAM latency), so sharing the SMs between them is faster than running
 // one after the other.
-template <class T, int LPN, int CPL, int VEC, bool RAGGED, bool MAPPED, bool HEAVY>
+template <class T, int LPN, int CPL, int VEC, bool RAGGED, int ROWS, bool HEAVY>
 __global__ void __launch_bounds__(kBlockThreads, (CPL * VEC * sizeof(T) <= 16 ? COMET_MINB_GATHER : 2))
 seg_gather_kernel(const SegGatherArgs a, const HeavyArgs h) {
   using L = Lanes<T, LPN, CPL, VEC, RAGGED>;
@@ -187,7 +191,7 @@ seg_gather_kernel(const SegGatherArgs a, const HeavyArgs h) {
     }
   }
 
-  SegGatherPolicy<T, LPN, CPL, VEC, RAGGED, MAPPED, HEAVY> p(a, ln, i0, j0);
+  SegGatherPolicy<T, LPN, CPL, VEC, RAGGED, ROWS, HEAVY> p(a, ln, i0, j0);
   walk_tile(ln, p, j0, j1, smem);
   while (p.segment() < i1) p.flush();                    // end markers that close the tile
 
@@ -495,12 +499,12 @@ int32_t choose_tile_items(int64_t total_items, int workers_per_block, bool uneve
   return (int32_t)t;
 }
 
-template <class T, int LPN, int CPL, int VEC, bool RAGGED, bool MAPPED, bool HEAVY>
+template <class T, int LPN, int CPL, int VEC, bool RAGGED, int ROWS, bool HEAVY>
 static comet_status_t launch_mapped(Context *ctx, const SegGatherArgs &a, const HeavyArgs &h, int64_t blocks,
                                     cudaStream_t stream) {
   using L = Lanes<T, LPN, CPL, VEC, RAGGED>;
   constexpr size_t smem = RingLayout<L, false>::kBlockBytes;
-  auto kernel = seg_gather_kernel<T, LPN, CPL, VEC, RAGGED, MAPPED, HEAVY>;
+  auto kernel = seg_gather_kernel<T, LPN, CPL, VEC, RAGGED, ROWS, HEAVY>;
   if (smem > 48 * 1024)
     COMET_CUDA_TRY(ctx, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   kernel<<<(unsigned)(blocks + (HEAVY ? h.heavy_ctas : 0)), kBlockThreads, smem, stream>>>(a, h);
@@ -594,9 +598,10 @@ comet_status_t pad_rows2(Context *ctx, int dtype, const void *src0, int64_t rows
 }
 
 // `heavy` (optional): the long-row plan of an SpMM; its scratch precedes the carries of this launch. pad (RAGGED): the
-// first `pad` rows of B are copied into scratch as whole pieces and gathered from there.
+// first `pad` rows of B are copied into scratch as whole pieces and gathered from there. cleared: out_row is given and C
+// holds zeros.
 template <class T, int LPN, int CPL, int VEC, bool RAGGED = false>
-static comet_status_t launch_one(Context *ctx, SegGatherArgs a, HeavyArgs *heavy, int64_t pad, cudaStream_t stream) {
+static comet_status_t launch_one(Context *ctx, SegGatherArgs a, HeavyArgs *heavy, bool cleared, int64_t pad, cudaStream_t stream) {
   constexpr int WORKERS = kBlockThreads / LPN;
   const int64_t total = a.M + a.N;
   a.tile_items = choose_tile_items(total, WORKERS, a.out_row != nullptr, 8);
@@ -644,7 +649,7 @@ static comet_status_t launch_one(Context *ctx, SegGatherArgs a, HeavyArgs *heavy
       st = spmm_heavy_prepare(ctx, &h, a.seg_end - 1, a.crd, a.val, scratch, stream);
       if (st != COMET_OK) return st;
       a.skip_len = h.threshold;
-      st = launch_mapped<T, LPN, CPL, VEC, false, false, true>(ctx, a, h, blocks, stream);
+      st = launch_mapped<T, LPN, CPL, VEC, false, kRowsAll, true>(ctx, a, h, blocks, stream);
       if (st != COMET_OK) return st;
       const int heavy_blocks = kSmCount * 8;
       const unsigned fix_blocks = (unsigned)(heavy_blocks + fixup_blocks(a.num_tiles, a.R));
@@ -654,8 +659,9 @@ static comet_status_t launch_one(Context *ctx, SegGatherArgs a, HeavyArgs *heavy
       return COMET_OK;
     }
   }
-  st = a.out_row ? launch_mapped<T, LPN, CPL, VEC, RAGGED, true, false>(ctx, a, h, blocks, stream)
-                 : launch_mapped<T, LPN, CPL, VEC, RAGGED, false, false>(ctx, a, h, blocks, stream);
+  st = !a.out_row ? launch_mapped<T, LPN, CPL, VEC, RAGGED, kRowsAll, false>(ctx, a, h, blocks, stream)
+       : cleared  ? launch_mapped<T, LPN, CPL, VEC, RAGGED, kRowsMapped, false>(ctx, a, h, blocks, stream)
+                  : launch_mapped<T, LPN, CPL, VEC, RAGGED, kRowsFilled, false>(ctx, a, h, blocks, stream);
   if (st != COMET_OK) return st;
   carry_fixup_launch(kDtype, a.carry_val, a.carry_seg, a.num_tiles, a.R, a.carry_ld, a.C, a.ldc, a.out_row, true, stream);
   COMET_LAUNCH_CHECK(ctx);
@@ -705,7 +711,6 @@ static comet_status_t seg_gather_typed(Context *ctx, const int32_t *seg_end, con
     a.B = B + done; a.ldb = ldb; a.C = C + done; a.ldc = ldc;
     a.out_row = out_row; a.out_rows = out_rows;
     a.wide_store = c_ok;
-    a.cleared = cleared;
     comet_status_t st = COMET_OK;
     const int64_t rem = R - done;
     if ((b_ok || pad) && !scalar) {
@@ -717,23 +722,23 @@ static comet_status_t seg_gather_typed(Context *ctx, const int32_t *seg_end, con
       const bool exact = b_ok && c_ok && (pieces & (pieces - 1)) == 0;
       if (pieces > 32) {
         if constexpr (sizeof(T) == 8)                      // fp32 chunks are at most 32 pieces
-          st = exact ? launch_one<T, 32, 2, PER>(ctx, a, heavy, 0, stream) : launch_one<T, 32, 2, PER, true>(ctx, a, heavy, p, stream);
-      } else if (exact && pieces == 32) st = launch_one<T, 32, 1, PER>(ctx, a, heavy, 0, stream);
-      else if (exact && pieces == 16) st = launch_one<T, 16, 1, PER>(ctx, a, heavy, 0, stream);
-      else if (exact && pieces == 8) st = launch_one<T, 8, 1, PER>(ctx, a, heavy, 0, stream);
-      else if (exact && pieces == 4) st = launch_one<T, 4, 1, PER>(ctx, a, heavy, 0, stream);
-      else if (exact && pieces == 2) st = launch_one<T, 2, 1, PER>(ctx, a, heavy, 0, stream);
-      else if (exact && pieces == 1) st = launch_one<T, 1, 1, PER>(ctx, a, heavy, 0, stream);
-      else if (pieces > 16) st = launch_one<T, 32, 1, PER, true>(ctx, a, heavy, p, stream);
-      else if (pieces > 8) st = launch_one<T, 16, 1, PER, true>(ctx, a, heavy, p, stream);
-      else if (pieces > 4) st = launch_one<T, 8, 1, PER, true>(ctx, a, heavy, p, stream);
-      else if (pieces > 2) st = launch_one<T, 4, 1, PER, true>(ctx, a, heavy, p, stream);
-      else st = launch_one<T, 2, 1, PER, true>(ctx, a, heavy, p, stream);
+          st = exact ? launch_one<T, 32, 2, PER>(ctx, a, heavy, cleared, 0, stream) : launch_one<T, 32, 2, PER, true>(ctx, a, heavy, cleared, p, stream);
+      } else if (exact && pieces == 32) st = launch_one<T, 32, 1, PER>(ctx, a, heavy, cleared, 0, stream);
+      else if (exact && pieces == 16) st = launch_one<T, 16, 1, PER>(ctx, a, heavy, cleared, 0, stream);
+      else if (exact && pieces == 8) st = launch_one<T, 8, 1, PER>(ctx, a, heavy, cleared, 0, stream);
+      else if (exact && pieces == 4) st = launch_one<T, 4, 1, PER>(ctx, a, heavy, cleared, 0, stream);
+      else if (exact && pieces == 2) st = launch_one<T, 2, 1, PER>(ctx, a, heavy, cleared, 0, stream);
+      else if (exact && pieces == 1) st = launch_one<T, 1, 1, PER>(ctx, a, heavy, cleared, 0, stream);
+      else if (pieces > 16) st = launch_one<T, 32, 1, PER, true>(ctx, a, heavy, cleared, p, stream);
+      else if (pieces > 8) st = launch_one<T, 16, 1, PER, true>(ctx, a, heavy, cleared, p, stream);
+      else if (pieces > 4) st = launch_one<T, 8, 1, PER, true>(ctx, a, heavy, cleared, p, stream);
+      else if (pieces > 2) st = launch_one<T, 4, 1, PER, true>(ctx, a, heavy, cleared, p, stream);
+      else st = launch_one<T, 2, 1, PER, true>(ctx, a, heavy, cleared, p, stream);
     } else {
       a.R = (int32_t)(rem < 128 ? rem : 128);
-      if (a.R > 64) st = launch_one<T, 32, 4, 1>(ctx, a, heavy, 0, stream);
-      else if (a.R > 32) st = launch_one<T, 32, 2, 1>(ctx, a, heavy, 0, stream);
-      else st = launch_one<T, 32, 1, 1>(ctx, a, heavy, 0, stream);
+      if (a.R > 64) st = launch_one<T, 32, 4, 1>(ctx, a, heavy, cleared, 0, stream);
+      else if (a.R > 32) st = launch_one<T, 32, 2, 1>(ctx, a, heavy, cleared, 0, stream);
+      else st = launch_one<T, 32, 1, 1>(ctx, a, heavy, cleared, 0, stream);
     }
     if (st != COMET_OK) return st;
     done += a.R;

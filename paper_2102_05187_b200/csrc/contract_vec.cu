@@ -204,14 +204,16 @@ seg_gather_kernel(const SegGatherArgs a, const HeavyArgs h) {
 }
 
 // Adds the carries onto the stored rows. The tiles that stopped inside one segment are consecutive (a run); the sum of
-// a run is added to the segment's row, which has no other writer by now. One thread per tile and column: the thread at
-// the head of a run adds it up, several tiles in flight. What bounds this is latency, and a run of thousands of tiles
-// (a slice that holds most of a tensor) would be a serial chain: a run of more than run_short() tiles is therefore added
-// by the whole CTA of its head, and (cut) runs are cut at every multiple of kRunPiece tiles: a piece's sum stays in the
-// slot of its first tile, and the CTA that finishes the last piece of a run adds the pieces (each counts itself done; none
-// waits). Every order is fixed. Measured, runs followed by one thread -> as here: 0.85 M entries, R = 4, 60 % of them in one
-// slice 918 -> 84 us (whole CSF MTTKRP); 14.9 M entries, R = 32 3.05 -> 0.39 ms (COO); 100 M entries, heaviest slice 0.5 %
-// 2.90 -> 2.84 ms.
+// a run is added to the segment's row, which has no other writer by now. One thread per tile and pair of columns: the
+// threads at the head of a run add it up, several tiles in flight. What bounds this is latency, and a run of thousands of
+// tiles (a slice that holds most of a tensor) would be a serial chain: a run of more than run_short() tiles is therefore
+// added by the whole CTA of its head, and (cut) runs are cut at the multiples of kRunPiece tiles behind which they go on for
+// kRunSpare tiles and more: a piece's sum stays in the slot of its first tile, and the CTA that finishes the last piece of a
+// run adds the pieces (each counts itself done; none waits). Every order is fixed. Finishing a piece costs about 4 us, and
+// some run crosses a multiple almost always: with short runs cut too, MTTKRP of 90,000 entries (CSF, R = 6) took 31.3 us
+// instead of 26.7, of 78,000 (COO, R = 5) 20.7 instead of 15.8. Measured, runs followed by one thread -> as here: 0.85 M
+// entries, R = 4, 60 % of them in one slice 918 -> 84 us (whole CSF MTTKRP); 14.9 M entries, R = 32 3.05 -> 0.39 ms (COO);
+// 100 M entries, heaviest slice 0.5 % 2.90 -> 2.84 ms.
 // Tiles up to which a thread follows a run. Beyond, the run takes its CTA about 3 us, and a CTA takes the runs of its tiles one
 // after the other, while the threads follow theirs side by side, 0.7 us per eight tiles: the narrower the rows, the more
 // tiles (and runs) a CTA has. A power-law matrix of 19.5 M entries times a vector: 135 us with 12 for every width, 106 us
@@ -232,6 +234,13 @@ struct FixupArgs {
   int32_t *done;                                 // per multiple of kRunPiece: pieces of the run first cut there that are summed
                                                  // (zero at the start; NULL: runs are not cut)
 };
+
+constexpr int32_t kRunSpare = 512;
+// Whether a run of segment `seg` that crosses tile t, a multiple of kRunPiece, is cut there. (The tiles in between are the
+// run's too.)
+__device__ __forceinline__ bool run_cut_at(const FixupArgs &f, int64_t t, int32_t seg) {
+  return t + kRunSpare < f.num_tiles && __ldg(f.carry_seg + t + kRunSpare) == seg;
+}
 
 template <class T>
 __device__ __forceinline__ void add_to_row(const FixupArgs &f, int32_t seg, int32_t c, double sum) {
@@ -272,7 +281,7 @@ template <class T>
 __device__ __forceinline__ void finish_piece(const FixupArgs &f, int32_t first, int32_t seg, double *s_part, int32_t *s_old) {
   auto cut_at = [&](int64_t m) {                 // the run is cut at multiple m
     const int64_t t = m * kRunPiece;
-    return m > 0 && t < f.num_tiles && __ldg(f.carry_seg + t) == seg && __ldg(f.carry_seg + t - 1) == seg;
+    return m > 0 && run_cut_at(f, t, seg) && __ldg(f.carry_seg + t - 1) == seg;
   };
   __threadfence();
   __syncthreads();
@@ -323,9 +332,10 @@ __device__ __forceinline__ void carry_fixup_role(const FixupArgs &f, int64_t blo
     const int32_t seg_before = tile > 0 ? __ldg(f.carry_seg + tile - 1) : -2;
     const int32_t seg = __ldg(f.carry_seg + tile);
     const bool head = seg >= 0 && seg_before != seg;
-    if (head || (seg >= 0 && cut && tile % kRunPiece == 0)) {
-      const int32_t edge = cut ? (tile / kRunPiece + 1) * kRunPiece : f.num_tiles;
-      const int32_t limit = edge < f.num_tiles ? edge : f.num_tiles;       // the run is followed up to here
+    if (head || (seg >= 0 && cut && tile % kRunPiece == 0 && run_cut_at(f, tile, seg))) {
+      const int32_t edge = (tile / kRunPiece + 1) * kRunPiece;
+      const bool on = cut && run_cut_at(f, edge, seg);                     // the run goes on in a piece of its own
+      const int32_t limit = on ? edge : f.num_tiles;                       // it is followed up to here
       auto carry = [&](int32_t t) {
         const double *at = f.carry_val + (int64_t)t * f.carry_ld + c;
         return f.carry_ld == 1 ? make_double2(__ldcs(at), 0.0) : __ldcs(reinterpret_cast<const double2 *>(at));
@@ -352,8 +362,6 @@ __device__ __forceinline__ void carry_fixup_role(const FixupArgs &f, int64_t blo
       }
       is_long = LONG && more;                    // every thread of the tile sees the same run
       if (!is_long) {
-        const bool on = cut && edge < f.num_tiles && edge - tile <= short_run && __ldg(f.carry_seg + edge - 1) == seg &&
-                        __ldg(f.carry_seg + edge) == seg;
         if (head && !on) {
           const int64_t row = f.out_row ? (int64_t)__ldg(f.out_row + seg) : (int64_t)seg;
           T *const dst = static_cast<T *>(f.C) + row * f.ldc + c;
@@ -384,8 +392,9 @@ __device__ __forceinline__ void carry_fixup_role(const FixupArgs &f, int64_t blo
         finish_piece<T>(f, first, seg, s_part, &s_old);
         continue;
       }
-      const int32_t edge = cut ? (first / kRunPiece + 1) * kRunPiece : f.num_tiles;
-      const int32_t limit = edge < f.num_tiles ? edge : f.num_tiles;
+      const int32_t edge = (first / kRunPiece + 1) * kRunPiece;
+      const bool on = cut && run_cut_at(f, edge, seg);
+      const int32_t limit = on ? edge : f.num_tiles;
       int32_t count = short_run, more;
       do {
         const int32_t at = first + count + threadIdx.x;
@@ -395,7 +404,6 @@ __device__ __forceinline__ void carry_fixup_role(const FixupArgs &f, int64_t blo
       const double sum = cta_slot_sum(f, first, 1, count, s_part);
       if (threadIdx.x < f.R) {
         const bool head = first == 0 || __ldg(f.carry_seg + first - 1) != seg;
-        const bool on = cut && limit < f.num_tiles && first + count == limit && __ldg(f.carry_seg + limit) == seg;
         if (head && !on) add_to_row<T>(f, seg, threadIdx.x, sum);
         else f.carry_val[(int64_t)first * f.carry_ld + threadIdx.x] = sum;
         if (threadIdx.x == 0) s_old = head && !on;

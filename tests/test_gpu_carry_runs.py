@@ -1,6 +1,6 @@
-"""The carry fix-up: segments that span from one tile to thousands of them, with run lengths around 12 and 20 tiles (added by
-one thread or by a whole CTA) and around multiples of 1,024 (where runs are cut in large problems). Small tiles are
-forced, so that small inputs reach every case."""
+"""The carry fix-up: segments that span from one tile to thousands of them, with run lengths around the number of tiles up to
+which threads follow a run (12 to 104, by width; a whole CTA adds longer ones) and around the multiples of 1,024 tiles at which
+long runs are cut in large problems. Small tiles are forced, so that small inputs reach every case."""
 import numpy as np
 import pytest
 import torch
@@ -38,6 +38,47 @@ def test_spmm_runs(lengths, R):
     assert torch.equal(first, comet.spmm(A, dev(B))), "not reproducible"
 
 
+def _rows_of_runs(runs):
+    """Row lengths so that the run of carries of each (head, tiles) pair starts in tile `head` and takes `tiles` tiles: an
+    entry and the end of a row are an item each, a tile holds TILE of them."""
+    lengths, at = [], 0                                      # items so far
+    for head, tiles in runs:
+        assert at <= TILE * head
+        while at % TILE:                                     # rows without entries up to a tile boundary
+            lengths.append(0)
+            at += 1
+        while at < TILE * head:                              # rows that end with their tile
+            lengths.append(TILE - 1)
+            at += TILE
+        lengths += [2, TILE * (head + tiles) + 2 - (at + 3)]  # ends 2 items into the tile behind the run
+        at = TILE * (head + tiles) + 3
+    return lengths + [TILE - 1] * 700
+
+
+@pytest.mark.parametrize("R,limit", [(1, 104), (4, 100), (5, 36), (16, 36), (24, 28), (100, 12)])
+def test_runs_at_the_limits(R, limit):
+    """Runs of `limit` tiles and one less and more, heads as many tiles in front of a multiple of 1,024, and runs that go on
+    511, 512 and 513 tiles behind one (cut from 513 tiles on), alone and over several multiples."""
+    at = {"short": [(5, limit - 1), (5 + limit, limit), (10 + 2 * limit, limit + 1)],
+          "cut": [(1024 - limit + d, limit - d + 512 + e) for d in (-1, 0, 1) for e in (-1, 0, 1)]}
+    for k, (head, tiles) in enumerate([(1024, 512), (1024, 513), (1024, 514), (1000, 2600), (1023, 1)] + at["cut"]):
+        runs = at["short"] + [(head, tiles), (head + tiles + 1, 3), (4096 - limit, limit + 2)]
+        lengths = _rows_of_runs(runs)
+        rng = np.random.default_rng(100 * R + k)
+        cols = max(lengths) + 3
+        r = np.repeat(np.arange(len(lengths)), lengths).astype(np.int32)
+        c = np.concatenate([(rng.integers(cols) + np.arange(n)) % cols for n in lengths if n]).astype(np.int32)
+        order = np.lexsort((c, r))
+        r, c = r[order], c[order]
+        v, B = rng.uniform(-1, 1, r.size), rng.uniform(-1, 1, (cols, R))
+        want, norm = oracle.spmm([r, c], v, (len(lengths), cols), B)
+        ptr = np.concatenate([[0], np.cumsum(lengths)]).astype(np.int32)
+        A = comet.SpTensor.from_arrays((len(lengths), cols), (0, 1), (D, CU), [None, dev(ptr)], [None, dev(c)], dev(v))
+        first = comet.spmm(A, dev(B))
+        assert_close(first, want, norm, what=f"run of {tiles} tiles from tile {head}")
+        assert torch.equal(first, comet.spmm(A, dev(B))), "not reproducible"
+
+
 @pytest.mark.parametrize("dtype", [np.float64, np.float32])
 @pytest.mark.parametrize("kernel", ["stream", "stream2", "resident"])
 def test_vector_runs(kernel, dtype, monkeypatch):
@@ -63,8 +104,7 @@ def test_vector_runs(kernel, dtype, monkeypatch):
 @pytest.mark.parametrize("attr", [(CU, CU, CU), (CN, S, S)])
 @pytest.mark.parametrize("R,n", [(4, 17000), (33, 180000), (128, 60000)])
 def test_mttkrp_heavy_slice(attr, R, n):
-    """A slice with most of the entries among slices of one entry, of about 20 tiles and of about 1,024 (R = 4: one launch;
-    R = 33 and 128: the runs are cut)."""
+    """A slice with most of the entries among slices of one entry, of about 20 tiles and of about 1,024; long runs are cut."""
     rng = np.random.default_rng(R)
     dims = (12, 811, 399)
     cell = rng.permutation(dims[1] * dims[2])[:n]

@@ -623,9 +623,15 @@ static comet_status_t launch_one(Context *ctx, SegGatherArgs a, HeavyArgs *heavy
     heavy_bytes = spmm_heavy_plan(sizeof(T) == 4 ? COMET_F32 : COMET_F64, a.M, a.N, heavy->cols, a.B, a.ldb, a.R, a.C, a.ldc,
                                   a.tile_items, &h);
   static const bool use_part = !(getenv("COMET_SEG_PARTITION") && atoi(getenv("COMET_SEG_PARTITION")) == 0);
-  const size_t part_bytes = use_part && a.num_tiles >= 1024 ? align_up((size_t)(a.num_tiles + 1) * sizeof(int32_t), 256) : 0;
   constexpr int kDtype = sizeof(T) == 4 ? COMET_F32 : COMET_F64;
   const size_t pad_bytes = RAGGED && pad ? padded_bytes(kDtype, pad, a.R) : 0;
+  // The split at the tile boundaries as a launch of its own costs 3 us; a worker that finds its own boundaries takes
+  // log2(M) / log2(LPN) dependent loads. So it pays from about a thousand tiles with few lanes (or beside padded copies or
+  // the long-row plan, which need the launch anyway), from many thousands with more: with the launch from 1,024 tiles at every
+  // width, SpMM of 89,000 entries in 16-lane workers took 21.7 us instead of 12.5, of 45,000 in whole warps 16.6 instead of
+  // 13.9; from 16,384 tiles on both are the same. In 2-lane workers the launch takes 25,000 entries from 22 to 13 us.
+  const int64_t part_least = LPN <= 4 || pad_bytes || heavy_bytes ? 1024 : 16384;
+  const size_t part_bytes = use_part && a.num_tiles >= part_least ? align_up((size_t)(a.num_tiles + 1) * sizeof(int32_t), 256) : 0;
   char *scratch = (char *)scratch_get(ctx, pad_bytes + heavy_bytes + carry_bytes(a.num_tiles, a.carry_ld) + part_bytes, stream);
   if (!scratch) return COMET_ERR_ALLOC;
   PrepareArgs prep{};

@@ -690,7 +690,13 @@ static bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 
 // lanes, a column each) run on B as it is. What the scalar shapes lose is lanes (R = 10: 22 of 32 idle) and requests in
 // flight. Measured, scalar -> ragged: 4 M entries in 200,000 rows, R = 3 / 10 / 25 / 50 / 100 fp64 134 -> 68, 137 -> 77, 155
 // -> 122, 194 -> 167, 463 -> 403 us, fp32 129 -> 70, 132 -> 77, 136 -> 109, 187 -> 151, 304 -> 208 us; a power-law
-// matrix of 3.2 M entries, R = 50, fp32 156 -> 145 us.
+// matrix of 3.2 M entries, R = 50, fp32 156 -> 145 us. Small inputs have the scalar shapes too, unless the ragged one is a
+// whole warp that reads B as it is: many narrow workers to a CTA leave few CTAs, and each finds its tile with few lanes. Over
+// some thousand random inputs the two are level between 150,000 (up to 4 lanes) and 500,000 entries (16 lanes, or copies);
+// below, the ragged ones took up to 1.7 times as long (34,700 entries, fp64, R = 24 20.7 us, scalar 12.1; 97,000, R = 20 27.8,
+// scalar 18.6).
+constexpr int64_t kRaggedLeast = 250000;
+
 template <class T>
 static comet_status_t seg_gather_typed(Context *ctx, const int32_t *seg_end, const int32_t *crd, const T *val,
                                        int64_t M, int64_t N, const T *B, int64_t ldb, int64_t R, T *C, int64_t ldc,
@@ -700,16 +706,19 @@ static comet_status_t seg_gather_typed(Context *ctx, const int32_t *seg_end, con
   HeavyArgs hint{};                                        // SpMM on [D,CU]: long rows by column phases
   hint.cols = b_rows;
   HeavyArgs *heavy = long_rows && !out_row && b_rows > 0 && R <= 128 ? &hint : nullptr;
-  const bool b_ok = aligned16(B) && ldb % PER == 0 && R % PER == 0, c_ok = aligned16(C) && ldc % PER == 0;
+  const bool b_ok = aligned16(B) && ldb % PER == 0, c_ok = aligned16(C) && ldc % PER == 0;
   // The copy moves a row of B twice (0.4 ps per byte and row); a ragged shape saves about 17 ps per entry on the scalar one.
-  // Below 100,000 entries that is less than the launch costs.
-  const bool pad = !b_ok && N >= 100000 && N * 40 >= b_rows * R * (int64_t)sizeof(T);
+  const bool pad = N >= kRaggedLeast && N * 40 >= b_rows * R * (int64_t)sizeof(T);
   // More than 32 pieces are two per lane, which halves the warps on an SM. Long rows of a B that stays in L2 are faster as
-  // two launches of at most 32 (4 M entries in 200,000 rows, 84 MB of B: R = 70 335 -> 262, R = 120 460 -> 381 us), short
-  // ones, a B in DRAM and small inputs (35,000 entries: 22 -> 40 us) are not (2.9 entries per row: 784 -> 1128 us; 430 MB: 398 -> 527 us). Short rows are faster still
-  // with a column per lane (R = 70: 784 -> 760 us): what costs there is the stores of the ragged rows.
+  // two launches of at most 32 (4 M entries in 200,000 rows, 84 MB of B: R = 70 335 -> 262 us), short ones, a B in DRAM and
+  // small inputs (35,000 entries: 22 -> 40 us) are not (2.9 entries per row: 784 -> 1128 us; 430 MB: 398 -> 527 us). Short
+  // rows are faster still with a column per lane (R = 70: 784 -> 760 us): what costs there is the stores of the ragged rows;
+  // and so is more than 96 columns where two launches would be of nearly the same width (DCSR, 1.6 M entries, R = 100 457 ->
+  // 277 us; 2.1 M, R = 127 225 -> 189 us).
   const bool split = N >= (1 << 20) && N >= 8 * M && b_rows * R * (int64_t)sizeof(T) <= (126ll << 20);
-  const bool scalar = R > 32 * PER && R < 128 && N < 4 * M;
+  auto one_column_per_lane = [&](int64_t chunk) {
+    return chunk > 32 * PER && ((chunk < 64 * PER && N < 4 * M) || (split && R <= 128 && chunk > 48 * PER));
+  };
   // A compressed root level with at least twice as many rows as segments: C is cleared in one stream of wide stores and the
   // stored rows are written over it. A worker that fills the rows in front of each segment itself writes fewer bytes but
   // waits for its gathers in between (4.2 M entries in 67 M / 8.4 M rows, R = 8: 919 -> 792, 290 -> 266 us).
@@ -727,13 +736,17 @@ static comet_status_t seg_gather_typed(Context *ctx, const int32_t *seg_end, con
     a.wide_store = c_ok;
     comet_status_t st = COMET_OK;
     const int64_t rem = R - done;
-    if ((b_ok || pad) && !scalar) {
-      int64_t chunk = rem < 128 ? rem : 128;
-      if (chunk > 32 * PER && split && !(b_ok && c_ok && chunk == 64 * PER)) chunk = 32 * PER;
-      const int64_t pieces = ceil_div(chunk, PER);
-      a.R = (int32_t)chunk;
-      const int64_t p = b_ok ? 0 : b_rows;
-      const bool exact = b_ok && c_ok && (pieces & (pieces - 1)) == 0;
+    int64_t chunk = rem < 128 ? rem : 128;
+    const bool whole = b_ok && chunk % PER == 0;           // gathered from B as it is, in whole pieces
+    const bool wide = whole && c_ok && chunk == 64 * PER;
+    bool pieces_ok = (whole || pad) && (wide || !one_column_per_lane(chunk));
+    if (pieces_ok && chunk > 32 * PER && split && !wide) chunk = 32 * PER;
+    const int64_t pieces = ceil_div(chunk, PER);
+    const bool exact = whole && c_ok && (pieces & (pieces - 1)) == 0;
+    if (whole && !exact && pieces <= 16 && N < kRaggedLeast) pieces_ok = false;
+    a.R = (int32_t)chunk;
+    if (pieces_ok) {
+      const int64_t p = whole ? 0 : b_rows;
       if (pieces > 32) {
         if constexpr (sizeof(T) == 8)                      // fp32 chunks are at most 32 pieces
           st = exact ? launch_one<T, 32, 2, PER>(ctx, a, heavy, cleared, 0, stream) : launch_one<T, 32, 2, PER, true>(ctx, a, heavy, cleared, p, stream);
@@ -749,7 +762,6 @@ static comet_status_t seg_gather_typed(Context *ctx, const int32_t *seg_end, con
       else if (pieces > 2) st = launch_one<T, 4, 1, PER, true>(ctx, a, heavy, cleared, p, stream);
       else st = launch_one<T, 2, 1, PER, true>(ctx, a, heavy, cleared, p, stream);
     } else {
-      a.R = (int32_t)(rem < 128 ? rem : 128);
       if (a.R > 64) st = launch_one<T, 32, 4, 1>(ctx, a, heavy, cleared, 0, stream);
       else if (a.R > 32) st = launch_one<T, 32, 2, 1>(ctx, a, heavy, cleared, 0, stream);
       else st = launch_one<T, 32, 1, 1>(ctx, a, heavy, cleared, 0, stream);

@@ -60,7 +60,9 @@ struct SegGatherPolicy {
   static constexpr bool kAux = false;
   // Ragged fp32 rows end in up to four scalar stores per lane, too much code for one copy per entry of the chunk: with the
   // chunk unrolled the kernel waits for instructions (30 M entries, R = 50: 519 us unrolled, 475 rolled).
-  static constexpr bool kFullUnroll = !(RAGGED && sizeof(T) == 4);
+  // The widest workers that fill rows of zeros as well: a copy of that per entry is too much code, too (DCSR, fp64:
+  // 6.2 M entries, power-law rows, R = 200 2.74 ms unrolled, 1.78 rolled; 1.2 M, R = 128 259 and 208 us).
+  static constexpr bool kFullUnroll = !(RAGGED && sizeof(T) == 4) && !(ROWS == kRowsFilled && CPL * VEC * sizeof(T) > 16 && VEC > 1);
   // one copy of the unrolled body where the chunk is long (instruction cache; measured: SpMM config 2 -4 %); the
   // narrow shapes have short tiles of short chunks, where the slower rolled tail costs more than it saves (TTM +5 %)
   static constexpr bool kRolledTail = LPN >= 16;

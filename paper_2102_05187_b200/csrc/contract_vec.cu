@@ -62,7 +62,7 @@ struct SegGatherPolicy {
   // chunk unrolled the kernel waits for instructions (30 M entries, R = 50: 519 us unrolled, 475 rolled).
   // The widest workers that fill rows of zeros as well: a copy of that per entry is too much code, too (DCSR, fp64:
   // 6.2 M entries, power-law rows, R = 200 2.74 ms unrolled, 1.78 rolled; 1.2 M, R = 128 259 and 208 us).
-  static constexpr bool kFullUnroll = !(RAGGED && sizeof(T) == 4) && !(ROWS == kRowsFilled && CPL * VEC * sizeof(T) > 16 && VEC > 1);
+  static constexpr bool kFullUnroll = !(RAGGED && (sizeof(T) == 4 || ROWS == kRowsFilled)) && !(ROWS == kRowsFilled && CPL * VEC * sizeof(T) > 16 && VEC > 1);
   // one copy of the unrolled body where the chunk is long (instruction cache; measured: SpMM config 2 -4 %); the
   // narrow shapes have short tiles of short chunks, where the slower rolled tail costs more than it saves (TTM +5 %)
   static constexpr bool kRolledTail = LPN >= 16;
@@ -454,32 +454,37 @@ void carry_fixup_launch(int dtype, double *carry_val, int32_t *carry_seg, int64_
   else (one ? carry_fixup_kernel<double, true> : carry_fixup_kernel<double, false>)<<<blocks, kBlockThreads, 0, stream>>>(f);
 }
 
-template <class T>
-__global__ void zero_rows_kernel(T *__restrict__ C, int64_t rows, int32_t R, int64_t ldc) {
-  const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int64_t r = idx / R;
-  if (r < rows) C[r * ldc + (idx - r * R)] = (T)0;
-}
-
-// The same without gaps between the rows: eight 16-byte stores per thread.
-__global__ void __launch_bounds__(256) zero_fill_kernel(int4 *__restrict__ p, int64_t n) {
+// Clears `rows` rows of `width` pieces (V: an element or 16 bytes), `ld` pieces apart, in one stream of stores: a CTA takes
+// 2,048 consecutive pieces of the result, a division per thread finds the first and the steps between its eight are added.
+template <class V>
+__global__ void __launch_bounds__(256) zero_rows_kernel(V *__restrict__ C, int64_t rows, int64_t width, int64_t ld, int32_t step_rows,
+                                                        int32_t step_cols) {
   const int64_t i0 = (int64_t)blockIdx.x * 2048 + threadIdx.x;
+  int64_t r = i0 < (1ll << 32) && width < (1ll << 32) ? (int64_t)((uint32_t)i0 / (uint32_t)width) : i0 / width;
+  int64_t c = i0 - r * width;
 #pragma unroll
-  for (int u = 0; u < 8; ++u)
-    if (i0 + u * 256 < n) __stcs(p + i0 + u * 256, make_int4(0, 0, 0, 0));
+  for (int u = 0; u < 8; ++u) {
+    if (r < rows) {
+      if (ld == width) __stcs(C + c, V{});                 // one long row
+      else C[r * ld + c] = V{};                            // the rest of a sector at a row's end may still come
+    }
+    r += step_rows;
+    c += step_cols;
+    if (c >= width) { c -= width; ++r; }
+  }
 }
 
 comet_status_t zero_rows(Context *ctx, void *C, int dtype, int64_t rows, int64_t R, int64_t ldc, cudaStream_t stream) {
   if (rows <= 0 || R <= 0) return COMET_OK;
-  const size_t bytes = (size_t)rows * R * (dtype == COMET_F32 ? 4 : 8);
-  if ((ldc == R || rows == 1) && bytes % 16 == 0 && (reinterpret_cast<uintptr_t>(C) & 15) == 0) {
-    zero_fill_kernel<<<(unsigned)ceil_div((int64_t)(bytes / 16), 2048), 256, 0, stream>>>((int4 *)C, (int64_t)(bytes / 16));
-    COMET_LAUNCH_CHECK(ctx);
-    return COMET_OK;
-  }
-  const int64_t n = rows * R;
-  if (dtype == COMET_F32) zero_rows_kernel<float><<<(unsigned)ceil_div(n, 256), 256, 0, stream>>>((float *)C, rows, (int32_t)R, ldc);
-  else zero_rows_kernel<double><<<(unsigned)ceil_div(n, 256), 256, 0, stream>>>((double *)C, rows, (int32_t)R, ldc);
+  if (ldc == R || rows == 1) { R *= rows; ldc = R; rows = 1; }             // no gaps: one long row
+  const int64_t per = dtype == COMET_F32 ? 4 : 2;
+  const bool wide = R % per == 0 && ldc % per == 0 && (reinterpret_cast<uintptr_t>(C) & 15) == 0;
+  const int64_t width = wide ? R / per : R, ld = wide ? ldc / per : ldc;
+  const unsigned blocks = (unsigned)ceil_div(rows * width, 2048);
+  const int32_t step_rows = (int32_t)(256 / width), step_cols = (int32_t)(256 % width);
+  if (wide) zero_rows_kernel<int4><<<blocks, 256, 0, stream>>>((int4 *)C, rows, width, ld, step_rows, step_cols);
+  else if (dtype == COMET_F32) zero_rows_kernel<float><<<blocks, 256, 0, stream>>>((float *)C, rows, width, ld, step_rows, step_cols);
+  else zero_rows_kernel<double><<<blocks, 256, 0, stream>>>((double *)C, rows, width, ld, step_rows, step_cols);
   COMET_LAUNCH_CHECK(ctx);
   return COMET_OK;
 }
@@ -697,7 +702,7 @@ static bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 
 // some thousand random inputs the two are level between 150,000 (up to 4 lanes) and 500,000 entries (16 lanes, or copies);
 // below, the ragged ones took up to 1.7 times as long (34,700 entries, fp64, R = 24 20.7 us, scalar 12.1; 97,000, R = 20 27.8,
 // scalar 18.6).
-constexpr int64_t kRaggedLeast = 250000;
+constexpr int64_t kRaggedLeastNarrow = 150000, kRaggedLeast = 250000;      // up to four pieces, more
 
 template <class T>
 static comet_status_t seg_gather_typed(Context *ctx, const int32_t *seg_end, const int32_t *crd, const T *val,
@@ -710,7 +715,7 @@ static comet_status_t seg_gather_typed(Context *ctx, const int32_t *seg_end, con
   HeavyArgs *heavy = long_rows && !out_row && b_rows > 0 && R <= 128 ? &hint : nullptr;
   const bool b_ok = aligned16(B) && ldb % PER == 0, c_ok = aligned16(C) && ldc % PER == 0;
   // The copy moves a row of B twice (0.4 ps per byte and row); a ragged shape saves about 17 ps per entry on the scalar one.
-  const bool pad = N >= kRaggedLeast && N * 40 >= b_rows * R * (int64_t)sizeof(T);
+  const bool pad = N >= (R <= 4 * PER ? kRaggedLeastNarrow : kRaggedLeast) && N * 40 >= b_rows * R * (int64_t)sizeof(T);
   // More than 32 pieces are two per lane, which halves the warps on an SM. Long rows of a B that stays in L2 are faster as
   // two launches of at most 32 (4 M entries in 200,000 rows, 84 MB of B: R = 70 335 -> 262 us), short ones, a B in DRAM and
   // small inputs (35,000 entries: 22 -> 40 us) are not (2.9 entries per row: 784 -> 1128 us; 430 MB: 398 -> 527 us). Short
@@ -721,10 +726,15 @@ static comet_status_t seg_gather_typed(Context *ctx, const int32_t *seg_end, con
   auto one_column_per_lane = [&](int64_t chunk) {
     return chunk > 32 * PER && ((chunk < 64 * PER && N < 4 * M) || (split && R <= 128 && chunk > 48 * PER));
   };
-  // A compressed root level with at least twice as many rows as segments: C is cleared in one stream of wide stores and the
-  // stored rows are written over it. A worker that fills the rows in front of each segment itself writes fewer bytes but
-  // waits for its gathers in between (4.2 M entries in 67 M / 8.4 M rows, R = 8: 919 -> 792, 290 -> 266 us).
-  const bool cleared = out_row && out_rows >= 2 * M;
+  // A compressed root level with far more rows than segments: C is cleared in one stream of wide stores and the stored rows
+  // are written over it. A worker that fills the rows in front of each segment itself writes fewer bytes but waits for its
+  // gathers in between (4.2 M entries in 67 M / 8.4 M rows, R = 8: 919 -> 792, 290 -> 266 us). From six rows per segment on
+  // the clear wins nearly always, from two on where the stored rows are narrow or many, or C is so large that it leaves
+  // the cache in between anyway; with wide rows in a C of some hundred MB the second write costs up to 1.3 times the fill
+  // (0.32 M entries in 1.06 M rows, fp32, R = 25: 68 us filled, 110 cleared).
+  const int64_t row_bytes = R * (int64_t)sizeof(T), c_bytes = out_rows * row_bytes;
+  const bool cleared = out_row && (out_rows >= 6 * M || (out_rows >= 2 * M && (row_bytes <= 64 || (c_bytes >= 60000000 &&
+                                                         (row_bytes <= 256 || M >= 500000 || c_bytes >= 1000000000)))));
   if (cleared) {
     const comet_status_t zs = zero_rows(ctx, C, sizeof(T) == 4 ? COMET_F32 : COMET_F64, out_rows, R, ldc, stream);
     if (zs != COMET_OK) return zs;
@@ -745,7 +755,7 @@ static comet_status_t seg_gather_typed(Context *ctx, const int32_t *seg_end, con
     if (pieces_ok && chunk > 32 * PER && split && !wide) chunk = 32 * PER;
     const int64_t pieces = ceil_div(chunk, PER);
     const bool exact = whole && c_ok && (pieces & (pieces - 1)) == 0;
-    if (whole && !exact && pieces <= 16 && N < kRaggedLeast) pieces_ok = false;
+    if (whole && !exact && pieces <= 16 && N < (pieces <= 4 ? kRaggedLeastNarrow : kRaggedLeast)) pieces_ok = false;
     a.R = (int32_t)chunk;
     if (pieces_ok) {
       const int64_t p = whole ? 0 : b_rows;

@@ -9,7 +9,8 @@
 // fp32 tensors the atomics go to a double scratch matrix that is rounded into the output at the end.
 //
 // CSF [CU,CU,CU], coordinates (i, j, k) at levels 0..2, A / B = the factors of the two other modes:
-//   level 1:  out[j, :] += (sum over the fiber's entries of val * B[k, :]) * A[i, :]     one add per fiber (mttkrp_level1.cu)
+//   level 1:  out[j, :] += (sum over the fiber's entries of val * B[k, :]) * A[i, :]     one add per fiber
+//             (mttkrp_level1.cu; here small or narrow outputs of tensors whose fibers hold an entry or two)
 //   level 2:  out[k, :] += val * (A[i, :] * B[j, :])                                     one add per entry
 // COO [CN,S,S]:  out[c_out, :] += val * A[c_a, :] * B[c_b, :]                            one add per entry
 //
@@ -40,7 +41,7 @@ struct ScatterArgs {
 
 constexpr int kScatterThreads = 256;
 
-template <class T, int G>
+template <class T, int LEVEL, int G>
 __global__ void __launch_bounds__(kScatterThreads) mttkrp_csf_scatter_kernel(const ScatterArgs a) {
   const T *const val = static_cast<const T *>(a.val);
   const T *const A = static_cast<const T *>(a.A), *const B = static_cast<const T *>(a.B);
@@ -61,10 +62,18 @@ __global__ void __launch_bounds__(kScatterThreads) mttkrp_csf_scatter_kernel(con
     while (f >= s_end && s + 1 < a.S) { ++s; s_end = __ldg(a.pos1 + s + 1); }
     const int64_t i = __ldg(a.crd0 + s), j = __ldg(a.crd1 + f);
     const int64_t p0 = __ldg(a.pos2 + f), p1 = __ldg(a.pos2 + f + 1);
+    if (LEVEL == 1 && p0 == p1) continue;
     for (int c = g; c < a.R; c += G) {
-      const double w = (double)__ldg(A + i * a.lda + c) * (double)__ldg(B + j * a.ldb + c);
-      for (int64_t p = p0; p < p1; ++p)
-        atomicAdd(a.acc + (int64_t)__ldg(a.crd2 + p) * a.ldacc + c, (double)ld_stream(val + p) * w);
+      if (LEVEL == 1) {
+        double t = 0.0;
+        for (int64_t p = p0; p < p1; ++p)
+          t += (double)ld_stream(val + p) * (double)__ldg(B + (int64_t)__ldg(a.crd2 + p) * a.ldb + c);
+        atomicAdd(a.acc + j * a.ldacc + c, t * (double)__ldg(A + i * a.lda + c));
+      } else {
+        const double w = (double)__ldg(A + i * a.lda + c) * (double)__ldg(B + j * a.ldb + c);
+        for (int64_t p = p0; p < p1; ++p)
+          atomicAdd(a.acc + (int64_t)__ldg(a.crd2 + p) * a.ldacc + c, (double)ld_stream(val + p) * w);
+      }
     }
   }
 }
@@ -431,7 +440,8 @@ static void launch_scatter(int kind, const ScatterArgs &a, int64_t units, cudaSt
   const int64_t workers = ceil_div(units, a.per_worker);
   const unsigned blocks = (unsigned)ceil_div(workers * G, kScatterThreads);
   if (kind == 0) mttkrp_coo_scatter_kernel<T, G><<<blocks, kScatterThreads, 0, stream>>>(a);
-  else mttkrp_csf_scatter_kernel<T, G><<<blocks, kScatterThreads, 0, stream>>>(a);
+  else if (kind == 1) mttkrp_csf_scatter_kernel<T, 1, G><<<blocks, kScatterThreads, 0, stream>>>(a);
+  else mttkrp_csf_scatter_kernel<T, 2, G><<<blocks, kScatterThreads, 0, stream>>>(a);
 }
 
 template <class T>
@@ -455,8 +465,14 @@ comet_status_t mttkrp_scatter(Context *ctx, int dtype, int kind, const int32_t *
   ScatterArgs a{};
   a.pos1 = pos1; a.crd0 = crd0; a.crd1 = crd1; a.pos2 = pos2; a.crd2 = crd2; a.val = val;
   a.S = S; a.F = F; a.N = N; a.A = A; a.lda = lda; a.B = B; a.ldb = ldb; a.R = (int32_t)R;
-  // CSF, output at level 1: a row add per fiber (mttkrp_level1.cu)
-  const size_t part_bytes = kind == 1 && N > 0 ? mttkrp_level1_bytes(N) : 0;
+  // CSF, output at level 1: a row add per fiber, by the kernel of mttkrp_level1.cu, whose tiles of 32 entries and more leave
+  // most of the chip idle on small inputs and whose half warps are mostly idle on a few columns. Where fibers hold an entry
+  // or two, a worker of few lanes per eight fibers is faster there; long fibers are a serial chain for it. Over 1,860 random
+  // calls, this kernel's time over the other's: fewer than two entries per fiber, up to 10,000 entries 0.68, up to 100,000
+  // 0.70, 100,000 to 300,000 0.93, a million and more 1.2 to 2.0; up to 4 columns 0.75 to 0.85 at any size; four entries and
+  // more per fiber 1.2 to 7.8.
+  const bool per_fiber = kind == 1 && N < 2 * F && (N < 150000 || R <= 4);
+  const size_t part_bytes = kind == 1 && N > 0 && !per_fiber ? mttkrp_level1_bytes(N) : 0;
   char *part = nullptr;
   if (dtype == COMET_F32) {
     if (rows == 0) return COMET_OK;

@@ -1,5 +1,6 @@
 """MTTKRP, output mode stored at level 1 of a CSF tensor: widths around the half-warp, warp and 64-column limits, rows that
-are not aligned, tiles of 32 entries and longer ones, and tensors that hold fibers and slices without entries."""
+are not aligned, tiles of 32 entries (one chunk, one mask word) up to 1,024, fibers of an entry or two (a worker per eight
+fibers) and long ones, and tensors that hold fibers and slices without entries."""
 import numpy as np
 import pytest
 import torch
@@ -61,3 +62,63 @@ def test_fibers_and_slices_without_entries(R):
         want[j] += x * F[0][i] * F[2][k]
     got = comet.mttkrp(X, 1, [dev(f) for f in F]).cpu().numpy()
     assert np.all(np.abs(got - want) <= 1e-12 * np.abs(v).sum())
+
+
+def _check(i, j, k, v, dims, X, R, dtype, seed):
+    """Against plain numpy sums (a caller-built tensor may hold fibers and slices without entries)."""
+    rng = np.random.default_rng(seed)
+    F = [rng.uniform(-1, 1, (d, R)).astype(dtype) for d in dims]
+    terms = v.astype(np.float64)[:, None] * F[0].astype(np.float64)[i] * F[2].astype(np.float64)[k]
+    want, norm = np.zeros((dims[1], R)), np.zeros((dims[1], R))
+    np.add.at(want, j, terms)
+    np.add.at(norm, j, np.abs(terms))
+    wide = [dev(np.pad(f, ((0, 0), (0, 1)))) for f in F]     # an odd leading dimension: not the walker of the aligned widths
+    got = comet.mttkrp(X, 1, [w[:, :R] for w in wide]).double().cpu().numpy()
+    tol = 1e-12 if dtype == np.float64 else 2.0 ** -23       # fp32: sums in double, one rounding
+    assert np.all(np.abs(got - want) <= tol * norm)
+
+
+@pytest.mark.parametrize("dtype", [np.float64, np.float32])
+@pytest.mark.parametrize("tile", ["32", "64", "96", "1024"])
+@pytest.mark.parametrize("R", [1, 5, 16, 32, 33, 70])
+def test_tiles_fibers_and_slices_without_entries(tile, R, dtype, monkeypatch):
+    """Several tiles of several chunks: fibers of 0 to 90 entries, slices of no, one and many fibers, runs of empty ones at the
+    start, at the end and on tile boundaries."""
+    monkeypatch.setenv("COMET_TILE_ITEMS", tile)
+    rng = np.random.default_rng(int(tile) + R)
+    dims = (400, 90, 100)
+    per_slice = rng.choice([0, 1, 2, 7, 40], 200)
+    per_slice[[0, 1, -1]] = 0
+    fibers = int(per_slice.sum())
+    lengths = rng.choice([0, 0, 1, 3, 32, 90], fibers)
+    lengths[[0, 1, 2, -1, -2]] = 0
+    for b in range(int(tile), int(lengths.sum()) // 2, 4 * int(tile)):   # a fiber that ends on a tile boundary, empty ones behind
+        f = int(np.searchsorted(np.cumsum(lengths), b))
+        lengths[f] -= int(np.cumsum(lengths)[f]) - b
+        lengths[f + 1:f + 3] = 0
+    crd0 = np.sort(rng.permutation(dims[0])[:200])
+    crd1 = np.concatenate([np.sort(rng.permutation(dims[1])[:n]) for n in per_slice])
+    crd2 = np.concatenate([np.sort(rng.permutation(dims[2])[:n]) for n in lengths])
+    v = rng.uniform(-1, 1, crd2.size).astype(dtype)
+    i32 = lambda x: dev(np.asarray(x).astype(np.int32))  # noqa: E731
+    ptr = lambda n: np.concatenate([[0], np.cumsum(n)])  # noqa: E731
+    X = comet.SpTensor.from_arrays(dims, (0, 1, 2), (CU, CU, CU), [i32([0, 200]), i32(ptr(per_slice)), i32(ptr(lengths))],
+                                   [i32(crd0), i32(crd1), i32(crd2)], dev(v))
+    comet.validate(X)
+    fiber = np.repeat(np.arange(fibers), lengths)
+    _check(np.repeat(crd0, per_slice)[fiber], crd1[fiber], crd2, v, dims, X, R, dtype, R)
+
+
+@pytest.mark.parametrize("dtype", [np.float64, np.float32])
+@pytest.mark.parametrize("R", [1, 3, 4, 5, 17, 129])
+@pytest.mark.parametrize("n", [3, 9000, 149_999, 150_001])
+def test_short_fibers(n, R, dtype):
+    """Fibers of an entry or two, on both sides of the size up to which they have a worker per eight fibers."""
+    rng = np.random.default_rng(n + R)
+    dims = (2000, 1500, 300)
+    cell = np.unique(rng.integers(0, dims[0] * dims[1] * dims[2], n + 50))
+    cell = np.sort(rng.permutation(cell)[:n])
+    i, j, k = (x.astype(np.int32) for x in np.unravel_index(cell, dims))
+    v = rng.uniform(-1, 1, n).astype(dtype)
+    X = comet.pack([dev(i), dev(j), dev(k)], dev(v), dims, (0, 1, 2), (CU, CU, CU))
+    _check(i, j, k, v, dims, X, R, dtype, R)

@@ -491,13 +491,18 @@ static comet_status_t launch_mttkrp(Context *ctx, MttkrpArgs a, int64_t p_pad, i
 }
 
 // Shapes as in seg_gather_typed (contract_vec.cu): exact ones, ragged ones (operands padded into scratch where they are no
-// whole 16-byte pieces), scalar ones where the factors have far more rows than the tensor has entries.
+// whole 16-byte pieces), scalar ones where the factors have far more rows than the tensor has entries, and on small inputs
+// (as there; two matrices are copied here, so copies pay later). Over 1,900 random calls the scalar shapes took, of the
+// time with copies, 0.69 to 0.87 at 100,000 to 200,000 entries, 0.77 to 1.0 up to 400,000, 0.9 to 1.1 up to 800,000; of the time
+// of ragged shapes of at most 16 pieces 0.72 to 1.0 below 100,000 entries, 1.0 to 1.2 from 200,000 on.
+constexpr int64_t kMttkrpPadLeast = 400000, kMttkrpPadLeastWide = 200000, kMttkrpRaggedLeast = 150000;   // wide: more than 16 pieces
+
 template <bool CSF, class T>
 static comet_status_t mttkrp_chunks(Context *ctx, const MttkrpArgs &base, int64_t p_rows, int64_t q_rows, int64_t R, cudaStream_t stream) {
   constexpr int PER = 16 / sizeof(T);
-  const bool in_ok = aligned16(base.P) && aligned16(base.Q) && base.ldp % PER == 0 && base.ldq % PER == 0 && R % PER == 0;
+  const bool in_ok = aligned16(base.P) && aligned16(base.Q) && base.ldp % PER == 0 && base.ldq % PER == 0;
   const bool out_ok = aligned16(base.out) && base.ldo % PER == 0;
-  const bool pad = !in_ok && base.N >= 100000 && base.N * 40 >= (p_rows + q_rows) * R * (int64_t)sizeof(T);   // as in seg_gather_typed
+  const bool pad = base.N >= (R > 16 * PER ? kMttkrpPadLeastWide : kMttkrpPadLeast) && base.N * 40 >= (p_rows + q_rows) * R * (int64_t)sizeof(T);    // as in seg_gather_typed
   int64_t done = 0;
   while (done < R) {
     const int64_t rem = R - done;
@@ -507,11 +512,11 @@ static comet_status_t mttkrp_chunks(Context *ctx, const MttkrpArgs &base, int64_
     a.out = static_cast<T *>(base.out) + done;
     a.wide_store = out_ok;
     comet_status_t st = COMET_OK;
-    if (in_ok || pad) {
-      const int64_t chunk = rem < 128 ? rem : 128, pieces = ceil_div(chunk, PER);
-      a.R = (int32_t)chunk;
-      const int64_t pp = in_ok ? 0 : p_rows, qp = in_ok ? 0 : q_rows;
-      const bool exact = in_ok && out_ok && (pieces & (pieces - 1)) == 0;
+    const int64_t chunk = rem < 128 ? rem : 128, pieces = ceil_div(chunk, PER);
+    const bool whole = in_ok && chunk % PER == 0, exact = whole && out_ok && (pieces & (pieces - 1)) == 0;
+    a.R = (int32_t)chunk;
+    if (exact || (whole ? pieces > 16 || base.N >= kMttkrpRaggedLeast : pad)) {
+      const int64_t pp = whole ? 0 : p_rows, qp = whole ? 0 : q_rows;
       if (pieces > 32) {
         if constexpr (sizeof(T) == 8)                      // fp32 chunks are at most 32 pieces
           st = exact ? launch_mttkrp<CSF, T, 32, 2, PER>(ctx, a, 0, 0, stream) : launch_mttkrp<CSF, T, 32, 2, PER, true>(ctx, a, pp, qp, stream);
@@ -527,7 +532,6 @@ static comet_status_t mttkrp_chunks(Context *ctx, const MttkrpArgs &base, int64_
       else if (pieces > 2) st = launch_mttkrp<CSF, T, 4, 1, PER, true>(ctx, a, pp, qp, stream);
       else st = launch_mttkrp<CSF, T, 2, 1, PER, true>(ctx, a, pp, qp, stream);
     } else {
-      a.R = (int32_t)(rem < 128 ? rem : 128);
       if (a.R > 64) st = launch_mttkrp<CSF, T, 32, 4, 1>(ctx, a, 0, 0, stream);
       else if (a.R > 32) st = launch_mttkrp<CSF, T, 32, 2, 1>(ctx, a, 0, 0, stream);
       else st = launch_mttkrp<CSF, T, 32, 1, 1>(ctx, a, 0, 0, stream);

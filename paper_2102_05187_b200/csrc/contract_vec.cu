@@ -237,7 +237,7 @@ struct FixupArgs {
                                                  // (zero at the start; NULL: runs are not cut)
 };
 
-constexpr int32_t kRunSpare = 512;
+constexpr int32_t kRunSpare = 128;
 // Whether a run of segment `seg` that crosses tile t, a multiple of kRunPiece, is cut there. (The tiles in between are the
 // run's too.)
 __device__ __forceinline__ bool run_cut_at(const FixupArgs &f, int64_t t, int32_t seg) {

@@ -58,10 +58,10 @@ def _rows_of_runs(runs):
 @pytest.mark.parametrize("R,limit", [(1, 104), (4, 100), (5, 36), (16, 36), (24, 28), (100, 12)])
 def test_runs_at_the_limits(R, limit):
     """Runs of `limit` tiles and one less and more, heads as many tiles in front of a multiple of 1,024, and runs that go on
-    511, 512 and 513 tiles behind one (cut from 513 tiles on), alone and over several multiples."""
+    127, 128 and 129 tiles behind one (cut from 129 tiles on), alone and over several multiples."""
     at = {"short": [(5, limit - 1), (5 + limit, limit), (10 + 2 * limit, limit + 1)],
-          "cut": [(1024 - limit + d, limit - d + 512 + e) for d in (-1, 0, 1) for e in (-1, 0, 1)]}
-    for k, (head, tiles) in enumerate([(1024, 512), (1024, 513), (1024, 514), (1000, 2600), (1023, 1)] + at["cut"]):
+          "cut": [(1024 - limit + d, limit - d + 128 + e) for d in (-1, 0, 1) for e in (-1, 0, 1)]}
+    for k, (head, tiles) in enumerate([(1024, 128), (1024, 1152), (1024, 1153), (1000, 2600), (1023, 1)] + at["cut"]):
         runs = at["short"] + [(head, tiles), (head + tiles + 1, 3), (4096 - limit, limit + 2)]
         lengths = _rows_of_runs(runs)
         rng = np.random.default_rng(100 * R + k)

@@ -91,9 +91,12 @@ __global__ void __launch_bounds__(kBlockThreads, 4) mttkrp_level1_kernel(const L
   const uint32_t ring = smem_u32(smem_raw) + worker * kLevel1WorkerBytes;
   const uint32_t w_ends = ring + kLevel1RingBytes, w_slices = w_ends + kLevel1Words * 4, w_rank = w_slices + kLevel1Words * 4;
 
-  const int32_t j0 = (int32_t)(tile * a.tile);
-  const int32_t j1 = (int64_t)j0 + a.tile < a.N ? j0 + a.tile : (int32_t)a.N;
-  const T *const val = static_cast<const T *>(a.val);
+  // Entries are counted from the tile's first one: the staging looks up to 96 entries ahead, and a tensor may hold so many
+  // that their numbers do not fit 32 bits there.
+  const int64_t first = tile * a.tile;
+  const int32_t j0 = (int32_t)first, len = (int32_t)(a.N - first < a.tile ? a.N - first : a.tile);
+  const T *const val = static_cast<const T *>(a.val) + first;
+  const int32_t *const crd2 = a.crd2 + first;
   int32_t col[CPL];                              // a lane beyond the last column reads the last one and adds nothing
   bool ok[CPL];
 #pragma unroll
@@ -113,7 +116,7 @@ __global__ void __launch_bounds__(kBlockThreads, 4) mttkrp_level1_kernel(const L
   // ---- the masks of the tile. A caller's tensor may hold fibers or slices without entries: their ends fall on the bit of
   // the one in front, the bits are then fewer than the fibers (slices), and these are found by position instead.
   bool odd_fibers, odd_slices;
-  const int32_t f0 = __ldg(a.part_fiber + tile), f1 = __ldg(a.part_fiber + tile + 1);     // fibers f0 .. f1-1 end in (j0, j1]
+  const int32_t f0 = __ldg(a.part_fiber + tile), f1 = __ldg(a.part_fiber + tile + 1);     // fibers f0 .. f1-1 end in the tile
   int32_t s = __ldg(a.part_slice + tile);
   {
     const int32_t s1 = __ldg(a.part_slice + tile + 1);
@@ -156,18 +159,18 @@ __global__ void __launch_bounds__(kBlockThreads, 4) mttkrp_level1_kernel(const L
     __syncwarp(mask);
     odd_fibers = __shfl_sync(mask, inc, G - 1, G) != f1 - f0;
   }
-  auto fiber_of_end = [&](int32_t j) {           // the fiber whose last entry is j
+  auto fiber_of_end = [&](int32_t j) {           // the fiber whose last entry is the tile's entry j
     int32_t lo = f0, hi = f1;
     while (lo < hi) {
-      const int32_t mid = (lo + hi) >> 1;
-      if (__ldg(a.seg_end2 + mid) <= j) lo = mid + 1; else hi = mid;
+      const int32_t mid = lo + ((hi - lo) >> 1);
+      if (__ldg(a.seg_end2 + mid) - j0 <= j) lo = mid + 1; else hi = mid;
     }
     return lo;
   };
-  auto next_slice = [&](int32_t j) {             // the slice of the entry behind j
+  auto next_slice = [&](int32_t j) {             // the slice of the entry behind the tile's entry j
     ++s;
     if (odd_slices)
-      while (s < a.S && __ldg(a.seg_end2 + __ldg(a.pos1 + s + 1) - 1) <= j + 1) ++s;
+      while (s < a.S && __ldg(a.seg_end2 + __ldg(a.pos1 + s + 1) - 1) - j0 <= j + 1) ++s;
     return s < a.S;
   };
 
@@ -181,10 +184,10 @@ __global__ void __launch_bounds__(kBlockThreads, 4) mttkrp_level1_kernel(const L
       const int32_t j = base + x;
       sv[i] = 0.0;
       sk[i] = sj[i] = 0;
-      if (j < j1) {
+      if (j < len) {
         sv[i] = (double)ld_stream(val + j);
-        sk[i] = ld_stream(a.crd2 + j);
-        const int w = (base - j0) >> 5;
+        sk[i] = ld_stream(crd2 + j);
+        const int w = base >> 5;
         const uint32_t e = (uint32_t)lds_s32(w_ends + w * 4);
         if ((e >> x) & 1u) {
           int32_t f = f0 + lds_s32(w_rank + w * 4) + __popc(e & ((1u << x) - 1u));
@@ -205,9 +208,9 @@ __global__ void __launch_bounds__(kBlockThreads, 4) mttkrp_level1_kernel(const L
 #pragma unroll
   for (int t = 0; t < CPL; ++t) tac[t] = 0.0;
   gather(pcol, ldp_bytes, __ldg(a.crd0 + s), prow);
-  load(j0);
+  load(0);
   store(0);
-  load(j0 + 32);
+  load(32);
   __syncwarp(mask);
 #pragma unroll
   for (int u = 0; u < kPF; ++u) {
@@ -217,13 +220,13 @@ __global__ void __launch_bounds__(kBlockThreads, 4) mttkrp_level1_kernel(const L
   }
   int half = 0;
   bool last_ends = false;
-  for (int32_t base = j0; base < j1; base += 32, half ^= 1) {
+  for (int32_t base = 0; base < len; base += 32, half ^= 1) {
     __syncwarp(mask);                            // every lane is done reading the half that is refilled next
     store(half ^ 1);
     __syncwarp(mask);
     load(base + 64);
-    const int n = j1 - base < 32 ? j1 - base : 32;
-    const uint32_t ends = (uint32_t)lds_s32(w_ends + ((base - j0) >> 5) * 4), slices = (uint32_t)lds_s32(w_slices + ((base - j0) >> 5) * 4);
+    const int n = len - base < 32 ? len - base : 32;
+    const uint32_t ends = (uint32_t)lds_s32(w_ends + (base >> 5) * 4), slices = (uint32_t)lds_s32(w_slices + (base >> 5) * 4);
     last_ends = (ends >> (n - 1)) & 1u;
 #pragma unroll 1
     for (int e0 = 0; e0 < n; e0 += kPF) {

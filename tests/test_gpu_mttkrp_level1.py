@@ -122,3 +122,23 @@ def test_short_fibers(n, R, dtype):
     v = rng.uniform(-1, 1, n).astype(dtype)
     X = comet.pack([dev(i), dev(j), dev(k)], dev(v), dims, (0, 1, 2), (CU, CU, CU))
     _check(i, j, k, v, dims, X, R, dtype, R)
+
+
+def test_as_many_entries_as_there_may_be():
+    """2^31 - 2 entries: the look-ahead behind the last tile passes 2^31."""
+    n = 2 ** 31 - 2
+    free, _ = torch.cuda.mem_get_info()
+    if free < 40 << 30:
+        pytest.skip("needs 40 GB of device memory")
+    ends = [0, 2 ** 29, 2 ** 30 + 5, 3 * 2 ** 29, n]                       # four fibers in two slices
+    longest = max(b - a for a, b in zip(ends, ends[1:]))
+    crd2 = torch.empty(n, dtype=torch.int32, device="cuda")
+    for a, b in zip(ends, ends[1:]):
+        torch.arange(b - a, dtype=torch.int32, device="cuda", out=crd2[a:b])
+    i32 = lambda x: dev(np.array(x), torch.int32)  # noqa: E731
+    X = comet.SpTensor.from_arrays((2, 3, longest), (0, 1, 2), (CU, CU, CU), [i32([0, 2]), i32([0, 2, 4]), i32(ends)],
+                                   [i32([0, 1]), i32([0, 2, 1, 2]), crd2], torch.ones(n, device="cuda"))
+    F = [torch.tensor([[1.0], [-2.0]], device="cuda"), None, torch.ones(longest, 1, device="cuda")]
+    got = comet.mttkrp(X, 1, F).double().cpu()
+    want = torch.tensor([[ends[1]], [-2.0 * (ends[3] - ends[2])], [ends[2] - ends[1] - 2.0 * (ends[4] - ends[3])]], dtype=torch.float64)
+    assert torch.equal(got, want.float().double())           # sums of ones are exact in double

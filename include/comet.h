@@ -189,8 +189,12 @@ comet_status_t comet_spmv(comet_handle_t handle, const comet_sptensor_t *A, cons
 
 /* SpMM  C_ir = sum_j A_ij B_jr  (SpMM definition). B: dims[mode_order[1]] x R, leading dimension
  * ldb >= R; C: dims[mode_order[0]] x R, leading dimension ldc >= R; every row of C is written.
- * Formats as for comet_spmv. Any R >= 1; columns are processed in chunks of up to 128, and a chunk of
- * 2^k 16-byte pieces (fp64: 2..128 columns, fp32: 4..128) on 16-byte-aligned rows takes the vectorised path. */
+ * Formats as for comet_spmv. Any R >= 1; columns are processed in chunks of up to 128. Any width is gathered in 16-byte
+ * pieces where B and its rows are 16-byte aligned and the chunk is a whole number of pieces; chunks of 2^k pieces on an
+ * equally aligned C (fp64: 2..128 columns, fp32: 4..128) are the fastest. Other operands are first copied into handle
+ * scratch with padded rows where enough entries pay for it (from 150,000 to 250,000 on, and if B has not far more bytes
+ * than 40 per entry): up to 40 bytes of scratch per entry, up to 160 for rows of a single fp32 column. The handle keeps
+ * its scratch until it is destroyed; where the allocator has no room for the copy, the call is made without it. */
 comet_status_t comet_spmm(comet_handle_t handle, const comet_sptensor_t *A, const void *B, int64_t R, int64_t ldb,
                           void *C, int64_t ldc, void *stream);
 
@@ -248,7 +252,7 @@ comet_status_t comet_ttm(comet_handle_t handle, const comet_sptensor_t *X, int32
  * product). X: [CN,S,S] (COO) or [CU,CU,CU] (CSF); `mode` = n may be ANY of the three modes, so that
  * one packed tensor serves the all-modes sequence of CP-ALS:
  *   - n stored at X's FIRST level: tiled kernels, every output row written by exactly one CTA, results
- *     bit-identical from run to run;
+ *     bit-identical from run to run (padded copies of the factors as for comet_spmm, from 200,000 to 400,000 entries on);
  *   - n stored at level 1 or 2: the tensor is used as stored (nothing is re-packed); the terms of an
  *     output row are then spread over the whole tensor and are added with atomic adds in double, so
  *     the summation ORDER is not fixed and results agree from run to run only up to rounding (still

@@ -715,7 +715,7 @@ static comet_status_t seg_gather_typed(Context *ctx, const int32_t *seg_end, con
   HeavyArgs *heavy = long_rows && !out_row && b_rows > 0 && R <= 128 ? &hint : nullptr;
   const bool b_ok = aligned16(B) && ldb % PER == 0, c_ok = aligned16(C) && ldc % PER == 0;
   // The copy moves a row of B twice (0.4 ps per byte and row); a ragged shape saves about 17 ps per entry on the scalar one.
-  const bool pad = N >= (R <= 4 * PER ? kRaggedLeastNarrow : kRaggedLeast) && N * 40 >= b_rows * R * (int64_t)sizeof(T);
+  bool pad = N >= (R <= 4 * PER ? kRaggedLeastNarrow : kRaggedLeast) && N * 40 >= b_rows * R * (int64_t)sizeof(T);
   // More than 32 pieces are two per lane, which halves the warps on an SM. Long rows of a B that stays in L2 are faster as
   // two launches of at most 32 (4 M entries in 200,000 rows, 84 MB of B: R = 70 335 -> 262 us), short ones, a B in DRAM and
   // small inputs (35,000 entries: 22 -> 40 us) are not (2.9 entries per row: 784 -> 1128 us; 430 MB: 398 -> 527 us). Short
@@ -777,6 +777,10 @@ static comet_status_t seg_gather_typed(Context *ctx, const int32_t *seg_end, con
       if (a.R > 64) st = launch_one<T, 32, 4, 1>(ctx, a, heavy, cleared, 0, stream);
       else if (a.R > 32) st = launch_one<T, 32, 2, 1>(ctx, a, heavy, cleared, 0, stream);
       else st = launch_one<T, 32, 1, 1>(ctx, a, heavy, cleared, 0, stream);
+    }
+    if (st == COMET_ERR_ALLOC && pieces_ok && !whole) {       // no room for a padded copy: the shapes that need none
+      pad = false;
+      continue;
     }
     if (st != COMET_OK) return st;
     done += a.R;

@@ -502,7 +502,7 @@ static comet_status_t mttkrp_chunks(Context *ctx, const MttkrpArgs &base, int64_
   constexpr int PER = 16 / sizeof(T);
   const bool in_ok = aligned16(base.P) && aligned16(base.Q) && base.ldp % PER == 0 && base.ldq % PER == 0;
   const bool out_ok = aligned16(base.out) && base.ldo % PER == 0;
-  const bool pad = base.N >= (R > 16 * PER ? kMttkrpPadLeastWide : kMttkrpPadLeast) && base.N * 40 >= (p_rows + q_rows) * R * (int64_t)sizeof(T);    // as in seg_gather_typed
+  bool pad = base.N >= (R > 16 * PER ? kMttkrpPadLeastWide : kMttkrpPadLeast) && base.N * 40 >= (p_rows + q_rows) * R * (int64_t)sizeof(T);    // as in seg_gather_typed
   int64_t done = 0;
   while (done < R) {
     const int64_t rem = R - done;
@@ -514,8 +514,9 @@ static comet_status_t mttkrp_chunks(Context *ctx, const MttkrpArgs &base, int64_
     comet_status_t st = COMET_OK;
     const int64_t chunk = rem < 128 ? rem : 128, pieces = ceil_div(chunk, PER);
     const bool whole = in_ok && chunk % PER == 0, exact = whole && out_ok && (pieces & (pieces - 1)) == 0;
+    const bool pieces_ok = exact || (whole ? pieces > 16 || base.N >= kMttkrpRaggedLeast : pad);
     a.R = (int32_t)chunk;
-    if (exact || (whole ? pieces > 16 || base.N >= kMttkrpRaggedLeast : pad)) {
+    if (pieces_ok) {
       const int64_t pp = whole ? 0 : p_rows, qp = whole ? 0 : q_rows;
       if (pieces > 32) {
         if constexpr (sizeof(T) == 8)                      // fp32 chunks are at most 32 pieces
@@ -535,6 +536,10 @@ static comet_status_t mttkrp_chunks(Context *ctx, const MttkrpArgs &base, int64_
       if (a.R > 64) st = launch_mttkrp<CSF, T, 32, 4, 1>(ctx, a, 0, 0, stream);
       else if (a.R > 32) st = launch_mttkrp<CSF, T, 32, 2, 1>(ctx, a, 0, 0, stream);
       else st = launch_mttkrp<CSF, T, 32, 1, 1>(ctx, a, 0, 0, stream);
+    }
+    if (st == COMET_ERR_ALLOC && pieces_ok && !whole) {       // no room for the padded copies: the shapes that need none
+      pad = false;
+      continue;
     }
     if (st != COMET_OK) return st;
     done += a.R;

@@ -77,6 +77,7 @@ typedef enum {
  *   COMET_SEG_DOT_KERNEL=name   SpMV/TTV kernel: resident | stream | stream2 (default: chosen by size)
  *   COMET_STREAM_SPAN=n         entries per span of the SpMV/TTV stream kernels (multiple of 128)
  *   COMET_PACK_CSR=1|0          forces / forbids the histogram CSR packing of comet_pack_ex (COMET_PACK_CSR_HISTOGRAM)
+ *   COMET_PACK_SMALL=0          comet_pack of small inputs without the one cooperative launch (as where the driver refuses it)
  *   COMET_SEG_PARTITION=0       matrix-operand kernels search their tile boundaries themselves (no pre-pass)
  *   COMET_CSF_FORM=fold|expand  root-mode CSF MTTKRP: per-fiber or per-entry form (default: by mean fiber length)
  *   COMET_MTTKRP_HOT_ROWS=0|1   per-entry MTTKRP (CSF leaf mode, COO non-root modes): never / always keep the most popular output rows in shared memory

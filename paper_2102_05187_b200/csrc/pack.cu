@@ -16,7 +16,7 @@
 //                order (64-bit ones gathered through the sorted indices). Equal adjacent keys are duplicates
 //                and are reported.
 //
-// No inter-CTA waiting anywhere: every scan is reduce / scan-of-sums / apply in separate launches.
+// No inter-CTA waiting in this file (small inputs take the cooperative launch of pack_small.cu, which has grid barriers): every scan is reduce / scan-of-sums / apply in separate launches.
 #include "common.cuh"
 #include "kernels.cuh"
 #include "pack_common.cuh"
@@ -370,9 +370,6 @@ __global__ void dup_merge_kernel(const uint64_t *__restrict__ keys, const uint32
 }
 
 // ------------------------------------------------------------------------------------------------ levels
-constexpr int kLevelThreads = 256;
-constexpr int kLevelItems = 8;
-constexpr int kLevelTile = kLevelThreads * kLevelItems;
 
 // Per tile: how many nodes each counted level opens; duplicates (equal adjacent keys) are flagged.
 // Counters are indexed by level (slots of uncounted levels stay unused); ORDER is a template parameter
@@ -779,17 +776,22 @@ extern "C" comet_status_t comet_pack_ex(comet_handle_t handle, int32_t order, co
   uint32_t *pay_a = nullptr;           // fp32 values as raw bits, else entry indices
   uint32_t *table = nullptr;           // digit counts during the sort, then the scanned node counts per tile and level
   const void *sorted_val = nullptr;    // the values in sorted order, once some array holds them so
-  if (!(flags & COMET_PACK_SUM_DUPLICATES) && pack_small_applies(ctx, order, total_bits, n)) {
+  bool small = !(flags & COMET_PACK_SUM_DUPLICATES) && pack_small_applies(ctx, order, total_bits, n);
+  if (small) {
     char *block = (char *)tmp.get(pack_small_bytes(order, n));
     if (!block) return COMET_ERR_ALLOC;
     PackSmallSorted sorted;
     const comet_status_t st = pack_small_sort(ctx, order, coords, key, plan,
                                               dtype == COMET_F32 ? static_cast<const uint32_t *>(coo_val) : nullptr, n, block,
                                               &sorted, s);
-    if (st != COMET_OK) return st;
-    keys_a = sorted.keys; pay_a = sorted.pay; table = sorted.counts;
-    if (dtype == COMET_F32) sorted_val = pay_a;
-  } else {
+    small = st != COMET_ERR_UNSUPPORTED_FORMAT;
+    if (small) {
+      if (st != COMET_OK) return st;
+      keys_a = sorted.keys; pay_a = sorted.pay; table = sorted.counts;
+      if (dtype == COMET_F32) sorted_val = pay_a;
+    }
+  }
+  if (!small) {
     keys_a = (uint64_t *)tmp.get((size_t)(n + 1) * 8);
     uint64_t *keys_b = (uint64_t *)tmp.get((size_t)(n + 1) * 8);
     pay_a = (uint32_t *)tmp.get((size_t)(n + 1) * 4);

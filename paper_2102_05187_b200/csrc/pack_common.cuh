@@ -71,6 +71,12 @@ __device__ __forceinline__ bool is_head(uint64_t k, uint64_t kprev, bool first, 
   return first || (k >> shift) != (kprev >> shift);
 }
 
+// Entries per tile of the level counts: level_count_kernel and level_emit_kernel (pack.cu) and the one launch of
+// pack_small.cu count and place nodes in the same tiles.
+constexpr int kLevelThreads = 256;
+constexpr int kLevelItems = 8;
+constexpr int kLevelTile = kLevelThreads * kLevelItems;
+
 struct LevelOut {
   int32_t *pos[COMET_MAX_ORDER];
   int32_t *crd[COMET_MAX_ORDER];
@@ -81,7 +87,9 @@ struct LevelOut {
 
 // Small inputs (pack_small.cu): keys, sort and level counts in one cooperative launch. `tmp` holds pack_small_bytes();
 // the call waits for the stream, after which the handle's pinned words hold what pack.cu reads from them (0 range error, 1
-// duplicate, 8 + l nodes of level l) and `out` the sorted entries and the scanned counts per 2,048-entry tile.
+// duplicate, 8 + l nodes of level l) and `out` the sorted entries and the scanned counts per tile of kLevelTile entries.
+// COMET_ERR_UNSUPPORTED_FORMAT: the driver refused the launch, as it does where the context has fewer SMs than the device
+// (nothing was written; COMET_PACK_SMALL=0 stands for such a refusal): take the general path.
 struct PackSmallSorted {
   uint64_t *keys;
   uint32_t *pay;

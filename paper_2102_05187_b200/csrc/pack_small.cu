@@ -14,6 +14,8 @@
 // The barriers are cooperative groups' (the launch guarantees that all CTAs are resident); nothing else waits.
 #include <cooperative_groups.h>
 
+#include <stdlib.h>
+
 #include "common.cuh"
 #include "kernels.cuh"
 #include "pack_common.cuh"
@@ -145,23 +147,25 @@ __global__ void __launch_bounds__(kSmallThreads, 1) pack_small_kernel(const Smal
     grid.sync();
   }
 
-  // node counts per 2,048 entries (the tiles of pack.cu's emit kernel), duplicates
+  // node counts per tile of pack.cu's emit kernel, duplicates
   const uint64_t *keys = a.keys[cur];
   bool dup = false;
   for (uint32_t lv = blockIdx.x; lv < a.level_tiles; lv += gridDim.x) {
     uint32_t mine[ORDER];
 #pragma unroll
     for (int l = 0; l < ORDER; ++l) mine[l] = 0;
-    uint64_t k[4], kp[4];
+    constexpr int kRounds = kLevelTile / kSmallThreads;
+    static_assert(kRounds * kSmallThreads == kLevelTile, "whole rounds of the CTA per level tile");
+    uint64_t k[kRounds], kp[kRounds];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const uint32_t p = lv * 2048 + u * kSmallThreads + tid, q = p < a.n ? p : a.n - 1;
+    for (int u = 0; u < kRounds; ++u) {
+      const uint32_t p = lv * kLevelTile + u * kSmallThreads + tid, q = p < a.n ? p : a.n - 1;
       k[u] = __ldcg(keys + q);
       kp[u] = __ldcg(keys + (q > 0 ? q - 1 : 0));
     }
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const uint32_t p = lv * 2048 + u * kSmallThreads + tid;
+    for (int u = 0; u < kRounds; ++u) {
+      const uint32_t p = lv * kLevelTile + u * kSmallThreads + tid;
       if (p < a.n) {
         dup |= (p > 0) & (k[u] == kp[u]);
 #pragma unroll
@@ -218,7 +222,7 @@ bool pack_small_applies(Context *ctx, int order, int total_bits, int64_t n) {
 // keys_a/b and pay_a/b, the digit table and the level counts
 size_t pack_small_bytes(int order, int64_t n) {
   return 2 * align_up((size_t)n * 8, 256) + 2 * align_up((size_t)n * 4, 256) + (size_t)kSmCount * 256 * 4 +
-         align_up((size_t)order * ceil_div(n, 2048) * 4, 256);
+         align_up((size_t)order * ceil_div(n, kLevelTile) * 4, 256);
 }
 
 template <int ORDER>
@@ -240,7 +244,7 @@ static cudaError_t run_small(const CoordPtrs &c, const KeyLayout &k, const Level
   for (int x = 0; x < 2; ++x) a.pay[x] = (uint32_t *)take((size_t)n * 4);
   a.table = (uint32_t *)take((size_t)kSmCount * 256 * 4);
   a.counts = (uint32_t *)tmp;
-  a.level_tiles = (uint32_t)ceil_div(n, 2048);
+  a.level_tiles = (uint32_t)ceil_div(n, kLevelTile);
   const int at = ((k.total_bits + 7) / 8) & 1;     // the buffer that the last digit's scatter writes
   out->keys = a.keys[at];
   out->pay = a.pay[at];
@@ -251,10 +255,16 @@ static cudaError_t run_small(const CoordPtrs &c, const KeyLayout &k, const Level
 
 comet_status_t pack_small_sort(Context *ctx, int order, const CoordPtrs &c, const KeyLayout &k, const LevelPlan &plan,
                                const uint32_t *val32, int64_t n, char *tmp, PackSmallSorted *out, cudaStream_t s) {
+  const char *allowed = getenv("COMET_PACK_SMALL");
   cudaError_t e;
-  if (order == 2) e = run_small<2>(c, k, plan, val32, n, tmp, ctx->h_pinned, out, s);
+  if (allowed && allowed[0] == '0') e = cudaErrorCooperativeLaunchTooLarge;
+  else if (order == 2) e = run_small<2>(c, k, plan, val32, n, tmp, ctx->h_pinned, out, s);
   else if (order == 3) e = run_small<3>(c, k, plan, val32, n, tmp, ctx->h_pinned, out, s);
   else e = run_small<4>(c, k, plan, val32, n, tmp, ctx->h_pinned, out, s);
+  if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported) {
+    cudaGetLastError();
+    return COMET_ERR_UNSUPPORTED_FORMAT;
+  }
   if (e != cudaSuccess) return cuda_fail(ctx, e);
   ctx->launches += 1;
   COMET_CUDA_TRY(ctx, cudaStreamSynchronize(s));

@@ -68,3 +68,23 @@ def test_errors_are_reported_and_leave_the_handle_usable(n, attr):
             comet.pack([c.cuda() for c in bad], val.cuda(), dims, (0, 1, 2), attr)
         assert e.value.status == status
     _check([c.numpy() for c in coords], val.numpy(), dims, (0, 1, 2), attr)
+
+
+@pytest.mark.parametrize("n", [1, 2047, 2049, 100_003])
+@pytest.mark.parametrize("order", [2, 3, 4])
+def test_general_path_where_the_launch_is_refused(n, order, monkeypatch):
+    """A context with fewer SMs than the device refuses the cooperative launch: the general path packs the same."""
+    dims = {2: (3001, 4099), 3: (257, 300, 191), 4: (67, 61, 59, 64)}[order]
+    coords, val = synth.random_coo(dims, n, n + order)
+    coords, val = [c.numpy() for c in coords], val.numpy()
+    handle = comet.default_handle()
+
+    def launches():
+        before = handle.kernel_launches()
+        for attr in FORMATS[order]:
+            _check(coords, val, dims, tuple(range(order)), attr)
+        return handle.kernel_launches() - before
+
+    one = launches()
+    monkeypatch.setenv("COMET_PACK_SMALL", "0")
+    assert launches() > one, "the one launch was taken all the same"

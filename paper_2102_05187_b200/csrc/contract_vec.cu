@@ -489,7 +489,7 @@ comet_status_t zero_rows(Context *ctx, void *C, int dtype, int64_t rows, int64_t
   return COMET_OK;
 }
 
-int32_t choose_tile_items(int64_t total_items, int workers_per_block, bool uneven, int32_t least) {
+int32_t choose_tile_items(int64_t total_items, int workers_per_block, bool uneven, int32_t least, int32_t most) {
   if (const char *e = getenv("COMET_TILE_ITEMS")) {
     int v = atoi(e);
     if (v >= 8 && v <= (1 << 20)) return v;
@@ -501,15 +501,19 @@ int32_t choose_tile_items(int64_t total_items, int workers_per_block, bool uneve
   // 8.2 M, R = 49 306 / 298 / 307 / 320 us; DCSR, 94 % of the rows empty, R = 8 1037 / 960 / 928 / 919 us.
   const int64_t slots = (int64_t)kSmCount * 4 * workers_per_block;
   int64_t t = ceil_div(total_items, slots * (uneven ? 8 : 4));
-  // That many tiles only where they are not too short: as long as half a CTA's worth of tiles per SM allows, up to 160 items
-  // (32 where the work is uneven), and not below `least` items. Measured with a limit of 32 / 96 / 160 / 256 items: SpMM, 2 M
+  // That many tiles only where they are not too short: as long as half a CTA's worth of tiles per SM allows, up to `most` items
+  // and not below `least`. `most` is 160, but 32 where the work is uneven and where a worker has one or two lanes: a CTA then has
+  // 128 or 256 of them, and long tiles leave few CTAs. Measured with a limit of 32 / 96 / 160 / 256 items: SpMM, 2 M
   // entries, R = 16 53.5 / 51.2 / 43.5 / 48.1 us; MTTKRP, CSF, 2 M, R = 16 94 / 89 / 78 / 86 us; COO 76 / 64 / 54 / 52 us. With
   // `least` 32 / 16 / 8 / 4: 20,000 entries, fp64, R = 4 31.7 / 17.3 / 15.5 / 15.8 us; the head of a CSF tile costs more (60,000
   // entries: 28 us with 32, 31 with 8).
-  const int64_t most = uneven ? 32 : 160;
   int64_t low = ceil_div(total_items, (int64_t)kSmCount * 2 * workers_per_block);
   low = low < least ? least : low < most ? low : most;
   if (t < low) t = low;
+  if (!uneven && most == 32 && t == most) {                // many workers to a CTA: whole waves, or the last one is nearly empty
+    const int64_t waves = total_items / (slots * t);
+    if (waves >= 1) t = ceil_div(total_items, slots * waves);
+  }
   if (t > 512) t = 512;
   return (int32_t)t;
 }
@@ -619,7 +623,7 @@ template <class T, int LPN, int CPL, int VEC, bool RAGGED = false>
 static comet_status_t launch_one(Context *ctx, SegGatherArgs a, HeavyArgs *heavy, bool cleared, int64_t pad, cudaStream_t stream) {
   constexpr int WORKERS = kBlockThreads / LPN;
   const int64_t total = a.M + a.N;
-  a.tile_items = choose_tile_items(total, WORKERS, a.out_row != nullptr, 8);
+  a.tile_items = choose_tile_items(total, WORKERS, a.out_row != nullptr, 8, a.out_row || (!RAGGED && LPN <= 2) ? 32 : 160);
   a.num_tiles = ceil_div(total, a.tile_items);
   a.own_len = a.tile_items / 4;
   a.carry_ld = (int32_t)align_up((size_t)a.R, 2);

@@ -440,7 +440,7 @@ static comet_status_t launch_mttkrp(Context *ctx, MttkrpArgs a, int64_t p_pad, i
   constexpr int WORKERS = kBlockThreads / LPN;
   const int64_t total = CSF ? a.F + a.N : a.N;
   using L = Lanes<T, LPN, CPL, VEC, RAGGED>;
-  a.tile_items = choose_tile_items(total, WORKERS, false, CSF ? 32 : 8);
+  a.tile_items = choose_tile_items(total, WORKERS, false, CSF ? 32 : 8, LPN <= 2 ? 32 : 160);
   if (CSF && a.tile_items > kCsfTileCap) a.tile_items = kCsfTileCap;          // one mask bit per leaf entry of a tile
   a.num_tiles = ceil_div(total, a.tile_items);
   a.carry_ld = (int32_t)align_up((size_t)a.R, 2);

@@ -78,6 +78,7 @@ typedef enum {
  *   COMET_STREAM_SPAN=n         entries per span of the SpMV/TTV stream kernels (multiple of 128)
  *   COMET_PACK_CSR=1|0          forces / forbids the histogram CSR packing of comet_pack_ex (COMET_PACK_CSR_HISTOGRAM)
  *   COMET_PACK_SMALL=0          comet_pack of small inputs without the one cooperative launch (as where the driver refuses it)
+ *   COMET_PACK_SPLIT=0|1        comet_pack of larger inputs: never / always split by sampled keys (default: from 600,000 entries on)
  *   COMET_SEG_PARTITION=0       matrix-operand kernels search their tile boundaries themselves (no pre-pass)
  *   COMET_CSF_FORM=fold|expand  root-mode CSF MTTKRP: per-fiber or per-entry form (default: by mean fiber length)
  *   COMET_MTTKRP_HOT_ROWS=0|1   per-entry MTTKRP (CSF leaf mode, COO non-root modes): never / always keep the most popular output rows in shared memory
@@ -137,7 +138,10 @@ int64_t comet_kernel_launches(comet_handle_t handle);
  * coordinate bit widths (ceil(log2(extent)) per mode) sum to <= 63. Input order is arbitrary; duplicates and out-of-range
  * coordinates are detected on the device and reported (COMET_ERR_DUPLICATE_COORD,
  * COMET_ERR_COORD_OUT_OF_RANGE); `out` is then left zeroed. On success `out` owns its arrays
- * (allocated through the handle's allocator) until comet_sptensor_free. Synchronises `stream` once.  *
+ * (allocated through the handle's allocator) until comet_sptensor_free. Synchronises `stream` once (twice for an input that
+ * takes the general path after the one for larger inputs could not hold it). From 600,000 entries on a call takes about 80 bytes
+ * of temporary memory per entry from the allocator, or, where it has no room for them, 24.
+ *
  * ELLPACK (named in the Tensor Storage Format section among the formats the four attributes compose; the paper
  * does not spell the composition out, this is the reading used): order 2 with h_attr = {COMET_D, COMET_S} gives a
  * descriptor of THREE levels [D, D, S]: the rows (dense), K slots per row (dense; listed as a third "mode" of

@@ -2,6 +2,10 @@
 // runtime function performs; Tensor Storage Format section for what each attribute stores), and
 // comet_validate for caller-built descriptors.
 //
+// Three paths: small inputs take the cooperative launch of pack_small.cu, larger ones of distinct keys the sampled splits of
+// pack_split.cu; what is described here is the general one (summed duplicates, more than 114 M entries, no room for the
+// splits' records) and the level passes that all share.
+//
 //   1. keys      one 64-bit key per entry: the coordinates in storage-level order, level 0 in the most
 //                significant bits (so key order = lexicographic order); coordinates are range-checked.
 //   2. sort      stable LSD radix sort of (key, 32-bit payload), 8 bits per pass, only over the bits in use; the
@@ -34,8 +38,6 @@ constexpr int kSortWarps = kSortThreads / 32;
 constexpr int kScanThreads = 256;
 constexpr int kScanItems = 8;
 constexpr int kScanTile = kScanThreads * kScanItems;
-
-enum { kStatusRange = 0, kStatusDuplicate = 1, kStatusInvalid = 2 };   // words of Context::d_status
 
 // ------------------------------------------------------------------------------------------------ keys
 // Where a sort pass reads its (key, payload) pairs. The payload is one 32-bit word that travels with the key
@@ -643,6 +645,10 @@ struct TempBlocks {
     if (q) p[n++] = q;
     return q;
   }
+  void adopt(TempBlocks &other) {    // at most one block
+    for (int i = 0; i < other.n; ++i) p[n++] = other.p[i];
+    other.n = 0;
+  }
   ~TempBlocks() { for (int i = 0; i < n; ++i) ctx_free(ctx, p[i], s); }
 };
 
@@ -771,6 +777,48 @@ extern "C" comet_status_t comet_pack_ex(comet_handle_t handle, int32_t order, co
   const int64_t table_len = radix_sort_table_words(n);
   const int64_t counts_len = (int64_t)COMET_MAX_ORDER * level_tiles;
 
+  // exact allocation of the result for n entries, `counts`: nodes of the counted levels
+  const size_t val_size = dtype == COMET_F32 ? 4 : 8;
+  void *owner = nullptr;
+  LevelOut lo{};
+  auto allocate = [&](const uint32_t *counts) -> comet_status_t {
+    owner = owner_new();
+    if (!owner) return COMET_ERR_ALLOC;
+    bool alloc_ok = true;
+    out->order = order;
+    out->dtype = dtype;
+    out->nnz = n;
+    int64_t parents = 1;
+    for (int l = 0; l < order; ++l) {
+      out->dims[l] = h_dims[l];
+      out->mode_order[l] = h_mode_order[l];
+      out->attr[l] = h_attr[l];
+      const int64_t nodes = plan.counted[l] >= 0 ? (int64_t)counts[l] : n;
+      if (plan.counted[l] >= 0) lo.nodes[l] = (uint32_t)nodes;
+      int64_t pos_len = 0, crd_len = 0;
+      if (h_attr[l] == COMET_D) { pos_len = 1; parents = key.dim[l]; }
+      else if (h_attr[l] == COMET_CU) { pos_len = parents + 1; crd_len = nodes; parents = nodes; }
+      else if (h_attr[l] == COMET_CN) { pos_len = 2; crd_len = n; parents = n; }
+      else { crd_len = n; }
+      out->pos_len[l] = pos_len;
+      out->crd_len[l] = crd_len;
+      if (pos_len) { out->pos[l] = (int32_t *)owner_alloc(ctx, owner, (size_t)pos_len * 4, s); alloc_ok &= out->pos[l] != nullptr; }
+      if (crd_len) { out->crd[l] = (int32_t *)owner_alloc(ctx, owner, (size_t)crd_len * 4, s); alloc_ok &= out->crd[l] != nullptr; }
+      lo.pos[l] = out->pos[l];
+      lo.crd[l] = out->crd[l];
+    }
+    if (n > 0) { out->val = owner_alloc(ctx, owner, (size_t)n * val_size, s); alloc_ok &= out->val != nullptr; }
+    lo.val = out->val;
+    lo.dim0 = key.dim[0];
+    return alloc_ok ? COMET_OK : COMET_ERR_ALLOC;
+  };
+  auto drop = [&](comet_status_t st) {           // what was allocated goes back
+    if (owner) owner_release(ctx, owner, s);
+    owner = nullptr;
+    memset(out, 0, sizeof(*out));
+    return st;
+  };
+
   TempBlocks tmp(ctx, s);
   uint64_t *keys_a = nullptr;
   uint32_t *pay_a = nullptr;           // fp32 values as raw bits, else entry indices
@@ -791,7 +839,66 @@ extern "C" comet_status_t comet_pack_ex(comet_handle_t handle, int32_t order, co
       if (dtype == COMET_F32) sorted_val = pay_a;
     }
   }
-  if (!small) {
+  // node counts of the counted levels: per-tile counts -> scanned offsets (kept in `table`) + totals beside the status words
+  uint32_t *d_nodes = reinterpret_cast<uint32_t *>(ctx->d_status) + 8;
+  auto count_nodes = [&](uint32_t *scan_tmp) -> comet_status_t {
+    if (order == 2) level_count_kernel<2><<<(unsigned)level_tiles, kLevelThreads, 0, s>>>(keys_a, n, plan, level_tiles, table, ctx->d_status);
+    else if (order == 3) level_count_kernel<3><<<(unsigned)level_tiles, kLevelThreads, 0, s>>>(keys_a, n, plan, level_tiles, table, ctx->d_status);
+    else level_count_kernel<4><<<(unsigned)level_tiles, kLevelThreads, 0, s>>>(keys_a, n, plan, level_tiles, table, ctx->d_status);
+    COMET_LAUNCH_CHECK(ctx);
+    for (int l = 0; l < order; ++l) {
+      if (plan.counted[l] < 0) continue;
+      comet_status_t st = exclusive_scan(ctx, table + (int64_t)l * level_tiles, table + (int64_t)l * level_tiles,
+                                         level_tiles, scan_tmp, d_nodes + l, s);
+      if (st != COMET_OK) return st;
+    }
+    return COMET_OK;
+  };
+  auto read_status = [&]() -> comet_status_t {   // the one synchronisation: status words and node counts
+    COMET_CUDA_TRY(ctx, cudaMemcpyAsync(ctx->h_pinned, ctx->d_status, 16 * sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+    COMET_CUDA_TRY(ctx, cudaStreamSynchronize(s));
+    return COMET_OK;
+  };
+  // Larger inputs of distinct keys: split by samples and sorted in shared memory, in the tensor's arrays at once where no
+  // level needs a count. Where there is no room for its records, or a region was too small, the radix sort packs them.
+  bool split = !small && !(flags & COMET_PACK_SUM_DUPLICATES) && pack_split_applies(order, total_bits, n);
+  if (split) {
+    TempBlocks block(ctx, s);
+    const bool direct = plan.ncounted == 0 && (h_attr[0] == COMET_CN || order == 2);
+    char *records = (char *)block.get(pack_split_bytes(n));
+    uint32_t *scan_tmp = nullptr;
+    if (records && !direct) {
+      table = (uint32_t *)tmp.get((size_t)counts_len * 4);
+      scan_tmp = (uint32_t *)tmp.get((size_t)scan_tmp_words(counts_len) * 4);
+    }
+    split = records && (direct || (table && scan_tmp));
+    if (split) {
+      comet_status_t st = direct ? allocate(nullptr) : COMET_OK;
+      if (st != COMET_OK) return drop(st);
+      st = [&]() -> comet_status_t {
+        COMET_CUDA_TRY(ctx, cudaMemsetAsync(ctx->d_status, 0, 16 * sizeof(int32_t), s));
+        PackSplitSorted sorted{};
+        comet_status_t q = pack_split_sort(ctx, order, coords, key, plan, coo_val, dtype, n, records, direct ? &lo : nullptr, &sorted, s);
+        if (q != COMET_OK) return q;
+        if (!direct) {
+          keys_a = sorted.keys;
+          sorted_val = sorted.val;
+          q = count_nodes(scan_tmp);
+          if (q != COMET_OK) return q;
+        }
+        return read_status();
+      }();
+      if (st != COMET_OK) return drop(st);
+      if (ctx->h_pinned[kStatusRange]) return drop(COMET_ERR_COORD_OUT_OF_RANGE);
+      split = !ctx->h_pinned[kStatusOverflow];
+      if (!split) drop(COMET_OK);
+      else if (ctx->h_pinned[kStatusDuplicate]) return drop(COMET_ERR_DUPLICATE_COORD);
+      else if (direct) { out->owner = owner; return COMET_OK; }
+      else tmp.adopt(block);
+    }
+  }
+  if (!small && !split) {
+    sorted_val = nullptr;
     keys_a = (uint64_t *)tmp.get((size_t)(n + 1) * 8);
     uint64_t *keys_b = (uint64_t *)tmp.get((size_t)(n + 1) * 8);
     pay_a = (uint32_t *)tmp.get((size_t)(n + 1) * 4);
@@ -802,7 +909,6 @@ extern "C" comet_status_t comet_pack_ex(comet_handle_t handle, int32_t order, co
     if (!keys_a || !keys_b || !pay_a || !pay_b || !table || !scan_tmp) return COMET_ERR_ALLOC;
 
     COMET_CUDA_TRY(ctx, cudaMemsetAsync(ctx->d_status, 0, 16 * sizeof(int32_t), s));
-    uint32_t *d_nodes = reinterpret_cast<uint32_t *>(ctx->d_status) + 8;   // node counts live beside the status words
 
     if (n > 0) {
       {
@@ -842,57 +948,19 @@ extern "C" comet_status_t comet_pack_ex(comet_handle_t handle, int32_t order, co
         n = distinct;
         level_tiles = ceil_div(n > 0 ? n : 1, kLevelTile);
       }
-      // node counts of the counted levels: per-tile counts -> scanned offsets (kept in `table`) + totals
-      if (order == 2) level_count_kernel<2><<<(unsigned)level_tiles, kLevelThreads, 0, s>>>(keys_a, n, plan, level_tiles, table, ctx->d_status);
-      else if (order == 3) level_count_kernel<3><<<(unsigned)level_tiles, kLevelThreads, 0, s>>>(keys_a, n, plan, level_tiles, table, ctx->d_status);
-      else level_count_kernel<4><<<(unsigned)level_tiles, kLevelThreads, 0, s>>>(keys_a, n, plan, level_tiles, table, ctx->d_status);
-      COMET_LAUNCH_CHECK(ctx);
-      for (int l = 0; l < order; ++l) {
-        if (plan.counted[l] < 0) continue;
-        comet_status_t st = exclusive_scan(ctx, table + (int64_t)l * level_tiles, table + (int64_t)l * level_tiles,
-                                           level_tiles, scan_tmp, d_nodes + l, s);
-        if (st != COMET_OK) return st;
-      }
+      const comet_status_t st = count_nodes(scan_tmp);
+      if (st != COMET_OK) return st;
     }
-    // the one synchronisation: status words and node counts
-    COMET_CUDA_TRY(ctx, cudaMemcpyAsync(ctx->h_pinned, ctx->d_status, 16 * sizeof(int32_t), cudaMemcpyDeviceToHost, s));
-    COMET_CUDA_TRY(ctx, cudaStreamSynchronize(s));
+    const comet_status_t st = read_status();
+    if (st != COMET_OK) return st;
   }
   if (ctx->h_pinned[kStatusRange]) return COMET_ERR_COORD_OUT_OF_RANGE;
   if (ctx->h_pinned[kStatusDuplicate]) return COMET_ERR_DUPLICATE_COORD;
 
-  // exact allocation
-  void *owner = owner_new();
-  if (!owner) return COMET_ERR_ALLOC;
-  LevelOut lo{};
-  bool alloc_ok = true;
-  out->order = order;
-  out->dtype = dtype;
-  out->nnz = n;
-  int64_t parents = 1;
-  for (int l = 0; l < order; ++l) {
-    out->dims[l] = h_dims[l];
-    out->mode_order[l] = h_mode_order[l];
-    out->attr[l] = h_attr[l];
-    const int64_t nodes = plan.counted[l] >= 0 ? (int64_t)reinterpret_cast<uint32_t *>(ctx->h_pinned)[8 + l] : n;
-    if (plan.counted[l] >= 0) lo.nodes[l] = (uint32_t)nodes;
-    int64_t pos_len = 0, crd_len = 0;
-    if (h_attr[l] == COMET_D) { pos_len = 1; parents = key.dim[l]; }
-    else if (h_attr[l] == COMET_CU) { pos_len = parents + 1; crd_len = nodes; parents = nodes; }
-    else if (h_attr[l] == COMET_CN) { pos_len = 2; crd_len = n; parents = n; }
-    else { crd_len = n; }
-    out->pos_len[l] = pos_len;
-    out->crd_len[l] = crd_len;
-    if (pos_len) { out->pos[l] = (int32_t *)owner_alloc(ctx, owner, (size_t)pos_len * 4, s); alloc_ok &= out->pos[l] != nullptr; }
-    if (crd_len) { out->crd[l] = (int32_t *)owner_alloc(ctx, owner, (size_t)crd_len * 4, s); alloc_ok &= out->crd[l] != nullptr; }
-    lo.pos[l] = out->pos[l];
-    lo.crd[l] = out->crd[l];
+  {
+    const comet_status_t st = allocate(reinterpret_cast<uint32_t *>(ctx->h_pinned) + 8);
+    if (st != COMET_OK) return drop(st);
   }
-  const size_t val_size = dtype == COMET_F32 ? 4 : 8;
-  if (n > 0) { out->val = owner_alloc(ctx, owner, (size_t)n * val_size, s); alloc_ok &= out->val != nullptr; }
-  lo.val = out->val;
-  lo.dim0 = key.dim[0];
-  if (!alloc_ok) { owner_release(ctx, owner, s); memset(out, 0, sizeof(*out)); return COMET_ERR_ALLOC; }
 
   // An empty tensor has no tiles: only the closing role runs. A dense root may have a long empty tail to write.
   const int64_t emit_tiles = n > 0 ? level_tiles : 0;
@@ -917,7 +985,7 @@ extern "C" comet_status_t comet_pack_ex(comet_handle_t handle, int32_t order, co
   }
   ctx->launches += 1;
   cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) { owner_release(ctx, owner, s); memset(out, 0, sizeof(*out)); return cuda_fail(ctx, e); }
+  if (e != cudaSuccess) return drop(cuda_fail(ctx, e));
   out->owner = owner;
   return COMET_OK;
 }

@@ -5,6 +5,8 @@
 
 namespace comet {
 
+enum { kStatusRange = 0, kStatusDuplicate = 1, kStatusInvalid = 2, kStatusOverflow = 3 };   // words of Context::d_status
+
 struct KeyLayout {
   int order;
   int shift[COMET_MAX_ORDER];      // bit position of level l's coordinate inside the key
@@ -99,5 +101,18 @@ bool pack_small_applies(Context *ctx, int order, int total_bits, int64_t n);
 size_t pack_small_bytes(int order, int64_t n);
 comet_status_t pack_small_sort(Context *ctx, int order, const CoordPtrs &c, const KeyLayout &k, const LevelPlan &plan,
                                const uint32_t *val32, int64_t n, char *tmp, PackSmallSorted *out, cudaStream_t s);
+
+// Larger inputs of distinct keys (pack_split.cu): split by sampled keys, sorted in shared memory. `tmp` holds
+// pack_split_bytes(); nothing waits. direct null: `sorted` receives the sorted keys and values (inside `tmp`); otherwise the
+// tensor's arrays, which are written (CSR [D,CU] and sorted coordinates [CN,S..]: no level needs a count). The status words
+// tell afterwards: with kStatusOverflow the input did not fit this path and what was written is void.
+struct PackSplitSorted {
+  uint64_t *keys;
+  void *val;
+};
+bool pack_split_applies(int order, int total_bits, int64_t n);
+size_t pack_split_bytes(int64_t n);
+comet_status_t pack_split_sort(Context *ctx, int order, const CoordPtrs &c, const KeyLayout &k, const LevelPlan &plan, const void *val,
+                               int dtype, int64_t n, char *tmp, const LevelOut *direct, PackSplitSorted *sorted, cudaStream_t s);
 
 }  // namespace comet

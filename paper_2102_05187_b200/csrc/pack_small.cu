@@ -8,8 +8,8 @@
 // so that its emit kernel can follow. The node counts and the error flags go straight to the handle's pinned host words.
 // What bounds it is the latency of the steps (about 9 us per digit: two grid barriers, two rounds through L2, the ranking).
 // Measured against the general path, whole comet_pack calls: 500 entries, order 3 162 -> 52 us; 60,000 entries of order 3
-// (four digits) packed and contracted once 325 -> 112 us; 0.42 M entries, five digits 323 -> 135 us. The limit of 16
-// entries per thread is what a thread can hold in registers.
+// (four digits) packed and contracted once 325 -> 112 us; 0.42 M entries, five digits 323 -> 135 us. Beyond 8 entries per
+// thread pack_split.cu is faster (620,000 entries 142 us here with 16, 106 there).
 //
 // The barriers are cooperative groups' (the launch guarantees that all CTAs are resident); nothing else waits.
 #include <cooperative_groups.h>
@@ -26,8 +26,8 @@ namespace cg = cooperative_groups;
 
 constexpr int kSmallThreads = 512;
 constexpr int kSmallWarps = kSmallThreads / 32;
-constexpr int kSmallMaxItems = 16;
-constexpr int64_t kSmallMax = (int64_t)kSmCount * kSmallThreads * kSmallMaxItems;     // 1.2 M entries
+constexpr int kSmallMaxItems = 8;
+constexpr int64_t kSmallMax = (int64_t)kSmCount * kSmallThreads * kSmallMaxItems;     // 0.6 M entries
 
 template <int ORDER> struct SmallArgs {
   CoordPtrs c;
@@ -204,7 +204,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1) pack_small_kernel(const Smal
 
 static int small_items(int64_t n) {
   const int64_t per = ceil_div(n, (int64_t)kSmCount * kSmallThreads);
-  return per <= 2 ? 2 : per <= 4 ? 4 : per <= 8 ? 8 : 16;
+  return per <= 2 ? 2 : per <= 4 ? 4 : 8;
 }
 
 bool pack_small_applies(Context *ctx, int order, int total_bits, int64_t n) {
@@ -230,7 +230,7 @@ static cudaError_t launch_small(SmallArgs<ORDER> a, int items, cudaStream_t s) {
   a.tiles = (uint32_t)ceil_div((int64_t)a.n, (int64_t)kSmallThreads * items);
   void *args[] = {&a};
   const void *kernel = items == 2 ? (const void *)pack_small_kernel<ORDER, 2> : items == 4 ? (const void *)pack_small_kernel<ORDER, 4>
-                     : items == 8 ? (const void *)pack_small_kernel<ORDER, 8> : (const void *)pack_small_kernel<ORDER, 16>;
+                                         : (const void *)pack_small_kernel<ORDER, 8>;
   return cudaLaunchCooperativeKernel(kernel, dim3(a.tiles), dim3(kSmallThreads), args, 0, s);
 }
 

@@ -489,33 +489,43 @@ comet_status_t zero_rows(Context *ctx, void *C, int dtype, int64_t rows, int64_t
   return COMET_OK;
 }
 
-int32_t choose_tile_items(int64_t total_items, int workers_per_block, bool uneven, int32_t least, int32_t most) {
+static int32_t forced_tile_items() {
   if (const char *e = getenv("COMET_TILE_ITEMS")) {
     int v = atoi(e);
     if (v >= 8 && v <= (1 << 20)) return v;
   }
-  // Four tiles per resident worker (148 SMs x 4 CTAs), eight where their work is uneven (rows of zeros to write),
-  // capped so that the last tiles do not leave the chip idle; rounded
-  // up, so that the last wave is not nearly empty. Every tile boundary costs a carry and two searches. Measured with
-  // 2 / 4 / 6 / 8 tiles: 3.2 M entries, R = 50, fp32 147 / 153 / 160 / 165 us; 30 M, R = 16 404 / 381 / 386 / 394 us;
-  // 8.2 M, R = 49 306 / 298 / 307 / 320 us; DCSR, 94 % of the rows empty, R = 8 1037 / 960 / 928 / 919 us.
+  return 0;
+}
+
+// Items per tile where tiles cost the same: one tile per resident worker (148 SMs x ctas_per_sm CTAs), so that the launch is one
+// full wave, or the fewest full waves of tiles of at most `most` items. Every tile costs a boundary, a cold start and a carry,
+// and a wave that is partly filled costs a whole one. With about 4 tiles per worker, rounded to at most 160 items on
+// mid-sized inputs, -> as here: SpMM, fp64, 3.1 M entries, R = 32 99.7 -> 79.0 us, 5.6 M, R = 10 116.7 -> 106.6, 5 M, R = 64 350
+// -> 322; TTM, R = 16, 3 M 74.3 -> 57.7, R = 32, 10 M 224 -> 196; MTTKRP, CSF, 3 M, R = 16 124 -> 107.5, COO, 20 M, R = 32 629 -> 592;
+// two waves 88 / 114 / 335, 60.6 / 205, 114. (`most`: 512 entries of MTTKRP are added in a row, 1,024 of SpMM and TTM.)
+// Small inputs take up to twice the items of a full wave, while that is at most `brief`: half a wave of 48 items is faster than a
+// full one of 24 (200,000 entries, R = 32 18.9 and 20.3 us; 0.4 M, fp32 26.2 and 29.2), of 96 no longer (0.8 M 46.8, 41.0).
+int32_t choose_tile_items(int64_t total_items, int workers_per_block, int ctas_per_sm, int32_t least, int32_t brief, int32_t most) {
+  if (const int32_t forced = forced_tile_items()) return forced;
+  const int64_t workers = (int64_t)kSmCount * ctas_per_sm * workers_per_block;
+  const int64_t waves = ceil_div(total_items, workers * most);
+  int64_t t = ceil_div(total_items, workers * waves);
+  if (t < brief) t = 2 * t < brief ? 2 * t : brief;
+  return (int32_t)(t < least ? least : t);
+}
+
+// The same where tiles are uneven: beside the long rows of an SpMM, whose entries the tiles leave out, and where rows are
+// mapped (a DCSR matrix: rows of zeros in front of the stored ones, stores far apart). Four tiles per resident worker, or eight, so that the last ones do not leave the
+// chip idle. DCSR, 94 % of the rows empty, R = 8, 2 / 4 / 6 / 8 tiles 1037 / 960 / 928 / 919 us; 5.6 M entries in power-law rows,
+// R = 32, one / two / four / eight 478 / 456 / 454 / 422 us; 4.2 M rows in a cleared C, R = 8, one wave 788, eight tiles 762.
+static int32_t choose_uneven_tile_items(int64_t total_items, int workers_per_block, int per_worker) {
+  if (const int32_t forced = forced_tile_items()) return forced;
   const int64_t slots = (int64_t)kSmCount * 4 * workers_per_block;
-  int64_t t = ceil_div(total_items, slots * (uneven ? 8 : 4));
-  // That many tiles only where they are not too short: as long as half a CTA's worth of tiles per SM allows, up to `most` items
-  // and not below `least`. `most` is 160, but 32 where the work is uneven and where a worker has one or two lanes: a CTA then has
-  // 128 or 256 of them, and long tiles leave few CTAs. Measured with a limit of 32 / 96 / 160 / 256 items: SpMM, 2 M
-  // entries, R = 16 53.5 / 51.2 / 43.5 / 48.1 us; MTTKRP, CSF, 2 M, R = 16 94 / 89 / 78 / 86 us; COO 76 / 64 / 54 / 52 us. With
-  // `least` 32 / 16 / 8 / 4: 20,000 entries, fp64, R = 4 31.7 / 17.3 / 15.5 / 15.8 us; the head of a CSF tile costs more (60,000
-  // entries: 28 us with 32, 31 with 8).
+  int64_t t = ceil_div(total_items, slots * per_worker);
   int64_t low = ceil_div(total_items, (int64_t)kSmCount * 2 * workers_per_block);
-  low = low < least ? least : low < most ? low : most;
+  low = low < 8 ? 8 : low < 32 ? low : 32;
   if (t < low) t = low;
-  if (!uneven && most == 32 && t == most) {                // many workers to a CTA: whole waves, or the last one is nearly empty
-    const int64_t waves = total_items / (slots * t);
-    if (waves >= 1) t = ceil_div(total_items, slots * waves);
-  }
-  if (t > 512) t = 512;
-  return (int32_t)t;
+  return (int32_t)(t < 512 ? t : 512);
 }
 
 template <class T, int LPN, int CPL, int VEC, bool RAGGED, int ROWS, bool HEAVY>
@@ -623,16 +633,20 @@ template <class T, int LPN, int CPL, int VEC, bool RAGGED = false>
 static comet_status_t launch_one(Context *ctx, SegGatherArgs a, HeavyArgs *heavy, bool cleared, int64_t pad, cudaStream_t stream) {
   constexpr int WORKERS = kBlockThreads / LPN;
   const int64_t total = a.M + a.N;
-  a.tile_items = choose_tile_items(total, WORKERS, a.out_row != nullptr, 8, a.out_row || (!RAGGED && LPN <= 2) ? 32 : 160);
-  a.num_tiles = ceil_div(total, a.tile_items);
-  a.own_len = a.tile_items / 4;
   a.carry_ld = (int32_t)align_up((size_t)a.R, 2);
-  const size_t val_bytes = align_up((size_t)a.num_tiles * a.carry_ld * sizeof(double), 256);
+  constexpr int kCtas = CPL * VEC * sizeof(T) <= 16 ? COMET_MINB_GATHER : 2;
+  a.tile_items = a.out_row ? choose_uneven_tile_items(total, WORKERS, 8)
+                           : choose_tile_items(total, WORKERS, kCtas, 8, LPN <= 2 ? 32 : 48, 1024);
   size_t heavy_bytes = 0;
   HeavyArgs h{};
-  if (!RAGGED && kHeavyShape<T, LPN, CPL, VEC> && heavy && !a.out_row)
-    heavy_bytes = spmm_heavy_plan(sizeof(T) == 4 ? COMET_F32 : COMET_F64, a.M, a.N, heavy->cols, a.B, a.ldb, a.R, a.C, a.ldc,
-                                  a.tile_items, &h);
+  if (!RAGGED && kHeavyShape<T, LPN, CPL, VEC> && heavy && !a.out_row) {
+    const int32_t tile = choose_uneven_tile_items(total, WORKERS, 4);
+    heavy_bytes = spmm_heavy_plan(sizeof(T) == 4 ? COMET_F32 : COMET_F64, a.M, a.N, heavy->cols, a.B, a.ldb, a.R, a.C, a.ldc, tile, &h);
+    if (heavy_bytes) a.tile_items = tile;
+  }
+  a.num_tiles = ceil_div(total, a.tile_items);
+  a.own_len = a.tile_items / 4;
+  const size_t val_bytes = align_up((size_t)a.num_tiles * a.carry_ld * sizeof(double), 256);
   static const bool use_part = !(getenv("COMET_SEG_PARTITION") && atoi(getenv("COMET_SEG_PARTITION")) == 0);
   constexpr int kDtype = sizeof(T) == 4 ? COMET_F32 : COMET_F64;
   const size_t pad_bytes = RAGGED && pad ? padded_bytes(kDtype, pad, a.R) : 0;

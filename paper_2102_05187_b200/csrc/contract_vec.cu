@@ -56,7 +56,8 @@ constexpr int kRowsAll = 0, kRowsFilled = 1, kRowsMapped = 2;
 template <class T, int LPN, int CPL, int VEC, bool RAGGED, int ROWS, bool PASS_THROUGH = false>
 struct SegGatherPolicy {
   using L = Lanes<T, LPN, CPL, VEC, RAGGED>;
-  static constexpr int kPF = COMET_PF_GATHER;
+  // PASS_THROUGH: the general rows beside the long ones, which come from DRAM: eight rows in flight (walk_tile_async)
+  static constexpr int kPF = PASS_THROUGH && CPL == 1 ? 2 * COMET_PF_GATHER : COMET_PF_GATHER;
   static constexpr bool kAux = false;
   // Ragged fp32 rows end in up to four scalar stores per lane, too much code for one copy per entry of the chunk: with the
   // chunk unrolled the kernel waits for instructions (30 M entries, R = 50: 519 us unrolled, 475 rolled).
@@ -92,6 +93,14 @@ struct SegGatherPolicy {
   __device__ __forceinline__ void fetch(int32_t j, Entry16 &e, int32_t &) const {
     e.v = (double)ld_stream(static_cast<const T *>(a.val) + j);
     e.a = ld_stream(a.crd + j);
+  }
+  __device__ __forceinline__ void fetch_async(int32_t j, uint32_t entry, bool there) const {
+    if (sizeof(T) == 8) copy_async8(entry, static_cast<const T *>(a.val) + j, there);
+    else copy_async4(entry, static_cast<const T *>(a.val) + j, there);
+    copy_async4(entry + 8, a.crd + j, there);
+  }
+  __device__ __forceinline__ void settle(uint32_t entry) const {       // values are read as doubles
+    if (sizeof(T) == 4) sts_f64(entry, (double)__int_as_float(lds_s32(entry)));
   }
   __device__ __forceinline__ void prefetch(int32_t c, int32_t, Slot &s) const {
     const T *row = reinterpret_cast<const T *>(bcol + (int64_t)c * (int32_t)(a.ldb * sizeof(T)));
@@ -141,7 +150,7 @@ seg_gather_kernel(const SegGatherArgs a, const HeavyArgs h) {
   const int worker = threadIdx.x / LPN;
   const int64_t tile = (int64_t)(blockIdx.x - (HEAVY ? h.heavy_ctas : 0)) * L::kWorkers + worker;
   if (tile >= a.num_tiles) return;                       // whole groups leave together
-  const uint32_t smem = smem_u32(smem_raw) + worker * RingLayout<L, false>::kWorkerBytes;
+  const uint32_t smem = smem_u32(smem_raw) + worker * (HEAVY ? AsyncRing<L>::kWorkerBytes : RingLayout<L, false>::kWorkerBytes);
   const L ln(a.R, a.wide_store);
   if (tile == 0) clear_piece_counts(a.carry_seg, a.num_tiles, ln.g, LPN);
 
@@ -194,7 +203,8 @@ seg_gather_kernel(const SegGatherArgs a, const HeavyArgs h) {
   }
 
   SegGatherPolicy<T, LPN, CPL, VEC, RAGGED, ROWS, HEAVY> p(a, ln, i0, j0);
-  walk_tile(ln, p, j0, j1, smem);
+  if constexpr (HEAVY) walk_tile_async(ln, p, j0, j1, smem);
+  else walk_tile(ln, p, j0, j1, smem);
   while (p.segment() < i1) p.flush();                    // end markers that close the tile
 
   // leaf entries of a segment that ends in a later tile: the open segment starts in front of the tile's end
@@ -532,7 +542,8 @@ template <class T, int LPN, int CPL, int VEC, bool RAGGED, int ROWS, bool HEAVY>
 static comet_status_t launch_mapped(Context *ctx, const SegGatherArgs &a, const HeavyArgs &h, int64_t blocks,
                                     cudaStream_t stream) {
   using L = Lanes<T, LPN, CPL, VEC, RAGGED>;
-  constexpr size_t smem = RingLayout<L, false>::kBlockBytes;
+  constexpr size_t ring = RingLayout<L, false>::kBlockBytes, async_ring = HEAVY ? AsyncRing<L>::kBlockBytes : 0;
+  constexpr size_t smem = ring > async_ring ? ring : async_ring;
   auto kernel = seg_gather_kernel<T, LPN, CPL, VEC, RAGGED, ROWS, HEAVY>;
   if (smem > 48 * 1024)
     COMET_CUDA_TRY(ctx, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));

@@ -51,6 +51,7 @@ __device__ __forceinline__ double lds_f64(uint32_t addr) {
   asm volatile("ld.shared.f64 %0, [%1];" : "=d"(v) : "r"(addr));
   return v;
 }
+__device__ __forceinline__ void sts_f64(uint32_t addr, double v) { asm volatile("st.shared.f64 [%0], %1;" ::"r"(addr), "d"(v) : "memory"); }
 __device__ __forceinline__ void lds_coords(uint32_t entry_addr, int32_t &a, int32_t &b) {   // words 2, 3 of an entry
   asm volatile("ld.shared.v2.b32 {%0, %1}, [%2+8];" : "=r"(a), "=r"(b) : "r"(entry_addr));
 }
@@ -409,6 +410,85 @@ __device__ __forceinline__ void walk_tile(const L &ln, Policy &p, int32_t j0, in
     if (n >= kChunk) walk_chunk<L, Policy, false>(p, win, cur, nxt, cur_aux, nxt_aux, kChunk);
     else walk_chunk<L, Policy, true>(p, win, cur, nxt, cur_aux, nxt_aux, n);
   }
+}
+
+// ---------------------------------------------------------------------------------------------- asynchronous staging
+// The same walk with the leaf entries copied into the ring by cp.async: no registers hold entries on their way, so that the
+// window of rows in flight can be twice as deep at the same occupancy. The ring has four chunks: the one being walked, the
+// one the window looks ahead into, and two on their way. Policy interface: as above with fetch_async(j, entry address,
+// there) instead of fetch, and settle(entry address), which a lane calls for the entries it copied once they have arrived.
+// For the gathers that go to DRAM (SpMM beside its long rows: 1103 -> 1040 us); where the rows come from L2 the copies
+// cost more than the deeper window gives (TTM of 30 M entries, R = 16 353 -> 385 us with four rows in flight, 413 with eight).
+constexpr int kAsyncChunk = 8, kRingChunks = 4;
+__device__ __forceinline__ void copy_async8(uint32_t dst, const void *src, bool there) {      // zeros where nothing is
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(dst), "l"(src), "r"(there ? 8 : 0) : "memory");
+}
+__device__ __forceinline__ void copy_async4(uint32_t dst, const void *src, bool there) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(there ? 4 : 0) : "memory");
+}
+template <class L> struct AsyncRing {
+  static constexpr int kWorkerBytes = kRingChunks * kAsyncChunk * 16 + 16;                    // skewed like RingLayout
+  static constexpr size_t kBlockBytes = (size_t)L::kWorkers * kWorkerBytes;
+};
+
+template <class L, class Policy>
+__device__ __forceinline__ void walk_tile_async(const L &ln, Policy &p, int32_t j0, int32_t j1, uint32_t smem) {
+  constexpr int kChunk = kAsyncChunk, kPF = Policy::kPF;
+  constexpr uint32_t kMask = kRingChunks * kChunk - 1;
+  static_assert(kChunk % kPF == 0 && L::LPN >= kChunk && !Policy::kAux, "a lane copies an entry of a chunk at most");
+  if (j0 >= j1) return;
+  auto slot = [&](int32_t x) { return smem + ((uint32_t)x & kMask) * 16; };                   // of the tile's entry x
+  auto ask = [&](int32_t x0) {                             // entries x0 .. x0 + kChunk - 1; those past the tile's end become zeros
+    if (ln.g < kChunk) {
+      const int32_t j = j0 + x0 + ln.g;
+      p.fetch_async(j < j1 ? j : j0, slot(x0 + ln.g), j < j1);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  auto settle = [&](int32_t x0) { if (ln.g < kChunk) p.settle(slot(x0 + ln.g)); };
+  ask(0);
+  ask(kChunk);
+  ask(2 * kChunk);
+  asm volatile("cp.async.wait_group 2;" ::: "memory");
+  settle(0);
+  ln.sync();
+
+  typename Policy::Slot win[kPF];
+  auto look = [&](uint32_t at, typename Policy::Slot &s) {
+    int32_t ca, cb;
+    lds_coords(at, ca, cb);
+    p.prefetch(ca, cb, s);
+  };
+#pragma unroll
+  for (int u = 0; u < kPF; ++u) look(smem + u * 16, win[u]);
+  const int32_t len = j1 - j0;
+  for (int32_t x0 = 0; x0 < len; x0 += kChunk) {
+    asm volatile("cp.async.wait_group 1;" ::: "memory");   // this lane's part of the next chunk is there
+    settle(x0 + kChunk);
+    ln.sync();                                             // every lane's; and the chunk walked last is free
+    ask(x0 + 3 * kChunk);
+    const uint32_t cur = slot(x0), nxt = slot(x0 + kChunk);
+    p.begin_chunk(j0 + x0);
+    const int n = len - x0;
+    if (n >= kChunk) {
+#pragma unroll
+      for (int q = 0; q < kChunk; ++q) {
+        p.consume(q, lds_f64(cur + q * 16), 0, win[q % kPF]);
+        look(q + kPF < kChunk ? cur + (q + kPF) * 16 : nxt + (q + kPF - kChunk) * 16, win[q % kPF]);
+      }
+    } else {                                               // the last chunk looks ahead inside itself only
+#pragma unroll 1
+      for (int q0 = 0; q0 < n; q0 += kPF)
+#pragma unroll
+        for (int u = 0; u < kPF; ++u) {
+          const int q = q0 + u;
+          if (q >= n) break;
+          p.consume(q, lds_f64(cur + q * 16), 0, win[u]);
+          if (q + kPF < n) look(cur + (q + kPF) * 16, win[u]);
+        }
+    }
+  }
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
 }
 
 }  // namespace comet

@@ -32,8 +32,9 @@ struct SegGatherArgs {
   int64_t ldb;
   void *C;                  // output rows (T), already offset to this launch's first column
   int64_t ldc;
-  const int32_t *out_row;   // NULL: segment s -> row s. Else segment s -> row out_row[s] (ascending) and the
-  int64_t out_rows;         //   rows in between (and up to out_rows) are zero-filled by the flushing worker
+  const int32_t *out_row;   // NULL: segment s -> row s. Else segment s -> row out_row[s] (ascending); the rows in between
+  int64_t out_rows;         //   (and up to out_rows) hold zeros already or are cleared by the CTAs from gap_from on
+  int64_t gap_from;
   int32_t R;                // columns handled by this launch
   bool wide_store;          // ragged shapes: rows of C take 16-byte stores
   int32_t tile_items;
@@ -47,10 +48,9 @@ struct SegGatherArgs {
                             //      path of SpMM): neither walked nor stored here. Never below tile_items.
 };
 
-// Where the rows of C go: segment s to row s; through out_row, the rows in between filled with zeros; or through out_row into
-// a C that holds zeros already. Three kernels, not a test: it sat in the body that is unrolled for every entry of a chunk, and
-// a DCSR matrix of 6.6 M entries in 2.1 M of 2.2 M rows, fp32, R = 31, took 1,060 us with it, 853 without.
-constexpr int kRowsAll = 0, kRowsFilled = 1, kRowsMapped = 2;
+// Where the rows of C go: segment s to row s, or through out_row. Two kernels, not a test, as the closing of a segment sits in
+// the body that is unrolled for every entry of a chunk.
+constexpr int kRowsAll = 0, kRowsMapped = 1;
 
 // What the walker does with one leaf entry: close the segments that end in front of it, accumulate.
 template <class T, int LPN, int CPL, int VEC, bool RAGGED, int ROWS, bool PASS_THROUGH = false>
@@ -61,9 +61,7 @@ struct SegGatherPolicy {
   static constexpr bool kAux = false;
   // Ragged fp32 rows end in up to four scalar stores per lane, too much code for one copy per entry of the chunk: with the
   // chunk unrolled the kernel waits for instructions (30 M entries, R = 50: 519 us unrolled, 475 rolled).
-  // The widest workers that fill rows of zeros as well: a copy of that per entry is too much code, too (DCSR, fp64:
-  // 6.2 M entries, power-law rows, R = 200 2.74 ms unrolled, 1.78 rolled; 1.2 M, R = 128 259 and 208 us).
-  static constexpr bool kFullUnroll = !(RAGGED && (sizeof(T) == 4 || ROWS == kRowsFilled)) && !(ROWS == kRowsFilled && CPL * VEC * sizeof(T) > 16 && VEC > 1);
+  static constexpr bool kFullUnroll = !(RAGGED && sizeof(T) == 4);
   // one copy of the unrolled body where the chunk is long (instruction cache; measured: SpMM config 2 -4 %); the
   // narrow shapes have short tiles of short chunks, where the slower rolled tail costs more than it saves (TTM +5 %)
   static constexpr bool kRolledTail = LPN >= 16;
@@ -109,21 +107,12 @@ struct SegGatherPolicy {
   }
   __device__ __forceinline__ void begin_chunk(int32_t b) { rel_end -= b - base; base = b; }
 
-  // Stores the open segment (and, for a compressed root level, zero-fills the rows in front of it).
-  __device__ __forceinline__ void flush() {
+  __device__ __forceinline__ void flush() {      // stores the open segment
     T *cmat = static_cast<T *>(a.C) + ln.col0;
-    if (ROWS != kRowsAll) {
-      const int64_t i = seg;
-      const int64_t r = __ldg(a.out_row + i);
-      if (ROWS == kRowsFilled) {
-        const int64_t lo = (i > 0) ? (int64_t)__ldg(a.out_row + i - 1) + 1 : 0;
-        ln.zero_rows(cmat, a.ldc, lo, r);
-        if (i == a.M - 1) ln.zero_rows(cmat, a.ldc, r + 1, a.out_rows);
-      }
-      ln.store_row(cmat + r * a.ldc, acc);
-    } else {
-      ln.store_row(cmat + (int64_t)seg * a.ldc, acc);
-    }
+    // (asking for the row, or the next end, when the segment opens takes the registers that the window needs: 65 -> 76 us on
+    // 2 M entries, R = 16; TTM 345 -> 399)
+    const int64_t row = ROWS == kRowsMapped ? (int64_t)__ldg(a.out_row + seg) : (int64_t)seg;
+    ln.store_row(cmat + row * a.ldc, acc);
     ln.zero(acc);
     ++seg;
     rel_end = end_of_open();
@@ -133,6 +122,54 @@ struct SegGatherPolicy {
     ln.fma_rows(v, s.r, acc);
   }
 };
+
+// Clears those of kGapRows rows of C that no segment owns (block b: rows b * kGapRows and on). The stored rows of the block are
+// marked in shared memory, then consecutive threads clear consecutive pieces of the others: about the same work for
+// every block wherever the empty rows lie. As CTAs of the gather kernel, whose rows are other ones, this costs no launch.
+// When the workers filled the rows in front of each segment that they closed, the code for that sat in every entry of the
+// unrolled chunk, and a tile with a long gap held its workers up: DCSR, power-law rows, all of them stored, fp64, 5.6 M entries,
+// R = 32 435 us, as here 130; fp32, 4.5 M, R = 31 196 and 135; 2 M entries in 491,000 of 500,000 rows, R = 16 98 and 59.
+constexpr int kGapRows = 1024;         // 256 / 512 / 1,024 / 2,048 rows: 6.6 M entries in 2.1 M of 2.2 M rows, fp32, R = 31 393 / 375 / 355 / 434 us
+template <class T>
+__device__ __forceinline__ void gap_role(const SegGatherArgs &a, int64_t block, unsigned char *smem) {
+  static_assert(kGapRows % kBlockThreads == 0 && kGapRows / 32 <= kBlockThreads, "");
+  uint32_t *const bits = reinterpret_cast<uint32_t *>(smem), *const empties = bits + kGapRows / 32;
+  uint16_t *const empty = reinterpret_cast<uint16_t *>(empties + 1);        // the empty rows, in any order
+  const int64_t r0 = block * kGapRows;
+  const int lane = threadIdx.x & 31;
+  if (threadIdx.x <= kGapRows / 32) bits[threadIdx.x] = 0;                  // and their number
+  int64_t lo = 0, hi = a.M;                                // the first segment whose row is r0 or behind it
+  while (lo < hi) {
+    const int64_t stride = (hi - lo + 31) / 32;
+    const int64_t q = lo + (int64_t)lane * stride + stride - 1;
+    const int full = __popc(__ballot_sync(0xffffffffu, q < hi && __ldg(a.out_row + q) < r0));
+    lo += (int64_t)full * stride;
+    const int64_t cap = lo + stride - 1;
+    if (cap < hi) hi = cap;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int t = 0; t < kGapRows / kBlockThreads; ++t) {     // rows are distinct: at most kGapRows of them lie in the block
+    const int64_t mine = lo + t * kBlockThreads + threadIdx.x;
+    const int64_t at = mine < a.M ? (int64_t)__ldg(a.out_row + mine) - r0 : kGapRows;
+    if (at < kGapRows) atomicOr(&bits[at >> 5], 1u << (at & 31));
+  }
+  __syncthreads();
+  const int rows = (int)(a.out_rows - r0 < kGapRows ? a.out_rows - r0 : kGapRows);
+  constexpr int PER = 16 / sizeof(T);
+  const bool wide = a.wide_store && a.R % PER == 0;
+  const int width = wide ? a.R / PER : a.R;
+  T *const C = static_cast<T *>(a.C) + r0 * a.ldc;
+  for (int r = threadIdx.x; r < rows; r += kBlockThreads)
+    if (!((bits[r >> 5] >> (r & 31)) & 1u)) empty[atomicAdd(empties, 1u)] = (uint16_t)r;
+  __syncthreads();
+  const int work = (int)*empties * width;
+  for (int i = threadIdx.x; i < work; i += kBlockThreads) {
+    const int e = i / width, c = i - e * width, r = empty[e];
+    if (wide) __stcs(reinterpret_cast<int4 *>(C + (int64_t)r * a.ldc) + c, make_int4(0, 0, 0, 0));
+    else __stcs(C + (int64_t)r * a.ldc + c, (T)0);
+  }
+}
 
 // HEAVY: the first h.heavy_ctas CTAs of the grid work on the long rows of an SpMM (spmm_heavy.cuh) while the
 // others walk the general tiles and skip those rows. The two roles are bound by different things (the long rows
@@ -145,6 +182,10 @@ seg_gather_kernel(const SegGatherArgs a, const HeavyArgs h) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   if (HEAVY && (int)blockIdx.x < h.heavy_ctas) {
     heavy_role<T, LPN, CPL, VEC>(h, smem_raw);
+    return;
+  }
+  if (ROWS == kRowsMapped && (int64_t)blockIdx.x >= a.gap_from) {
+    gap_role<T>(a, (int64_t)blockIdx.x - a.gap_from, smem_raw);
     return;
   }
   const int worker = threadIdx.x / LPN;
@@ -524,8 +565,8 @@ int32_t choose_tile_items(int64_t total_items, int workers_per_block, int ctas_p
   return (int32_t)(t < least ? least : t);
 }
 
-// The same where tiles are uneven: beside the long rows of an SpMM, whose entries the tiles leave out, and where rows are
-// mapped (a DCSR matrix: rows of zeros in front of the stored ones, stores far apart). Four tiles per resident worker, or eight, so that the last ones do not leave the
+// The same where tiles are uneven: beside the long rows of an SpMM, whose entries the tiles leave out, and where the rows of a
+// cleared C are written far apart. Four tiles per resident worker, or eight, so that the last ones do not leave the
 // chip idle. DCSR, 94 % of the rows empty, R = 8, 2 / 4 / 6 / 8 tiles 1037 / 960 / 928 / 919 us; 5.6 M entries in power-law rows,
 // R = 32, one / two / four / eight 478 / 456 / 454 / 422 us; 4.2 M rows in a cleared C, R = 8, one wave 788, eight tiles 762.
 static int32_t choose_uneven_tile_items(int64_t total_items, int workers_per_block, int per_worker) {
@@ -646,7 +687,7 @@ static comet_status_t launch_one(Context *ctx, SegGatherArgs a, HeavyArgs *heavy
   const int64_t total = a.M + a.N;
   a.carry_ld = (int32_t)align_up((size_t)a.R, 2);
   constexpr int kCtas = CPL * VEC * sizeof(T) <= 16 ? COMET_MINB_GATHER : 2;
-  a.tile_items = a.out_row ? choose_uneven_tile_items(total, WORKERS, 8)
+  a.tile_items = a.out_row && cleared ? choose_uneven_tile_items(total, WORKERS, 8)
                            : choose_tile_items(total, WORKERS, kCtas, 8, LPN <= 2 ? 32 : 48, 1024);
   size_t heavy_bytes = 0;
   HeavyArgs h{};
@@ -709,9 +750,10 @@ static comet_status_t launch_one(Context *ctx, SegGatherArgs a, HeavyArgs *heavy
       return COMET_OK;
     }
   }
+  a.gap_from = blocks;
+  const int64_t gap_blocks = a.out_row && !cleared ? ceil_div(a.out_rows, (int64_t)kGapRows) : 0;
   st = !a.out_row ? launch_mapped<T, LPN, CPL, VEC, RAGGED, kRowsAll, false>(ctx, a, h, blocks, stream)
-       : cleared  ? launch_mapped<T, LPN, CPL, VEC, RAGGED, kRowsMapped, false>(ctx, a, h, blocks, stream)
-                  : launch_mapped<T, LPN, CPL, VEC, RAGGED, kRowsFilled, false>(ctx, a, h, blocks, stream);
+                  : launch_mapped<T, LPN, CPL, VEC, RAGGED, kRowsMapped, false>(ctx, a, h, blocks + gap_blocks, stream);
   if (st != COMET_OK) return st;
   carry_fixup_launch(kDtype, a.carry_val, a.carry_seg, a.num_tiles, a.R, a.carry_ld, a.C, a.ldc, a.out_row, true, stream);
   COMET_LAUNCH_CHECK(ctx);
@@ -755,15 +797,13 @@ static comet_status_t seg_gather_typed(Context *ctx, const int32_t *seg_end, con
   auto one_column_per_lane = [&](int64_t chunk) {
     return chunk > 32 * PER && ((chunk < 64 * PER && N < 4 * M) || (split && R <= 128 && chunk > 48 * PER));
   };
-  // A compressed root level with far more rows than segments: C is cleared in one stream of wide stores and the stored rows
-  // are written over it. A worker that fills the rows in front of each segment itself writes fewer bytes but waits for its
-  // gathers in between (4.2 M entries in 67 M / 8.4 M rows, R = 8: 919 -> 792, 290 -> 266 us). From six rows per segment on
-  // the clear wins nearly always, from two on where the stored rows are narrow or many, or C is so large that it leaves
-  // the cache in between anyway; with wide rows in a C of some hundred MB the second write costs up to 1.3 times the fill
-  // (0.32 M entries in 1.06 M rows, fp32, R = 25: 68 us filled, 110 cleared).
+  // A compressed root level whose empty rows are cleared by CTAs of the gather launch (gap_role), which write them once, or
+  // C is cleared as a whole in one stream of wide stores first (7.5 TB/s where the others reach 4.5) and the stored rows are written over
+  // it: narrow rows, or few stored ones in a large C. Gaps -> stream: 4.2 M entries in 67 M / 8.4 M rows, R = 8 1018 -> 765, 269 ->
+  // 232 us; 1 M in 5 M, fp32, R = 4 92 -> 65; but 1 M in 3 M, R = 64 331 -> 395; 0.32 M in 1.06 M, R = 25 82 -> 97; 0.1 M in 1 M, R = 16
+  // 35 -> 39.
   const int64_t row_bytes = R * (int64_t)sizeof(T), c_bytes = out_rows * row_bytes;
-  const bool cleared = out_row && (out_rows >= 6 * M || (out_rows >= 2 * M && (row_bytes <= 64 || (c_bytes >= 60000000 &&
-                                                         (row_bytes <= 256 || M >= 500000 || c_bytes >= 1000000000)))));
+  const bool cleared = out_row && ((out_rows >= 2 * M && row_bytes <= 64 && c_bytes >= 20000000) || (out_rows >= 6 * M && c_bytes >= 200000000));
   if (cleared) {
     const comet_status_t zs = zero_rows(ctx, C, sizeof(T) == 4 ? COMET_F32 : COMET_F64, out_rows, R, ldc, stream);
     if (zs != COMET_OK) return zs;
@@ -822,6 +862,7 @@ comet_status_t seg_gather(Context *ctx, int dtype, const int32_t *seg_end, const
                           const int32_t *out_row, int64_t out_rows, int64_t b_rows, bool long_rows, cudaStream_t stream) {
   if (ldb >= (1ll << 28)) return COMET_ERR_INDEX_OVERFLOW;      // row offsets are formed as int32 bytes * int32 index
   if (M == 0) return out_row ? zero_rows(ctx, C, dtype, out_rows, R, ldc, stream) : COMET_OK;
+  if (out_row && M == out_rows) out_row = nullptr;         // every row is stored: segment s is row s
   if (dtype == COMET_F32)
     return seg_gather_typed<float>(ctx, seg_end, crd, (const float *)val, M, N, (const float *)B, ldb, R, (float *)C, ldc,
                                    out_row, out_rows, b_rows, long_rows, stream);

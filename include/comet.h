@@ -140,7 +140,7 @@ int64_t comet_kernel_launches(comet_handle_t handle);
  * COMET_ERR_COORD_OUT_OF_RANGE); `out` is then left zeroed. On success `out` owns its arrays
  * (allocated through the handle's allocator) until comet_sptensor_free. Synchronises `stream` once (twice for an input that
  * takes the general path after the one for larger inputs could not hold it). From 600,000 entries on a call takes about 80 bytes
- * of temporary memory per entry from the allocator, or, where it has no room for them, 24.
+ * of temporary memory per entry from the allocator, or, where it has no room for them or for the tensor beside them, 24.
  *
  * ELLPACK (named in the Tensor Storage Format section among the formats the four attributes compose; the paper
  * does not spell the composition out, this is the reading used): order 2 with h_attr = {COMET_D, COMET_S} gives a

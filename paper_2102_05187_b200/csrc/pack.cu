@@ -645,11 +645,10 @@ struct TempBlocks {
     if (q) p[n++] = q;
     return q;
   }
-  void adopt(TempBlocks &other) {    // at most one block
-    for (int i = 0; i < other.n; ++i) p[n++] = other.p[i];
-    other.n = 0;
+  void release() {
+    while (n > 0) ctx_free(ctx, p[--n], s);
   }
-  ~TempBlocks() { for (int i = 0; i < n; ++i) ctx_free(ctx, p[i], s); }
+  ~TempBlocks() { release(); }
 };
 
 }  // namespace
@@ -860,41 +859,48 @@ extern "C" comet_status_t comet_pack_ex(comet_handle_t handle, int32_t order, co
     return COMET_OK;
   };
   // Larger inputs of distinct keys: split by samples and sorted in shared memory, in the tensor's arrays at once where no
-  // level needs a count. Where there is no room for its records, or a region was too small, the radix sort packs them.
+  // level needs a count. Where there is no room for its records, or for the tensor beside them, or a region was too small, all
+  // of that goes back and the radix sort packs them, in less than a third of the memory.
   bool split = !small && !(flags & COMET_PACK_SUM_DUPLICATES) && pack_split_applies(order, total_bits, n);
+  TempBlocks records(ctx, s);
   if (split) {
-    TempBlocks block(ctx, s);
     const bool direct = plan.ncounted == 0 && (h_attr[0] == COMET_CN || order == 2);
-    char *records = (char *)block.get(pack_split_bytes(n));
-    uint32_t *scan_tmp = nullptr;
-    if (records && !direct) {
-      table = (uint32_t *)tmp.get((size_t)counts_len * 4);
-      scan_tmp = (uint32_t *)tmp.get((size_t)scan_tmp_words(counts_len) * 4);
-    }
-    split = records && (direct || (table && scan_tmp));
-    if (split) {
-      comet_status_t st = direct ? allocate(nullptr) : COMET_OK;
-      if (st != COMET_OK) return drop(st);
-      st = [&]() -> comet_status_t {
-        COMET_CUDA_TRY(ctx, cudaMemsetAsync(ctx->d_status, 0, 16 * sizeof(int32_t), s));
-        PackSplitSorted sorted{};
-        comet_status_t q = pack_split_sort(ctx, order, coords, key, plan, coo_val, dtype, n, records, direct ? &lo : nullptr, &sorted, s);
+    const comet_status_t st = [&]() -> comet_status_t {
+      char *block = (char *)records.get(pack_split_bytes(n));
+      uint32_t *scan_tmp = nullptr;
+      if (block && !direct) {
+        table = (uint32_t *)records.get((size_t)counts_len * 4);
+        scan_tmp = (uint32_t *)records.get((size_t)scan_tmp_words(counts_len) * 4);
+      }
+      if (!block || (!direct && (!table || !scan_tmp))) return COMET_ERR_ALLOC;
+      comet_status_t q = direct ? allocate(nullptr) : COMET_OK;
+      if (q != COMET_OK) return q;
+      COMET_CUDA_TRY(ctx, cudaMemsetAsync(ctx->d_status, 0, 16 * sizeof(int32_t), s));
+      PackSplitSorted sorted{};
+      q = pack_split_sort(ctx, order, coords, key, plan, coo_val, dtype, n, block, direct ? &lo : nullptr, &sorted, s);
+      if (q != COMET_OK) return q;
+      if (!direct) {
+        keys_a = sorted.keys;
+        sorted_val = sorted.val;
+        q = count_nodes(scan_tmp);
         if (q != COMET_OK) return q;
-        if (!direct) {
-          keys_a = sorted.keys;
-          sorted_val = sorted.val;
-          q = count_nodes(scan_tmp);
-          if (q != COMET_OK) return q;
-        }
-        return read_status();
-      }();
-      if (st != COMET_OK) return drop(st);
-      if (ctx->h_pinned[kStatusRange]) return drop(COMET_ERR_COORD_OUT_OF_RANGE);
+      }
+      q = read_status();
+      if (q != COMET_OK) return q;
+      if (ctx->h_pinned[kStatusRange]) return COMET_ERR_COORD_OUT_OF_RANGE;
       split = !ctx->h_pinned[kStatusOverflow];
-      if (!split) drop(COMET_OK);
-      else if (ctx->h_pinned[kStatusDuplicate]) return drop(COMET_ERR_DUPLICATE_COORD);
-      else if (direct) { out->owner = owner; return COMET_OK; }
-      else tmp.adopt(block);
+      if (!split) return COMET_OK;
+      if (ctx->h_pinned[kStatusDuplicate]) return COMET_ERR_DUPLICATE_COORD;
+      return direct ? COMET_OK : allocate(reinterpret_cast<uint32_t *>(ctx->h_pinned) + 8);
+    }();
+    if (st == COMET_ERR_ALLOC) split = false;
+    else if (st != COMET_OK) return drop(st);
+    if (!split) {
+      drop(COMET_OK);
+      records.release();
+    } else if (direct) {
+      out->owner = owner;
+      return COMET_OK;
     }
   }
   if (!small && !split) {
@@ -957,7 +963,7 @@ extern "C" comet_status_t comet_pack_ex(comet_handle_t handle, int32_t order, co
   if (ctx->h_pinned[kStatusRange]) return COMET_ERR_COORD_OUT_OF_RANGE;
   if (ctx->h_pinned[kStatusDuplicate]) return COMET_ERR_DUPLICATE_COORD;
 
-  {
+  if (!owner) {
     const comet_status_t st = allocate(reinterpret_cast<uint32_t *>(ctx->h_pinned) + 8);
     if (st != COMET_OK) return drop(st);
   }

@@ -686,7 +686,7 @@ static comet_status_t launch_one(Context *ctx, SegGatherArgs a, HeavyArgs *heavy
   constexpr int WORKERS = kBlockThreads / LPN;
   const int64_t total = a.M + a.N;
   a.carry_ld = (int32_t)align_up((size_t)a.R, 2);
-  constexpr int kCtas = CPL * VEC * sizeof(T) <= 16 ? COMET_MINB_GATHER : 2;
+  constexpr int kCtas = resident_ctas(CPL * VEC * sizeof(T) <= 16 ? COMET_MINB_GATHER : 2, RingLayout<Lanes<T, LPN, CPL, VEC, RAGGED>, false>::kBlockBytes);
   a.tile_items = a.out_row && cleared ? choose_uneven_tile_items(total, WORKERS, 8)
                            : choose_tile_items(total, WORKERS, kCtas, 8, LPN <= 2 ? 32 : 48, 1024);
   size_t heavy_bytes = 0;

@@ -114,8 +114,13 @@ struct CooPolicy {
   }
 };
 
+// CTAs per SM that the register budget is held to. Two pieces of 16 bytes a lane: the unrolled chunk takes 246 registers, in
+// the ragged form, which rolls it, 118 (COO of 0.24 M entries, fp64, R = 100 36 us with four tiles per worker, 46 in a wave of one CTA, 37 of two).
+template <class T, int CPL, int VEC, bool RAGGED>
+constexpr int kCooCtas = CPL * VEC * sizeof(T) <= 16 ? COMET_MINB_COO : RAGGED || VEC == 1 ? 2 : 1;
+
 template <class T, int LPN, int CPL, int VEC, bool RAGGED>
-__global__ void __launch_bounds__(kBlockThreads, (CPL * VEC * sizeof(T) <= 16 ? COMET_MINB_COO : 1)) mttkrp_coo_kernel(const MttkrpArgs a) {
+__global__ void __launch_bounds__(kBlockThreads, (kCooCtas<T, CPL, VEC, RAGGED>)) mttkrp_coo_kernel(const MttkrpArgs a) {
   using L = Lanes<T, LPN, CPL, VEC, RAGGED>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int worker = threadIdx.x / LPN;
@@ -440,7 +445,9 @@ static comet_status_t launch_mttkrp(Context *ctx, MttkrpArgs a, int64_t p_pad, i
   constexpr int WORKERS = kBlockThreads / LPN;
   const int64_t total = CSF ? a.F + a.N : a.N;
   using L = Lanes<T, LPN, CPL, VEC, RAGGED>;
-  constexpr int kCtas = CPL * VEC * sizeof(T) <= 16 ? 4 : CSF ? 2 : 1;
+  constexpr size_t smem = CSF ? RingLayout<L, false>::kBlockBytes + (size_t)WORKERS * kCsfWorkerBytes
+                              : RingLayout<L, true>::kBlockBytes;
+  constexpr int kCtas = resident_ctas(!CSF ? kCooCtas<T, CPL, VEC, RAGGED> : CPL * VEC * sizeof(T) <= 16 ? COMET_MINB_CSF : 2, smem);
   a.tile_items = choose_tile_items(total, WORKERS, kCtas, CSF ? 32 : 8, LPN <= 2 ? 32 : 48, 512);
   // A COO tile is that many entries: whole chunks, or every tile ends in one that is walked as a loop (100 M entries, tiles of
   // 503 entries 2916 us, of 512 2847).
@@ -474,8 +481,6 @@ static comet_status_t launch_mttkrp(Context *ctx, MttkrpArgs a, int64_t p_pad, i
     a.part_slice = ps;
   }
   const unsigned blocks = (unsigned)ceil_div(a.num_tiles, WORKERS);
-  constexpr size_t smem = CSF ? RingLayout<L, false>::kBlockBytes + (size_t)WORKERS * kCsfWorkerBytes
-                              : RingLayout<L, true>::kBlockBytes;
   // CSF with short fibers (mean length below 4): the per-entry form; COMET_CSF_FORM=fold / expand forces one
   bool expand = CSF && a.N < 4 * a.F;
   if (const char *e = getenv("COMET_CSF_FORM")) expand = CSF && (e[0] == 'e' ? true : (e[0] == 'f' ? false : expand));

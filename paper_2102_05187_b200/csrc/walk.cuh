@@ -243,6 +243,14 @@ template <class L, bool AUX> struct RingLayout {
   static constexpr size_t kBlockBytes = (size_t)L::kWorkers * kWorkerBytes;
 };
 
+// CTAs that an SM holds beside each other: as many as their registers allow, or their shared memory (228 KB, of which each CTA
+// takes another KB). Workers of one or two lanes are many to a CTA, each with a ring of its own. What a wave is follows from it: CSF
+// MTTKRP of 9 M entries, fp32, R = 8 274 us with four tiles per worker, 330 in one of four CTAs where three fit, 255 in one of three.
+constexpr int resident_ctas(int by_registers, size_t smem) {
+  const int by_memory = (int)(228 * 1024 / (smem + 1024));
+  return by_memory < by_registers ? by_memory : by_registers;
+}
+
 // A policy that declares `static constexpr bool kPositional = true` is told WHERE the entry it prefetches sits
 // (position `at` of the current or of the next chunk) through prefetch_at(at, in_current_chunk, a, b, slot):
 // for policies that keep per-chunk information about the entries (the CSF fiber-end masks).

@@ -50,3 +50,44 @@ def test_mttkrp_coo(items, off):
     want, norm = oracle.mttkrp(c, v, dims, 0, F)
     A = upload_packed(oracle.pack(c, v, dims, (0, 1, 2), (CN, S, S)))
     assert_close(comet.mttkrp(A, 0, [None] + [dev(f) for f in F[1:]]), want, norm, what="mttkrp")
+
+
+def _tensor(total, dims, fibers, seed):
+    """3-order coordinates sorted by storage order: `fibers` fibers that hold total - fibers entries, so that the merge list of a
+    kernel that has a marker per fiber holds `total` items."""
+    n = total - fibers
+    rng = np.random.default_rng(seed)
+    f = np.sort(rng.choice(dims[0] * dims[1], fibers, replace=False))
+    cells = np.arange(fibers) * dims[2]                      # an entry in every fiber, the others anywhere
+    more = np.setdiff1d(rng.choice(fibers * dims[2], n + fibers, replace=False), cells)
+    cells = np.sort(np.concatenate([cells, rng.permutation(more)[:n - fibers]]))
+    assert cells.size == n
+    row = f[cells // dims[2]]
+    return [(row // dims[1]).astype(np.int32), (row % dims[1]).astype(np.int32), (cells % dims[2]).astype(np.int32)], rng.uniform(-1, 1, n)
+
+
+# Lanes a worker: one (a CTA to an SM, four waves), two (three CTAs to an SM), 16, and 32 with two pieces.
+@pytest.mark.parametrize("R,workers,ctas,items", [(2, 256, 4, 31), (2, 256, 4, 33), (4, 128, 3, 23), (4, 128, 3, 33), (32, 16, 4, 35),
+                                                  (32, 16, 4, 36), (32, 16, 4, 64), (64, 8, 4, 23), (64, 8, 4, 24), (128, 8, 2, 33), (128, 8, 2, 49)])
+@pytest.mark.parametrize("off", [0, 1])
+def test_mttkrp_csf(R, workers, ctas, items, off):
+    total, dims = 148 * ctas * workers * items + off, (97, 89, 4003)
+    c, v = _tensor(total, dims, min(8001, total // 10), items)
+    F = [None] + [synth.random_dense((d, R), 4 + i).numpy() for i, d in enumerate(dims[1:])]
+    want, norm = oracle.mttkrp(c, v, dims, 0, F)
+    A = upload_packed(oracle.pack(c, v, dims, (0, 1, 2), (CU, CU, CU)))
+    assert_close(comet.mttkrp(A, 0, [None] + [dev(f) for f in F[1:]]), want, norm, what="mttkrp")
+
+
+# One lane (two CTAs to an SM, two waves beyond 32 items), two, 16 (whole chunks in many waves only), 32 with two pieces whole (one CTA)
+# and ragged (two).
+@pytest.mark.parametrize("R,workers,ctas,items", [(2, 256, 2, 11), (2, 256, 2, 12), (2, 256, 2, 33), (4, 128, 4, 23), (4, 128, 4, 24), (32, 16, 4, 47),
+                                                  (32, 16, 4, 48), (32, 16, 4, 129), (128, 8, 1, 31), (128, 8, 1, 33), (100, 8, 2, 23), (100, 8, 2, 24)])
+def test_mttkrp_coo_widths(R, workers, ctas, items):
+    dims = (301, 97, 211)
+    coords, val = synth.random_coo(dims, 148 * ctas * workers * items + 1, 3)
+    c, v = [x.numpy() for x in coords], val.numpy()
+    F = [None] + [synth.random_dense((d, R), 4 + i).numpy() for i, d in enumerate(dims[1:])]
+    want, norm = oracle.mttkrp(c, v, dims, 0, F)
+    A = upload_packed(oracle.pack(c, v, dims, (0, 1, 2), (CN, S, S)))
+    assert_close(comet.mttkrp(A, 0, [None] + [dev(f) for f in F[1:]]), want, norm, what="mttkrp")

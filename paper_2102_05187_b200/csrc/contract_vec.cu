@@ -549,20 +549,20 @@ static int32_t forced_tile_items() {
 }
 
 // Items per tile where tiles cost the same: one tile per resident worker (148 SMs x ctas_per_sm CTAs), so that the launch is one
-// full wave, or the fewest full waves of tiles of at most `most` items. Every tile costs a boundary, a cold start and a carry,
-// and a wave that is partly filled costs a whole one. With about 4 tiles per worker, rounded to at most 160 items on
-// mid-sized inputs, -> as here: SpMM, fp64, 3.1 M entries, R = 32 99.7 -> 79.0 us, 5.6 M, R = 10 116.7 -> 106.6, 5 M, R = 64 350
+// full wave, or, beyond `once` items, full waves, `waves` or more, of tiles of at most `most`. Every tile costs a boundary, a cold
+// start and a carry, and a wave that is partly filled costs a whole one. With about 4 tiles per worker, rounded to at most 160 items
+// on mid-sized inputs, -> as here: SpMM, fp64, 3.1 M entries, R = 32 99.7 -> 79.0 us, 5.6 M, R = 10 116.7 -> 106.6, 5 M, R = 64 350
 // -> 322; TTM, R = 16, 3 M 74.3 -> 57.7, R = 32, 10 M 224 -> 196; MTTKRP, CSF, 3 M, R = 16 124 -> 107.5, COO, 20 M, R = 32 629 -> 592;
-// two waves 88 / 114 / 335, 60.6 / 205, 114. (`most`: 512 entries of MTTKRP are added in a row, 1,024 of SpMM and TTM.)
+// two waves 88 / 114 / 335, 60.6 / 205, 114.
 // Small inputs take up to twice the items of a full wave, while that is at most `brief`: half a wave of 48 items is faster than a
 // full one of 24 (200,000 entries, R = 32 18.9 and 20.3 us; 0.4 M, fp32 26.2 and 29.2), of 96 no longer (0.8 M 46.8, 41.0).
-int32_t choose_tile_items(int64_t total_items, int workers_per_block, int ctas_per_sm, int32_t least, int32_t brief, int32_t most) {
+int32_t choose_tile_items(int64_t total_items, int workers_per_block, int ctas_per_sm, const TileRule &r) {
   if (const int32_t forced = forced_tile_items()) return forced;
-  const int64_t workers = (int64_t)kSmCount * ctas_per_sm * workers_per_block;
-  const int64_t waves = ceil_div(total_items, workers * most);
-  int64_t t = ceil_div(total_items, workers * waves);
-  if (t < brief) t = 2 * t < brief ? 2 * t : brief;
-  return (int32_t)(t < least ? least : t);
+  auto with_ctas = [&](int64_t ctas) { return ceil_div(total_items, kSmCount * ctas * workers_per_block); };
+  int64_t t = with_ctas(ctas_per_sm);
+  if (t > r.once) t = with_ctas(ctas_per_sm * (ceil_div(t, r.most) > r.waves ? ceil_div(t, r.most) : r.waves));
+  if (t < r.brief) t = 2 * t < r.brief ? 2 * t : r.brief;
+  return (int32_t)(t < r.least ? r.least : t);
 }
 
 // The same where tiles are uneven: beside the long rows of an SpMM, whose entries the tiles leave out, and where the rows of a
@@ -678,17 +678,26 @@ comet_status_t pad_rows2(Context *ctx, int dtype, const void *src0, int64_t rows
   return prepare_run(ctx, dtype, a, stream);
 }
 
+// A worker of one lane reads its tile's entries by itself, 32 such tiles to a warp: where they are long, no two lanes read from
+// one line, and all the lines are more than the L1 holds. 12 to 18 entries are best at every size: SpMM of 9 M entries, fp64, R = 2
+// 522 us in one wave, 517 with four tiles per worker, 228 as here; fp32, R = 4 452, 453 and 183; TTM, fp64 518, 368 and 224. Two lanes and more: 1,024 entries are added in a row at most.
+template <int LPN>
+constexpr TileRule gather_tile_rule() {
+  return LPN == 1 ? TileRule{8, 16, 20, 1, 16} : LPN == 2 ? TileRule{8, 32, 1024, 1, 1024} : TileRule{8, 48, 1024, 1, 1024};
+}
+
 // `heavy` (optional): the long-row plan of an SpMM; its scratch precedes the carries of this launch. pad (RAGGED): the
 // first `pad` rows of B are copied into scratch as whole pieces and gathered from there. cleared: out_row is given and C
 // holds zeros.
 template <class T, int LPN, int CPL, int VEC, bool RAGGED = false>
-static comet_status_t launch_one(Context *ctx, SegGatherArgs a, HeavyArgs *heavy, bool cleared, int64_t pad, cudaStream_t stream) {
+static comet_status_t launch_one(Context *ctx, SegGatherArgs a, HeavyArgs *heavy, bool cleared, int64_t pad, cudaStream_t stream, int32_t at_least = 0) {
   constexpr int WORKERS = kBlockThreads / LPN;
   const int64_t total = a.M + a.N;
   a.carry_ld = (int32_t)align_up((size_t)a.R, 2);
   constexpr int kCtas = resident_ctas(CPL * VEC * sizeof(T) <= 16 ? COMET_MINB_GATHER : 2, RingLayout<Lanes<T, LPN, CPL, VEC, RAGGED>, false>::kBlockBytes);
   a.tile_items = a.out_row && cleared ? choose_uneven_tile_items(total, WORKERS, 8)
-                           : choose_tile_items(total, WORKERS, kCtas, 8, LPN <= 2 ? 32 : 48, 1024);
+                           : choose_tile_items(total, WORKERS, kCtas, gather_tile_rule<LPN>());
+  if (a.tile_items < at_least) a.tile_items = at_least;
   size_t heavy_bytes = 0;
   HeavyArgs h{};
   if (!RAGGED && kHeavyShape<T, LPN, CPL, VEC> && heavy && !a.out_row) {
@@ -710,6 +719,8 @@ static comet_status_t launch_one(Context *ctx, SegGatherArgs a, HeavyArgs *heavy
   const int64_t part_least = LPN <= 4 || pad_bytes || heavy_bytes ? 1024 : 16384;
   const size_t part_bytes = use_part && a.num_tiles >= part_least ? align_up((size_t)(a.num_tiles + 1) * sizeof(int32_t), 256) : 0;
   char *scratch = (char *)scratch_get(ctx, pad_bytes + heavy_bytes + carry_bytes(a.num_tiles, a.carry_ld) + part_bytes, stream);
+  // many short tiles have many carries: with no room for them, longer tiles
+  if (!scratch && LPN == 1 && a.tile_items < 512) return launch_one<T, LPN, CPL, VEC, RAGGED>(ctx, a, heavy, cleared, pad, stream, 512);
   if (!scratch) return COMET_ERR_ALLOC;
   PrepareArgs prep{};
   if (pad_bytes) {

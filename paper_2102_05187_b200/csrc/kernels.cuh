@@ -104,7 +104,12 @@ comet_status_t ell_spmm(Context *ctx, const comet_sptensor_t *A, const void *B, 
 comet_status_t elementwise_mul(Context *ctx, const comet_sptensor_t *A, const void *B, const int64_t *h_strides, void *out,
                                cudaStream_t s);
 
-int32_t choose_tile_items(int64_t total_items, int workers_per_block, int ctas_per_sm, int32_t least, int32_t brief, int32_t most);
+struct TileRule {
+  int32_t least;             // items of a tile at least
+  int32_t brief;             // small inputs: tiles up to this size, rather than a full wave of shorter ones
+  int32_t once, waves, most; // one full wave up to `once` items; beyond, `waves` or more of tiles of at most `most`
+};
+int32_t choose_tile_items(int64_t total_items, int workers_per_block, int ctas_per_sm, const TileRule &rule);
 
 // Block list of a library-owned tensor (what comet_sptensor_free releases).
 void *owner_new();

@@ -102,3 +102,20 @@ def test_no_room_for_padded_copies(R):
         assert_close(comet.mttkrp(X, 0, [None, dev(F[1]), dev(F[2])]), want, norm)
     assert (refused or handle.refused) if R == 131 else (refused and handle.refused), "the limit was not met"
     handle.lib.comet_destroy(handle._h)
+
+
+def test_no_room_for_the_carries_of_short_tiles():
+    """Workers of one lane (rows of B of 16 bytes) take tiles of 16 entries; with no room for their carries, long ones."""
+    handle = _LimitedHandle(2 << 20)
+    rows, cols, n = 100_000, 1000, 2_000_000
+    rng = np.random.default_rng(2)
+    cell = np.unique(rng.integers(0, rows * cols, n + 50_000))[:n]
+    r, c = (cell // cols).astype(np.int32), (cell % cols).astype(np.int32)
+    v, B = rng.uniform(-1, 1, n), rng.uniform(-1, 1, (cols, 2))
+    want, norm = oracle.spmm([r, c], v, (rows, cols), B)
+    pk = oracle.pack([r, c], v, (rows, cols), (0, 1), (D, CU))
+    A = comet.SpTensor.from_arrays(pk.dims, pk.mode_order, pk.attr, [dev(p, torch.int32) for p in pk.pos],
+                                   [None, dev(pk.crd[1], torch.int32)], dev(pk.val), handle=handle)
+    assert_close(comet.spmm(A, dev(B)), want, norm)
+    assert handle.refused == 1, "the limit was not met"
+    handle.lib.comet_destroy(handle._h)

@@ -66,6 +66,20 @@ def _tensor(total, dims, fibers, seed):
     return [(row // dims[1]).astype(np.int32), (row % dims[1]).astype(np.int32), (cells % dims[2]).astype(np.int32)], rng.uniform(-1, 1, n)
 
 
+# Lanes a worker: one (three CTAs to an SM; tiles of 16 beyond 20), two, eight (two CTAs to an SM below 24 items in a full wave, three
+# below 64; three waves beyond 192 where fibers are long on average).
+@pytest.mark.parametrize("R,workers,ctas,items", [(2, 256, 3, 11), (2, 256, 3, 12), (2, 256, 3, 20), (2, 256, 3, 21), (4, 128, 4, 23), (4, 128, 4, 24),
+                                                  (16, 32, 4, 7), (16, 32, 4, 23), (16, 32, 4, 24), (16, 32, 4, 63), (16, 32, 4, 64), (16, 32, 4, 192)])
+@pytest.mark.parametrize("off", [0, 1])
+def test_ttm(R, workers, ctas, items, off):
+    total, dims = 148 * ctas * workers * items + off, (97, 89, 4003)
+    c, v = _tensor(total, dims, total // 40 if total < 320_000 else 8001, items)
+    U = synth.random_dense((dims[2], R), 5).numpy()
+    _, want, norm = oracle.ttm(c, v, dims, 2, U)
+    A = upload_packed(oracle.pack(c, v, dims, (0, 1, 2), (CU, CU, CU)))
+    assert_close(comet.ttm(A, 2, dev(U)).val.reshape(want.shape), want, norm, what="ttm")
+
+
 # Lanes a worker: one (a CTA to an SM, four waves), two (three CTAs to an SM), 16, and 32 with two pieces.
 @pytest.mark.parametrize("R,workers,ctas,items", [(2, 256, 4, 31), (2, 256, 4, 33), (4, 128, 3, 23), (4, 128, 3, 33), (32, 16, 4, 35),
                                                   (32, 16, 4, 36), (32, 16, 4, 64), (64, 8, 4, 23), (64, 8, 4, 24), (128, 8, 2, 33), (128, 8, 2, 49)])

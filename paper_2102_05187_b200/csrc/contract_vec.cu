@@ -554,14 +554,17 @@ static int32_t forced_tile_items() {
 // on mid-sized inputs, -> as here: SpMM, fp64, 3.1 M entries, R = 32 99.7 -> 79.0 us, 5.6 M, R = 10 116.7 -> 106.6, 5 M, R = 64 350
 // -> 322; TTM, R = 16, 3 M 74.3 -> 57.7, R = 32, 10 M 224 -> 196; MTTKRP, CSF, 3 M, R = 16 124 -> 107.5, COO, 20 M, R = 32 629 -> 592;
 // two waves 88 / 114 / 335, 60.6 / 205, 114.
-// Small inputs take up to twice the items of a full wave, while that is at most `brief`: half a wave of 48 items is faster than a
-// full one of 24 (200,000 entries, R = 32 18.9 and 20.3 us; 0.4 M, fp32 26.2 and 29.2), of 96 no longer (0.8 M 46.8, 41.0).
+// Small inputs, whose full wave would be of tiles below `brief` items, take `few` CTAs per SM, mid-sized ones three of four: fewer
+// and longer tiles, but whole CTAs per SM, or some SMs have one more than the others (COO MTTKRP, 1 M entries, fp64, R = 8 28.4 us
+// with two, 35.0 with 2.2). SpMM of every width class, uniform and power-law rows, time over that of two CTAs per SM: full-wave
+// tiles of 10 to 16 items 1.00 with three and 1.05 with four; 20 to 30 0.96 and 1.01; 45 to 60 0.95 and 0.95; 76 0.91 and 0.92.
 int32_t choose_tile_items(int64_t total_items, int workers_per_block, int ctas_per_sm, const TileRule &r) {
   if (const int32_t forced = forced_tile_items()) return forced;
   auto with_ctas = [&](int64_t ctas) { return ceil_div(total_items, kSmCount * ctas * workers_per_block); };
   int64_t t = with_ctas(ctas_per_sm);
   if (t > r.once) t = with_ctas(ctas_per_sm * (ceil_div(t, r.most) > r.waves ? ceil_div(t, r.most) : r.waves));
-  if (t < r.brief) t = 2 * t < r.brief ? 2 * t : r.brief;
+  else if (t < r.brief) t = with_ctas(r.few);
+  else if (ctas_per_sm == 4 && t < (workers_per_block < 64 ? 64 : 32)) t = with_ctas(3);
   return (int32_t)(t < r.least ? r.least : t);
 }
 
@@ -683,7 +686,7 @@ comet_status_t pad_rows2(Context *ctx, int dtype, const void *src0, int64_t rows
 // 522 us in one wave, 517 with four tiles per worker, 228 as here; fp32, R = 4 452, 453 and 183; TTM, fp64 518, 368 and 224. Two lanes and more: 1,024 entries are added in a row at most.
 template <int LPN>
 constexpr TileRule gather_tile_rule() {
-  return LPN == 1 ? TileRule{8, 16, 20, 1, 16} : LPN == 2 ? TileRule{8, 32, 1024, 1, 1024} : TileRule{8, 48, 1024, 1, 1024};
+  return LPN == 1 ? TileRule{8, 12, 2, 20, 1, 16} : TileRule{8, 24, 2, 1024, 1, 1024};
 }
 
 // `heavy` (optional): the long-row plan of an SpMM; its scratch precedes the carries of this launch. pad (RAGGED): the

@@ -106,7 +106,7 @@ comet_status_t elementwise_mul(Context *ctx, const comet_sptensor_t *A, const vo
 
 struct TileRule {
   int32_t least;             // items of a tile at least
-  int32_t brief;             // small inputs: tiles up to this size, rather than a full wave of shorter ones
+  int32_t brief, few;        // where a full wave is of tiles below `brief` items, `few` CTAs per SM
   int32_t once, waves, most; // one full wave up to `once` items; beyond, `waves` or more of tiles of at most `most`
 };
 int32_t choose_tile_items(int64_t total_items, int workers_per_block, int ctas_per_sm, const TileRule &rule);

@@ -441,10 +441,12 @@ static bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 
 
 // 512 entries are added in a row at most. Workers of one lane have rings and marks that leave two CTAs to an SM (COO), or one
 // (CSF), and four times as many tiles as a wave has workers all the same: a CTA is short of warps then, and its tiles are short.
-template <bool CSF, int LPN>
+// COO pays more per tile (slices are found entry by entry): two CTAs per SM up to twice the size, one where two is all.
+template <bool CSF, int LPN, int CTAS>
 constexpr TileRule mttkrp_tile_rule() {
-  if (CSF) return LPN == 1 ? TileRule{32, 32, 0, 4, 512} : LPN == 2 ? TileRule{32, 32, 512, 1, 512} : TileRule{32, 48, 512, 1, 512};
-  return LPN == 1 ? TileRule{8, 32, 0, 2, 512} : LPN == 2 ? TileRule{8, 32, 512, 1, 512} : TileRule{8, 48, 512, 1, 512};
+  if (CSF) return LPN == 1 ? TileRule{32, 0, 1, 0, 4, 512} : TileRule{32, LPN == 16 ? 36 : 24, 2, 512, 1, 512};
+  if (LPN == 1) return TileRule{8, 12, 1, 32, 2, 512};
+  return CTAS == 4 ? TileRule{8, LPN > 2 ? 48 : 24, 2, 512, 1, 512} : TileRule{32, 30, 1, 512, 1, 512};
 }
 
 // p_pad / q_pad (RAGGED): so many rows of P / Q are copied into scratch as whole pieces and gathered from there.
@@ -456,7 +458,7 @@ static comet_status_t launch_mttkrp(Context *ctx, MttkrpArgs a, int64_t p_pad, i
   constexpr size_t smem = CSF ? RingLayout<L, false>::kBlockBytes + (size_t)WORKERS * kCsfWorkerBytes
                               : RingLayout<L, true>::kBlockBytes;
   constexpr int kCtas = resident_ctas(!CSF ? kCooCtas<T, CPL, VEC, RAGGED> : CPL * VEC * sizeof(T) <= 16 ? COMET_MINB_CSF : 2, smem);
-  a.tile_items = choose_tile_items(total, WORKERS, kCtas, mttkrp_tile_rule<CSF, LPN>());
+  a.tile_items = choose_tile_items(total, WORKERS, kCtas, mttkrp_tile_rule<CSF, LPN, kCtas>());
   // A COO tile is that many entries: whole chunks, or every tile ends in one that is walked as a loop (100 M entries, tiles of
   // 503 entries 2916 us, of 512 2847).
   if (!CSF && a.tile_items >= 4 * L::kChunk && !getenv("COMET_TILE_ITEMS")) a.tile_items = (int32_t)align_up((size_t)a.tile_items, L::kChunk);

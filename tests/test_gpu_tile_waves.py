@@ -80,6 +80,26 @@ def test_ttm(R, workers, ctas, items, off):
     assert_close(comet.ttm(A, 2, dev(U)).val.reshape(want.shape), want, norm, what="ttm")
 
 
+@pytest.mark.parametrize("R,dtype,workers", [(25, "f64", 16), (25, "f32", 32), (37, "f64", 8)])      # copies of B, the last lane masked
+@pytest.mark.parametrize("items", [48, 49])
+@pytest.mark.parametrize("off", [-1, 1])
+def test_spmm_ragged(R, dtype, workers, items, off):
+    items = items * 32 // workers                             # enough entries for the ragged shapes: 250,000 and more
+    rows, t = 2003, torch.float32 if dtype == "f32" else torch.float64
+    n = SLOTS * workers * items + off - rows
+    rng = np.random.default_rng(items)
+    cols = 1 + 2 * n // rows
+    cells = np.sort(rng.choice(rows * cols, n, replace=False))
+    c = [(cells // cols).astype(np.int32), (cells % cols).astype(np.int32)]
+    val, B = rng.uniform(-1, 1, n).astype(np.float32).astype(np.float64), synth.random_dense((cols, R), 5).numpy().astype(np.float32).astype(np.float64)
+    want, norm = oracle.spmm(c, val, (rows, cols), B)
+    pk = oracle.pack(c, val, (rows, cols), (0, 1), (D, CU))
+    A = comet.SpTensor.from_arrays(pk.dims, pk.mode_order, pk.attr, [dev(p, torch.int32) for p in pk.pos],
+                                   [None, dev(pk.crd[1], torch.int32)], dev(pk.val, t))
+    # fp32: sums in double, rounded when stored and once more where a carry is added
+    assert_close(comet.spmm(A, dev(B, t)), want, norm, tol=1e-12 if dtype == "f64" else 3 * 2.0 ** -24, what="spmm")
+
+
 # Lanes a worker: one (a CTA to an SM, four waves), two (three CTAs to an SM), 16, and 32 with two pieces.
 @pytest.mark.parametrize("R,workers,ctas,items", [(2, 256, 4, 31), (2, 256, 4, 33), (4, 128, 3, 23), (4, 128, 3, 33), (32, 16, 4, 35),
                                                   (32, 16, 4, 36), (32, 16, 4, 64), (64, 8, 4, 23), (64, 8, 4, 24), (128, 8, 2, 33), (128, 8, 2, 49)])

@@ -684,22 +684,28 @@ comet_status_t pad_rows2(Context *ctx, int dtype, const void *src0, int64_t rows
 // A worker of one lane reads its tile's entries by itself, 32 such tiles to a warp: where they are long, no two lanes read from
 // one line, and all the lines are more than the L1 holds. 12 to 18 entries are best at every size: SpMM of 9 M entries, fp64, R = 2
 // 522 us in one wave, 517 with four tiles per worker, 228 as here; fp32, R = 4 452, 453 and 183; TTM, fp64 518, 368 and 224. Two lanes and more: 1,024 entries are added in a row at most.
+// Where a tensor's fibers are long on average (`mixed`), some tiles may hold nothing but short ones, which store a row per entry or
+// two, and in one wave the launch waits for those: three waves from 192 items on (16 lanes: 400), for the workers that do not fill a warp. Slices
+// of very different sizes, 22 entries per fiber, 9 M, fp64, R = 10 135 us with four tiles per worker, 162 in one wave, 146 as here; fp32,
+// R = 50, 5.5 M 186, 210 and 173. With short fibers everywhere tiles are alike (8 per fiber, 3.2 M, fp64, R = 32 95 us with four tiles
+// per worker, 74 in one wave, 92 in three); in matrices the long rows cost what the short ones do.
 template <int LPN>
-constexpr TileRule gather_tile_rule() {
-  return LPN == 1 ? TileRule{8, 12, 2, 20, 1, 16} : TileRule{8, 24, 2, 1024, 1, 1024};
+constexpr TileRule gather_tile_rule(bool mixed) {
+  if (LPN == 1) return TileRule{8, 12, 2, 20, 1, 16};
+  return mixed && LPN < 32 ? TileRule{8, 24, 2, LPN == 16 ? 400 : 192, 3, 640} : TileRule{8, 24, 2, 1024, 1, 1024};
 }
 
 // `heavy` (optional): the long-row plan of an SpMM; its scratch precedes the carries of this launch. pad (RAGGED): the
 // first `pad` rows of B are copied into scratch as whole pieces and gathered from there. cleared: out_row is given and C
-// holds zeros.
+// holds zeros. fibers: segments are fibers of a tensor.
 template <class T, int LPN, int CPL, int VEC, bool RAGGED = false>
-static comet_status_t launch_one(Context *ctx, SegGatherArgs a, HeavyArgs *heavy, bool cleared, int64_t pad, cudaStream_t stream, int32_t at_least = 0) {
+static comet_status_t launch_one(Context *ctx, SegGatherArgs a, HeavyArgs *heavy, bool cleared, bool fibers, int64_t pad, cudaStream_t stream, int32_t at_least = 0) {
   constexpr int WORKERS = kBlockThreads / LPN;
   const int64_t total = a.M + a.N;
   a.carry_ld = (int32_t)align_up((size_t)a.R, 2);
   constexpr int kCtas = resident_ctas(CPL * VEC * sizeof(T) <= 16 ? COMET_MINB_GATHER : 2, RingLayout<Lanes<T, LPN, CPL, VEC, RAGGED>, false>::kBlockBytes);
   a.tile_items = a.out_row && cleared ? choose_uneven_tile_items(total, WORKERS, 8)
-                           : choose_tile_items(total, WORKERS, kCtas, gather_tile_rule<LPN>());
+                           : choose_tile_items(total, WORKERS, kCtas, gather_tile_rule<LPN>(fibers && a.N >= 12 * a.M));
   if (a.tile_items < at_least) a.tile_items = at_least;
   size_t heavy_bytes = 0;
   HeavyArgs h{};
@@ -723,7 +729,7 @@ static comet_status_t launch_one(Context *ctx, SegGatherArgs a, HeavyArgs *heavy
   const size_t part_bytes = use_part && a.num_tiles >= part_least ? align_up((size_t)(a.num_tiles + 1) * sizeof(int32_t), 256) : 0;
   char *scratch = (char *)scratch_get(ctx, pad_bytes + heavy_bytes + carry_bytes(a.num_tiles, a.carry_ld) + part_bytes, stream);
   // many short tiles have many carries: with no room for them, longer tiles
-  if (!scratch && LPN == 1 && a.tile_items < 512) return launch_one<T, LPN, CPL, VEC, RAGGED>(ctx, a, heavy, cleared, pad, stream, 512);
+  if (!scratch && LPN == 1 && a.tile_items < 512) return launch_one<T, LPN, CPL, VEC, RAGGED>(ctx, a, heavy, cleared, fibers, pad, stream, 512);
   if (!scratch) return COMET_ERR_ALLOC;
   PrepareArgs prep{};
   if (pad_bytes) {
@@ -793,7 +799,7 @@ template <class T>
 static comet_status_t seg_gather_typed(Context *ctx, const int32_t *seg_end, const int32_t *crd, const T *val,
                                        int64_t M, int64_t N, const T *B, int64_t ldb, int64_t R, T *C, int64_t ldc,
                                        const int32_t *out_row, int64_t out_rows, int64_t b_rows, bool long_rows,
-                                       cudaStream_t stream) {
+                                       bool fibers, cudaStream_t stream) {
   constexpr int PER = 16 / sizeof(T);                      // elements per 128-bit piece
   HeavyArgs hint{};                                        // SpMM on [D,CU]: long rows by column phases
   hint.cols = b_rows;
@@ -844,22 +850,22 @@ static comet_status_t seg_gather_typed(Context *ctx, const int32_t *seg_end, con
       const int64_t p = whole ? 0 : b_rows;
       if (pieces > 32) {
         if constexpr (sizeof(T) == 8)                      // fp32 chunks are at most 32 pieces
-          st = exact ? launch_one<T, 32, 2, PER>(ctx, a, heavy, cleared, 0, stream) : launch_one<T, 32, 2, PER, true>(ctx, a, heavy, cleared, p, stream);
-      } else if (exact && pieces == 32) st = launch_one<T, 32, 1, PER>(ctx, a, heavy, cleared, 0, stream);
-      else if (exact && pieces == 16) st = launch_one<T, 16, 1, PER>(ctx, a, heavy, cleared, 0, stream);
-      else if (exact && pieces == 8) st = launch_one<T, 8, 1, PER>(ctx, a, heavy, cleared, 0, stream);
-      else if (exact && pieces == 4) st = launch_one<T, 4, 1, PER>(ctx, a, heavy, cleared, 0, stream);
-      else if (exact && pieces == 2) st = launch_one<T, 2, 1, PER>(ctx, a, heavy, cleared, 0, stream);
-      else if (exact && pieces == 1) st = launch_one<T, 1, 1, PER>(ctx, a, heavy, cleared, 0, stream);
-      else if (pieces > 16) st = launch_one<T, 32, 1, PER, true>(ctx, a, heavy, cleared, p, stream);
-      else if (pieces > 8) st = launch_one<T, 16, 1, PER, true>(ctx, a, heavy, cleared, p, stream);
-      else if (pieces > 4) st = launch_one<T, 8, 1, PER, true>(ctx, a, heavy, cleared, p, stream);
-      else if (pieces > 2) st = launch_one<T, 4, 1, PER, true>(ctx, a, heavy, cleared, p, stream);
-      else st = launch_one<T, 2, 1, PER, true>(ctx, a, heavy, cleared, p, stream);
+          st = exact ? launch_one<T, 32, 2, PER>(ctx, a, heavy, cleared, fibers, 0, stream) : launch_one<T, 32, 2, PER, true>(ctx, a, heavy, cleared, fibers, p, stream);
+      } else if (exact && pieces == 32) st = launch_one<T, 32, 1, PER>(ctx, a, heavy, cleared, fibers, 0, stream);
+      else if (exact && pieces == 16) st = launch_one<T, 16, 1, PER>(ctx, a, heavy, cleared, fibers, 0, stream);
+      else if (exact && pieces == 8) st = launch_one<T, 8, 1, PER>(ctx, a, heavy, cleared, fibers, 0, stream);
+      else if (exact && pieces == 4) st = launch_one<T, 4, 1, PER>(ctx, a, heavy, cleared, fibers, 0, stream);
+      else if (exact && pieces == 2) st = launch_one<T, 2, 1, PER>(ctx, a, heavy, cleared, fibers, 0, stream);
+      else if (exact && pieces == 1) st = launch_one<T, 1, 1, PER>(ctx, a, heavy, cleared, fibers, 0, stream);
+      else if (pieces > 16) st = launch_one<T, 32, 1, PER, true>(ctx, a, heavy, cleared, fibers, p, stream);
+      else if (pieces > 8) st = launch_one<T, 16, 1, PER, true>(ctx, a, heavy, cleared, fibers, p, stream);
+      else if (pieces > 4) st = launch_one<T, 8, 1, PER, true>(ctx, a, heavy, cleared, fibers, p, stream);
+      else if (pieces > 2) st = launch_one<T, 4, 1, PER, true>(ctx, a, heavy, cleared, fibers, p, stream);
+      else st = launch_one<T, 2, 1, PER, true>(ctx, a, heavy, cleared, fibers, p, stream);
     } else {
-      if (a.R > 64) st = launch_one<T, 32, 4, 1>(ctx, a, heavy, cleared, 0, stream);
-      else if (a.R > 32) st = launch_one<T, 32, 2, 1>(ctx, a, heavy, cleared, 0, stream);
-      else st = launch_one<T, 32, 1, 1>(ctx, a, heavy, cleared, 0, stream);
+      if (a.R > 64) st = launch_one<T, 32, 4, 1>(ctx, a, heavy, cleared, fibers, 0, stream);
+      else if (a.R > 32) st = launch_one<T, 32, 2, 1>(ctx, a, heavy, cleared, fibers, 0, stream);
+      else st = launch_one<T, 32, 1, 1>(ctx, a, heavy, cleared, fibers, 0, stream);
     }
     if (st == COMET_ERR_ALLOC && pieces_ok && !whole) {       // no room for a padded copy: the shapes that need none
       pad = false;
@@ -873,15 +879,15 @@ static comet_status_t seg_gather_typed(Context *ctx, const int32_t *seg_end, con
 
 comet_status_t seg_gather(Context *ctx, int dtype, const int32_t *seg_end, const int32_t *crd, const void *val,
                           int64_t M, int64_t N, const void *B, int64_t ldb, int64_t R, void *C, int64_t ldc,
-                          const int32_t *out_row, int64_t out_rows, int64_t b_rows, bool long_rows, cudaStream_t stream) {
+                          const int32_t *out_row, int64_t out_rows, int64_t b_rows, bool long_rows, bool fibers, cudaStream_t stream) {
   if (ldb >= (1ll << 28)) return COMET_ERR_INDEX_OVERFLOW;      // row offsets are formed as int32 bytes * int32 index
   if (M == 0) return out_row ? zero_rows(ctx, C, dtype, out_rows, R, ldc, stream) : COMET_OK;
   if (out_row && M == out_rows) out_row = nullptr;         // every row is stored: segment s is row s
   if (dtype == COMET_F32)
     return seg_gather_typed<float>(ctx, seg_end, crd, (const float *)val, M, N, (const float *)B, ldb, R, (float *)C, ldc,
-                                   out_row, out_rows, b_rows, long_rows, stream);
+                                   out_row, out_rows, b_rows, long_rows, fibers, stream);
   return seg_gather_typed<double>(ctx, seg_end, crd, (const double *)val, M, N, (const double *)B, ldb, R, (double *)C,
-                                  ldc, out_row, out_rows, b_rows, long_rows, stream);
+                                  ldc, out_row, out_rows, b_rows, long_rows, fibers, stream);
 }
 
 }  // namespace comet

@@ -441,9 +441,12 @@ static bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 
 
 // 512 entries are added in a row at most. Workers of one lane have rings and marks that leave two CTAs to an SM (COO), or one
 // (CSF), and four times as many tiles as a wave has workers all the same: a CTA is short of warps then, and its tiles are short.
+// `mixed`: an output mode at level 1 whose fibers are long on average; tiles of short ones make an atomic row add per entry or two (as
+// gather_tile_rule; 9 M entries in slices of different sizes, fp64, R = 4 172 us with four tiles per worker, 223 in one wave, 181 here).
 // COO pays more per tile (slices are found entry by entry): two CTAs per SM up to twice the size, one where two is all.
 template <bool CSF, int LPN, int CTAS>
-constexpr TileRule mttkrp_tile_rule() {
+constexpr TileRule mttkrp_tile_rule(bool mixed) {
+  if (CSF && mixed && LPN > 1) return TileRule{32, 24, 2, 192, 3, 512};
   if (CSF) return LPN == 1 ? TileRule{32, 0, 1, 0, 4, 512} : TileRule{32, LPN == 16 ? 36 : 24, 2, 512, 1, 512};
   if (LPN == 1) return TileRule{8, 12, 1, 32, 2, 512};
   return CTAS == 4 ? TileRule{8, LPN > 2 ? 48 : 24, 2, 512, 1, 512} : TileRule{32, 30, 1, 512, 1, 512};
@@ -458,7 +461,7 @@ static comet_status_t launch_mttkrp(Context *ctx, MttkrpArgs a, int64_t p_pad, i
   constexpr size_t smem = CSF ? RingLayout<L, false>::kBlockBytes + (size_t)WORKERS * kCsfWorkerBytes
                               : RingLayout<L, true>::kBlockBytes;
   constexpr int kCtas = resident_ctas(!CSF ? kCooCtas<T, CPL, VEC, RAGGED> : CPL * VEC * sizeof(T) <= 16 ? COMET_MINB_CSF : 2, smem);
-  a.tile_items = choose_tile_items(total, WORKERS, kCtas, mttkrp_tile_rule<CSF, LPN, kCtas>());
+  a.tile_items = choose_tile_items(total, WORKERS, kCtas, mttkrp_tile_rule<CSF, LPN, kCtas>(CSF && a.level1 && a.N >= 12 * a.F));
   // A COO tile is that many entries: whole chunks, or every tile ends in one that is walked as a loop (100 M entries, tiles of
   // 503 entries 2916 us, of 512 2847).
   if (!CSF && a.tile_items >= 4 * L::kChunk && !getenv("COMET_TILE_ITEMS")) a.tile_items = (int32_t)align_up((size_t)a.tile_items, L::kChunk);

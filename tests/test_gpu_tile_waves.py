@@ -125,3 +125,13 @@ def test_mttkrp_coo_widths(R, workers, ctas, items):
     want, norm = oracle.mttkrp(c, v, dims, 0, F)
     A = upload_packed(oracle.pack(c, v, dims, (0, 1, 2), (CN, S, S)))
     assert_close(comet.mttkrp(A, 0, [None] + [dev(f) for f in F[1:]]), want, norm, what="mttkrp")
+
+
+@pytest.mark.parametrize("items", [192, 193])                 # whole warps; beyond 192 three waves of the row adds of long fibers
+def test_mttkrp_level1(items):
+    total, dims, R = SLOTS * 8 * items, (97, 89, 4003), 64
+    c, v = _tensor(total, dims, 8001, items)
+    F = [synth.random_dense((d, R), 4 + i).numpy() for i, d in enumerate(dims)]
+    want, norm = oracle.mttkrp(c, v, dims, 1, F)
+    A = upload_packed(oracle.pack(c, v, dims, (0, 1, 2), (CU, CU, CU)))
+    assert_close(comet.mttkrp(A, 1, [dev(f) for f in F]), want, norm, what="mttkrp")

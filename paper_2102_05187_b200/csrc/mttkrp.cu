@@ -463,8 +463,11 @@ static comet_status_t launch_mttkrp(Context *ctx, MttkrpArgs a, int64_t p_pad, i
   constexpr int kCtas = resident_ctas(!CSF ? kCooCtas<T, CPL, VEC, RAGGED> : CPL * VEC * sizeof(T) <= 16 ? COMET_MINB_CSF : 2, smem);
   a.tile_items = choose_tile_items(total, WORKERS, kCtas, mttkrp_tile_rule<CSF, LPN, kCtas>(CSF && a.level1 && a.N >= 12 * a.F));
   // A COO tile is that many entries: whole chunks, or every tile ends in one that is walked as a loop (100 M entries, tiles of
-  // 503 entries 2916 us, of 512 2847).
-  if (!CSF && a.tile_items >= 4 * L::kChunk && !getenv("COMET_TILE_ITEMS")) a.tile_items = (int32_t)align_up((size_t)a.tile_items, L::kChunk);
+  // 503 entries 2916 us, of 512 2847). With few waves the longer tiles leave the last one partly empty, which costs more
+  // (2 to 6 M entries, R = 8 to 64, one or two waves up to 9 %), but for workers of one or two lanes, 16 or 32 to a warp, of which some
+  // would walk the loop at any time (9 M entries, fp64, R = 4, tiles of 119 entries 277 us, of 120 221).
+  const bool many_waves = total >= (int64_t)8 * kSmCount * kCtas * WORKERS * a.tile_items;
+  if (!CSF && (many_waves || LPN <= 2) && a.tile_items >= 4 * L::kChunk && !getenv("COMET_TILE_ITEMS")) a.tile_items = (int32_t)align_up((size_t)a.tile_items, L::kChunk);
   if (CSF && a.tile_items > kCsfTileCap) a.tile_items = kCsfTileCap;          // one mask bit per leaf entry of a tile
   a.num_tiles = ceil_div(total, a.tile_items);
   a.carry_ld = (int32_t)align_up((size_t)a.R, 2);

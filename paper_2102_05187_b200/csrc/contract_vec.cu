@@ -572,13 +572,15 @@ int32_t choose_tile_items(int64_t total_items, int workers_per_block, int ctas_p
 // cleared C are written far apart. Four tiles per resident worker, or eight, so that the last ones do not leave the
 // chip idle. DCSR, 94 % of the rows empty, R = 8, 2 / 4 / 6 / 8 tiles 1037 / 960 / 928 / 919 us; 5.6 M entries in power-law rows,
 // R = 32, one / two / four / eight 478 / 456 / 454 / 422 us; 4.2 M rows in a cleared C, R = 8, one wave 788, eight tiles 762.
-static int32_t choose_uneven_tile_items(int64_t total_items, int workers_per_block, int per_worker) {
+// Not that many where the tiles would be below `low` items, while half of the workers have one: beside long rows 160 (1.4 M entries in
+// equal rows, fp32, R = 64 95 us with at least 32, 80 with 160; power-law rows, fp64, R = 128 184 and 180), in a cleared C 32.
+static int32_t choose_uneven_tile_items(int64_t total_items, int workers_per_block, int per_worker, int32_t low) {
   if (const int32_t forced = forced_tile_items()) return forced;
   const int64_t slots = (int64_t)kSmCount * 4 * workers_per_block;
   int64_t t = ceil_div(total_items, slots * per_worker);
-  int64_t low = ceil_div(total_items, (int64_t)kSmCount * 2 * workers_per_block);
-  low = low < 8 ? 8 : low < 32 ? low : 32;
-  if (t < low) t = low;
+  const int64_t half = ceil_div(total_items, (int64_t)kSmCount * 2 * workers_per_block);
+  const int64_t least = half < 8 ? 8 : half < low ? half : low;
+  if (t < least) t = least;
   return (int32_t)(t < 512 ? t : 512);
 }
 
@@ -704,13 +706,13 @@ static comet_status_t launch_one(Context *ctx, SegGatherArgs a, HeavyArgs *heavy
   const int64_t total = a.M + a.N;
   a.carry_ld = (int32_t)align_up((size_t)a.R, 2);
   constexpr int kCtas = resident_ctas(CPL * VEC * sizeof(T) <= 16 ? COMET_MINB_GATHER : 2, RingLayout<Lanes<T, LPN, CPL, VEC, RAGGED>, false>::kBlockBytes);
-  a.tile_items = a.out_row && cleared ? choose_uneven_tile_items(total, WORKERS, 8)
+  a.tile_items = a.out_row && cleared ? choose_uneven_tile_items(total, WORKERS, 8, 32)
                            : choose_tile_items(total, WORKERS, kCtas, gather_tile_rule<LPN>(fibers && a.N >= 12 * a.M));
   if (a.tile_items < at_least) a.tile_items = at_least;
   size_t heavy_bytes = 0;
   HeavyArgs h{};
   if (!RAGGED && kHeavyShape<T, LPN, CPL, VEC> && heavy && !a.out_row) {
-    const int32_t tile = choose_uneven_tile_items(total, WORKERS, 4);
+    const int32_t tile = choose_uneven_tile_items(total, WORKERS, 4, 160);
     heavy_bytes = spmm_heavy_plan(sizeof(T) == 4 ? COMET_F32 : COMET_F64, a.M, a.N, heavy->cols, a.B, a.ldb, a.R, a.C, a.ldc, tile, &h);
     if (heavy_bytes) a.tile_items = tile;
   }

@@ -706,8 +706,9 @@ static comet_status_t launch_one(Context *ctx, SegGatherArgs a, HeavyArgs *heavy
   const int64_t total = a.M + a.N;
   a.carry_ld = (int32_t)align_up((size_t)a.R, 2);
   constexpr int kCtas = resident_ctas(CPL * VEC * sizeof(T) <= 16 ? COMET_MINB_GATHER : 2, RingLayout<Lanes<T, LPN, CPL, VEC, RAGGED>, false>::kBlockBytes);
-  a.tile_items = a.out_row && cleared ? choose_uneven_tile_items(total, WORKERS, 8, 32)
-                           : choose_tile_items(total, WORKERS, kCtas, gather_tile_rule<LPN>(fibers && a.N >= 12 * a.M));
+  TileRule rule = gather_tile_rule<LPN>(fibers && a.N >= 12 * a.M);
+  if (a.out_row && !cleared && kCtas == 2) { rule.brief = 96; rule.few = 1; }           // the CTAs that clear rows run beside them
+  a.tile_items = a.out_row && cleared && LPN > 1 ? choose_uneven_tile_items(total, WORKERS, 8, 32) : choose_tile_items(total, WORKERS, kCtas, rule);
   if (a.tile_items < at_least) a.tile_items = at_least;
   size_t heavy_bytes = 0;
   HeavyArgs h{};
@@ -822,10 +823,13 @@ static comet_status_t seg_gather_typed(Context *ctx, const int32_t *seg_end, con
   // A compressed root level whose empty rows are cleared by CTAs of the gather launch (gap_role), which write them once, or
   // C is cleared as a whole in one stream of wide stores first (7.5 TB/s where the others reach 4.5) and the stored rows are written over
   // it: narrow rows, or few stored ones in a large C. Gaps -> stream: 4.2 M entries in 67 M / 8.4 M rows, R = 8 1018 -> 765, 269 ->
-  // 232 us; 1 M in 5 M, fp32, R = 4 92 -> 65; but 1 M in 3 M, R = 64 331 -> 395; 0.32 M in 1.06 M, R = 25 82 -> 97; 0.1 M in 1 M, R = 16
-  // 35 -> 39.
+  // 232 us; 1 M in 5 M, fp32, R = 4 92 -> 65; 0.13 M in 0.76 M, R = 19 57 -> 46; 0.16 M in 1.6 M, fp32, R = 2 29 -> 23; 3.2 M in 7 M, R = 25 606
+  // -> 530; 5.5 M in 7.3 M, fp32, R = 4 294 -> 227; but 1 M in 3 M, R = 64 331 -> 395; 0.32 M in 1.06 M, R = 25 82 -> 97; 42,000 in 282,000,
+  // fp32, R = 32 the stream takes 1.4 times as long.
   const int64_t row_bytes = R * (int64_t)sizeof(T), c_bytes = out_rows * row_bytes;
-  const bool cleared = out_row && ((out_rows >= 2 * M && row_bytes <= 64 && c_bytes >= 20000000) || (out_rows >= 6 * M && c_bytes >= 200000000));
+  const bool cleared = out_row && (out_rows >= 6 * M ? c_bytes >= (row_bytes <= 64 ? 10000000 : 100000000)
+                                   : out_rows >= 2 * M ? (row_bytes <= 64 && c_bytes >= 20000000) || (row_bytes <= 256 && c_bytes >= 1000000000)
+                                                       : 2 * out_rows >= 3 * M && row_bytes <= 16 && c_bytes >= 50000000);
   if (cleared) {
     const comet_status_t zs = zero_rows(ctx, C, sizeof(T) == 4 ? COMET_F32 : COMET_F64, out_rows, R, ldc, stream);
     if (zs != COMET_OK) return zs;

@@ -65,3 +65,19 @@ def test_cleared_c(cuda_device):
     C = torch.full((rows, R), float("nan"), dtype=torch.float64, device="cuda")
     comet.spmm(A, dev(B), C)
     assert_close(C, want, norm, what="cleared")
+
+
+@pytest.mark.parametrize("rows,stored,R", [(700_001, 90_000, 2), (700_001, 100_000, 19), (3_200_003, 2_100_000, 2)])
+def test_cleared_where_gaps_are_many_and_rows_narrow(rows, stored, R, cuda_device):
+    """The rules by which C is cleared first: narrow rows of which few are stored, few stored rows in a large C, 16-byte rows."""
+    cols = 400
+    rng = np.random.default_rng(rows)
+    i = np.sort(rng.choice(rows, stored, replace=False)).astype(np.int32)
+    j = rng.integers(0, cols, stored).astype(np.int32)
+    val = rng.uniform(-1, 1, stored)
+    B = synth.random_dense((cols, R), 5).numpy()
+    want, norm = oracle.spmm([i, j], val, (rows, cols), B)
+    A = upload_packed(oracle.pack([i, j], val, (rows, cols), (0, 1), (CU, CU)))
+    C = torch.full((rows, R), float("nan"), dtype=torch.float64, device="cuda")
+    comet.spmm(A, dev(B), C)
+    assert_close(C, want, norm, what="cleared")

@@ -152,3 +152,19 @@ def test_input_whose_samples_mislead(attr):
     before = handle.kernel_launches()
     _check([(key // 1000).astype(np.int32), (key % 1000).astype(np.int32)], rng.uniform(-1, 1, n), (900, 1000), (0, 1), attr)
     assert handle.kernel_launches() - before > 12, "the radix sort was expected to follow"
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.float64])
+def test_many_coarse_buckets(dtype, monkeypatch):
+    """512 coarse buckets: the first split writes its runs record by record, not as bulk copies. Cells: multiples of an odd number
+    modulo 2^36, which are distinct and in no order."""
+    monkeypatch.delenv("COMET_PACK_SMALL")
+    monkeypatch.delenv("COMET_PACK_SPLIT")
+    n, rows = 46_300_007, 1 << 18
+    key = torch.arange(n, dtype=torch.int64, device="cuda") * (0x9E3779B97F4A7C15 - (1 << 64)) & ((1 << 36) - 1)
+    val = (torch.arange(n, dtype=torch.int64, device="cuda") % 16_777_213).to(dtype)
+    A = comet.pack([(key >> 18).to(torch.int32), (key & (rows - 1)).to(torch.int32)], val, (rows, rows), (0, 1), (D, CU))
+    key, order = torch.sort(key)
+    assert torch.equal(A.crd(1), (key & (rows - 1)).to(torch.int32))
+    assert torch.equal(A.pos(1)[1:], torch.cumsum(torch.bincount(key >> 18, minlength=rows), 0).to(torch.int32)) and int(A.pos(1)[0]) == 0
+    assert torch.equal(A.val, val[order])

@@ -100,6 +100,20 @@ def test_spmm_ragged(R, dtype, workers, items, off):
     assert_close(comet.spmm(A, dev(B, t)), want, norm, tol=1e-12 if dtype == "f64" else 3 * 2.0 ** -24, what="spmm")
 
 
+@pytest.mark.parametrize("off", [0, 1])                       # one full wave of the longest tiles; two waves of half as long ones
+def test_spmm_second_wave(off):
+    rows, R = 2003, 128
+    n = 148 * 2 * 8 * 1024 + off - rows                       # 32 lanes with two pieces: two CTAs of eight workers to an SM
+    rng = np.random.default_rng(off)
+    cols = 1 + 2 * n // rows
+    cells = np.sort(rng.choice(rows * cols, n, replace=False))
+    c = [(cells // cols).astype(np.int32), (cells % cols).astype(np.int32)]
+    val, B = rng.uniform(-1, 1, n), synth.random_dense((cols, R), 5).numpy()
+    want, norm = oracle.spmm(c, val, (rows, cols), B)
+    A = upload_packed(oracle.pack(c, val, (rows, cols), (0, 1), (D, CU)))
+    assert_close(comet.spmm(A, dev(B)), want, norm, what="spmm")
+
+
 # Lanes a worker: one (a CTA to an SM, four waves), two (three CTAs to an SM), 16, and 32 with two pieces.
 @pytest.mark.parametrize("R,workers,ctas,items", [(2, 256, 4, 31), (2, 256, 4, 33), (4, 128, 3, 23), (4, 128, 3, 33), (32, 16, 4, 35),
                                                   (32, 16, 4, 36), (32, 16, 4, 64), (64, 8, 4, 23), (64, 8, 4, 24), (128, 8, 2, 33), (128, 8, 2, 49)])
@@ -135,3 +149,15 @@ def test_mttkrp_level1(items):
     want, norm = oracle.mttkrp(c, v, dims, 1, F)
     A = upload_packed(oracle.pack(c, v, dims, (0, 1, 2), (CU, CU, CU)))
     assert_close(comet.mttkrp(A, 1, [dev(f) for f in F]), want, norm, what="mttkrp")
+
+
+@pytest.mark.parametrize("form", ["coo", "csf"])
+@pytest.mark.parametrize("off", [0, 1])
+def test_mttkrp_second_wave(form, off):
+    dims, R = (97, 89, 4003), 64                              # whole warps, four CTAs to an SM, tiles of at most 512
+    total, fibers = SLOTS * 8 * 512 + off, 8001
+    c, v = _tensor(total if form == "csf" else total + fibers, dims, fibers, off)
+    F = [None] + [synth.random_dense((d, R), 4 + i).numpy() for i, d in enumerate(dims[1:])]
+    want, norm = oracle.mttkrp(c, v, dims, 0, F)
+    A = upload_packed(oracle.pack(c, v, dims, (0, 1, 2), (CU, CU, CU) if form == "csf" else (CN, S, S)))
+    assert_close(comet.mttkrp(A, 0, [None] + [dev(f) for f in F[1:]]), want, norm, what="mttkrp")

@@ -109,8 +109,8 @@ struct SegGatherPolicy {
 
   __device__ __forceinline__ void flush() {      // stores the open segment
     T *cmat = static_cast<T *>(a.C) + ln.col0;
-    // (asking for the row, or the next end, when the segment opens takes the registers that the window needs: 65 -> 76 us on
-    // 2 M entries, R = 16; TTM 345 -> 399)
+    // (asking for the row, or the next end, when the segment opens takes the registers that the window needs: this kernel
+    // alone 65 -> 76 us on 2 M entries, R = 16; TTM of 30 M 345 -> 399)
     const int64_t row = ROWS == kRowsMapped ? (int64_t)__ldg(a.out_row + seg) : (int64_t)seg;
     ln.store_row(cmat + row * a.ldc, acc);
     ln.zero(acc);
@@ -132,7 +132,7 @@ struct SegGatherPolicy {
 constexpr int kGapRows = 1024;         // 256 / 512 / 1,024 / 2,048 rows: 6.6 M entries in 2.1 M of 2.2 M rows, fp32, R = 31 393 / 375 / 355 / 434 us
 template <class T>
 __device__ __forceinline__ void gap_role(const SegGatherArgs &a, int64_t block, unsigned char *smem) {
-  static_assert(kGapRows % kBlockThreads == 0 && kGapRows / 32 <= kBlockThreads, "");
+  static_assert(kGapRows % kBlockThreads == 0 && kGapRows / 32 < kBlockThreads, "");
   uint32_t *const bits = reinterpret_cast<uint32_t *>(smem), *const empties = bits + kGapRows / 32;
   uint16_t *const empty = reinterpret_cast<uint16_t *>(empties + 1);        // the empty rows, in any order
   const int64_t r0 = block * kGapRows;
@@ -590,6 +590,7 @@ static comet_status_t launch_mapped(Context *ctx, const SegGatherArgs &a, const 
   using L = Lanes<T, LPN, CPL, VEC, RAGGED>;
   constexpr size_t ring = RingLayout<L, false>::kBlockBytes, async_ring = HEAVY ? AsyncRing<L>::kBlockBytes : 0;
   constexpr size_t smem = ring > async_ring ? ring : async_ring;
+  static_assert(ROWS != kRowsMapped || smem >= kGapRows / 8 + 4 + kGapRows * 2, "gap_role: marks, their number, the empty rows");
   auto kernel = seg_gather_kernel<T, LPN, CPL, VEC, RAGGED, ROWS, HEAVY>;
   if (smem > 48 * 1024)
     COMET_CUDA_TRY(ctx, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));

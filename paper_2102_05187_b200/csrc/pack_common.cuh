@@ -1,4 +1,4 @@
-// What the two packing paths share (pack.cu: any size; pack_small.cu: one launch for small inputs).
+// What the packing paths share (pack.cu: any size; pack_small.cu: one launch for small inputs; pack_split.cu: larger ones).
 #pragma once
 
 #include "common.cuh"

@@ -3,23 +3,26 @@
 // The keys of a packing are distinct (equal ones are an error), so nothing has to be stable and an entry moves three
 // times whatever the number of key bits, where the radix sort of pack.cu moves it once per 8 bits and gathers 64-bit
 // values at the end. Splitters are sampled, not digits, so that power-law modes make no large pieces:
-//   1. one CTA sorts a sample of the keys, 32 per coarse bucket (32 to 512 buckets);
+//   1. a sample of the keys, 32 per coarse bucket (32 to 512 buckets), is put in order;
 //   2. every tile of 4,096 entries forms its keys, finds each one's bucket in a search tree of the splitters, counts,
 //      takes room in every bucket with one atomic add, and writes its runs as records of key and value (16 bytes);
 //   3. a CTA per coarse bucket samples and sorts again: splitters of fine buckets of about 1,400 entries;
 //   4. the same split inside every coarse bucket, into regions of 3,584 records per fine bucket;
 //   5. a CTA per fine bucket: the 32 samples of the bucket and linear interpolation between them give each entry one
-//      of 512 cells of about three entries in key order, and a count of the smaller keys of its cell gives its place.
+//      of 2,048 cells in key order (64 between two samples, less than one entry each on average), and a count of the
+//      smaller keys of its cell gives its place.
 // Formats whose levels all have an entry per node (CSR, sorted coordinates) are written by step 5 itself; the others
 // get sorted keys and values, for the level kernels of pack.cu.
 //
-// A bucket that its region cannot hold (2.5 times the expected size: about one packing in ten thousand, or an input
-// with very many equal coordinates) raises a flag, nothing is written beyond a region, and pack.cu sorts again.
-// No CTA waits for another.
+// A bucket that its region cannot hold (2.5 times the expected size) raises a flag, nothing is written beyond a region, and
+// pack.cu sorts again. How often, from the distribution of the samples' spacings (Beta) summed over the buckets: at most
+// one packing of distinct keys in 50,000 up to 40 M entries, 2 in 10,000 up to 90 M, 1 in 1,000 at 100 M and 9 in 1,000 at the
+// limit of 114.7 M, where a coarse bucket has up to 256 fine ones and still 4,096 samples. Which entries are sampled depends on their
+// number alone, so that an input whose order misleads the samples does so on every call. No CTA waits for another.
 //
 // The splits are bound by the steps that their barriers keep apart (search 40 us, counting 15 to 25, copies out 20 to 40,
-// reading and ordering the records 80, of 160; load/store pipe 50 to 85 %), the last step by the load/store pipe (74 %) and
-// instruction issue (55 %). Measured against the radix sort, whole comet_pack calls: 19.8 M entries to CSR, fp64 1431 ->
+// reading and ordering the records 80, of 160; L1 59 %, issue 42 to 52 %, most stalls at barriers), the last step by the same, the
+// load/store pipe (71 %) and instruction issue (53 %). Measured against the radix sort, whole comet_pack calls: 19.8 M entries to CSR, fp64 1431 ->
 // 726 us, fp32 1215 -> 712; 100 M to sorted coordinates 9157 -> 4020; 50 M to CSF 3957 -> 2360; 3 M to CSF 423 -> 250.
 // Tiles of 2,048 records, three to five CTAs per SM and a CTA per tile all gave 160 to 190 us for a split.
 #include "common.cuh"
@@ -85,7 +88,8 @@ static SplitShape split_shape(int64_t n, int total_bits) {
   return s;
 }
 
-__device__ __forceinline__ uint32_t sample_hash(uint32_t x) {       // spreads sample numbers over 32 bits
+// Spreads sample numbers over 32 bits: lowbias32 of C. Wellons' "Hash Prospector", shifts and multipliers as published.
+__device__ __forceinline__ uint32_t sample_hash(uint32_t x) {
   x ^= x >> 16; x *= 0x7feb352du;
   x ^= x >> 15; x *= 0x846ca68bu;
   return x ^ (x >> 16);

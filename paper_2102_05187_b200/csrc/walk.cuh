@@ -212,12 +212,6 @@ template <class T_, int LPN_, int CPL_, int VEC_, bool RAGGED_ = false> struct L
         for (int e = 0; e < VEC; ++e)
           if (!RAGGED || col0 + t * kStride + e < R) row[t * kStride + e] = acc[t][e];
   }
-  // rows lo .. hi-1 of a matrix whose lane-piece-0 pointer of row 0 is `base`
-  __device__ __forceinline__ void zero_rows(T *base, int64_t ld, int64_t lo, int64_t hi) const {
-    double z[CPL][VEC];
-    zero(z);
-    for (int64_t r = lo; r < hi; ++r) store_row(base + r * ld, z);
-  }
   __device__ __forceinline__ void fma_rows(double v, const T (&row)[CPL][VEC], double (&acc)[CPL][VEC]) const {
 #pragma unroll
     for (int t = 0; t < CPL; ++t)
@@ -425,8 +419,9 @@ __device__ __forceinline__ void walk_tile(const L &ln, Policy &p, int32_t j0, in
 // window of rows in flight can be twice as deep at the same occupancy. The ring has four chunks: the one being walked, the
 // one the window looks ahead into, and two on their way. Policy interface: as above with fetch_async(j, entry address,
 // there) instead of fetch, and settle(entry address), which a lane calls for the entries it copied once they have arrived.
-// For the gathers that go to DRAM (SpMM beside its long rows: 1103 -> 1040 us); where the rows come from L2 the copies
-// cost more than the deeper window gives (TTM of 30 M entries, R = 16 353 -> 385 us with four rows in flight, 413 with eight).
+// For the gathers that go to DRAM (SpMM beside its long rows, whole calls of 19.8 M entries, R = 64 1114 -> 1055 us); where the rows
+// come from L2 the copies cost more than the deeper window gives (TTM of 30 M entries, R = 16, this kernel alone 353 -> 385 us with
+// four rows in flight, 413 with eight).
 constexpr int kAsyncChunk = 8, kRingChunks = 4;
 __device__ __forceinline__ void copy_async8(uint32_t dst, const void *src, bool there) {      // zeros where nothing is
   asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(dst), "l"(src), "r"(there ? 8 : 0) : "memory");

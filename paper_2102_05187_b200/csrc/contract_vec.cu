@@ -710,6 +710,8 @@ static comet_status_t launch_one(Context *ctx, SegGatherArgs a, HeavyArgs *heavy
   TileRule rule = gather_tile_rule<LPN>(fibers && a.N >= 12 * a.M);
   if (a.out_row && !cleared && kCtas == 2) { rule.brief = 96; rule.few = 1; }           // the CTAs that clear rows run beside them
   a.tile_items = a.out_row && cleared && LPN > 1 ? choose_uneven_tile_items(total, WORKERS, 8, 32) : choose_tile_items(total, WORKERS, kCtas, rule);
+  // a bound on the carries, which the handle's scratch keeps (up to 40 bytes per tile): four million short tiles
+  if (LPN == 1 && at_least < total >> 22) at_least = (int32_t)(total >> 22);
   if (a.tile_items < at_least) a.tile_items = at_least;
   size_t heavy_bytes = 0;
   HeavyArgs h{};
